@@ -645,8 +645,11 @@ static cldiam_status radix_sort_impl(K* keys, uint32_t* vals, K* keys_alt, uint3
 // Two passes over sorted (key, value) pairs: the first counts each tile's run
 // heads (ballots), an exclusive scan turns the counts into each tile's first
 // output index, and the second gives the heads consecutive indices r and
-// writes them; for each run the minimum value is folded in with one store per
-// run inside a warp, or one atomicMin per run piece per warp otherwise.
+// writes them; each run's minimum is reduced over the lanes of a warp first, so
+// it costs one store per run inside a warp, or one atomicMin per warp it spans.
+// (With one atomicMin per item, runs of millions of equal keys -- the cluster
+// pairs of a power-law graph's quotient -- queue at one address: 522M items in
+// 16.9M runs took 202 ms on R-MAT 24; UQNEW ms with the reduction.)
 // Output per unique key: row_out[r] = key / div (if row_out), col_out[r*cs] =
 // key % div, w_out[r*cs] = min value (w_out pre-filled with 0xFFFFFFFF).
 // Keys >= sentinel are ignored (they sort last).
@@ -735,47 +738,67 @@ __global__ void __launch_bounds__(UQ_THREADS, 4)
     }
     __syncthreads();
     const uint32_t tbase = s_prefix + s_woff[w];
-    // Run minima: a head stores its run's key and its own value, then (after a block barrier, so the
-    // stores come first) every other item of a run folds its value in with atomicMin.  The one run
-    // that may continue into the next tile has its head fold in with atomicMin too (w_out holds
-    // 0xFFFFFFFF beforehand), as do items whose run began in an earlier tile.
-    const size_t tend = min(cnt, (size_t)(tile + 1) * UQ_TILE);
-    const K lastkey = keys[tend - 1];
-    const bool crosses = tend < cnt && keys[tend] == lastkey && lastkey < sentinel;
+    // Run minima.  A warp holds 256 consecutive items, so a run's piece in it is reduced over the lanes (and
+    // carried from one group of 32 to the next) before anything is written: a run that begins and ends in
+    // the warp is one plain store, a run shared with other warps one atomicMin per warp (w_out holds
+    // 0xFFFFFFFF beforehand).
     const auto row_of = [&](K kk) -> uint64_t { return (uint64_t)kk / div; };
+    const K wnext = base + UQ_ITEMS * 32 < cnt ? keys[base + UQ_ITEMS * 32] : sentinel;  // item after the warp's
+    const K wlast = __shfl_sync(0xffffffffu, key[UQ_ITEMS - 1], 31);
+    const bool goes_on = wnext < sentinel && wnext == wlast;  // the warp's last run continues in the next warp
+    uint32_t carry = 0xFFFFFFFFu;  // minimum of the run open at the previous group's end
+    bool carry_head = false;       // its head is in this warp
 #pragma unroll
     for (int i = 0; i < UQ_ITEMS; ++i) {
         const size_t idx = base + (size_t)i * 32 + l;
         const bool valid = key[i] < sentinel;
+        const bool f = (head_bits >> i) & 1u;
         K before = __shfl_up_sync(0xffffffffu, key[i], 1);
-        if (l == 0) before = idx > 0 ? keys[idx - 1] : sentinel;
-        const uint32_t f = (head_bits >> i) & 1u;
-        if (!valid || !f) continue;
-        const uint32_t r = tbase + ex[i];
-        if (crosses && key[i] == lastkey) atomicMin(&w_out[(size_t)r * cs], val[i]);
-        else w_out[(size_t)r * cs] = val[i];
-        const uint64_t q = row_of(key[i]);
-        if (row_out) row_out[r] = (uint32_t)q;
-        col_out[(size_t)r * cs] = (uint32_t)((uint64_t)key[i] - q * div);
-        if (off_out) {
-            const uint64_t q0 = idx == 0 ? 0ull : row_of(before) + 1ull;  // rows after the previous run's row
-            for (uint64_t qq = q0; qq <= q && qq <= nrows; ++qq) off_out[qq] = r;
-        }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < UQ_ITEMS; ++i) {
-        const size_t idx = base + (size_t)i * 32 + l;
-        const bool valid = key[i] < sentinel;
         K after = __shfl_down_sync(0xffffffffu, key[i], 1);
-        if (l == 31) after = (idx + 1 < cnt) ? keys[idx + 1] : sentinel;
-        if (!valid) continue;
-        const uint32_t f = (head_bits >> i) & 1u;
-        const uint32_t r = tbase + ex[i] + f - 1u;
-        if (!f) atomicMin(&w_out[(size_t)r * cs], val[i]);
+        if (l == 0) before = idx > 0 && idx <= cnt ? keys[idx - 1] : sentinel;
+        if (l == 31) after = idx + 1 < cnt ? keys[idx + 1] : sentinel;
+        // segment starts: run heads, and every invalid item (they sort last) on its own
+        const unsigned word = __ballot_sync(0xffffffffu, f || !valid);
+        uint32_t v = val[i];
+        if (l == 0 && !(word & 1u)) v = min(v, carry);
+        if (word == 0) {
+            v = __reduce_min_sync(0xffffffffu, v);
+        } else {
+            const unsigned above = l == 31 ? 0u : word & (0xfffffffeu << l);
+            const uint32_t tail = above ? (uint32_t)__ffs(above) - 2u : 31u;  // this lane's segment ends here
+#pragma unroll
+            for (uint32_t o = 1; o < 32; o <<= 1) {
+                const uint32_t t = __shfl_down_sync(0xffffffffu, v, o);
+                if (l + o <= tail) v = min(v, t);
+            }
+        }
+        const uint32_t last = word ? 31u - (uint32_t)__clz(word) : 0u;  // start lane of the group's last segment
+        const unsigned next0 = __shfl_sync(0xffffffffu, (unsigned)(i + 1 < UQ_ITEMS ? head_bits >> (i + 1) : 0u), 0) & 1u;
+        const bool next_valid = i + 1 < UQ_ITEMS && __shfl_sync(0xffffffffu, key[i + 1 < UQ_ITEMS ? i + 1 : i], 0) < sentinel;
+        const bool cont = i + 1 < UQ_ITEMS ? next_valid && !next0 : goes_on;  // the last segment's run goes on
+        const uint32_t vlast = __shfl_sync(0xffffffffu, v, last);
+        const bool start = valid && (f || (l == 0 && !(word & 1u)));
+        if (start && !(i + 1 < UQ_ITEMS && cont && l == last)) {
+            const uint32_t r = tbase + ex[i] + (f ? 0u : 0xFFFFFFFFu);  // a piece without its head: the run before
+            const bool whole = (f || carry_head) && !(i + 1 == UQ_ITEMS && cont && l == last);
+            if (whole) w_out[(size_t)r * cs] = v;
+            else atomicMin(&w_out[(size_t)r * cs], v);
+        }
+        carry_head = cont && (word != 0 || carry_head);
+        carry = cont ? vlast : 0xFFFFFFFFu;
+        if (valid && f) {
+            const uint32_t r = tbase + ex[i];
+            const uint64_t q = row_of(key[i]);
+            if (row_out) row_out[r] = (uint32_t)q;
+            col_out[(size_t)r * cs] = (uint32_t)((uint64_t)key[i] - q * div);
+            if (off_out) {
+                const uint64_t q0 = idx == 0 ? 0ull : row_of(before) + 1ull;  // rows after the previous run's row
+                for (uint64_t qq = q0; qq <= q && qq <= nrows; ++qq) off_out[qq] = r;
+            }
+        }
         // the last run: the remaining rows end at the total
-        if (off_out && !(after < sentinel))
-            for (uint64_t qq = row_of(key[i]) + 1; qq <= nrows; ++qq) off_out[qq] = (uint64_t)r + 1;
+        if (off_out && valid && !(after < sentinel))
+            for (uint64_t qq = row_of(key[i]) + 1; qq <= nrows; ++qq) off_out[qq] = (uint64_t)(tbase + ex[i] + (f ? 1u : 0u));
     }
 }
 
