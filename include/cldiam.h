@@ -94,7 +94,7 @@ typedef struct {
                                         D_u (while D_u < Delta); D_v = d_v <= final Delta         */
 
 /* cldiam_opts.quotient_mode (same result either way) */
-#define CLDIAM_QUOTIENT_AUTO 0  /* dense while k <= 4096, else radix sort (default) */
+#define CLDIAM_QUOTIENT_AUTO 0  /* dense while k <= 4096 or k^2 <= nnz, else radix sort (default) */
 #define CLDIAM_QUOTIENT_SORT 1  /* radix sort of (cid_u, cid_v) keys + segmented min */
 #define CLDIAM_QUOTIENT_DENSE 2 /* atomicMin into a k x k matrix (k <= 65535)        */
 
@@ -370,7 +370,8 @@ typedef struct {
                                       of all adjacency entries; < 0 = never; 0 = 0.3                */
     uint32_t relax_ctas_per_sm;    /* CTAs per SM of the growing-step kernels; 0 = all that fit     */
     uint32_t dense_quotient_k;     /* CLDIAM_QUOTIENT_AUTO: dense k x k de-duplication up to this k
-                                      (<= 65535), radix sort above; 0 = 4096                       */
+                                      (<= 65535), above it (if >= 4096) while k^2 <= nnz, then by
+                                      radix sort; 0 = 4096                                          */
     uint32_t apsp_sources_per_cta; /* quotient diameter by batched SSSP: sources per CTA, 1, 4 or 8;
                                       0 = by k (8 below 2,048 nodes, else 4)                       */
     uint32_t apsp_fw_density;      /* quotient diameter by Floyd-Warshall when nnz >= k^2 / this,

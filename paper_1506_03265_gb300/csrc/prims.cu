@@ -648,8 +648,8 @@ static cldiam_status radix_sort_impl(K* keys, uint32_t* vals, K* keys_alt, uint3
 // writes them; each run's minimum is reduced over the lanes of a warp first, so
 // it costs one store per run inside a warp, or one atomicMin per warp it spans.
 // (With one atomicMin per item, runs of millions of equal keys -- the cluster
-// pairs of a power-law graph's quotient -- queue at one address: 522M items in
-// 16.9M runs took 202 ms on R-MAT 24; UQNEW ms with the reduction.)
+// pairs of a power-law graph's quotient -- queue at one address: the 521M items
+// of R-MAT 24 took 202 ms; the whole quotient by sort went from 225 to 20-24 ms.)
 // Output per unique key: row_out[r] = key / div (if row_out), col_out[r*cs] =
 // key % div, w_out[r*cs] = min value (w_out pre-filled with 0xFFFFFFFF).
 // Keys >= sentinel are ignored (they sort last).

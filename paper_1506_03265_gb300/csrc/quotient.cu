@@ -6,9 +6,9 @@
 // sort on the 2 log2 k significant key bits groups equal pairs, whose run
 // heads become the quotient entries and an atomicMin over each run keeps the
 // minimum.  Because the CSR is symmetric the result is symmetric, sorted by
-// (row, col).  While k is small enough for a dense k x k matrix to stay in
-// L2, the pairs are instead folded into that matrix with atomicMin and read
-// out row by row, which gives the same sorted CSR.
+// (row, col).  While a dense k x k matrix is small (k <= 4,096, or k^2 <= nnz),
+// the pairs are instead folded into that matrix with atomicMin and read out
+// row by row, which gives the same sorted CSR.
 #include "cluster_dev.cuh"
 #include "internal.cuh"
 #include "prof.cuh"
@@ -384,9 +384,17 @@ cldiam_status quotient(const cldiam_clustering* c, cldiam_quotient** out) {
     q->c = c;
     q->stream = c->g->stream;
     q->max_fw_k = c->max_fw_k;
-    // dense deduplication while the k x k matrix fits in L2 (auto) or when asked; radix sort otherwise
-    const bool dense = c->quotient_mode == CLDIAM_QUOTIENT_DENSE ||
-                       (c->quotient_mode == CLDIAM_QUOTIENT_AUTO && c->k <= tuning_for(c->g->nnz).dense_quotient_k);
+    // Dense deduplication when asked, up to the tuning knob's k, and above it while k^2 <= nnz (unless the knob was
+    // set below its default, which asks for the sort): the matrix is then at most half of the CSR's bytes and less
+    // than the sort's buffers.  Whole quotient by sort / dense, ms: R-MAT 24 (521M entries) k = 6,158 23.5 / 2.1,
+    // k = 23,065 24.3 / 5.8; R-MAT 22 (128M) k = 7,633 5.5 / 0.81; road mesh 4096^2 (60M) k = 7,473 0.76 / 0.64; with
+    // k^2 = 1.9 nnz the road mesh is faster by sort (k = 10,836 0.76 / 1.01), as is a mesh at 5.5 nnz (k = 4,679
+    // 0.197 / 0.223).
+    bool dense = c->quotient_mode == CLDIAM_QUOTIENT_DENSE;
+    if (c->quotient_mode == CLDIAM_QUOTIENT_AUTO) {
+        const uint32_t cap = tuning_for(c->g->nnz).dense_quotient_k;
+        dense = c->k <= cap || (cap >= 4096u && c->k <= 65535u && (uint64_t)c->k * c->k <= c->g->nnz);
+    }
     if (dense && c->k > 65535u) {
         free_quotient(q);
         return fail(CLDIAM_ERR_UNSUPPORTED, "dense quotient deduplication needs k <= 65535");
