@@ -81,104 +81,156 @@ __global__ void k_fw_scatter(const uint64_t* __restrict__ off, const uint32_t* _
     if (wd && wide) atomicExch(wide, 1u);
 }
 
-// Tiles are T x T = 64 x 64; a CTA of 256 threads gives each thread a 4 x 4
-// block (rows 4*ty.., cols 4*tx..).  Within the pivot tile and the pivot
-// row / column tiles, iteration p reads row p and column p, which iteration p
-// itself cannot change (D[p][p] = 0), so one barrier per p suffices.
+// Tiles are T x T = 64 x 64; 256 threads hold a tile as 4 x 4 registers each (rows 4*ty.., cols 4*tx..).
 constexpr int FT = 64;
 constexpr int FQ = 4;       // 4 x 4 entries per thread
 constexpr int FTH = 256;    // 16 x 16 threads
-constexpr int FP = FT + 1;  // padded shared row
+constexpr int FS = 32;      // columns (row tiles) or rows (column tiles) of a phase 2 strip
+constexpr int FA = FT + 4;  // padded row of a transposed tile, 16-byte aligned
 
-__device__ __forceinline__ void fw_load_tile(uint32_t (*t)[FP], const uint32_t* M, uint32_t kp, uint32_t ti,
-                                             uint32_t tj) {
-    for (int i = threadIdx.x; i < FT * FT; i += FTH) {
-        int y = i / FT, x = i % FT;
-        t[y][x] = M[((size_t)ti * FT + y) * kp + (size_t)tj * FT + x];
+__device__ __forceinline__ void fw_load4x4(uint32_t (&c)[FQ][FQ], const uint32_t* M, uint32_t kp, size_t y, size_t x) {
+#pragma unroll
+    for (int i = 0; i < FQ; ++i) {
+        const uint4 v = *reinterpret_cast<const uint4*>(&M[(y + i) * kp + x]);
+        c[i][0] = v.x; c[i][1] = v.y; c[i][2] = v.z; c[i][3] = v.w;
     }
 }
-__device__ __forceinline__ void fw_store_tile(uint32_t (*t)[FP], uint32_t* M, uint32_t kp, uint32_t ti, uint32_t tj) {
-    for (int i = threadIdx.x; i < FT * FT; i += FTH) {
-        int y = i / FT, x = i % FT;
-        M[((size_t)ti * FT + y) * kp + (size_t)tj * FT + x] = t[y][x];
+__device__ __forceinline__ void fw_store4x4(const uint32_t (&c)[FQ][FQ], uint32_t* M, uint32_t kp, size_t y, size_t x) {
+#pragma unroll
+    for (int i = 0; i < FQ; ++i)
+        *reinterpret_cast<uint4*>(&M[(y + i) * kp + x]) = make_uint4(c[i][0], c[i][1], c[i][2], c[i][3]);
+}
+template <bool FAST>
+__device__ __forceinline__ void fw_relax4x4(uint32_t (&c)[FQ][FQ], const uint4 av, const uint4 bv, bool& ovf) {
+    const uint32_t a[FQ] = {av.x, av.y, av.z, av.w};
+    const uint32_t b[FQ] = {bv.x, bv.y, bv.z, bv.w};
+#pragma unroll
+    for (int i = 0; i < FQ; ++i)
+#pragma unroll
+        for (int j = 0; j < FQ; ++j) c[i][j] = fw_relax<FAST>(c[i][j], a[i], b[j], ovf);
+}
+
+// Phase 1: closes the pivot tile held in registers.  Iteration p needs row p and column p, which it cannot change
+// itself (D[p][p] = 0): their owners publish them in one of two shared buffers, one barrier per p.  A serial chain
+// of 64 barriers on one CTA; with the tile in shared memory (16 read-modify-writes per thread and p) it took 40 us,
+// from registers 7 us.
+struct FwLine {
+    __align__(16) uint32_t row[2][FT], col[2][FT];
+};
+template <bool FAST>
+__device__ __forceinline__ void fw_close(uint32_t (&c)[FQ][FQ], FwLine& s, int ty, int tx, bool& ovf) {
+    for (int p4 = 0; p4 < FT / FQ; ++p4) {
+#pragma unroll
+        for (int j = 0; j < FQ; ++j) {
+            const int b = j & 1;
+            if (ty == p4) *reinterpret_cast<uint4*>(&s.row[b][tx * FQ]) = make_uint4(c[j][0], c[j][1], c[j][2], c[j][3]);
+            if (tx == p4) *reinterpret_cast<uint4*>(&s.col[b][ty * FQ]) = make_uint4(c[0][j], c[1][j], c[2][j], c[3][j]);
+            __syncthreads();
+            fw_relax4x4<FAST>(c, *reinterpret_cast<const uint4*>(&s.col[b][ty * FQ]),
+                              *reinterpret_cast<const uint4*>(&s.row[b][tx * FQ]), ovf);
+        }
     }
 }
 
-// phase 1: the pivot tile against itself
 template <bool FAST>
 __global__ void __launch_bounds__(FTH) k_fw_phase1(uint32_t* __restrict__ M, uint32_t kp, uint32_t r,
                                                    uint32_t* __restrict__ ovf_flag) {
-    __shared__ uint32_t t[FT][FP];
+    __shared__ FwLine line;
     const int ty = threadIdx.x / 16, tx = threadIdx.x % 16;
-    fw_load_tile(t, M, kp, r, r);
-    __syncthreads();
+    const size_t y = (size_t)r * FT + ty * FQ, x = (size_t)r * FT + tx * FQ;
+    uint32_t c[FQ][FQ];
+    fw_load4x4(c, M, kp, y, x);
     bool ovf = false;
-    for (int p = 0; p < FT; ++p) {
-        uint32_t a[FQ], b[FQ];
-#pragma unroll
-        for (int q = 0; q < FQ; ++q) {
-            a[q] = t[ty * FQ + q][p];
-            b[q] = t[p][tx * FQ + q];
-        }
-#pragma unroll
-        for (int i = 0; i < FQ; ++i)
-#pragma unroll
-            for (int j = 0; j < FQ; ++j) {
-                uint32_t& c = t[ty * FQ + i][tx * FQ + j];
-                c = fw_relax<FAST>(c, a[i], b[j], ovf);
-            }
-        __syncthreads();
-    }
-    fw_store_tile(t, M, kp, r, r);
-    if (ovf) atomicExch(ovf_flag, 1u);
+    fw_close<FAST>(c, line, ty, tx, ovf);
+    fw_store4x4(c, M, kp, y, x);
+    if (!FAST && ovf) atomicExch(ovf_flag, 1u);
 }
 
-// phase 2: tiles in pivot row r (blockIdx.y == 0) and pivot column r (blockIdx.y == 1)
-template <bool FAST>
-__global__ void __launch_bounds__(FTH) k_fw_phase2(uint32_t* __restrict__ M, uint32_t kp, uint32_t r,
-                                                   uint32_t* __restrict__ ovf_flag) {
-    __shared__ uint32_t piv[FT][FP];
-    __shared__ uint32_t t[FT][FP];
+// Phase 2, tiles in pivot row r (blockIdx.y == 0) and pivot column r (blockIdx.y == 1).
+// Fast form: the pivot tile is closed, so one min-plus product with the tile as it was gives the same values as 64
+// dependent iterations (any path through the pivot nodes is one closed hop and one old entry), without a barrier
+// per p.  A tile is cut into two strips of 32, one CTA of 128 threads each, since 2 (nt - 1) tiles alone leave half
+// of the SMs idle: 47 us as dependent iterations, 5.2 us so (nt = 32).
+__global__ void __launch_bounds__(FTH / 2) k_fw_phase2_fast(uint32_t* __restrict__ M, uint32_t kp, uint32_t r) {
+    __shared__ __align__(16) uint32_t At[FT][FA];  // left operand, transposed (row strip: the whole pivot tile)
+    __shared__ __align__(16) uint32_t B[FT][FT];
+    const bool is_row = blockIdx.y == 0;
+    uint32_t o = blockIdx.x >> 1;
+    const uint32_t strip = blockIdx.x & 1;
+    if (o >= r) ++o;
+    // output block: 64 rows x 32 columns of a row tile, or 32 rows x 64 columns of a column tile
+    const size_t y0 = (size_t)(is_row ? r : o) * FT + (is_row ? 0 : strip * FS);
+    const size_t x0 = (size_t)(is_row ? o : r) * FT + (is_row ? strip * FS : 0);
+    const int h = is_row ? FT : FS, w = is_row ? FS : FT;
+    for (int i = threadIdx.x; i < h * FT; i += FTH / 2) At[i % FT][i / FT] = M[(y0 + i / FT) * kp + (size_t)r * FT + i % FT];
+    for (int i = threadIdx.x; i < FT * w; i += FTH / 2) B[i / w][i % w] = M[((size_t)r * FT + i / w) * kp + x0 + i % w];
+    const int tx = threadIdx.x % (w / FQ), ty = threadIdx.x / (w / FQ);
+    uint32_t c[FQ][FQ];
+    fw_load4x4(c, M, kp, y0 + ty * FQ, x0 + tx * FQ);
+    __syncthreads();
+    bool ovf = false;
+#pragma unroll 8
+    for (int p = 0; p < FT; ++p)
+        fw_relax4x4<true>(c, *reinterpret_cast<const uint4*>(&At[p][ty * FQ]),
+                          *reinterpret_cast<const uint4*>(&B[p][tx * FQ]), ovf);
+    fw_store4x4(c, M, kp, y0 + ty * FQ, x0 + tx * FQ);
+}
+
+// Checked form: dependent iterations (a product with the old tile would look at larger candidate sums and report
+// OVERFLOW on inputs that these accept), the tile in registers, row or column p published as in phase 1.
+__global__ void __launch_bounds__(FTH) k_fw_phase2_checked(uint32_t* __restrict__ M, uint32_t kp, uint32_t r,
+                                                           uint32_t* __restrict__ ovf_flag) {
+    __shared__ __align__(16) uint32_t piv[FT][FA];  // row tiles: the pivot tile transposed; column tiles: as it is
+    __shared__ __align__(16) uint32_t line[2][FT];
     const int ty = threadIdx.x / 16, tx = threadIdx.x % 16;
     const bool is_row = blockIdx.y == 0;
     uint32_t o = blockIdx.x;
     if (o >= r) ++o;
-    const uint32_t ti = is_row ? r : o, tj = is_row ? o : r;
-    fw_load_tile(piv, M, kp, r, r);
-    fw_load_tile(t, M, kp, ti, tj);
-    __syncthreads();
-    bool ovf = false;
-    for (int p = 0; p < FT; ++p) {
-        uint32_t a[FQ], b[FQ];
-#pragma unroll
-        for (int q = 0; q < FQ; ++q) {
-            // row tile: min(t, piv[y][p] + t[p][x]); column tile: min(t, t[y][p] + piv[p][x])
-            a[q] = is_row ? piv[ty * FQ + q][p] : t[ty * FQ + q][p];
-            b[q] = is_row ? t[p][tx * FQ + q] : piv[p][tx * FQ + q];
-        }
-#pragma unroll
-        for (int i = 0; i < FQ; ++i)
-#pragma unroll
-            for (int j = 0; j < FQ; ++j) {
-                uint32_t& c = t[ty * FQ + i][tx * FQ + j];
-                c = fw_relax<FAST>(c, a[i], b[j], ovf);
-            }
-        __syncthreads();
+    const size_t y = (size_t)(is_row ? r : o) * FT + ty * FQ, x = (size_t)(is_row ? o : r) * FT + tx * FQ;
+    for (int i = threadIdx.x; i < FT * FT; i += FTH) {
+        const uint32_t v = M[((size_t)r * FT + i / FT) * kp + (size_t)r * FT + i % FT];
+        if (is_row) piv[i % FT][i / FT] = v;
+        else piv[i / FT][i % FT] = v;
     }
-    fw_store_tile(t, M, kp, ti, tj);
+    uint32_t c[FQ][FQ];
+    fw_load4x4(c, M, kp, y, x);
+    bool ovf = false;
+    for (int p4 = 0; p4 < FT / FQ; ++p4) {
+#pragma unroll
+        for (int j = 0; j < FQ; ++j) {
+            const int b = j & 1, p = p4 * FQ + j;
+            if (is_row && ty == p4)
+                *reinterpret_cast<uint4*>(&line[b][tx * FQ]) = make_uint4(c[j][0], c[j][1], c[j][2], c[j][3]);
+            if (!is_row && tx == p4)
+                *reinterpret_cast<uint4*>(&line[b][ty * FQ]) = make_uint4(c[0][j], c[1][j], c[2][j], c[3][j]);
+            __syncthreads();
+            const uint32_t* a = is_row ? piv[p] : line[b];
+            const uint32_t* bb = is_row ? line[b] : piv[p];
+            fw_relax4x4<false>(c, *reinterpret_cast<const uint4*>(a + ty * FQ),
+                               *reinterpret_cast<const uint4*>(bb + tx * FQ), ovf);
+        }
+    }
+    fw_store4x4(c, M, kp, y, x);
     if (ovf) atomicExch(ovf_flag, 1u);
 }
 
-// phase 3: every other tile from its pivot-column and pivot-row tiles; no barrier inside the p loop.
-// The pivot-column tile is held transposed, so a thread reads its 4 rows of column p as one vector.
-constexpr int FA = FT + 4;  // padded row of the transposed tile, 16-byte aligned
+// Phase 3: every other tile from its pivot-column and pivot-row tiles; no barrier inside the p loop.  The
+// pivot-column tile is held transposed, so a thread reads its 4 rows of column p as one vector.  Bound by the
+// integer add-min rate.  The first CTA takes the next pivot tile and closes it when it is done (phase 1 of the next
+// round), hidden behind the other tiles instead of a launch of its own.
 template <bool FAST>
 __global__ void __launch_bounds__(FTH) k_fw_phase3(uint32_t* __restrict__ M, uint32_t kp, uint32_t r,
                                                    uint32_t* __restrict__ ovf_flag) {
     __shared__ __align__(16) uint32_t At[FT][FA];
     __shared__ __align__(16) uint32_t B[FT][FT];
+    __shared__ FwLine line;
     const int ty = threadIdx.x / 16, tx = threadIdx.x % 16;
     uint32_t ti = blockIdx.y, tj = blockIdx.x;
+    // (in the grid's numbering, which leaves the pivot out, the next pivot is number r: swap it with number 0)
+    const bool has_next = r < gridDim.x;
+    const bool next = has_next && ti == 0 && tj == 0;
+    if (next) ti = tj = r;
+    else if (has_next && ti == r && tj == r) ti = tj = 0;
     if (ti >= r) ++ti;
     if (tj >= r) ++tj;
     for (int i = threadIdx.x; i < FT * FT; i += FTH) {
@@ -187,29 +239,30 @@ __global__ void __launch_bounds__(FTH) k_fw_phase3(uint32_t* __restrict__ M, uin
         B[y][x] = M[((size_t)r * FT + y) * kp + (size_t)tj * FT + x];
     }
     uint32_t c[FQ][FQ];
-#pragma unroll
-    for (int i = 0; i < FQ; ++i) {
-        const uint4 v = *reinterpret_cast<const uint4*>(&M[((size_t)ti * FT + ty * FQ + i) * kp + (size_t)tj * FT + tx * FQ]);
-        c[i][0] = v.x; c[i][1] = v.y; c[i][2] = v.z; c[i][3] = v.w;
-    }
+    const size_t y0 = (size_t)ti * FT + ty * FQ, x0 = (size_t)tj * FT + tx * FQ;
+    fw_load4x4(c, M, kp, y0, x0);
     __syncthreads();
     bool ovf = false;
 #pragma unroll 8
-    for (int p = 0; p < FT; ++p) {
-        const uint4 av = *reinterpret_cast<const uint4*>(&At[p][ty * FQ]);
-        const uint4 bv = *reinterpret_cast<const uint4*>(&B[p][tx * FQ]);
-        const uint32_t a[FQ] = {av.x, av.y, av.z, av.w};
-        const uint32_t b[FQ] = {bv.x, bv.y, bv.z, bv.w};
-#pragma unroll
-        for (int i = 0; i < FQ; ++i)
-#pragma unroll
-            for (int j = 0; j < FQ; ++j) c[i][j] = fw_relax<FAST>(c[i][j], a[i], b[j], ovf);
-    }
-#pragma unroll
-    for (int i = 0; i < FQ; ++i)
-        *reinterpret_cast<uint4*>(&M[((size_t)ti * FT + ty * FQ + i) * kp + (size_t)tj * FT + tx * FQ]) =
-            make_uint4(c[i][0], c[i][1], c[i][2], c[i][3]);
+    for (int p = 0; p < FT; ++p)
+        fw_relax4x4<FAST>(c, *reinterpret_cast<const uint4*>(&At[p][ty * FQ]),
+                          *reinterpret_cast<const uint4*>(&B[p][tx * FQ]), ovf);
+    if (next) fw_close<FAST>(c, line, ty, tx, ovf);
+    fw_store4x4(c, M, kp, y0, x0);
     if (!FAST && ovf) atomicExch(ovf_flag, 1u);
+}
+
+// all rounds of blocked Floyd-Warshall on the padded matrix of nt x nt tiles
+template <bool FAST>
+cldiam_status fw_rounds(uint32_t* M, uint32_t kp, uint32_t nt, uint32_t* ovf, cudaStream_t s) {
+    CLD_K(K_FW, s, k_fw_phase1<FAST><<<1, FTH, 0, s>>>(M, kp, 0, ovf));
+    for (uint32_t r = 0; r < nt && nt > 1; ++r) {
+        if constexpr (FAST) CLD_K(K_FW, s, k_fw_phase2_fast<<<dim3(2 * (nt - 1), 2), FTH / 2, 0, s>>>(M, kp, r));
+        else CLD_K(K_FW, s, k_fw_phase2_checked<<<dim3(nt - 1, 2), FTH, 0, s>>>(M, kp, r, ovf));
+        CLD_K(K_FW, s, k_fw_phase3<FAST><<<dim3(nt - 1, nt - 1), FTH, 0, s>>>(M, kp, r, ovf));
+    }
+    CLD_LAUNCH_CHECK();
+    return CLDIAM_OK;
 }
 
 // largest entry below `none` among the k x k real entries; *missing = 1 if some entry is `none`
@@ -456,14 +509,7 @@ cldiam_status fw_dense(uint32_t* M, uint32_t kp, uint32_t k, uint32_t nt, const 
     CLD_K(K_FW, s, k_fw_init<<<grid_for((size_t)kp * kp, 256), 256, 0, s>>>(M, kp, k, none));
     CLD_K(K_FW, s, k_fw_scatter<<<grid_for(k, 1, 64), 128, 0, s>>>(off, col, w, k, kp, M, FAST ? scal + 3 : nullptr));
     CLD_LAUNCH_CHECK();
-    for (uint32_t r = 0; r < nt; ++r) {
-        CLD_K(K_FW, s, k_fw_phase1<FAST><<<1, FTH, 0, s>>>(M, kp, r, scal));
-        if (nt > 1) {
-            CLD_K(K_FW, s, k_fw_phase2<FAST><<<dim3(nt - 1, 2), FTH, 0, s>>>(M, kp, r, scal));
-            CLD_K(K_FW, s, k_fw_phase3<FAST><<<dim3(nt - 1, nt - 1), FTH, 0, s>>>(M, kp, r, scal));
-        }
-        CLD_LAUNCH_CHECK();
-    }
+    CLD_TRY(fw_rounds<FAST>(M, kp, nt, scal, s));
     CLD_K(K_FW, s, k_fw_max_finite<<<grid_for((size_t)k * kp, 256), 256, 0, s>>>(M, kp, k, none, scal + 1,
                                                                                   FAST ? scal + 4 : nullptr));
     CLD_LAUNCH_CHECK();
@@ -622,14 +668,7 @@ cldiam_status apsp_max_noalloc(uint32_t k, const uint64_t* off, const uint32_t* 
         k_fw_init<<<grid_for((size_t)kp * kp, 256), 256, 0, s>>>(M, kp, k, INF);
         k_fw_scatter<<<grid_for(k, 1, 64), 128, 0, s>>>(off, col, w, k, kp, M, nullptr);
         CLD_LAUNCH_CHECK();
-        for (uint32_t r = 0; r < nt; ++r) {
-            k_fw_phase1<false><<<1, FTH, 0, s>>>(M, kp, r, ovf);
-            if (nt > 1) {
-                k_fw_phase2<false><<<dim3(nt - 1, 2), FTH, 0, s>>>(M, kp, r, ovf);
-                k_fw_phase3<false><<<dim3(nt - 1, nt - 1), FTH, 0, s>>>(M, kp, r, ovf);
-            }
-            CLD_LAUNCH_CHECK();
-        }
+        CLD_TRY(fw_rounds<false>(M, kp, nt, ovf, s));
         k_fw_max_finite<<<grid_for((size_t)k * kp, 256), 256, 0, s>>>(M, kp, k, INF, best, nullptr);
         CLD_LAUNCH_CHECK();
     }
