@@ -103,21 +103,27 @@ __global__ void k_assign_cid(uint32_t n, const uint32_t* __restrict__ center, co
 // entry (an unfrozen node that reads the candidates of its contracted
 // neighbours, kPullTag | v) reduces its candidates over its lanes first, so
 // it lowers its own key once per group segment.  No block barrier.
+// RESIDENT: the kernel runs many steps (k_grow), so node state is read past L1, whose lines may be older than a
+// stage's reset; a one-step launch reads through L1 (a stale line only lets an extra candidate through).  Its
+// positions and ids come from lists that other CTAs wrote earlier in the same launch, so they are checked against the
+// graph's sizes (n, nnz) before use; one outside them would set ctr->bad.
+template <int WARPS>
 struct PushSmem {
-    uint32_t spre[PT / 32][QC + 1];  // first positions of the entries after the chunk's first
-    uint32_t sbase[PT / 32][QC + 2];
-    unsigned long long skey[PT / 32][QC + 2];
-    uint32_t sbuf[PT / 32][PNB];
+    unsigned long long skey[WARPS][QC + 2];
+    uint32_t spre[WARPS][QC + 1];  // first positions of the entries after the chunk's first
+    uint32_t sbase[WARPS][QC + 2];
+    uint32_t sbuf[WARPS][PNB];
 };
 
+template <bool RESIDENT, int WARPS>
 __device__ __forceinline__ void dev_push(const uint32_t* __restrict__ fbase, const unsigned long long* __restrict__ fkey,
                                          const uint32_t* __restrict__ fpre, const uint32_t* __restrict__ cfirst,
                                          uint32_t nf, uint32_t E, const uint2* __restrict__ adj,
                                          const uint32_t* __restrict__ center, const uint32_t* __restrict__ Dcum,
                                          unsigned long long* __restrict__ key, uint32_t delta,
                                          uint32_t* __restrict__ stamp, uint32_t stepid,
-                                         uint32_t* __restrict__ next, Counters* ctr, PushSmem& smp, uint32_t br,
-                                         uint32_t nb) {
+                                         uint32_t* __restrict__ next, Counters* ctr, PushSmem<WARPS>& smp, uint32_t br,
+                                         uint32_t nb, uint32_t n = 0, uint32_t nnz = 0) {
     auto& spre = smp.spre;
     auto& sbase = smp.sbase;
     auto& skey = smp.skey;
@@ -127,14 +133,20 @@ __device__ __forceinline__ void dev_push(const uint32_t* __restrict__ fbase, con
     const unsigned le_mask = 0xffffffffu >> (31u - lane);
     WarpNext wn{sbuf[warp], 0};
     unsigned long long newly = 0;
+    bool bad = false;
     const uint32_t nq = (uint32_t)(((uint64_t)E + QC - 1) / QC);
-    const uint32_t nwarps = nb * (PT / 32);
-    for (uint32_t q = br * (PT / 32) + warp; q < nq; q += nwarps) {
+    const uint32_t nwarps = nb * WARPS;
+    for (uint32_t q = br * WARPS + warp; q < nq; q += nwarps) {
         const uint32_t p0 = q * QC, e1 = min(E, p0 + QC);
         // entry i0 holds p0; entries i0 + 1 .. il start inside (p0, p0 + QC] (at most QC of them)
         const uint32_t i0 = __ldcg(&cfirst[q]);
         const uint32_t il = q + 1 < nq ? __ldcg(&cfirst[q + 1]) : nf - 1;
+        if (RESIDENT && (i0 > il || il >= nf)) {
+            bad = true;
+            continue;
+        }
         const uint32_t ne = min(il - i0 + 1, (uint32_t)QC + 1);
+        if (RESIDENT) __syncwarp();  // the previous chunk's entries have been read
         for (uint32_t j = lane; j < ne; j += 32) {
             if (j) spre[warp][j - 1] = __ldcg(&fpre[i0 + j]);
             sbase[warp][j] = __ldcg(&fbase[i0 + j]);
@@ -154,7 +166,27 @@ __device__ __forceinline__ void dev_push(const uint32_t* __restrict__ fbase, con
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             const uint32_t p = p0 + 32u * u + lane;
-            ed[u] = p < e1 ? ld_stream_u2(adj + (sbase[warp][own[u]] + p), pol_stream) : make_uint2(0u, 0xFFFFFFFFu);
+            bool in = p < e1;
+            if (RESIDENT && in && (own[u] >= ne || sbase[warp][own[u]] + p >= nnz)) {
+                bad = true;
+                in = false;
+            }
+            ed[u] = in ? ld_stream_u2(adj + (sbase[warp][own[u]] + p), pol_stream) : make_uint2(0u, 0xFFFFFFFFu);
+        }
+        // RESIDENT: the groups' loads and exchanges are issued level by level for all four groups, since few warps
+        // share the latency (one group after another, a push took 14,000 cycles, so 8,200)
+        uint32_t pcu[4], pdu[4], tgt[4];
+        unsigned long long cnk[4];
+        if constexpr (RESIDENT) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                pcu[u] = kNone;
+                pdu[u] = 0;
+                if ((skey[warp][own[u]] & kPullTag) == kPullTag && ed[u].y <= delta) {
+                    pcu[u] = __ldcg(&center[ed[u].x]);
+                    if (Dcum) pdu[u] = __ldcg(&Dcum[ed[u].x]);
+                }
+            }
         }
         unsigned long long carry = kInfKey;  // pull entry still open at the previous group's end
 #pragma unroll
@@ -171,11 +203,16 @@ __device__ __forceinline__ void dev_push(const uint32_t* __restrict__ fbase, con
                     nk = (cand << 32) | (ku & 0xFFFFFFFFull);
                 }
             } else if (live && ed[u].y <= delta) {  // pull: candidate of a contracted neighbour
-                const uint32_t cu = __ldg(&center[ed[u].x]);
-                if (cu != kNone) {
-                    const uint64_t cand = (uint64_t)(Dcum ? __ldg(&Dcum[ed[u].x]) : 0u) + ed[u].y;
-                    if (cand <= delta) nk = (cand << 32) | cu;
+                uint32_t cu, du = 0;
+                if constexpr (RESIDENT) {
+                    cu = pcu[u];
+                    du = pdu[u];
+                } else {
+                    cu = __ldg(&center[ed[u].x]);
+                    if (cu != kNone && Dcum) du = __ldg(&Dcum[ed[u].x]);
                 }
+                const uint64_t cand = (uint64_t)du + ed[u].y;
+                if (cu != kNone && cand <= delta) nk = (cand << 32) | cu;
             }
             // pulling entries: one candidate per segment (all lanes of an entry share its kind)
             if (__any_sync(0xffffffffu, is_pull)) {
@@ -195,28 +232,61 @@ __device__ __forceinline__ void dev_push(const uint32_t* __restrict__ fbase, con
             } else {
                 carry = kInfKey;
             }
-            bool first = false;
-            if (nk != kInfKey) {
-                // the target's key and stamp in one round trip, through L1 (a stale line only lets an
-                // extra candidate through: keys only fall within a launch, and the atomics decide); most
-                // candidates lose to the current key
-                const unsigned long long cur = ld_keep_u64(&key[target], pol_keep);
-                const uint32_t stp = ld_keep_u32(&stamp[target], pol_keep);
-                if (nk < cur) {
-                    red_min_keep_u64(&key[target], nk, pol_keep);
-                    if (stp != stepid) {  // hubs see many lowerings: only the first ones exchange
-                        const uint32_t old = atomicExch(&stamp[target], stepid);
-                        first = old != stepid;
-                        newly += old == 0u ? 1 : 0;
+            if constexpr (RESIDENT) {
+                if (nk != kInfKey && target >= n) {
+                    bad = true;
+                    nk = kInfKey;
+                }
+                cnk[u] = nk;
+                tgt[u] = target;
+            } else {
+                bool first = false;
+                if (nk != kInfKey) {
+                    // the target's key and stamp in one round trip, through L1 (a stale line only lets an
+                    // extra candidate through: keys only fall within a launch, and the atomics decide); most
+                    // candidates lose to the current key
+                    const unsigned long long cur = ld_keep_u64(&key[target], pol_keep);
+                    const uint32_t stp = ld_keep_u32(&stamp[target], pol_keep);
+                    if (nk < cur) {
+                        red_min_keep_u64(&key[target], nk, pol_keep);
+                        if (stp != stepid) {  // hubs see many lowerings: only the first ones exchange
+                            const uint32_t old = atomicExch(&stamp[target], stepid);
+                            first = old != stepid;
+                            newly += old == 0u ? 1 : 0;
+                        }
                     }
                 }
+                wn.put(first, target, lane);
             }
-            wn.put(first, target, lane);
+        }
+        if constexpr (RESIDENT) {
+            unsigned long long cur[4];
+            uint32_t stp[4], old[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const bool has = cnk[u] != kInfKey;
+                cur[u] = has ? ld_cg_keep_u64(&key[tgt[u]], pol_keep) : 0ull;
+                stp[u] = has ? ld_cg_keep_u32(&stamp[tgt[u]], pol_keep) : stepid;
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                old[u] = stepid;
+                if (cnk[u] < cur[u]) {
+                    red_min_keep_u64(&key[tgt[u]], cnk[u], pol_keep);
+                    if (stp[u] != stepid) old[u] = atomicExch(&stamp[tgt[u]], stepid);
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                newly += old[u] == 0u ? 1 : 0;
+                wn.put(old[u] != stepid, tgt[u], lane);
+            }
         }
         if (wn.cnt >= (uint32_t)PW) wn.flush(next, &ctr->nnext, lane);
     }
     if (wn.cnt) wn.flush(next, &ctr->nnext, lane);
     warp_add_u64(&ctr->newly_covered, newly);
+    if (RESIDENT && __any_sync(0xffffffffu, bad) && lane == 0) atomicExch(&ctr->bad, 1u);
 }
 
 __global__ void __launch_bounds__(PT, 6) k_push(const uint32_t* __restrict__ fbase,
@@ -227,8 +297,8 @@ __global__ void __launch_bounds__(PT, 6) k_push(const uint32_t* __restrict__ fba
                                                 unsigned long long* __restrict__ key, uint32_t delta,
                                                 uint32_t* __restrict__ stamp, uint32_t stepid,
                                                 uint32_t* __restrict__ next, Counters* ctr) {
-    __shared__ PushSmem smp;
-    dev_push(fbase, fkey, fpre, cfirst, nf, E, adj, center, Dcum, key, delta, stamp, stepid, next, ctr, smp,
+    __shared__ PushSmem<PT / 32> smp;
+    dev_push<false>(fbase, fkey, fpre, cfirst, nf, E, adj, center, Dcum, key, delta, stamp, stepid, next, ctr, smp,
                     blockIdx.x, gridDim.x);
 }
 
@@ -357,6 +427,213 @@ __global__ void __launch_bounds__(PT, 6) k_pull(uint32_t n, uint32_t nnz, uint32
                     blockIdx.x, gridDim.x);
 }
 
+// ---------------------------------------------------------------- resident growth
+// Small steps are latency: as separate launches a step is a push, a snapshot, a counter reset and a counter read
+// that the host waits for, 37 us on a 1,001 x 1,001 mesh for frontiers of a few thousand entries.  k_grow runs them
+// in one launch: one thread-block cluster (its CTAs are resident together, and its barrier orders their memory)
+// takes growing steps back to back, every CTA deciding from the same counters, until a step is too large for it or
+// the growth ends; on small graphs it runs whole stages (draw, listing, doubling, contraction) too.
+// Bound by dependent L2 round trips (chunk table, entries, adjacency, keys, stamps, append; then the snapshot's): 16,000
+// cycles a step up to 65,000 entries, 33,000 at 100,000, of which a cluster barrier is 1,050.  Clustering alone, host
+// loop / resident: 64^2 mesh (44 steps) 1,602 / 504 us, 300^2 mesh (101) 3,101 / 1,326 us, 1,001^2 mesh (206) 7,405 /
+// 4,779 us, road mesh 4,096^2 (134) 12,520 / 11,555 us.  Above 2^18 entries a step of the whole device (push and
+// snapshot 13 to 40 us and 22 us between them) is the faster one; a whole-node pass over more than 2^17 nodes by 16
+// SMs likewise.
+constexpr int GT = 1024;                     // threads per CTA
+constexpr int GCTAS = 16;                    // CTAs of the cluster
+constexpr uint32_t kGrowEntries = 1u << 18;  // largest step: 16 passes of a warp's 128 positions over the cluster's warps
+constexpr uint32_t kGrowNodes = 1u << 17;    // whole stages up to this many nodes: 8 rounds of a node per thread
+constexpr uint32_t kGrowEpochs = 1u << 20;   // phases per launch, after which the host launches it again
+
+enum GrowPhase : uint32_t { kPhaseStage = 0, kPhaseStep = 1, kPhaseGrown = 2, kPhaseDone = 3, kPhaseFailed = 4 };
+
+// The control state of CLUSTER between phases, kept by the host and by every thread of k_grow alike.
+struct GrowState {
+    uint64_t U;           // unfrozen nodes at the stage's start
+    uint64_t covered;     // of them, nodes holding a key
+    uint64_t frozen_deg;  // adjacency entries of frozen nodes
+    uint64_t node_updates, edges_scanned, centers_drawn;
+    uint64_t unfrozen;    // what the last draw saw
+    uint32_t phase, stage, stepid, delta;
+    uint32_t nf, E, cur;  // the frontier and which pair of buffers holds it
+    uint32_t growth_steps;
+    uint32_t steps, stages, doublings, guard_exits;
+};
+
+struct GrowArgs {
+    const uint64_t* off;
+    const uint2* adj;
+    unsigned long long* key;
+    unsigned long long* keyS;
+    unsigned long long* fkey[2];
+    uint32_t *center, *D, *R, *stamp, *next;
+    uint32_t *fbase[2], *fpre[2], *cfirst[2];
+    Counters* ring;  // three counter blocks, zeroed
+    GrowState* out;
+    double tau, L;
+    uint64_t seed, nnz;
+    uint32_t n, step_cap, max_entries;
+    bool cumulative, pull_ok, stages;
+};
+
+struct GrowSmem {
+    PushSmem<GT / 32> push;
+    unsigned long long scratch[33];
+    Counters seen;
+};
+
+__device__ __forceinline__ void grow_barrier() {
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
+}
+
+__global__ void __launch_bounds__(GT, 1) k_grow(const GrowArgs a, GrowState g) {
+    extern __shared__ __align__(16) unsigned char grow_smem[];
+    GrowSmem& sm = *reinterpret_cast<GrowSmem*>(grow_smem);
+    const uint32_t br = blockIdx.x, nb = gridDim.x;  // one cluster: the CTA's rank and the cluster's size
+    uint32_t epoch = 0;
+    // Counter block of the current epoch (between two closing barriers).  An epoch clears the next one's block, last
+    // read two epochs ago: every CTA has passed the barrier that closed the epoch in between.
+    const auto ctr = [&]() { return a.ring + epoch % 3; };
+    const auto close_epoch = [&]() {  // every thread gets the epoch's counters
+        if (br == 0 && threadIdx.x < sizeof(Counters) / 8)
+            reinterpret_cast<unsigned long long*>(a.ring + (epoch + 1) % 3)[threadIdx.x] = 0ull;
+        grow_barrier();
+        if (threadIdx.x < sizeof(Counters) / 8)
+            reinterpret_cast<unsigned long long*>(&sm.seen)[threadIdx.x] =
+                __ldcg(reinterpret_cast<const unsigned long long*>(ctr()) + threadIdx.x);
+        __syncthreads();
+        ++epoch;
+    };
+    const auto rebuild = [&]() {
+        const bool pull = a.pull_ok && (a.nnz - g.frozen_deg) < g.frozen_deg;
+        dev_rebuild(a.n, a.key, a.center, a.cumulative ? a.D : nullptr, a.off, g.delta, pull, a.fbase[g.cur],
+                    a.fkey[g.cur], a.fpre[g.cur], a.cfirst[g.cur], ctr(), sm.scratch, br, nb);
+        close_epoch();
+        g.nf = (uint32_t)(sm.seen.front >> 32);
+        g.E = (uint32_t)sm.seen.front;
+    };
+    while (epoch < kGrowEpochs) {
+        if (g.phase == kPhaseStep) {
+            if (g.E > a.max_entries) break;
+            uint32_t updated = 0;
+            ++g.growth_steps;
+            ++g.stepid;
+            if (g.nf > 0) {
+                dev_push<true>(a.fbase[g.cur], a.fkey[g.cur], a.fpre[g.cur], a.cfirst[g.cur], g.nf, g.E, a.adj, a.center,
+                               a.cumulative ? a.D : nullptr, a.key, g.delta, a.stamp, g.stepid, a.next, ctr(), sm.push,
+                               br, nb, a.n, (uint32_t)a.nnz);
+                grow_barrier();
+                const uint32_t nn = min(__ldcg(&ctr()->nnext), a.n), o = g.cur ^ 1;
+                dev_snapshot(a.next, nn, a.key, a.off, g.delta, a.fbase[o], a.fkey[o], a.fpre[o], a.cfirst[o], ctr(),
+                             sm.scratch, br, nb, a.keyS, a.n);
+                close_epoch();
+                if (sm.seen.bad) {
+                    g.phase = kPhaseFailed;
+                    g.unfrozen = ~g.U;
+                    break;
+                }
+                updated = sm.seen.nnext;
+                g.covered += sm.seen.newly_covered;
+                g.edges_scanned += g.E;
+                g.nf = (uint32_t)(sm.seen.front >> 32);
+                g.E = (uint32_t)sm.seen.front;
+                g.cur = o;
+            }
+            g.steps++;
+            g.node_updates += updated;
+            if (!(updated != 0 && 2 * g.covered < g.U && (a.step_cap == 0 || g.growth_steps < a.step_cap)))
+                g.phase = kPhaseGrown;
+        } else if (!a.stages) {
+            break;
+        } else if (g.phase == kPhaseStage) {
+            uint64_t thr = 0;
+            if (!stage_threshold(g.U, a.tau, a.L, &thr)) {
+                g.phase = kPhaseDone;
+                break;
+            }
+            if (g.stage > kMaxStages) {
+                g.phase = kPhaseFailed;
+                break;
+            }
+            dev_select(a.n, a.center, a.key, a.seed, g.stage, thr, ctr(), br, nb, a.keyS);
+            close_epoch();
+            g.covered = sm.seen.selected;
+            g.centers_drawn += sm.seen.selected;
+            g.unfrozen = sm.seen.unfrozen;
+            if (g.unfrozen != g.U) {
+                g.phase = kPhaseFailed;
+                break;
+            }
+            rebuild();
+            g.growth_steps = 0;
+            g.phase = kPhaseStep;
+        } else if (g.phase == kPhaseGrown) {
+            if (2 * g.covered < g.U) {
+                // (connected graph: some covered or frozen node touches an uncovered one iff any exists)
+                if (g.delta < kDeltaMax && (g.covered > 0 || g.U < a.n)) {
+                    g.delta = (g.delta > kDeltaMax / 2) ? kDeltaMax : 2 * g.delta;
+                    g.doublings++;
+                    rebuild();
+                    g.growth_steps = 0;
+                    g.phase = kPhaseStep;
+                    continue;
+                }
+                g.guard_exits++;
+            }
+            dev_finalize_d(a.n, a.key, a.center, a.cumulative ? nullptr : a.R, a.D, ctr(), br, nb);
+            grow_barrier();
+            dev_finalize_freeze(a.n, a.key, a.center, a.R, a.D, a.off, ctr(), br, nb, a.keyS, a.cumulative);
+            close_epoch();
+            const bool overflow = sm.seen.overflow != 0;
+            g.U -= sm.seen.frozen;
+            g.frozen_deg += sm.seen.frozen_deg;
+            if (overflow) {
+                g.phase = kPhaseFailed;
+                g.unfrozen = g.U = 0;
+                break;
+            }
+            g.stages++;
+            ++g.stage;
+            g.phase = kPhaseStage;
+        } else {
+            break;
+        }
+    }
+    if (br == 0 && threadIdx.x == 0) *a.out = g;
+}
+
+// CTAs of k_grow's cluster on this device: 16 where such a cluster can be resident, else the portable 8, else 0 (not
+// used).  Decided once per device; concurrent first calls store the same value.
+int grow_cluster_size(int dev) {
+    static std::atomic<int> cached[64];  // 0 = not asked yet, else size + 1
+    if (dev < 0 || dev >= 64) return 0;
+    if (cached[dev].load() == 0) {
+        int size = 0;
+        if (cudaFuncSetAttribute(k_grow, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(GrowSmem)) ==
+                cudaSuccess &&
+            cudaFuncSetAttribute(k_grow, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
+            for (int c = GCTAS; c >= 8 && size == 0; c /= 2) {
+                cudaLaunchConfig_t cfg{};
+                cudaLaunchAttribute at{};
+                at.id = cudaLaunchAttributeClusterDimension;
+                at.val.clusterDim.x = (unsigned)c;
+                at.val.clusterDim.y = at.val.clusterDim.z = 1;
+                cfg.gridDim = dim3((unsigned)c);
+                cfg.blockDim = dim3(GT);
+                cfg.dynamicSmemBytes = sizeof(GrowSmem);
+                cfg.attrs = &at;
+                cfg.numAttrs = 1;
+                int m = 0;
+                if (cudaOccupancyMaxActiveClusters(&m, k_grow, &cfg) == cudaSuccess && m > 0) size = c;
+            }
+        }
+        cudaGetLastError();
+        cached[dev].store(size + 1);
+    }
+    return cached[dev].load() - 1;
+}
+
 // node state before the first stage: no center, D = R = 0, no stamp, no key
 __global__ void k_cluster_init(uint32_t n, uint32_t* __restrict__ center, uint32_t* __restrict__ D,
                                uint32_t* __restrict__ R, uint32_t* __restrict__ stamp,
@@ -472,7 +749,7 @@ cldiam_status cluster(cldiam_graph* g, double tau, uint64_t seed, const cldiam_o
     CLD_TRY(next.alloc(n, s));
     CLD_TRY(ctr.alloc(1, s));
     Counters* hc = static_cast<Counters*>(g->host.h);
-    static_assert(sizeof(Counters) <= 128, "counter block must fit the pinned area");
+    static_assert(sizeof(Counters) <= 128 && sizeof(GrowState) <= 128, "the read-back blocks must fit the pinned area");
 
     const unsigned gb = grid_for(n, 256);
     CLD_K(K_MISC, s, k_cluster_init<<<gb, 256, 0, s>>>(n, center.get(), D.get(), R.get(), stamp.get(), key.get(),
@@ -495,20 +772,17 @@ cldiam_status cluster(cldiam_graph* g, double tau, uint64_t seed, const cldiam_o
         return CLDIAM_OK;
     };
 
-    cldiam_result st{};
     const double L = std::log2((double)n);
-    uint64_t U = n;               // unfrozen nodes
-    uint64_t frozen_deg = 0;      // adjacency entries of frozen nodes
     const bool pull_ok = g->nnz < 0x80000000ull;  // push + pull entries must index below 2^32
-    uint32_t stage = 1, stepid = 0;
-    uint32_t* fv = fvA.get();
-    uint32_t* fp = fpA.get();
-    unsigned long long* fk = fkeyA.get();
-    uint32_t* fv2 = fvB.get();
-    uint32_t* fp2 = fpB.get();
-    unsigned long long* fk2 = fkeyB.get();
-    uint32_t* cf = cfA.get();
-    uint32_t* cf2 = cfB.get();
+    GrowState gs{};
+    gs.U = n;
+    gs.phase = kPhaseStage;
+    gs.stage = 1;
+    gs.delta = delta;
+    uint32_t* const fv[2] = {fvA.get(), fvB.get()};
+    uint32_t* const fp[2] = {fpA.get(), fpB.get()};
+    uint32_t* const cf[2] = {cfA.get(), cfB.get()};
+    unsigned long long* const fk[2] = {fkeyA.get(), fkeyB.get()};
     const unsigned max_relax_grid = (unsigned)num_sms() * 8;
     // the growing-step kernels loop over warp chunks: launch at most the resident CTAs (no partial second
     // wave after the first has finished its chunks)
@@ -531,104 +805,183 @@ cldiam_status cluster(cldiam_graph* g, double tau, uint64_t seed, const cldiam_o
     const unsigned push_grid = (unsigned)num_sms() * push_ctas;
     const unsigned pull_grid =
         (unsigned)std::min<uint64_t>((uint64_t)num_sms() * pull_ctas, (pull_chunks + PT / 32 - 1) / (PT / 32));
-    uint32_t nf = 0, E = 0;
     DBuf<uint32_t> rows_built;  // COO rows for the guard's edge scan when the graph keeps none
 
-    // list every relaxer (stage start, or after Delta doubled)
-    auto rebuild = [&]() -> cldiam_status {
-        const bool pull = pull_ok && (g->nnz - frozen_deg) < frozen_deg;
-        CLD_TRY(zero_field(offsetof(Counters, front), 8));
-        CLD_K(K_REBUILD, s, k_rebuild<<<gb, 256, 0, s>>>(n, key.get(), center.get(), cumulative ? D.get() : nullptr,
-                                                          g->off, delta, pull, fv, fk, fp, cf, ctr.get()));
-        CLD_LAUNCH_CHECK();
+    // Resident growth (k_grow): on connected graphs, unless a tuning knob asks for the grid kernels (a set number of
+    // CTAs) or for the dense form at a share of the adjacency that the step reaches (a share other than the default).
+    const int grow_ctas = g->connected && n >= 2 && g->nnz < 0xFFFFFFFFull && tun.relax_ctas_per_sm == 0 ? grow_cluster_size(dev) : 0;
+    const bool strict_pull = pull_dense && tun.pull_ratio != tuning_defaults_filled(cldiam_tuning{}).pull_ratio;
+    const uint32_t grow_entries =
+        strict_pull ? (uint32_t)std::min<double>(kGrowEntries, std::max(0.0, std::ceil((double)tun.pull_ratio * (double)g->nnz) - 1))
+                    : kGrowEntries;
+    const bool grow_stages = n <= kGrowNodes;
+    DBuf<Counters> ring;
+    DBuf<GrowState> gdev;
+    if (grow_ctas) {
+        CLD_TRY(ring.alloc(3, s));
+        CLD_TRY(gdev.alloc(1, s));
+    }
+    const auto grow = [&]() -> cldiam_status {
+        GrowArgs a{};
+        a.off = g->off;
+        a.adj = g->adj;
+        a.key = key.get();
+        a.keyS = keyS.get();
+        for (int i = 0; i < 2; ++i) {
+            a.fkey[i] = fk[i];
+            a.fbase[i] = fv[i];
+            a.fpre[i] = fp[i];
+            a.cfirst[i] = cf[i];
+        }
+        a.center = center.get();
+        a.D = D.get();
+        a.R = R.get();
+        a.stamp = stamp.get();
+        a.next = next.get();
+        a.ring = ring.get();
+        a.out = gdev.get();
+        a.tau = tau;
+        a.L = L;
+        a.seed = seed;
+        a.nnz = g->nnz;
+        a.n = n;
+        a.step_cap = step_cap;
+        a.max_entries = grow_entries;
+        a.cumulative = cumulative;
+        a.pull_ok = pull_ok;
+        a.stages = grow_stages;
+        CLD_CUDA(cudaMemsetAsync(ring.get(), 0, 3 * sizeof(Counters), s));
+        cudaLaunchConfig_t cfg{};
+        cudaLaunchAttribute at{};
+        at.id = cudaLaunchAttributeClusterDimension;
+        at.val.clusterDim.x = (unsigned)grow_ctas;
+        at.val.clusterDim.y = at.val.clusterDim.z = 1;
+        cfg.gridDim = dim3((unsigned)grow_ctas);
+        cfg.blockDim = dim3(GT);
+        cfg.dynamicSmemBytes = sizeof(GrowSmem);
+        cfg.stream = s;
+        cfg.attrs = &at;
+        cfg.numAttrs = 1;
+        const uint64_t scanned0 = gs.edges_scanned, updates0 = gs.node_updates;
+        CLD_K(K_RELAX, s, CLD_CUDA(cudaLaunchKernelEx(&cfg, k_grow, a, gs)));
+        GrowState* hg = static_cast<GrowState*>(g->host.h);
+        CLD_CUDA(cudaMemcpyAsync(hg, gdev.get(), sizeof(GrowState), cudaMemcpyDeviceToHost, s));
+        CLD_CUDA(cudaStreamSynchronize(s));
+        prof_flush();
+        gs = *hg;
+        prof_add_bytes(K_RELAX, 16.0 * (double)(gs.edges_scanned - scanned0) + 40.0 * (double)(gs.node_updates - updates0));
         return CLDIAM_OK;
     };
 
-    {
-        for (;;) {
+    // list every relaxer (stage start, or after Delta doubled)
+    auto rebuild = [&]() -> cldiam_status {
+        const bool pull = pull_ok && (g->nnz - gs.frozen_deg) < gs.frozen_deg;
+        CLD_TRY(zero_field(offsetof(Counters, front), 8));
+        CLD_K(K_REBUILD, s, k_rebuild<<<gb, 256, 0, s>>>(n, key.get(), center.get(), cumulative ? D.get() : nullptr,
+                                                          g->off, gs.delta, pull, fv[gs.cur], fk[gs.cur], fp[gs.cur],
+                                                          cf[gs.cur], ctr.get()));
+        CLD_LAUNCH_CHECK();
+        CLD_TRY(sync_counters());
+        gs.nf = (uint32_t)(hc->front >> 32);
+        gs.E = (uint32_t)hc->front;
+        gs.growth_steps = 0;
+        gs.phase = kPhaseStep;
+        return CLDIAM_OK;
+    };
+    const auto draw_mismatch = [&]() {
+        char buf[200];
+        snprintf(buf, sizeof buf, "the draw of stage %u saw %llu unfrozen nodes, the loop tracked %llu", gs.stage,
+                 (unsigned long long)gs.unfrozen, (unsigned long long)gs.U);
+        return fail(CLDIAM_ERR_DIVERGED, buf);
+    };
+
+    // Algorithm 1's loops as phases: a stage's draw, its growing steps one by one, and what follows when growth stops
+    while (gs.phase != kPhaseDone) {
+        if (grow_ctas && (gs.phase == kPhaseStep ? gs.nf > 0 && gs.E <= grow_entries : grow_stages)) {
+            CLD_TRY(grow());
+            if (gs.phase == kPhaseFailed) {
+                if (gs.stage > kMaxStages) return fail(CLDIAM_ERR_DIVERGED, "CLUSTER exceeded its stage limit");
+                if (gs.unfrozen == ~gs.U) return fail(CLDIAM_ERR_DIVERGED, "inconsistent frontier in a resident growing step");
+                if (gs.unfrozen != gs.U) return draw_mismatch();
+                return fail(CLDIAM_ERR_OVERFLOW, "a cluster distance bound reached 2^32 - 1");
+            }
+        } else if (gs.phase == kPhaseStage) {
             uint64_t thr = 0;
-            if (!stage_threshold(U, tau, L, &thr)) break;  // outer while test of Algorithm 1, center draw threshold
-            if (stage > kMaxStages) return fail(CLDIAM_ERR_DIVERGED, "CLUSTER exceeded its stage limit");
+            // outer while test of Algorithm 1, center draw threshold
+            if (!stage_threshold(gs.U, tau, L, &thr)) {
+                gs.phase = kPhaseDone;
+                break;
+            }
+            if (gs.stage > kMaxStages) return fail(CLDIAM_ERR_DIVERGED, "CLUSTER exceeded its stage limit");
 
             // selection + reset, then the stage's first frontier
             CLD_TRY(zero_field(offsetof(Counters, selected), 8));
             CLD_TRY(zero_field(offsetof(Counters, unfrozen), 8));
-            CLD_K(K_SELECT, s, k_select<<<gb, 256, 0, s>>>(n, center.get(), key.get(), seed, stage, thr, ctr.get(),
+            CLD_K(K_SELECT, s, k_select<<<gb, 256, 0, s>>>(n, center.get(), key.get(), seed, gs.stage, thr, ctr.get(),
                                                             keyS.get()));
             CLD_LAUNCH_CHECK();
             CLD_TRY(rebuild());
-            CLD_TRY(sync_counters());
-            if (hc->unfrozen != U) {
-                char buf[200];
-                snprintf(buf, sizeof buf, "the draw of stage %u saw %llu unfrozen nodes, the loop tracked %llu",
-                         stage, (unsigned long long)hc->unfrozen, (unsigned long long)U);
-                return fail(CLDIAM_ERR_DIVERGED, buf);
+            gs.unfrozen = hc->unfrozen;
+            if (gs.unfrozen != gs.U) return draw_mismatch();
+            gs.covered = hc->selected;
+            gs.centers_drawn += hc->selected;
+        } else if (gs.phase == kPhaseStep) {
+            uint32_t updated = 0;
+            ++gs.growth_steps;
+            ++gs.stepid;
+            const uint32_t c = gs.cur, o = gs.cur ^ 1;
+            if (gs.nf > 0) {
+                CLD_TRY(zero_field(offsetof(Counters, newly_covered), 24));  // newly_covered, front, nnext
+                // the dense form reads the whole adjacency: worth it when the relaxers hold a large share
+                const bool dense = pull_dense && (double)gs.E >= (double)tun.pull_ratio * (double)g->nnz;
+                if (dense) {
+                    CLD_K(K_PULL, s, k_pull<<<pull_grid, PT, 0, s>>>(n, (uint32_t)g->nnz, pull_chunks, crow.get(), g->off,
+                                                                      g->adj, cumulative ? center.get() : nullptr,
+                                                                      keyS.get(), key.get(), gs.delta, stamp.get(),
+                                                                      gs.stepid, next.get(), ctr.get()));
+                } else {
+                    const uint64_t warps = ((uint64_t)gs.E + QC - 1) / QC;
+                    const unsigned rg = (unsigned)std::min<uint64_t>((warps + PT / 32 - 1) / (PT / 32), push_grid);
+                    CLD_K(K_RELAX, s, k_push<<<rg, PT, 0, s>>>(fv[c], fk[c], fp[c], cf[c], gs.nf, gs.E, g->adj,
+                                                                center.get(), cumulative ? D.get() : nullptr, key.get(),
+                                                                gs.delta, stamp.get(), gs.stepid, next.get(), ctr.get()));
+                }
+                CLD_LAUNCH_CHECK();
+                CLD_K(K_SNAPSHOT, s, k_snapshot<<<max_relax_grid, 256, 0, s>>>(next.get(), key.get(), g->off, gs.delta,
+                                                                             fv[o], fk[o], fp[o], cf[o], ctr.get(),
+                                                                             keyS.get()));
+                CLD_LAUNCH_CHECK();
+                CLD_TRY(sync_counters());
+                updated = hc->nnext;
+                gs.covered += hc->newly_covered;
+                gs.edges_scanned += gs.E;
+                if (dense) {
+                    // algorithmic bytes of a dense step: per adjacency entry the (col, w) pair (8 B) and
+                    // the neighbour's snapshot key (8 B); per row its start and snapshot key (16 B); per
+                    // changed node its key, stamp and list slot (16 B)
+                    prof_add_bytes(K_PULL, 16.0 * (double)g->nnz + 16.0 * n + 16.0 * updated);
+                } else {
+                    // algorithmic bytes of a pushed step: per frontier entry its slot (4 + 8 + 4 B)
+                    // and row start (8 B); per adjacency entry the (col, w) pair (8 B) and the target's
+                    // key (8 B); per changed node its key, stamp and list slot (16 B)
+                    prof_add_bytes(K_RELAX, 24.0 * gs.nf + 16.0 * (double)gs.E + 16.0 * updated);
+                }
+                prof_add_bytes(K_SNAPSHOT, 4.0 * updated + 16.0 * updated + 16.0 * updated + 16.0 * (hc->front >> 32));
+                gs.cur = o;
+                gs.nf = (uint32_t)(hc->front >> 32);
+                gs.E = (uint32_t)hc->front;
             }
-            uint64_t covered = hc->selected;
-            nf = (uint32_t)(hc->front >> 32);
-            E = (uint32_t)hc->front;
-            st.centers_drawn += hc->selected;
-
-            for (;;) {
-                uint32_t updated, growth_steps = 0;
-                do {
-                    ++growth_steps;
-                    ++stepid;
-                    updated = 0;
-                    if (nf > 0) {
-                        CLD_TRY(zero_field(offsetof(Counters, newly_covered), 24));  // newly_covered, front, nnext
-                        // the dense form reads the whole adjacency: worth it when the relaxers hold a large share
-                        const bool dense = pull_dense && (double)E >= (double)tun.pull_ratio * (double)g->nnz;
-                        if (dense) {
-                            CLD_K(K_PULL, s, k_pull<<<pull_grid, PT, 0, s>>>(n, (uint32_t)g->nnz, pull_chunks, crow.get(),
-                                                                              g->off, g->adj,
-                                                                              cumulative ? center.get() : nullptr, keyS.get(),
-                                                                              key.get(), delta, stamp.get(), stepid,
-                                                                              next.get(), ctr.get()));
-                        } else {
-                            const uint64_t warps = ((uint64_t)E + QC - 1) / QC;
-                            const unsigned rg = (unsigned)std::min<uint64_t>((warps + PT / 32 - 1) / (PT / 32), push_grid);
-                            CLD_K(K_RELAX, s, k_push<<<rg, PT, 0, s>>>(fv, fk, fp, cf, nf, E, g->adj, center.get(),
-                                                                        cumulative ? D.get() : nullptr, key.get(), delta,
-                                                                        stamp.get(), stepid, next.get(), ctr.get()));
-                        }
-                        CLD_LAUNCH_CHECK();
-                        CLD_K(K_SNAPSHOT, s, k_snapshot<<<max_relax_grid, 256, 0, s>>>(next.get(), key.get(), g->off, delta,
-                                                                                     fv2, fk2, fp2, cf2, ctr.get(),
-                                                                                     keyS.get()));
-                        CLD_LAUNCH_CHECK();
-                        CLD_TRY(sync_counters());
-                        updated = hc->nnext;
-                        covered += hc->newly_covered;
-                        st.edges_scanned += E;
-                        if (dense) {
-                            // algorithmic bytes of a dense step: per adjacency entry the (col, w) pair (8 B) and
-                            // the neighbour's snapshot key (8 B); per row its start and snapshot key (16 B); per
-                            // changed node its key, stamp and list slot (16 B)
-                            prof_add_bytes(K_PULL, 16.0 * (double)g->nnz + 16.0 * n + 16.0 * updated);
-                        } else {
-                            // algorithmic bytes of a pushed step: per frontier entry its slot (4 + 8 + 4 B)
-                            // and row start (8 B); per adjacency entry the (col, w) pair (8 B) and the target's
-                            // key (8 B); per changed node its key, stamp and list slot (16 B)
-                            prof_add_bytes(K_RELAX, 24.0 * nf + 16.0 * (double)E + 16.0 * updated);
-                        }
-                        prof_add_bytes(K_SNAPSHOT, 4.0 * updated + 16.0 * updated + 16.0 * updated + 16.0 * (hc->front >> 32));
-                        std::swap(fv, fv2);
-                        std::swap(fp, fp2);
-                        std::swap(fk, fk2);
-                        std::swap(cf, cf2);
-                        nf = (uint32_t)(hc->front >> 32);
-                        E = (uint32_t)hc->front;
-                    }
-                    st.steps++;
-                    st.node_updates += updated;
-                } while (updated != 0 && 2 * covered < U && (step_cap == 0 || growth_steps < step_cap));
-                if (2 * covered >= U) break;
+            gs.steps++;
+            gs.node_updates += updated;
+            if (!(updated != 0 && 2 * gs.covered < gs.U && (step_cap == 0 || gs.growth_steps < step_cap)))
+                gs.phase = kPhaseGrown;
+        } else {
+            if (2 * gs.covered < gs.U) {
                 bool growable = false;
-                if (delta < kDeltaMax && g->connected) {
+                if (gs.delta < kDeltaMax && g->connected) {
                     // connected graph: some covered or frozen node touches an uncovered one iff any exists
-                    growable = covered > 0 || U < n;
-                } else if (delta < kDeltaMax && g->nnz) {
+                    growable = gs.covered > 0 || gs.U < n;
+                } else if (gs.delta < kDeltaMax && g->nnz) {
                     CLD_TRY(zero_field(offsetof(Counters, growable), 4));
                     if (!g->row && !rows_built.get()) {  // (graphs without a row array are connected LCCs)
                         CLD_TRY(rows_built.alloc(g->nnz, s));
@@ -641,16 +994,13 @@ cldiam_status cluster(cldiam_graph* g, double tau, uint64_t seed, const cldiam_o
                     CLD_TRY(sync_counters());
                     growable = hc->growable != 0;
                 }
-                if (!growable) {
-                    st.guard_exits++;
-                    break;
+                if (growable) {
+                    gs.delta = (gs.delta > kDeltaMax / 2) ? kDeltaMax : 2 * gs.delta;
+                    gs.doublings++;
+                    CLD_TRY(rebuild());
+                    continue;
                 }
-                delta = (delta > kDeltaMax / 2) ? kDeltaMax : 2 * delta;
-                st.doublings++;
-                CLD_TRY(rebuild());
-                CLD_TRY(sync_counters());
-                nf = (uint32_t)(hc->front >> 32);
-                E = (uint32_t)hc->front;
+                gs.guard_exits++;
             }
 
             // assign and contract
@@ -662,18 +1012,27 @@ cldiam_status cluster(cldiam_graph* g, double tau, uint64_t seed, const cldiam_o
             CLD_LAUNCH_CHECK();
             CLD_TRY(sync_counters());
             if (hc->overflow) return fail(CLDIAM_ERR_OVERFLOW, "a cluster distance bound reached 2^32 - 1");
-            U -= hc->frozen;
-            frozen_deg += hc->frozen_deg;
-            st.stages++;
-            ++stage;
+            gs.U -= hc->frozen;
+            gs.frozen_deg += hc->frozen_deg;
+            gs.stages++;
+            ++gs.stage;
+            gs.phase = kPhaseStage;
         }
-        CLD_K(K_FINALIZE, s, k_singletons<<<gb, 256, 0, s>>>(n, center.get(), D.get()));
-        CLD_LAUNCH_CHECK();
     }
+    CLD_K(K_FINALIZE, s, k_singletons<<<gb, 256, 0, s>>>(n, center.get(), D.get()));
+    CLD_LAUNCH_CHECK();
+    cldiam_result st{};
+    st.stages = gs.stages;
+    st.steps = gs.steps;
+    st.doublings = gs.doublings;
+    st.guard_exits = gs.guard_exits;
+    st.node_updates = gs.node_updates;
+    st.edges_scanned = gs.edges_scanned;
+    st.centers_drawn = gs.centers_drawn;
 
     CLD_TRY(relabel_clusters(g, center.get(), cid.get(), &st.k));
     prof_flush();
-    st.delta_end = delta;
+    st.delta_end = gs.delta;
 
     cl->center = center.detach();
     cl->D = D.detach();

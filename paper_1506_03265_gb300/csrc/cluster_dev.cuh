@@ -45,13 +45,13 @@ struct Counters {
     unsigned long long newly_covered;  // nodes that got their first key this step
     unsigned long long front;          // next frontier: (entries << 32) | adjacency entries
     uint32_t nnext;                    // changed nodes this step
-    uint32_t pad;
+    uint32_t bad;                      // a list of the resident growth held an id out of range
     // others
     uint32_t growable;                 // some covered/frozen node touches an uncovered one
     uint32_t overflow;                 // a D_v reached 2^32 - 1
     unsigned long long unfrozen;       // unfrozen nodes the stage's draw saw (checks the tracked |U|)
 };
-static_assert(offsetof(Counters, pad) + 4 - offsetof(Counters, newly_covered) == 24,
+static_assert(offsetof(Counters, bad) + 4 - offsetof(Counters, newly_covered) == 24,
               "the per-step counters form one block");
 
 constexpr int RC = 1024;  // adjacency entries per relax chunk of one CTA (the many-graph form)
@@ -460,7 +460,7 @@ __device__ __forceinline__ void dev_snapshot(const uint32_t* __restrict__ next, 
                                              uint32_t* __restrict__ fbase, unsigned long long* __restrict__ fkey,
                                              uint32_t* __restrict__ fpre, uint32_t* __restrict__ cfirst, Counters* ctr,
                                              unsigned long long* scratch, uint32_t br, uint32_t nb,
-                                             unsigned long long* __restrict__ keyS = nullptr) {
+                                             unsigned long long* __restrict__ keyS = nullptr, uint32_t n = kNone) {
     for (uint32_t base = br * blockDim.x; base < nn; base += nb * blockDim.x) {
         const uint32_t i = base + threadIdx.x;
         bool take = false;
@@ -468,12 +468,16 @@ __device__ __forceinline__ void dev_snapshot(const uint32_t* __restrict__ next, 
         unsigned long long k = 0;
         if (i < nn) {
             v = __ldcg(&next[i]);
-            k = __ldcg(&key[v]);
-            if (keyS) keyS[v] = k;  // the next step's start-of-step key
-            const uint64_t o = off[v];
-            b0 = (uint32_t)o;
-            deg = (uint32_t)(off[v + 1] - o);
-            take = (uint32_t)(k >> 32) < delta && deg > 0;
+            if (v < n) {
+                k = __ldcg(&key[v]);
+                if (keyS) keyS[v] = k;  // the next step's start-of-step key
+                const uint64_t o = off[v];
+                b0 = (uint32_t)o;
+                deg = (uint32_t)(off[v + 1] - o);
+                take = (uint32_t)(k >> 32) < delta && deg > 0;
+            } else {
+                atomicExch(&ctr->bad, 1u);
+            }
         }
         uint32_t slot = 0, pre = 0;
         front_append(&ctr->front, take, deg, slot, pre, scratch);

@@ -313,6 +313,11 @@ __device__ __forceinline__ unsigned long long ld_cg_keep_u64(const unsigned long
     asm volatile("ld.global.cg.L2::cache_hint.u64 %0, [%1], %2;" : "=l"(r) : "l"(p), "l"(pol));
     return r;
 }
+__device__ __forceinline__ uint32_t ld_cg_keep_u32(const uint32_t* p, uint64_t pol) {
+    uint32_t r;
+    asm volatile("ld.global.cg.L2::cache_hint.u32 %0, [%1], %2;" : "=r"(r) : "l"(p), "l"(pol));
+    return r;
+}
 __device__ __forceinline__ unsigned long long atom_min_keep_u64(unsigned long long* p, unsigned long long v,
                                                                 uint64_t pol) {
     unsigned long long old;
