@@ -18,6 +18,7 @@
 #include <atomic>
 #include <mutex>
 
+#include "cluster_dev.cuh"
 #include "internal.cuh"
 #include "prof.cuh"
 
@@ -500,6 +501,309 @@ cldiam_status launch_wl(uint32_t k, const uint64_t* off, const uint32_t* col, co
     return CLDIAM_OK;
 }
 
+// ---------------------------------------------------------------- diameter of a symmetric quotient by bounds
+// The largest distance needs the eccentricity of few nodes: after an exact SSSP from s every node v has
+// max(d(s, v), ecc(s) - d(s, v)) <= ecc(v) <= d(s, v) + ecc(s) (Takes and Kosters, "Determining the diameter of small
+// world networks", CIKM 2011), so a node whose upper bound does not exceed the largest eccentricity seen cannot hold
+// the diameter.  Batches of sources run until no node is left: first an even sample of the ids, then the nodes of the
+// largest upper and of the smallest lower bounds.  Two or three batches are enough on meshes,
+// road meshes and R-MAT graphs alike, whatever k is.
+// One CTA per source, so that a round costs little: the nodes improved in the last round are a list in shared memory,
+// their adjacency is one flattened range (a block scan of the degrees), and each warp takes 128 positions of it; an SSSP
+// on a road mesh's quotient (k = 4,082, 98,000 entries) is 12 to 20 rounds and 140,000 positions, bound by the issue
+// and latency of the position lookups and shared atomics.  Every source by the worklist above / bounds: road mesh
+// 4,096^2 2,702 / 1,082 us, R-MAT 24 (k = 4,023) 2,617 / 390 us, R-MAT 22 (k = 1,897) 354 / 107 us, 1,001^2 mesh
+// (k = 840) 269 / 168 us.
+struct BoundCtl {
+    unsigned long long wsum;  // sum over nodes of their heaviest entry
+    uint32_t wmax;
+    uint32_t wide;            // a path might reach 2^32 - 1: nothing is pruned, the caller takes every source
+    uint32_t nsrc;            // sources of the next batch
+    uint32_t best;            // largest eccentricity so far
+    uint32_t err;             // an SSSP exceeded its round limit
+    uint32_t pad;
+};
+constexpr uint32_t kBoundFirst = 152, kBoundNext = 304;  // sources of the first and of later batches
+
+// heaviest entry of every row, and the first sources
+__global__ void __launch_bounds__(256) k_bound_prep(const uint64_t* __restrict__ off, const uint32_t* __restrict__ w,
+                                                    uint32_t k, uint32_t nsrc, uint32_t* __restrict__ ub,
+                                                    uint32_t* __restrict__ lb, uint32_t* __restrict__ src,
+                                                    BoundCtl* ctl) {
+    const uint32_t warps = (gridDim.x * blockDim.x) >> 5, lane = lane_id();
+    unsigned long long sum = 0;
+    uint32_t mx = 0;
+    for (uint32_t v = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; v < k; v += warps) {
+        uint32_t m = 0;
+        for (uint64_t j = off[v] + lane; j < off[v + 1]; j += 32) m = max(m, w[j]);
+        m = __reduce_max_sync(0xffffffffu, m);
+        sum += m;
+        mx = max(mx, m);
+        if (lane == 0) {
+            ub[v] = INF;
+            lb[v] = 0;
+            if (v < nsrc) src[v] = (uint32_t)((uint64_t)v * k / nsrc);
+        }
+    }
+    if (lane == 0) {
+        atomicAdd(&ctl->wsum, sum);
+        atomicMax(&ctl->wmax, mx);
+        if (blockIdx.x == 0 && threadIdx.x == 0) ctl->nsrc = nsrc;
+    }
+}
+
+template <int T>
+struct BoundSmem {  // one tile of a round's list
+    uint32_t pre[T + 1];  // first positions of the nodes after the tile's first
+    uint32_t base[T];
+    uint32_t dist[T];
+    uint32_t wsum[T / 32];
+    uint32_t total, count[2];
+};
+
+// Largest distance from src[blockIdx.x], and the bounds it gives every node (ub only falls, lb only rises).
+template <int T>
+__global__ void __launch_bounds__(T) k_bound_sssp(const uint64_t* __restrict__ off, const uint32_t* __restrict__ col,
+                                                    const uint32_t* __restrict__ w, uint32_t k,
+                                                    const uint32_t* __restrict__ src, uint32_t* __restrict__ ub,
+                                                    uint32_t* __restrict__ lb, BoundCtl* ctl) {
+    extern __shared__ __align__(16) uint32_t sm[];
+    __shared__ BoundSmem<T> s;
+    // a stored distance is the length of a simple path, at most the sum of its nodes' heaviest entries
+    if (ctl->wsum + ctl->wmax >= 0xFFFFFFFFull) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) ctl->wide = 1;
+        return;
+    }
+    if (blockIdx.x >= ctl->nsrc) return;
+    const uint32_t words = (k + 31) / 32;
+    uint32_t* dist = sm;               // [k]
+    uint32_t* listed = dist + k;       // bit v: v is in the next list
+    uint32_t* soff = listed + words;   // [k + 1] row starts
+    uint16_t* list[2];
+    list[0] = reinterpret_cast<uint16_t*>(soff + k + 1);
+    list[1] = list[0] + k;
+    const uint32_t tid = threadIdx.x, warp = tid >> 5, lane = lane_id();
+    const unsigned le_mask = 0xffffffffu >> (31u - lane);
+    const uint32_t source = src[blockIdx.x];
+    for (uint32_t v = tid; v < k; v += T) dist[v] = v == source ? 0u : INF;
+    for (uint32_t v = tid; v <= k; v += T) soff[v] = (uint32_t)off[v];
+    for (uint32_t i = tid; i < words; i += T) listed[i] = 0;
+    if (tid == 0) {
+        list[0][0] = (uint16_t)source;
+        s.count[0] = 1;
+        s.count[1] = 0;
+    }
+    __syncthreads();
+    const uint32_t max_rounds = 4 * k + 64;  // far above any real count: a guard, reported as an error
+    for (uint32_t round = 0;; ++round) {
+        const uint32_t c = round & 1;
+        const uint32_t m = s.count[c];
+        if (m == 0) break;
+        if (round > max_rounds) {
+            if (tid == 0) atomicExch(&ctl->err, 1u);
+            break;
+        }
+        for (uint32_t t0 = 0; t0 < m; t0 += T) {
+            // the tile's nodes: taken off the list before their distance is read, so a later improvement lists them again
+            const uint32_t mt = min(m - t0, (uint32_t)T);
+            uint32_t deg = 0, b0 = 0, d = 0;
+            if (tid < mt) {
+                const uint32_t v = list[c][t0 + tid];
+                atomicAnd(&listed[v >> 5], ~(1u << (v & 31)));
+                d = atomicAdd(&dist[v], 0u);
+                b0 = soff[v];
+                deg = soff[v + 1] - b0;
+            }
+            const uint32_t incl = warp_incl_scan(deg);
+            if (lane == 31) s.wsum[warp] = incl;
+            __syncthreads();
+            uint32_t before = 0, total = 0;
+#pragma unroll
+            for (uint32_t i = 0; i < T / 32; ++i) {
+                const uint32_t x = s.wsum[i];
+                before += i < warp ? x : 0u;
+                total += x;
+            }
+            if (tid < mt) {
+                const uint32_t pre = before + incl - deg;
+                if (tid > 0) s.pre[tid - 1] = pre;
+                s.base[tid] = b0 - pre;
+                s.dist[tid] = d;
+            }
+            __syncthreads();
+            for (uint32_t p0 = warp * PW; p0 < total; p0 += (T / 32) * PW) {
+                // owner of p0: the number of later nodes that start at or before it
+                uint32_t B = 0, len = mt - 1;
+                while (len > 0) {
+                    const uint32_t step = (len + 31) / 32;
+                    const uint32_t at = (lane + 1) * step;  // probes the last of each piece
+                    const bool in = at <= len ? s.pre[B + at - 1] <= p0 : false;
+                    const uint32_t n_in = (uint32_t)__popc(__ballot_sync(0xffffffffu, in));
+                    B += n_in * step;
+                    len = min(step - 1, len - n_in * step);
+                }
+                // (the entries of all four groups are loaded before any is used)
+                uint32_t own[PWG], v[PWG], nd[PWG];
+#pragma unroll
+                for (int u = 0; u < PWG; ++u)
+                    B += (uint32_t)__popc(group_starts(s.pre + B, mt - 1 - B, p0 + 32u * u, B, lane, le_mask, &own[u]));
+#pragma unroll
+                for (int u = 0; u < PWG; ++u) {
+                    const uint32_t p = p0 + 32u * u + lane;
+                    v[u] = source;
+                    nd[u] = INF;
+                    if (p < total) {
+                        const uint32_t j = s.base[own[u]] + p;
+                        v[u] = __ldg(col + j);
+                        nd[u] = s.dist[own[u]] + __ldg(w + j);
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < PWG; ++u) {
+                    bool put = false;
+                    if (nd[u] < dist[v[u]] && nd[u] < atomicMin(&dist[v[u]], nd[u])) {
+                        const uint32_t bit = 1u << (v[u] & 31);
+                        put = !(atomicOr(&listed[v[u] >> 5], bit) & bit);
+                    }
+                    const unsigned pm = __ballot_sync(0xffffffffu, put);
+                    if (pm) {
+                        uint32_t at = 0;
+                        if (lane == 0) at = atomicAdd(&s.count[c ^ 1], (uint32_t)__popc(pm));
+                        at = __shfl_sync(0xffffffffu, at, 0);
+                        if (put) list[c ^ 1][at + (uint32_t)__popc(pm & lanemask_lt())] = (uint16_t)v[u];
+                    }
+                }
+            }
+            __syncthreads();
+        }
+        if (tid == 0) s.count[c] = 0;
+        __syncthreads();
+    }
+    uint32_t ecc = 0;
+    for (uint32_t v = tid; v < k; v += T) ecc = dist[v] != INF ? max(ecc, dist[v]) : ecc;
+    ecc = block_reduce(ecc, [](uint32_t a, uint32_t b) { return a > b ? a : b; }, 0u);
+    if (tid == 0) {
+        s.total = ecc;
+        atomicMax(&ctl->best, ecc);
+    }
+    __syncthreads();
+    ecc = s.total;
+    for (uint32_t v = tid; v < k; v += T) {
+        const uint32_t d = dist[v];
+        if (d == INF) continue;
+        const uint32_t hi = (uint32_t)min((uint64_t)d + ecc, (uint64_t)(INF - 1)), lo = max(d, ecc - d);
+        if (hi < ub[v]) atomicMin(&ub[v], hi);
+        if (lo > lb[v]) atomicMax(&lb[v], lo);
+    }
+}
+
+// Sources of the next batch (one CTA): every node whose upper bound exceeds the best eccentricity, or, when these are
+// more than `most`, half of the batch from the largest upper bounds among them and half from the smallest lower bounds
+// of all nodes with unknown eccentricity (thresholds by bisection over the value).
+__global__ void __launch_bounds__(1024) k_bound_select(uint32_t k, uint32_t most, const uint32_t* __restrict__ ub,
+                                                       const uint32_t* __restrict__ lb, uint32_t* __restrict__ src,
+                                                       BoundCtl* ctl) {
+    __shared__ uint32_t s_n;
+    if (ctl->wide || ctl->nsrc == 0) return;
+    const uint32_t best = ctl->best;
+    const auto count = [&](auto&& pred) -> uint32_t {  // nodes for which pred holds, at every thread
+        __syncthreads();
+        if (threadIdx.x == 0) s_n = 0;
+        __syncthreads();
+        uint32_t c = 0;
+        for (uint32_t v = threadIdx.x; v < k; v += blockDim.x) c += pred(v) ? 1u : 0u;
+        c = __reduce_add_sync(0xffffffffu, c);
+        if (lane_id() == 0 && c) atomicAdd(&s_n, c);
+        __syncthreads();
+        return s_n;
+    };
+    const uint32_t open = count([&](uint32_t v) { return ub[v] > best; });
+    uint32_t hi_from = best + 1, lo_to = 0;  // take ub >= hi_from; lb < lo_to
+    if (open > most) {
+        uint32_t a = best + 1, b = INF;  // largest t with at least half of a batch at or above it
+        while (a < b) {
+            const uint32_t mid = a + (b - a) / 2 + 1;
+            if (count([&](uint32_t v) { return ub[v] >= mid; }) >= most / 2) a = mid;
+            else b = mid - 1;
+        }
+        hi_from = a;
+        a = 0;
+        b = INF;  // smallest t with at least half of a batch below it
+        while (a < b) {
+            const uint32_t mid = a + (b - a) / 2;
+            if (count([&](uint32_t v) { return ub[v] > lb[v] && lb[v] < mid; }) >= most / 2) b = mid;
+            else a = mid + 1;
+        }
+        lo_to = a;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) s_n = 0;
+    __syncthreads();
+    for (int part = 0; part < 2; ++part) {
+        const uint32_t cap = open <= most || part == 1 ? most : most / 2;
+        for (uint32_t v = threadIdx.x; v < k; v += blockDim.x) {
+            const bool high = ub[v] > best && ub[v] >= hi_from, low = ub[v] > lb[v] && lb[v] < lo_to;
+            if (part == 0 ? high : low && !high) {
+                const uint32_t at = atomicAdd(&s_n, 1u);
+                if (at < cap) src[at] = v;
+            }
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) s_n = min(s_n, cap);
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) ctl->nsrc = s_n;
+}
+
+size_t bound_smem(uint32_t k) { return (size_t)k * 12 + 4 + (size_t)((k + 31) / 32) * 4; }
+constexpr size_t kBoundSmemMax = 208 * 1024;  // beside the static tile
+
+// Largest distance of a symmetric quotient by bounds; *done = false when a path might reach 2^32 - 1 (every source must
+// then be looked at, in the caller's checked form).
+cldiam_status bound_diameter(uint32_t k, const uint64_t* off, const uint32_t* col, const uint32_t* w, cudaStream_t s,
+                             uint64_t* phi, bool* done) {
+    static std::atomic<bool> attr[64];  // first call per device sets the attribute (idempotent)
+    int dev = 0;
+    CLD_CUDA(cudaGetDevice(&dev));
+    if (dev < 0 || dev >= 64 || !attr[dev]) {
+        const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
+        CLD_CUDA(cudaFuncSetAttribute(k_bound_sssp<512>, a, (int)kBoundSmemMax));
+        CLD_CUDA(cudaFuncSetAttribute(k_bound_sssp<1024>, a, (int)kBoundSmemMax));
+        if (dev >= 0 && dev < 64) attr[dev] = true;
+    }
+    *done = false;
+    DBuf<uint32_t> bounds, src;
+    DBuf<BoundCtl> ctl;
+    CLD_TRY(bounds.alloc(2 * (size_t)k, s));
+    CLD_TRY(src.alloc(kBoundNext, s));
+    CLD_TRY(ctl.alloc(1, s));
+    uint32_t *ub = bounds.get(), *lb = bounds.get() + k;
+    CLD_CUDA(cudaMemsetAsync(ctl.get(), 0, sizeof(BoundCtl), s));
+    uint32_t n = std::min(k, kBoundFirst);
+    CLD_K(K_FW, s, k_bound_prep<<<grid_for((size_t)k * 32, 256), 256, 0, s>>>(off, w, k, n, ub, lb, src.get(), ctl.get()));
+    BoundCtl h{};
+    do {
+        // most graphs are done after two or three batches: three are queued before the host looks
+        for (int i = 0; i < 3; ++i) {
+            // (three batches with 512 / 1,024 threads: k = 840 168 / 224 us, k = 1,897 126 / 107, k = 4,082 1,261 / 1,082)
+            if (k < 1536)
+                CLD_K(K_FW, s, k_bound_sssp<512><<<n, 512, bound_smem(k), s>>>(off, col, w, k, src.get(), ub, lb, ctl.get()));
+            else
+                CLD_K(K_FW, s, k_bound_sssp<1024><<<n, 1024, bound_smem(k), s>>>(off, col, w, k, src.get(), ub, lb,
+                                                                                 ctl.get()));
+            CLD_K(K_FW, s, k_bound_select<<<1, 1024, 0, s>>>(k, kBoundNext, ub, lb, src.get(), ctl.get()));
+            n = std::min(k, kBoundNext);
+        }
+        CLD_LAUNCH_CHECK();
+        CLD_CUDA(cudaMemcpyAsync(&h, ctl.get(), sizeof h, cudaMemcpyDeviceToHost, s));
+        CLD_CUDA(cudaStreamSynchronize(s));
+        if (h.err) return fail(CLDIAM_ERR_DIVERGED, "quotient SSSP exceeded its round limit");
+    } while (!h.wide && h.nsrc > 0);
+    *done = !h.wide;
+    *phi = h.best;
+    return CLDIAM_OK;
+}
+
 // Blocked Floyd-Warshall over the padded kp x kp matrix M in the given form; scal[0] = overflow
 // (checked form), scal[1] = largest finite distance, scal[3] = wide weight, scal[4] = unconnected pair.
 template <bool FAST>
@@ -564,6 +868,14 @@ cldiam_status apsp_max_device(uint32_t k, const uint64_t* off, const uint32_t* c
     bool sparse = (double)nnz * (double)tun.apsp_fw_density < (double)k * k;
     if (!sparse && k > max_fw_k) sparse = (double)nnz * 8.0 < (double)k * k;
     const SparsePlan plan = sparse ? sparse_plan(k, tun.apsp_sources_per_cta) : SparsePlan::kNone;
+    // A quotient built here (not validated: symmetric by construction) takes the bounds, unless a knob sets the
+    // sources per CTA; a caller's CSR is not checked for symmetry, which the bounds rely on, so it takes every source.
+    // (Up to one batch of nodes there is nothing to leave out: the worklist is faster, 17 against 37 us at k = 59.)
+    if (sparse && !validate && tun.apsp_sources_per_cta == 0 && k > kBoundFirst && k <= 65535u && bound_smem(k) <= kBoundSmemMax) {
+        bool done = false;
+        CLD_TRY(bound_diameter(k, off, col, w, s, phi, &done));
+        if (done) return CLDIAM_OK;
+    }
     if (plan == SparsePlan::kWorklist8) {
         CLD_TRY(launch_wl<8>(k, off, col, w, nnz, s, scal.get() + 1, scal.get(), scal.get() + 5));
     } else if (plan == SparsePlan::kWorklist4) {
