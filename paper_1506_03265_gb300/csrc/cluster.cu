@@ -751,7 +751,7 @@ cldiam_status cluster(cldiam_graph* g, double tau, uint64_t seed, const cldiam_o
     Counters* hc = static_cast<Counters*>(g->host.h);
     static_assert(sizeof(Counters) <= 128 && sizeof(GrowState) <= 128, "the read-back blocks must fit the pinned area");
 
-    const unsigned gb = grid_for(n, 256);
+    const unsigned gb = grid_for(n, 256), gn = grid_for(((size_t)n + NU - 1) / NU, 256);
     CLD_K(K_MISC, s, k_cluster_init<<<gb, 256, 0, s>>>(n, center.get(), D.get(), R.get(), stamp.get(), key.get(),
                                                         keyS.get()));
     CLD_LAUNCH_CHECK();
@@ -877,7 +877,7 @@ cldiam_status cluster(cldiam_graph* g, double tau, uint64_t seed, const cldiam_o
     auto rebuild = [&]() -> cldiam_status {
         const bool pull = pull_ok && (g->nnz - gs.frozen_deg) < gs.frozen_deg;
         CLD_TRY(zero_field(offsetof(Counters, front), 8));
-        CLD_K(K_REBUILD, s, k_rebuild<<<gb, 256, 0, s>>>(n, key.get(), center.get(), cumulative ? D.get() : nullptr,
+        CLD_K(K_REBUILD, s, k_rebuild<<<gn, 256, 0, s>>>(n, key.get(), center.get(), cumulative ? D.get() : nullptr,
                                                           g->off, gs.delta, pull, fv[gs.cur], fk[gs.cur], fp[gs.cur],
                                                           cf[gs.cur], ctr.get()));
         CLD_LAUNCH_CHECK();
@@ -917,7 +917,7 @@ cldiam_status cluster(cldiam_graph* g, double tau, uint64_t seed, const cldiam_o
             // selection + reset, then the stage's first frontier
             CLD_TRY(zero_field(offsetof(Counters, selected), 8));
             CLD_TRY(zero_field(offsetof(Counters, unfrozen), 8));
-            CLD_K(K_SELECT, s, k_select<<<gb, 256, 0, s>>>(n, center.get(), key.get(), seed, gs.stage, thr, ctr.get(),
+            CLD_K(K_SELECT, s, k_select<<<gn, 256, 0, s>>>(n, center.get(), key.get(), seed, gs.stage, thr, ctr.get(),
                                                             keyS.get()));
             CLD_LAUNCH_CHECK();
             CLD_TRY(rebuild());
@@ -1005,7 +1005,7 @@ cldiam_status cluster(cldiam_graph* g, double tau, uint64_t seed, const cldiam_o
 
             // assign and contract
             CLD_TRY(zero_field(offsetof(Counters, frozen), 16));  // frozen + frozen_deg
-            CLD_K(K_FINALIZE, s, k_finalize_d<<<gb, 256, 0, s>>>(n, key.get(), center.get(), cumulative ? nullptr : R.get(),
+            CLD_K(K_FINALIZE, s, k_finalize_d<<<gn, 256, 0, s>>>(n, key.get(), center.get(), cumulative ? nullptr : R.get(),
                                                                  D.get(), ctr.get()));
             CLD_K(K_FINALIZE, s, k_finalize_freeze<<<gb, 256, 0, s>>>(n, key.get(), center.get(), R.get(), D.get(), g->off,
                                                                       ctr.get(), keyS.get(), cumulative));

@@ -101,6 +101,43 @@ __device__ __forceinline__ void front_append(unsigned long long* ctr, bool pred,
     __syncthreads();
 }
 
+// The same for NC candidate entries per thread (bit j of `kinds` set: entry j of deg[j] positions is taken), in the
+// order entry 0 of every lane, entry 1 of every lane, ...: a warp's entries stay consecutive per j, so the writes of
+// the frontier arrays are coalesced.
+template <int NC>
+__device__ __forceinline__ void front_append_n(unsigned long long* ctr, uint32_t kinds, const uint32_t (&deg)[NC],
+                                               uint32_t (&slot)[NC], uint32_t (&pre)[NC], unsigned long long* scratch) {
+    const unsigned w = threadIdx.x >> 5, l = lane_id(), nw = blockDim.x >> 5;
+    uint32_t wc = 0, wd = 0;  // the warp's entries and positions so far
+#pragma unroll
+    for (int j = 0; j < NC; ++j) {
+        const bool p = (kinds >> j) & 1u;
+        const unsigned mask = __ballot_sync(0xffffffffu, p);
+        const uint32_t d = p ? deg[j] : 0u;
+        const uint32_t incl = warp_incl_scan(d);
+        slot[j] = wc + (uint32_t)__popc(mask & lanemask_lt());
+        pre[j] = wd + incl - d;
+        wc += (uint32_t)__popc(mask);
+        wd += __shfl_sync(0xffffffffu, incl, 31);
+    }
+    if (l == 31) scratch[w] = ((unsigned long long)wc << 32) | wd;
+    __syncthreads();
+    if (w == 0) {
+        const unsigned long long v = l < nw ? scratch[l] : 0ull;
+        const unsigned long long iv = warp_incl_scan(v);
+        if (l < nw) scratch[l] = iv - v;
+        if (l == 31) scratch[32] = iv ? atomicAdd(ctr, iv) : 0ull;
+    }
+    __syncthreads();
+    const unsigned long long at = scratch[32] + scratch[w];
+#pragma unroll
+    for (int j = 0; j < NC; ++j) {
+        slot[j] += (uint32_t)(at >> 32);
+        pre[j] += (uint32_t)at;
+    }
+    __syncthreads();
+}
+
 // ---------------------------------------------------------------- warp-chunk sweeps
 // The one-graph kernels that sweep a flattened range of positions (a
 // frontier's adjacency, or the whole CSR) give each warp PW consecutive
@@ -159,15 +196,35 @@ struct WarpNext {
     }
 };
 
+// Passes over every node (or every changed node) give each thread NU of them a block apart and issue the loads of each
+// level for all NU before the next level, one append per NU: with one node per thread and iteration the dependent
+// loads and the append's barriers set the time (n = 16.8M: listing 136 -> 92 us, draw 33 -> 29, bounds of the
+// contraction 41 -> 32; its freezing pass, 54 us, became slower, 67, and keeps one).
+// Nodes that the threads hold one each stay one per thread, so that they spread over all of them.
+constexpr uint32_t NU = 4;
+__device__ __forceinline__ uint32_t nodes_per_thread(uint32_t n, uint32_t nb) {
+    return (uint64_t)n > (uint64_t)nb * blockDim.x ? NU : 1u;
+}
+
 // a3: draw the new centers of this stage among unfrozen nodes, reset the others.
 __device__ __forceinline__ void dev_select(uint32_t n, const uint32_t* __restrict__ center,
                                            unsigned long long* __restrict__ key, uint64_t seed, uint32_t stage,
                                            uint64_t thr, Counters* ctr, uint32_t br, uint32_t nb,
                                            unsigned long long* __restrict__ keyS = nullptr) {
     unsigned long long cnt = 0, unfrozen = 0;
-    for (uint32_t base = br * blockDim.x; base < n; base += nb * blockDim.x) {
-        const uint32_t v = base + threadIdx.x;
-        if (v < n && __ldcg(&center[v]) == kNone) {
+    const uint32_t per = nodes_per_thread(n, nb);
+    const uint64_t stride = (uint64_t)nb * blockDim.x * per;
+    for (uint64_t base = (uint64_t)br * blockDim.x * per; base < n; base += stride) {
+        uint32_t c[NU];
+#pragma unroll
+        for (uint32_t u = 0; u < NU; ++u) {
+            const uint64_t v = base + u * blockDim.x + threadIdx.x;
+            c[u] = u < per && v < n ? __ldcg(&center[v]) : 0u;
+        }
+#pragma unroll
+        for (uint32_t u = 0; u < NU; ++u) {
+            const uint32_t v = (uint32_t)base + u * blockDim.x + threadIdx.x;  // < n where c[u] is kNone
+            if (c[u] != kNone) continue;
             const U4 r = philox4x32_10(seed, v, stage, 0u, 0u);
             const bool sel = (uint64_t)r.x < thr;
             key[v] = sel ? (unsigned long long)v : kInfKey;
@@ -192,42 +249,57 @@ __device__ __forceinline__ void dev_rebuild(uint32_t n, const unsigned long long
                                             unsigned long long* __restrict__ fkey, uint32_t* __restrict__ fpre,
                                             uint32_t* __restrict__ cfirst, Counters* ctr, unsigned long long* scratch,
                                             uint32_t br, uint32_t nb) {
-    for (uint32_t base = br * blockDim.x; base < n; base += nb * blockDim.x) {
-        const uint32_t v = base + threadIdx.x;
-        bool push = false, pl = false;
-        unsigned long long k = 0;
-        uint32_t deg = 0, b0 = 0;
-        if (v < n) {
-            const uint64_t o = off[v];
-            b0 = (uint32_t)o;
-            deg = (uint32_t)(off[v + 1] - o);
-            const uint32_t c = __ldcg(&center[v]);
-            if (deg > 0) {
-                if (c != kNone) {
-                    const uint32_t dd = Dcum ? __ldcg(&Dcum[v]) : 0u;  // (0, c_u), or (D_u, c_u) cumulative
-                    push = !pull && dd < delta;
-                    k = ((unsigned long long)dd << 32) | c;
-                } else {
-                    k = __ldcg(&key[v]);
-                    push = k != kInfKey && (uint32_t)(k >> 32) < delta;
-                    pl = pull;
-                }
+    const uint32_t per = nodes_per_thread(n, nb);
+    const uint64_t stride = (uint64_t)nb * blockDim.x * per;
+    for (uint64_t base = (uint64_t)br * blockDim.x * per; base < n; base += stride) {
+        uint32_t c[NU], b0[NU], deg[NU];
+        unsigned long long k[NU];
+#pragma unroll
+        for (uint32_t u = 0; u < NU; ++u) {
+            const uint64_t v = base + u * blockDim.x + threadIdx.x;
+            c[u] = 0;
+            k[u] = kInfKey;
+            b0[u] = deg[u] = 0;
+            if (u < per && v < n) {
+                const uint64_t o = off[v];
+                b0[u] = (uint32_t)o;
+                deg[u] = (uint32_t)(off[v + 1] - o);
+                c[u] = __ldcg(&center[v]);
             }
         }
-        uint32_t slot = 0, pre = 0;
-        front_append(&ctr->front, push, deg, slot, pre, scratch);
-        if (push) {
-            fbase[slot] = b0 - pre;
-            fkey[slot] = k;
-            fpre[slot] = pre;
-            if (cfirst) chunk_table_put(cfirst, slot, pre, deg);
+#pragma unroll
+        for (uint32_t u = 0; u < NU; ++u) {
+            const uint64_t v = base + u * blockDim.x + threadIdx.x;
+            if (c[u] == kNone) k[u] = __ldcg(&key[v]);
         }
-        front_append(&ctr->front, pl, deg, slot, pre, scratch);
-        if (pl) {
-            fbase[slot] = b0 - pre;
-            fkey[slot] = kPullTag | v;
-            fpre[slot] = pre;
-            if (cfirst) chunk_table_put(cfirst, slot, pre, deg);
+        uint32_t pushes = 0, pulls = 0;
+#pragma unroll
+        for (uint32_t u = 0; u < NU; ++u) {
+            const uint64_t v = base + u * blockDim.x + threadIdx.x;
+            if (deg[u] == 0) continue;  // (also past the end)
+            bool push;
+            if (c[u] != kNone) {
+                const uint32_t dd = Dcum ? __ldcg(&Dcum[v]) : 0u;  // (0, c_u), or (D_u, c_u) cumulative
+                push = !pull && dd < delta;
+                k[u] = ((unsigned long long)dd << 32) | c[u];
+            } else {
+                push = k[u] != kInfKey && (uint32_t)(k[u] >> 32) < delta;
+                pulls |= (pull ? 1u : 0u) << u;
+            }
+            pushes |= (push ? 1u : 0u) << u;
+        }
+        for (int kind = 0; kind < (pull ? 2 : 1); ++kind) {
+            const uint32_t kinds = kind ? pulls : pushes;
+            uint32_t slot[NU], pre[NU];
+            front_append_n<NU>(&ctr->front, kinds, deg, slot, pre, scratch);
+#pragma unroll
+            for (uint32_t u = 0; u < NU; ++u) {
+                if (!((kinds >> u) & 1u)) continue;
+                fbase[slot[u]] = b0[u] - pre[u];
+                fkey[slot[u]] = kind ? kPullTag | (base + u * blockDim.x + threadIdx.x) : k[u];
+                fpre[slot[u]] = pre[u];
+                if (cfirst) chunk_table_put(cfirst, slot[u], pre[u], deg[u]);
+            }
         }
     }
 }
@@ -506,16 +578,34 @@ __device__ __forceinline__ void dev_growable(const uint32_t* __restrict__ row, c
 __device__ __forceinline__ void dev_finalize_d(uint32_t n, const unsigned long long* __restrict__ key,
                                                const uint32_t* __restrict__ center, const uint32_t* __restrict__ R,
                                                uint32_t* __restrict__ D, Counters* ctr, uint32_t br, uint32_t nb) {
-    for (uint32_t v = br * blockDim.x + threadIdx.x; v < n; v += nb * blockDim.x) {
-        if (__ldcg(&center[v]) != kNone) continue;
-        const unsigned long long k = __ldcg(&key[v]);
-        if (k == kInfKey) continue;
-        uint64_t dv = (k >> 32) + (R ? (uint64_t)__ldcg(&R[(uint32_t)k]) : 0ull);  // cumulative mode: R null
-        if (dv >= 0xFFFFFFFFull) {
-            atomicExch(&ctr->overflow, 1u);
-            dv = 0xFFFFFFFEull;
+    const uint32_t per = nodes_per_thread(n, nb);
+    const uint64_t stride = (uint64_t)nb * blockDim.x * per;
+    for (uint64_t base = (uint64_t)br * blockDim.x * per; base < n; base += stride) {
+        unsigned long long k[NU];
+        uint32_t r[NU];
+        bool take[NU];
+#pragma unroll
+        for (uint32_t u = 0; u < NU; ++u) {
+            const uint64_t v = base + u * blockDim.x + threadIdx.x;
+            take[u] = u < per && v < n && __ldcg(&center[v]) == kNone;
         }
-        D[v] = (uint32_t)dv;
+#pragma unroll
+        for (uint32_t u = 0; u < NU; ++u) k[u] = take[u] ? __ldcg(&key[base + u * blockDim.x + threadIdx.x]) : kInfKey;
+#pragma unroll
+        for (uint32_t u = 0; u < NU; ++u) {
+            take[u] = take[u] && k[u] != kInfKey;
+            r[u] = take[u] && R ? __ldcg(&R[(uint32_t)k[u]]) : 0u;  // cumulative mode: R null
+        }
+#pragma unroll
+        for (uint32_t u = 0; u < NU; ++u) {
+            if (!take[u]) continue;
+            uint64_t dv = (k[u] >> 32) + (uint64_t)r[u];
+            if (dv >= 0xFFFFFFFFull) {
+                atomicExch(&ctr->overflow, 1u);
+                dv = 0xFFFFFFFEull;
+            }
+            D[base + u * blockDim.x + threadIdx.x] = (uint32_t)dv;
+        }
     }
 }
 
