@@ -993,4 +993,12 @@ cldiam_status apsp_max_noalloc(uint32_t k, const uint64_t* off, const uint32_t* 
     return CLDIAM_OK;
 }
 
+cldiam_status load_apsp_kernels() {
+    return load_kernels(k_bound_prep, k_bound_sssp<512>, k_bound_sssp<1024>, k_bound_select, k_fw_init, k_fw_validate,
+                        k_fw_scatter, k_fw_phase1<true>, k_fw_phase1<false>, k_fw_phase2_fast, k_fw_phase2_checked,
+                        k_fw_phase3<true>, k_fw_phase3<false>, k_fw_max_finite, k_apsp_wl<8, true>, k_apsp_wl<8, false>,
+                        k_apsp_wl<4, true>, k_apsp_wl<4, false>, k_apsp_wl<1, true>, k_apsp_wl<1, false>,
+                        k_apsp_msbf<1, true>, k_apsp_msbf<1, false>);
+}
+
 }  // namespace cld

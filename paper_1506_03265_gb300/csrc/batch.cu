@@ -1025,6 +1025,7 @@ struct cldiam_server {
     std::deque<uint32_t> bq;
     bool bstop = false;
     cld::Pinned bhost;  // counter block of the big lane's one-graph runs
+    bool counted = false;  // counted among the device's live servers
 };
 
 namespace cld {
@@ -1096,8 +1097,10 @@ static void big_lane(cldiam_server* sv) {
 
 cldiam_status server_free(cldiam_server* sv);
 
-// Servers alive in this process: while one is, its persistent kernel may hold SMs, so CLUSTER keeps its
-// host-driven stage loop (a cooperative launch would wait for every SM).
+// Servers alive on each device: a server's persistent kernel holds its SMs until it has been idle for long, and the
+// few SMs it leaves need not include a cluster's worth in one GPC, so thread-block clusters are not launched beside it.
+static std::atomic<int> g_live_servers[64];
+bool serving_kernel_alive(int dev) { return dev < 0 || dev >= 64 || g_live_servers[dev].load() > 0; }
 
 cldiam_status server_create(cldiam_arena* a, const cldiam_server_opts* o, cldiam_server** out) {
     if (!a || !out) return fail(CLDIAM_ERR_INVALID_ARG, "NULL arena or out");
@@ -1165,8 +1168,14 @@ cldiam_status server_create(cldiam_arena* a, const cldiam_server_opts* o, cldiam
     sv->big_graph.resize(sv->cap);
     sv->big_tau.resize(sv->cap);
     sv->big_seed.resize(sv->cap);
+    for (auto load : {load_prims_kernels, load_csr_kernels, load_cluster_kernels, load_quotient_kernels, load_apsp_kernels})
+        if ((st = load()) != CLDIAM_OK) return cleanup(st);
     {
         std::lock_guard<std::mutex> lk(sv->mu);
+        if (sv->device >= 0 && sv->device < 64) {
+            g_live_servers[sv->device].fetch_add(1);
+            sv->counted = true;
+        }
         if ((st = server_launch(sv)) != CLDIAM_OK) return cleanup(st);
     }
     sv->big = std::thread(big_lane, sv);
@@ -1243,6 +1252,7 @@ cldiam_status server_free(cldiam_server* sv) {
     }
     if (sv->kstream) cudaStreamSynchronize(sv->kstream);
     if (sv->bstream) cudaStreamSynchronize(sv->bstream);
+    if (sv->counted) g_live_servers[sv->device].fetch_sub(1);
     dfree(sv->head, sv->kstream);
     dfree(sv->wss, sv->kstream);
     dfree(sv->descs, sv->kstream);

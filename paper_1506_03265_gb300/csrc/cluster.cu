@@ -807,7 +807,7 @@ cldiam_status cluster(cldiam_graph* g, double tau, uint64_t seed, const cldiam_o
         (unsigned)std::min<uint64_t>((uint64_t)num_sms() * pull_ctas, (pull_chunks + PT / 32 - 1) / (PT / 32));
     DBuf<uint32_t> rows_built;  // COO rows for the guard's edge scan when the graph keeps none
 
-    // Resident growth (k_grow): on connected graphs, unless a tuning knob asks for the grid kernels (a set number of
+    // Resident growth (k_grow): on connected graphs, while no server's kernel holds the SMs, unless a tuning knob asks for the grid kernels (a set number of
     // CTAs) or for the dense form at a share of the adjacency that the step reaches (a share other than the default).
     const int grow_ctas = g->connected && n >= 2 && g->nnz < 0xFFFFFFFFull && tun.relax_ctas_per_sm == 0 ? grow_cluster_size(dev) : 0;
     const bool strict_pull = pull_dense && tun.pull_ratio != tuning_defaults_filled(cldiam_tuning{}).pull_ratio;
@@ -897,7 +897,7 @@ cldiam_status cluster(cldiam_graph* g, double tau, uint64_t seed, const cldiam_o
 
     // Algorithm 1's loops as phases: a stage's draw, its growing steps one by one, and what follows when growth stops
     while (gs.phase != kPhaseDone) {
-        if (grow_ctas && (gs.phase == kPhaseStep ? gs.nf > 0 && gs.E <= grow_entries : grow_stages)) {
+        if (grow_ctas && !serving_kernel_alive(dev) && (gs.phase == kPhaseStep ? gs.nf > 0 && gs.E <= grow_entries : grow_stages)) {
             CLD_TRY(grow());
             if (gs.phase == kPhaseFailed) {
                 if (gs.stage > kMaxStages) return fail(CLDIAM_ERR_DIVERGED, "CLUSTER exceeded its stage limit");
@@ -1042,6 +1042,11 @@ cldiam_status cluster(cldiam_graph* g, double tau, uint64_t seed, const cldiam_o
     *out = cl;
     owner.c = nullptr;
     return CLDIAM_OK;
+}
+
+cldiam_status load_cluster_kernels() {
+    return load_kernels(k_cluster_init, k_pull_rows, k_select, k_rebuild, k_snapshot, k_push, k_pull, k_growable,
+                        k_finalize_d, k_finalize_freeze, k_singletons, k_center_flags, k_assign_cid);
 }
 
 }  // namespace cld

@@ -101,6 +101,24 @@ inline unsigned grid_for(size_t n, int block, int max_blocks_per_sm = 8) {
     return (unsigned)b;
 }
 
+// ---------------------------------------------------------------- kernel loading
+// The runtime loads a kernel's code at its first use, and that load waits for the kernels already running: beside a
+// server's persistent kernel, for as long as it lives.  A server therefore has every kernel of the one-graph path loaded
+// before its own is launched (asking for a kernel's attributes loads it).
+template <class... K>
+cldiam_status load_kernels(K... k) {
+    cudaFuncAttributes a;
+    cudaError_t e = cudaSuccess;
+    (void)((e = cudaFuncGetAttributes(&a, k), e == cudaSuccess) && ...);
+    CLD_CUDA(e);
+    return CLDIAM_OK;
+}
+cldiam_status load_prims_kernels();     // sorts, scans, reductions
+cldiam_status load_cluster_kernels();
+cldiam_status load_quotient_kernels();
+cldiam_status load_apsp_kernels();
+cldiam_status load_csr_kernels();       // the row array of a graph without one
+
 // ---------------------------------------------------------------- Philox4x32-10
 // Salmon, Moraes, Dror, Shaw, "Parallel random numbers: as easy as 1, 2, 3"
 // (SC'11).  Ten rounds of two 32x32->64 multiplies with the round constants

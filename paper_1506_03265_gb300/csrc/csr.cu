@@ -936,4 +936,8 @@ cldiam_status delta0(const cldiam_graph* g, int mode, uint32_t explicit_value, u
     return CLDIAM_OK;
 }
 
+cldiam_status load_csr_kernels() {
+    return load_kernels(k_fill_rows);
+}
+
 }  // namespace cld

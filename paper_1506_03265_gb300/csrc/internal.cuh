@@ -96,6 +96,8 @@ cldiam_status server_replay(cldiam_server* sv, const uint32_t* ids, const double
                             const double* arrival, uint32_t count, int plain, cldiam_result* out, double* latency,
                             double* elapsed);
 uint64_t arena_device_bytes(const cldiam_arena* a);
+// a server's persistent kernel may hold SMs of device `dev` (no thread-block cluster should be launched beside it)
+bool serving_kernel_alive(int dev);
 cudaStream_t arena_stream(const cldiam_arena* a);
 
 cldiam_status arena_job_times(const cldiam_arena* a, uint32_t count, double* start_s, double* end_s);

@@ -1073,4 +1073,12 @@ cldiam_status radix_sort_pairs_u32(uint32_t* keys, uint32_t* vals, uint32_t* key
     return radix_sort_impl<uint32_t>(keys, vals, keys_alt, vals_alt, n, 0, bits, in_alt, s);
 }
 
+cldiam_status load_prims_kernels() {
+    return load_kernels(k_tile_reduce<uint32_t>, k_tile_scan<uint32_t>, k_tile_reduce<uint64_t>, k_tile_scan<uint64_t>,
+                        k_offsets_from_rows, k_reduce_max_u32, k_reduce_min_u32, k_reduce_sum_u32, k_os_hist<uint32_t>,
+                        k_os_hist<uint64_t>, k_os_hist_scan, k_os_pass<uint32_t, true, false>,
+                        k_os_pass<uint64_t, true, false>, k_os_pass<uint64_t, true, true>, k_unique_count<uint32_t>,
+                        k_unique_count<uint64_t>, k_unique_write<uint32_t>, k_unique_write<uint64_t>);
+}
+
 }  // namespace cld

@@ -410,4 +410,9 @@ cldiam_status quotient(const cldiam_clustering* c, cldiam_quotient** out) {
     return CLDIAM_OK;
 }
 
+cldiam_status load_quotient_kernels() {
+    return load_kernels(k_q_pack_cd, k_q_emit<uint32_t>, k_q_emit<uint64_t>, k_q_dense_emit, k_q_rows,
+                        k_q_dense_emit_chunks, k_q_dense_mirror, k_q_dense_count, k_q_dense_fill, k_q_widen);
+}
+
 }  // namespace cld
