@@ -18,6 +18,7 @@
 #include <atomic>
 #include <mutex>
 
+#include "bounds.cuh"
 #include "cluster_dev.cuh"
 #include "internal.cuh"
 #include "prof.cuh"
@@ -502,12 +503,9 @@ cldiam_status launch_wl(uint32_t k, const uint64_t* off, const uint32_t* col, co
 }
 
 // ---------------------------------------------------------------- diameter of a symmetric quotient by bounds
-// The largest distance needs the eccentricity of few nodes: after an exact SSSP from s every node v has
-// max(d(s, v), ecc(s) - d(s, v)) <= ecc(v) <= d(s, v) + ecc(s) (Takes and Kosters, "Determining the diameter of small
-// world networks", CIKM 2011), so a node whose upper bound does not exceed the largest eccentricity seen cannot hold
-// the diameter.  Batches of sources run until no node is left: first an even sample of the ids, then the nodes of the
-// largest upper and of the smallest lower bounds.  Two or three batches are enough on meshes,
-// road meshes and R-MAT graphs alike, whatever k is.
+// The largest distance needs the eccentricity of few nodes (bounds.cuh).  Batches of sources run until no node is left:
+// first an even sample of the ids, then the nodes of the largest upper and of the smallest lower bounds.  Two or three
+// batches are enough on meshes, road meshes and R-MAT graphs alike, whatever k is.
 // One CTA per source, so that a round costs little: the nodes improved in the last round are a list in shared memory,
 // their adjacency is one flattened range (a block scan of the degrees), and each warp takes 128 positions of it; an SSSP
 // on a road mesh's quotient (k = 4,082, 98,000 entries) is 12 to 20 rounds and 140,000 positions, bound by the issue
@@ -697,62 +695,13 @@ __global__ void __launch_bounds__(T) k_bound_sssp(const uint64_t* __restrict__ o
     }
 }
 
-// Sources of the next batch (one CTA): every node whose upper bound exceeds the best eccentricity, or, when these are
-// more than `most`, half of the batch from the largest upper bounds among them and half from the smallest lower bounds
-// of all nodes with unknown eccentricity (thresholds by bisection over the value).
 __global__ void __launch_bounds__(1024) k_bound_select(uint32_t k, uint32_t most, const uint32_t* __restrict__ ub,
                                                        const uint32_t* __restrict__ lb, uint32_t* __restrict__ src,
                                                        BoundCtl* ctl) {
     __shared__ uint32_t s_n;
     if (ctl->wide || ctl->nsrc == 0) return;
-    const uint32_t best = ctl->best;
-    const auto count = [&](auto&& pred) -> uint32_t {  // nodes for which pred holds, at every thread
-        __syncthreads();
-        if (threadIdx.x == 0) s_n = 0;
-        __syncthreads();
-        uint32_t c = 0;
-        for (uint32_t v = threadIdx.x; v < k; v += blockDim.x) c += pred(v) ? 1u : 0u;
-        c = __reduce_add_sync(0xffffffffu, c);
-        if (lane_id() == 0 && c) atomicAdd(&s_n, c);
-        __syncthreads();
-        return s_n;
-    };
-    const uint32_t open = count([&](uint32_t v) { return ub[v] > best; });
-    uint32_t hi_from = best + 1, lo_to = 0;  // take ub >= hi_from; lb < lo_to
-    if (open > most) {
-        uint32_t a = best + 1, b = INF;  // largest t with at least half of a batch at or above it
-        while (a < b) {
-            const uint32_t mid = a + (b - a) / 2 + 1;
-            if (count([&](uint32_t v) { return ub[v] >= mid; }) >= most / 2) a = mid;
-            else b = mid - 1;
-        }
-        hi_from = a;
-        a = 0;
-        b = INF;  // smallest t with at least half of a batch below it
-        while (a < b) {
-            const uint32_t mid = a + (b - a) / 2;
-            if (count([&](uint32_t v) { return ub[v] > lb[v] && lb[v] < mid; }) >= most / 2) b = mid;
-            else a = mid + 1;
-        }
-        lo_to = a;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) s_n = 0;
-    __syncthreads();
-    for (int part = 0; part < 2; ++part) {
-        const uint32_t cap = open <= most || part == 1 ? most : most / 2;
-        for (uint32_t v = threadIdx.x; v < k; v += blockDim.x) {
-            const bool high = ub[v] > best && ub[v] >= hi_from, low = ub[v] > lb[v] && lb[v] < lo_to;
-            if (part == 0 ? high : low && !high) {
-                const uint32_t at = atomicAdd(&s_n, 1u);
-                if (at < cap) src[at] = v;
-            }
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) s_n = min(s_n, cap);
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) ctl->nsrc = s_n;
+    const uint32_t n = bound_select(k, most, ctl->best, ub, lb, src, s_n);
+    if (threadIdx.x == 0) ctl->nsrc = n;
 }
 
 size_t bound_smem(uint32_t k) { return (size_t)k * 12 + 4 + (size_t)((k + 31) / 32) * 4; }

@@ -22,7 +22,8 @@
 #include <thread>
 #include <vector>
 
-#include "cluster_dev.cuh"
+#include "bounds.cuh"
+#include "grow.cuh"
 #include "internal.cuh"
 #include "prof.cuh"
 
@@ -35,8 +36,9 @@ namespace {
 // 2,000-graph mixture but 1.6x the time per large graph on one CTA, and its 111 R-MAT 16 graphs set the
 // tail (17.4k against 25.4k graphs/s)
 constexpr int kBatchCtasPerSm = 1;
-constexpr int BT = 1024 / kBatchCtasPerSm;  // threads per CTA
-constexpr int kRelaxU = 1024 / BT;          // positions per thread of a growing-step chunk (1,024 per chunk)
+constexpr int BT = GT;  // threads per CTA: those of the growth loop
+constexpr int BW = BT / 32;
+constexpr int kJobCtas = 8;  // CTAs that share a large job: the portable cluster size
 constexpr uint32_t kDenseCap = 1024;  // largest quotient deduplicated in the dense matrix
 constexpr uint64_t kSplitMinEntries = 1u << 16;  // graphs below this many entries always stay in the launch
 // makespan model of the many-graph split (GB300): seconds per unit of work (entry or node) on one 1,024-thread
@@ -71,7 +73,15 @@ struct Job {
     uint32_t pad;
 };
 
-struct Workspace {  // one slice per CTA
+// Results of a job's phases after CLUSTER, shared by its CTAs.
+struct FinishCtl {
+    unsigned long long entries;  // of the quotient
+    unsigned long long wsum;     // sum over quotient nodes of their heaviest entry
+    uint32_t wmax, rmax, best, nsrc, err, job;
+    uint32_t part[kJobCtas];     // centers in each CTA's share of the nodes
+};
+
+struct Workspace {  // one slice per CTA, or per group of CTAs that share a job
     unsigned long long* key;
     unsigned long long* fkey[2];
     uint32_t* center;
@@ -80,13 +90,14 @@ struct Workspace {  // one slice per CTA
     uint32_t* stamp;
     uint32_t* fbase[2];
     uint32_t* fpre[2];
+    uint32_t* cfirst[2];
     uint32_t* next;
-    uint32_t* cid;
     uint32_t* M;      // dense quotient, kDenseCap^2
     uint32_t* qoff;   // quotient CSR extracted from M
     uint32_t* qcol;
     uint32_t* qw;
-    Counters* ctr;
+    Counters* ring;   // three counter blocks
+    FinishCtl* fin;
 };
 
 struct JobOut {
@@ -133,357 +144,544 @@ __device__ __forceinline__ T block_all_reduce(T v, Op op, T ident, T* red) {
 }
 
 struct BatchSmem {
-    RelaxSmem relax;
-    uint32_t relax_next[relax_nbuf_words<kRelaxU>(BT / 32)];
-    unsigned long long scratch[33];
-    unsigned long long red64[33];
+    GrowArgs args;
     uint32_t red32[33];
     uint32_t woff[33];
-    uint32_t job;
-    uint32_t changed[3];
+    uint32_t word;
 };
 
-// cid[v] = rank of v's center among all centers (block-wide scan); returns k
-__device__ uint32_t block_relabel(uint32_t n, const uint32_t* __restrict__ center, uint32_t* __restrict__ rank,
-                                  uint32_t* __restrict__ cid, BatchSmem& sm) {
-    const unsigned w = threadIdx.x >> 5, l = lane_id(), nw = blockDim.x >> 5;
+constexpr uint32_t kFinishU = 4;  // nodes, rows' columns or entries per thread whose loads are issued together
+
+// Centers among nodes [lo, hi) (4,096 per iteration, 128 consecutive ones per warp): returns their number; with `rank`
+// also rank[c] = first + the number of smaller centers of the range.
+__device__ uint32_t block_centers(uint32_t lo, uint32_t hi, const uint32_t* center, uint32_t* rank, uint32_t first,
+                                  BatchSmem& sm) {
+    const unsigned w = threadIdx.x >> 5, l = lane_id();
     uint32_t running = 0;
-    for (uint32_t base = 0; base < n; base += blockDim.x) {
-        const uint32_t v = base + threadIdx.x;
-        const bool f = v < n && __ldcg(&center[v]) == v;
-        const unsigned bal = __ballot_sync(0xffffffffu, f);
-        if (l == 0) sm.woff[w] = (uint32_t)__popc(bal);
+    for (uint64_t base = lo; base < hi; base += BT * kFinishU) {
+        unsigned bal[kFinishU];
+        uint32_t mine = 0;
+        const uint64_t v0 = base + w * (32 * kFinishU) + l;
+        uint32_t c[kFinishU];
+#pragma unroll
+        for (uint32_t u = 0; u < kFinishU; ++u) c[u] = v0 + 32 * u < hi ? __ldcg(&center[v0 + 32 * u]) : kNone;
+#pragma unroll
+        for (uint32_t u = 0; u < kFinishU; ++u) {
+            bal[u] = __ballot_sync(0xffffffffu, c[u] != kNone && c[u] == (uint32_t)v0 + 32 * u);
+            mine += (uint32_t)__popc(bal[u]);
+        }
+        if (l == 0) sm.woff[w] = mine;
         __syncthreads();
         if (w == 0) {
-            const uint32_t c = l < nw ? sm.woff[l] : 0u;  // lanes past the warp count add nothing
-            const uint32_t incl = warp_incl_scan(c);
-            sm.woff[l] = incl - c;
+            const uint32_t x = l < BW ? sm.woff[l] : 0u;
+            const uint32_t incl = warp_incl_scan(x);
+            sm.woff[l] = incl - x;
             if (l == 31) sm.woff[32] = incl;
         }
         __syncthreads();
-        if (f) rank[v] = running + sm.woff[w] + (uint32_t)__popc(bal & lanemask_lt());
+        if (rank) {
+            uint32_t at = first + running + sm.woff[w];
+#pragma unroll
+            for (uint32_t u = 0; u < kFinishU; ++u) {
+                if ((bal[u] >> l) & 1u) rank[v0 + 32 * u] = at + (uint32_t)__popc(bal[u] & lanemask_lt());
+                at += (uint32_t)__popc(bal[u]);
+            }
+        }
         running += sm.woff[32];
         __syncthreads();
     }
-    for (uint32_t v = threadIdx.x; v < n; v += blockDim.x) cid[v] = __ldcg(&rank[__ldcg(&center[v])]);
-    __syncthreads();
     return running;
 }
 
-// exact max finite distance of the k-node quotient held densely in M (row stride k)
-__device__ uint32_t block_quotient_diameter(uint32_t k, uint32_t* __restrict__ M, const Workspace& ws,
-                                            uint32_t* dyn, BatchSmem& sm, bool& ovf, uint32_t fw_k) {
-    if (k <= 1) return 0;
-    uint32_t best = 0;
-    if (k <= min(fw_k, kSmemFwK)) {
-        // Floyd-Warshall in shared memory; row p and column p are fixed during iteration p
-        for (uint32_t i = threadIdx.x; i < k * k; i += blockDim.x) dyn[i] = __ldcg(&M[i]);
-        __syncthreads();
-        for (uint32_t p = 0; p < k; ++p) {
-            for (uint32_t idx = threadIdx.x; idx < k * k; idx += blockDim.x) {
-                const uint32_t i = idx / k, j = idx - i * k;
-                dyn[idx] = relax_min_u32(dyn[idx], dyn[i * k + p], dyn[p * k + j], ovf);
-            }
-            __syncthreads();
-        }
-        for (uint32_t i = threadIdx.x; i < k * k; i += blockDim.x)
-            if (dyn[i] != kNone && dyn[i] > best) best = dyn[i];
-    } else {
-        // quotient CSR from M (warp per row, ballot compaction keeps columns sorted), then
-        // batched exact SSSP on it
-        const unsigned w = threadIdx.x >> 5, l = lane_id(), nw = blockDim.x >> 5;
-        for (uint32_t a = w; a < k; a += nw) {
-            uint32_t c = 0;
-            for (uint32_t b0 = 0; b0 < k; b0 += 32) {
-                const uint32_t b = b0 + l;
-                c += __popc(__ballot_sync(0xffffffffu, b < k && b != a && __ldcg(&M[a * k + b]) != kNone));
-            }
-            if (l == 0) ws.qoff[a + 1] = c;
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            ws.qoff[0] = 0;
-            for (uint32_t a = 0; a < k; ++a) ws.qoff[a + 1] += ws.qoff[a];
-        }
-        __syncthreads();
-        for (uint32_t a = w; a < k; a += nw) {
-            uint32_t pos = __ldcg(&ws.qoff[a]);
-            for (uint32_t b0 = 0; b0 < k; b0 += 32) {
-                const uint32_t b = b0 + l;
-                const uint32_t x = (b < k && b != a) ? __ldcg(&M[a * k + b]) : kNone;
-                const unsigned bal = __ballot_sync(0xffffffffu, x != kNone);
-                if (x != kNone) {
-                    const uint32_t at = pos + (uint32_t)__popc(bal & lanemask_lt());
-                    ws.qcol[at] = b;
-                    ws.qw[at] = x;
-                }
-                pos += (uint32_t)__popc(bal);
-            }
-        }
-        __syncthreads();
-        // worklist multi-source Bellman-Ford, 8 sources at a time: dist[v][s] and one word of change
-        // bits per node (two rounds) in shared memory; a changed node pushes to its neighbours
-        constexpr uint32_t S = 8;
-        uint32_t* dist = dyn;  // k x S
-        uint32_t* chg0 = dyn + (size_t)k * S;
-        uint32_t* chg1 = chg0 + k;
-        for (uint32_t s0 = 0; s0 < k; s0 += S) {
-            for (uint32_t i = threadIdx.x; i < k * S; i += blockDim.x) dist[i] = (s0 + i % S == i / S) ? 0u : kNone;
-            for (uint32_t v = threadIdx.x; v < k; v += blockDim.x) {
-                chg0[v] = (v >= s0 && v < s0 + S) ? 1u << (v - s0) : 0u;
-                chg1[v] = 0;
-            }
-            __syncthreads();
-            for (uint32_t round = 0;; ++round) {
-                uint32_t* cur = (round & 1) ? chg1 : chg0;
-                uint32_t* nxt = (round & 1) ? chg0 : chg1;
-                for (uint32_t v = w; v < k; v += nw) {
-                    const uint32_t bits = cur[v];
-                    if (!bits) continue;
-                    const uint32_t beg = __ldcg(&ws.qoff[v]), end = __ldcg(&ws.qoff[v + 1]);
-                    for (uint32_t j = beg + l; j < end; j += 32) {
-                        const uint32_t u = __ldcg(&ws.qcol[j]), wj = __ldcg(&ws.qw[j]);
-                        for (uint32_t b = bits; b; b &= b - 1) {
-                            const uint32_t si = (uint32_t)__ffs(b) - 1;
-                            const uint32_t dv = dist[v * S + si];
-                            if (dv == kNone) continue;
-                            const uint64_t nd = (uint64_t)dv + wj;
-                            if (nd >= kNone) {
-                                ovf = true;
-                                continue;
-                            }
-                            uint32_t* du = &dist[u * S + si];
-                            if ((uint32_t)nd < *du && (uint32_t)nd < atomicMin(du, (uint32_t)nd))
-                                atomicOr(&nxt[u], 1u << si);
-                        }
-                    }
-                }
-                __syncthreads();
-                bool any = false;
-                for (uint32_t v = threadIdx.x; v < k; v += blockDim.x) {
-                    cur[v] = 0;
-                    any |= nxt[v] != 0;
-                }
-                if (!__syncthreads_or(any)) break;
-                if (round > k * S + 64) {  // distances only decrease: far above any real count, reported
-                    ovf = true;
-                    break;
-                }
-            }
-            for (uint32_t i = threadIdx.x; i < k * S; i += blockDim.x)
-                if (s0 + i % S < k && dist[i] != kNone && dist[i] > best) best = dist[i];
-            __syncthreads();
-        }
-    }
+// Floyd-Warshall of the k x k matrix M in shared memory (k <= kSmemFwK); row p and column p are fixed during iteration p
+__device__ uint32_t block_floyd_warshall(uint32_t k, const uint32_t* M, uint32_t* dyn, bool& ovf) {
+    const unsigned w = threadIdx.x >> 5, l = lane_id();
+    for (uint32_t i = threadIdx.x; i < k * k; i += BT) dyn[i] = __ldcg(&M[i]);
     __syncthreads();
-    return block_all_reduce(best, [](uint32_t a, uint32_t b) { return a > b ? a : b; }, 0u, sm.red32);
+    for (uint32_t p = 0; p < k; ++p) {
+        for (uint32_t i = w; i < k; i += BW) {
+            const uint32_t a = dyn[i * k + p];
+            for (uint32_t j = l; j < k; j += 32) dyn[i * k + j] = relax_min_u32(dyn[i * k + j], a, dyn[p * k + j], ovf);
+        }
+        __syncthreads();
+    }
+    uint32_t best = 0;
+    for (uint32_t i = threadIdx.x; i < k * k; i += BT)
+        if (dyn[i] != kNone && dyn[i] > best) best = dyn[i];
+    return best;
 }
 
-// One job: CLUSTER + quotient + Phi(G_C) of one arena graph by this CTA; thread 0 stores the result.
-// The end of a job on one CTA: singletons, relabel, the dense quotient and Phi(G_C); thread 0 stores
-// the result.  `res` holds the CLUSTER counters so far.
+// Every source of the quotient CSR by one CTA, with overflow checks (quotients whose path sums might reach 2^32 - 1):
+// worklist multi-source Bellman-Ford, 8 sources at a time: dist[v][s] and one word of change bits per node (two rounds)
+// in shared memory; a changed node pushes to its neighbours
+__device__ uint32_t block_all_sources(uint32_t k, const Workspace& ws, uint32_t* dyn, bool& ovf) {
+    const unsigned w = threadIdx.x >> 5, l = lane_id();
+    constexpr uint32_t S = 8;
+    uint32_t best = 0;
+    uint32_t* dist = dyn;  // k x S
+    uint32_t* chg0 = dyn + (size_t)k * S;
+    uint32_t* chg1 = chg0 + k;
+    for (uint32_t s0 = 0; s0 < k; s0 += S) {
+        for (uint32_t i = threadIdx.x; i < k * S; i += BT) dist[i] = (s0 + i % S == i / S) ? 0u : kNone;
+        for (uint32_t v = threadIdx.x; v < k; v += BT) {
+            chg0[v] = (v >= s0 && v < s0 + S) ? 1u << (v - s0) : 0u;
+            chg1[v] = 0;
+        }
+        __syncthreads();
+        for (uint32_t round = 0;; ++round) {
+            uint32_t* cur = (round & 1) ? chg1 : chg0;
+            uint32_t* nxt = (round & 1) ? chg0 : chg1;
+            for (uint32_t v = w; v < k; v += BW) {
+                const uint32_t bits = cur[v];
+                if (!bits) continue;
+                const uint32_t beg = __ldcg(&ws.qoff[v]), end = __ldcg(&ws.qoff[v + 1]);
+                for (uint32_t j = beg + l; j < end; j += 32) {
+                    const uint32_t u = __ldcg(&ws.qcol[j]), wj = __ldcg(&ws.qw[j]);
+                    for (uint32_t b = bits; b; b &= b - 1) {
+                        const uint32_t si = (uint32_t)__ffs(b) - 1;
+                        const uint32_t dv = dist[v * S + si];
+                        if (dv == kNone) continue;
+                        const uint64_t nd = (uint64_t)dv + wj;
+                        if (nd >= kNone) {
+                            ovf = true;
+                            continue;
+                        }
+                        uint32_t* du = &dist[u * S + si];
+                        if ((uint32_t)nd < *du && (uint32_t)nd < atomicMin(du, (uint32_t)nd))
+                            atomicOr(&nxt[u], 1u << si);
+                    }
+                }
+            }
+            __syncthreads();
+            bool any = false;
+            for (uint32_t v = threadIdx.x; v < k; v += BT) {
+                cur[v] = 0;
+                any |= nxt[v] != 0;
+            }
+            if (!__syncthreads_or(any)) break;
+            if (round > k * S + 64) {  // distances only decrease: far above any real count, reported
+                ovf = true;
+                break;
+            }
+        }
+        for (uint32_t i = threadIdx.x; i < k * S; i += BT)
+            if (s0 + i % S < k && dist[i] != kNone && dist[i] > best) best = dist[i];
+        __syncthreads();
+    }
+    return best;
+}
+
+// The quotient CSR as the SSSPs of one CTA read it: staged in shared memory when it fits beside them.
+struct QuotientView {
+    const uint32_t* off;   // [k + 1], shared
+    const uint16_t* scol;  // shared, or null
+    const uint32_t* sw;
+    const uint32_t* gcol;
+    const uint32_t* gw;
+};
+
+// Exact SSSP from `source` by one warp: dist[k] and one bit per node to be relaxed again, both its own; a lane relaxes
+// one node's entries, improved nodes get their bit back, until no bit is left.  No path sum can reach 2^32 - 1.  Returns
+// the largest distance at every lane; *err when the sweeps exceed their limit.
+__device__ uint32_t warp_sssp(uint32_t k, const QuotientView& q, uint32_t source, uint32_t* dist, uint32_t* bits,
+                              uint32_t* err) {
+    const uint32_t l = lane_id(), words = (k + 31) / 32;
+    for (uint32_t v = l; v < k; v += 32) dist[v] = v == source ? 0u : kNone;
+    for (uint32_t i = l; i < words; i += 32) bits[i] = i == source / 32 ? 1u << (source % 32) : 0u;
+    __syncwarp();
+    for (uint32_t sweep = 0;; ++sweep) {
+        bool any = false;
+        for (uint32_t i = 0; i < words; ++i) {
+            const uint32_t b = *(volatile uint32_t*)&bits[i];
+            if (!b) continue;
+            any = true;
+            __syncwarp();
+            if (l == 0) bits[i] = 0;
+            __syncwarp();
+            if ((b >> l) & 1u) {
+                const uint32_t v = 32 * i + l, d = *(volatile uint32_t*)&dist[v];
+                for (uint32_t j = q.off[v]; j < q.off[v + 1]; ++j) {
+                    const uint32_t u = q.scol ? q.scol[j] : __ldcg(&q.gcol[j]);
+                    const uint32_t nd = d + (q.scol ? q.sw[j] : __ldcg(&q.gw[j]));
+                    if (nd < *(volatile uint32_t*)&dist[u] && nd < atomicMin(&dist[u], nd))
+                        atomicOr(&bits[u / 32], 1u << (u % 32));
+                }
+            }
+            __syncwarp();
+        }
+        if (!any) break;
+        if (sweep > 4 * k + 64) {  // far above any real count: a guard, reported as an error
+            if (l == 0) atomicExch(err, 1u);
+            break;
+        }
+    }
+    uint32_t ecc = 0;
+    for (uint32_t v = l; v < k; v += 32) ecc = dist[v] != kNone ? max(ecc, dist[v]) : ecc;
+    return __reduce_max_sync(0xffffffffu, ecc);
+}
+
+constexpr size_t kBatchDyn = 208 * 1024;  // dynamic shared memory of a CTA
+static_assert(kBatchDyn >= sizeof(GrowSmem) && kBatchDyn >= (size_t)kSmemFwK * kSmemFwK * 4 &&
+                  kBatchDyn >= (size_t)kDenseCap * (8 * 4 + 8),
+              "the growth loop, the shared Floyd-Warshall matrix and the all-source SSSP share the dynamic memory");
+
+// Exact diameter of a symmetric quotient whose path sums cannot reach 2^32 - 1, by eccentricity bounds (bounds.cuh): a
+// warp per source, the warps of all CTAs of the job at once.  ub, lb and src are global scratch, ub and lb preset.
+template <class Barrier>
+__device__ void group_bound_diameter(uint32_t k, uint32_t entries, const Workspace& ws, uint32_t* ub, uint32_t* lb,
+                                     uint32_t* src, uint32_t* soff, BatchSmem& sm, uint32_t br, uint32_t nb,
+                                     Barrier barrier) {
+    // shared memory behind the offsets: the CSR if it leaves room for 16 warps, then dist and bits per warp
+    const uint32_t words = (k + 31) / 32, per = k + words;  // words of one warp's SSSP
+    uint32_t* mem = soff + k + 1;
+    const size_t room = kBatchDyn / 4 - (k + 1);
+    const size_t csr = entries + (entries + 1) / 2;
+    QuotientView q{soff, nullptr, nullptr, ws.qcol, ws.qw};
+    size_t left = room;
+    if (csr + 16 * (size_t)per <= room) {
+        uint32_t* sw = mem;
+        uint16_t* scol = reinterpret_cast<uint16_t*>(mem + entries);
+        for (uint32_t j = threadIdx.x; j < entries; j += BT) {
+            sw[j] = __ldcg(&ws.qw[j]);
+            scol[j] = (uint16_t)__ldcg(&ws.qcol[j]);
+        }
+        q.scol = scol;
+        q.sw = sw;
+        mem += csr;
+        left -= csr;
+    }
+    const uint32_t warps = (uint32_t)min((size_t)BW, left / per);  // sources at once in this CTA
+    const uint32_t w = threadIdx.x >> 5, l = lane_id();
+    __syncthreads();
+    uint32_t ns = min(k, warps * nb);
+    for (bool first = true; ns > 0; first = false) {
+        const uint32_t i = br * warps + w;
+        if (w < warps && i < ns) {
+            uint32_t* dist = mem + (size_t)w * per;
+            const uint32_t source = first ? (uint32_t)((uint64_t)i * k / ns) : __ldcg(&src[i]);
+            const uint32_t ecc = warp_sssp(k, q, source, dist, dist + k, &ws.fin->err);
+            if (l == 0) atomicMax(&ws.fin->best, ecc);
+            for (uint32_t v = l; v < k; v += 32) {
+                const uint32_t d = dist[v];
+                if (d == kNone) continue;
+                atomicMin(&ub[v], (uint32_t)min((uint64_t)d + ecc, (uint64_t)(kNone - 1)));
+                atomicMax(&lb[v], max(d, ecc - d));
+            }
+        }
+        barrier();
+        if (ns == k) break;  // every node was a source
+        if (br == 0) {
+            // (the SSSPs' memory is free between batches)
+            uint32_t* sub = mem;
+            uint32_t* slb = mem + k;
+            for (uint32_t v = threadIdx.x; v < k; v += BT) {
+                sub[v] = __ldcg(&ub[v]);
+                slb[v] = __ldcg(&lb[v]);
+            }
+            __syncthreads();
+            const uint32_t n = bound_select(k, warps * nb, __ldcg(&ws.fin->best), sub, slb, src, sm.word);
+            if (threadIdx.x == 0) ws.fin->nsrc = __ldcg(&ws.fin->err) ? 0u : n;
+        }
+        barrier();
+        ns = __ldcg(&ws.fin->nsrc);
+    }
+}
+
+// The end of a job: singletons, relabel, the dense quotient and Phi(G_C); CTA 0 stores the result.  `res` holds the
+// CLUSTER counters so far.  Every phase is split over the job's CTAs (br of nb), a barrier between phases.
+template <class Barrier>
 __device__ void finish_job(const Job& job, const ArenaDesc& d, const uint64_t* __restrict__ off,
                            const uint2* __restrict__ adj, const uint32_t* __restrict__ row, const Workspace& ws,
                            BatchSmem& sm, uint32_t* dyn, JobOut* out, cldiam_result res, uint32_t status,
-                           uint32_t delta) {
-    const unsigned tid = threadIdx.x;
-    const uint32_t n = d.n;
+                           uint32_t br, uint32_t nb, Barrier barrier) {
+    const unsigned tid = threadIdx.x, w = tid >> 5, l = lane_id();
+    const uint32_t n = d.n, gt = br * BT + tid, gw = br * BW + w;  // thread and warp among the job's
+    const uint32_t nt = nb * BT, nw = nb * BW;
+    FinishCtl* fin = ws.fin;
+    uint2* cd = reinterpret_cast<uint2*>(ws.fkey[0]);  // (cluster id, D) of every node
+    const auto pack = [](uint2 x) { return (unsigned long long)x.y << 32 | x.x; };
     if (status == kJobOk) {
-        dev_singletons(n, ws.center, ws.D, 0, 1);
-        __syncthreads();
-        res.delta_end = delta;
-        const uint32_t k = block_relabel(n, ws.center, ws.stamp, ws.cid, sm);  // stamp reused as rank
+        dev_singletons(n, ws.center, ws.D, br, nb);
+        barrier();
+        // cluster id = rank of the center among the centers: counts of the CTAs' shares, then ranks
+        const uint32_t share = (uint32_t)(((uint64_t)n + (uint64_t)nb * 4096 - 1) / ((uint64_t)nb * 4096) * 4096);
+        const uint32_t lo = min(n, br * share), hi = (uint32_t)min((uint64_t)n, (uint64_t)lo + share);
+        uint32_t first = 0, k = 0;
+        if (nb > 1) {
+            const uint32_t c = block_centers(lo, hi, ws.center, nullptr, 0, sm);
+            if (tid == 0) fin->part[br] = c;
+            barrier();
+            for (uint32_t i = 0; i < nb; ++i) {
+                const uint32_t x = __ldcg(&fin->part[i]);
+                first += i < br ? x : 0u;
+                k += x;
+            }
+        }
+        const uint32_t mine = block_centers(lo, hi, ws.center, ws.stamp, first, sm);  // stamp reused as rank
+        if (nb == 1) k = mine;
         res.k = k;
-        const uint32_t rmax =
-            block_all_reduce([&] {
-                uint32_t m = 0;
-                for (uint32_t v = tid; v < n; v += BT) m = max(m, __ldcg(&ws.D[v]));
-                return m;
-            }(), [](uint32_t a, uint32_t b) { return a > b ? a : b; }, 0u, sm.red32);
-        res.radius = rmax;
+        barrier();
+        uint32_t* ub = ws.R;
+        uint32_t* lb = ws.next;
+        uint32_t rmax = 0;
+        for (uint64_t base = gt; base < n; base += (uint64_t)nt * kFinishU) {
+            uint32_t c[kFinishU], dd[kFinishU];
+#pragma unroll
+            for (uint32_t u = 0; u < kFinishU; ++u) {
+                const uint64_t v = base + (uint64_t)u * nt;
+                c[u] = v < n ? __ldcg(&ws.center[v]) : 0u;
+                dd[u] = v < n ? __ldcg(&ws.D[v]) : 0u;
+            }
+#pragma unroll
+            for (uint32_t u = 0; u < kFinishU; ++u) c[u] = __ldcg(&ws.stamp[c[u]]);
+#pragma unroll
+            for (uint32_t u = 0; u < kFinishU; ++u) {
+                const uint64_t v = base + (uint64_t)u * nt;
+                if (v < n) cd[v] = make_uint2(c[u], dd[u]);
+                rmax = max(rmax, dd[u]);
+            }
+        }
+        rmax = __reduce_max_sync(0xffffffffu, rmax);
+        if (l == 0 && rmax) atomicMax(&fin->rmax, rmax);
         if (k > kDenseCap) {
             status = kJobNeedsPlain;
         } else {
-            // weighted quotient graph, deduplicated densely
+            // weighted quotient graph, deduplicated densely: each undirected edge once, into both of its entries
             uint32_t* M = ws.M;
-            for (uint32_t i = tid; i < k * k; i += BT) M[i] = (i / k == i % k) ? 0u : kNone;
-            __syncthreads();
-            bool ovf = false;
-            for (uint64_t i = tid; i < d.nnz; i += BT) {
-                const uint32_t u = row[i];
-                const uint2 e = adj[i];
-                const uint32_t a = __ldcg(&ws.cid[u]), b = __ldcg(&ws.cid[e.x]);
-                if (a != b) {
-                    uint64_t s = (uint64_t)__ldcg(&ws.D[u]) + e.y + __ldcg(&ws.D[e.x]);
-                    if (s >= 0xFFFFFFFFull) {
-                        ovf = true;
-                        s = 0xFFFFFFFEull;
-                    }
-                    atomicMin(&M[(size_t)a * k + b], (uint32_t)s);
-                }
+            for (uint32_t a = gw; a < k; a += nw)
+                for (uint32_t b = l; b < k; b += 32) M[a * k + b] = a == b ? 0u : kNone;
+            for (uint32_t v = gt; v < k; v += nt) {
+                ub[v] = kNone;
+                lb[v] = 0;
             }
-            __syncthreads();
-            const unsigned long long qe = block_all_reduce(
-                [&] {
-                    unsigned long long c = 0;
-                    for (uint32_t i = tid; i < k * k; i += BT) c += (i / k != i % k && __ldcg(&M[i]) != kNone);
-                    return c;
-                }(),
-                [](unsigned long long a, unsigned long long b) { return a + b; }, 0ull, sm.red64);
+            barrier();
+            bool ovf = false;
+            for (uint64_t base = gt; base < d.nnz; base += (uint64_t)nt * kFinishU) {
+                uint32_t r[kFinishU];
+                uint2 e[kFinishU];
+#pragma unroll
+                for (uint32_t u = 0; u < kFinishU; ++u) {
+                    const uint64_t i = base + (uint64_t)u * nt;
+                    r[u] = i < d.nnz ? row[i] : 0u;
+                    e[u] = i < d.nnz ? adj[i] : make_uint2(0u, 0u);
+                }
+                unsigned long long pu[kFinishU], pv[kFinishU];
+#pragma unroll
+                for (uint32_t u = 0; u < kFinishU; ++u) {
+                    const bool take = r[u] < e[u].x;
+                    pu[u] = take ? pack(__ldcg(&cd[r[u]])) : 0ull;
+                    pv[u] = take ? pack(__ldcg(&cd[e[u].x])) : 0ull;
+                }
+                uint32_t at[kFinishU], cur[kFinishU], s32[kFinishU];
+#pragma unroll
+                for (uint32_t u = 0; u < kFinishU; ++u) {
+                    const uint32_t a = (uint32_t)pu[u], b = (uint32_t)pv[u];
+                    uint64_t sw = (pu[u] >> 32) + e[u].y + (pv[u] >> 32);
+                    const bool take = r[u] < e[u].x && a != b;
+                    if (take && sw >= 0xFFFFFFFFull) {
+                        ovf = true;
+                        sw = 0xFFFFFFFEull;
+                    }
+                    s32[u] = (uint32_t)sw;
+                    at[u] = a * k + b;
+                    cur[u] = take ? __ldcg(&M[at[u]]) : 0u;
+                }
+#pragma unroll
+                for (uint32_t u = 0; u < kFinishU; ++u)
+                    if (s32[u] < cur[u]) {
+                        atomicMin(&M[at[u]], s32[u]);
+                        atomicMin(&M[(uint32_t)pv[u] * k + (uint32_t)pu[u]], s32[u]);
+                    }
+            }
+            if (__any_sync(0xffffffffu, ovf) && l == 0) atomicExch(&fin->err, 2u);
+            barrier();
+            // entries per row, and the guard of the bounds: sum over rows of the heaviest entry
+            unsigned long long entries = 0, wsum = 0;
+            uint32_t wmax = 0;
+            for (uint32_t a = gw; a < k; a += nw) {
+                uint32_t c = 0, m = 0;
+                for (uint32_t b0 = 0; b0 < k; b0 += 32 * kFinishU) {
+                    uint32_t x[kFinishU];
+#pragma unroll
+                    for (uint32_t u = 0; u < kFinishU; ++u) {
+                        const uint32_t b = b0 + 32 * u + l;
+                        x[u] = b < k && b != a ? __ldcg(&M[a * k + b]) : kNone;
+                    }
+#pragma unroll
+                    for (uint32_t u = 0; u < kFinishU; ++u) {
+                        c += x[u] != kNone ? 1u : 0u;
+                        m = x[u] != kNone ? max(m, x[u]) : m;
+                    }
+                }
+                c = __reduce_add_sync(0xffffffffu, c);
+                m = __reduce_max_sync(0xffffffffu, m);
+                if (l == 0) ws.qoff[a] = c;
+                entries += c;
+                wsum += m;
+                wmax = max(wmax, m);
+            }
+            if (l == 0 && entries) {
+                atomicAdd(&fin->entries, entries);
+                atomicAdd(&fin->wsum, wsum);
+                atomicMax(&fin->wmax, wmax);
+            }
+            barrier();
+            const uint32_t qe = (uint32_t)__ldcg(&fin->entries);
             res.quotient_edges = qe;
             bool ovf2 = false;
-            const uint32_t phi = block_quotient_diameter(k, M, ws, dyn, sm, ovf2, job.fw_k);
-            const uint32_t any_ovf = block_all_reduce((uint32_t)(ovf || ovf2),
-                                                      [](uint32_t a, uint32_t b) { return a | b; }, 0u, sm.red32);
-            if (any_ovf) status = kJobOverflow;
+            // No path sum of an SSSP can reach 2^32 - 1 when the sum of the rows' heaviest entries and one more entry do
+            // not; Floyd-Warshall also adds two paths.  Up to fw_k nodes it takes dense quotients, and those whose two
+            // paths might overflow, so that OVERFLOW is reported as it always was (sparse ones are faster by bounds).
+            const unsigned long long longest = __ldcg(&fin->wsum), heaviest = __ldcg(&fin->wmax);
+            const bool dense = (uint64_t)qe * 8 >= (uint64_t)k * k || 2 * longest + heaviest >= 0xFFFFFFFFull;
+            if (k > 1 && k <= min(job.fw_k, kSmemFwK) && dense) {
+                if (br == 0) {
+                    const uint32_t best = block_floyd_warshall(k, M, dyn, ovf2);
+                    const uint32_t m = __reduce_max_sync(0xffffffffu, best);
+                    if (l == 0) atomicMax(&fin->best, m);
+                }
+            } else if (k > 1) {
+                // quotient CSR from M: row starts by a block scan of the counts (k <= 1,024), in every CTA; a warp per
+                // row, ballot compaction keeps the columns sorted
+                uint32_t* soff = dyn;
+                const uint32_t c = tid < k ? __ldcg(&ws.qoff[tid]) : 0u;
+                const uint32_t incl = warp_incl_scan(c);
+                if (l == 31) sm.woff[w] = incl;
+                __syncthreads();
+                uint32_t before = 0;
+                for (uint32_t i = 0; i < w; ++i) before += sm.woff[i];
+                if (tid < k) soff[tid] = before + incl - c;
+                if (tid == 0) soff[k] = qe;
+                __syncthreads();
+                for (uint32_t a = gw; a < k; a += nw) {
+                    uint32_t pos = soff[a];
+                    for (uint32_t b0 = 0; b0 < k; b0 += 32 * kFinishU) {
+                        uint32_t x[kFinishU];
+#pragma unroll
+                        for (uint32_t u = 0; u < kFinishU; ++u) {
+                            const uint32_t b = b0 + 32 * u + l;
+                            x[u] = b < k && b != a ? __ldcg(&M[a * k + b]) : kNone;
+                        }
+#pragma unroll
+                        for (uint32_t u = 0; u < kFinishU; ++u) {
+                            const unsigned bal = __ballot_sync(0xffffffffu, x[u] != kNone);
+                            if (x[u] != kNone) {
+                                const uint32_t p = pos + (uint32_t)__popc(bal & lanemask_lt());
+                                ws.qcol[p] = b0 + 32 * u + l;
+                                ws.qw[p] = x[u];
+                            }
+                            pos += (uint32_t)__popc(bal);
+                        }
+                    }
+                }
+                barrier();
+                if (longest + heaviest < 0xFFFFFFFFull) {
+                    group_bound_diameter(k, qe, ws, ub, lb, ws.fbase[0], soff, sm, br, nb, barrier);
+                } else if (br == 0) {
+                    for (uint32_t i = tid; i <= k; i += BT) ws.qoff[i] = soff[i];
+                    __syncthreads();
+                    const uint32_t best = block_all_sources(k, ws, dyn, ovf2);
+                    const uint32_t m = __reduce_max_sync(0xffffffffu, best);
+                    if (l == 0) atomicMax(&fin->best, m);
+                }
+            }
+            if (__any_sync(0xffffffffu, ovf2) && l == 0) atomicExch(&fin->err, 2u);
+            barrier();
+            const uint32_t err = __ldcg(&fin->err), phi = __ldcg(&fin->best);
+            if (err) status = err == 1u ? kJobDiverged : kJobOverflow;
+            res.radius = __ldcg(&fin->rmax);
             res.phi_gc = phi;
-            res.phi_approx = (uint64_t)phi + 2ull * rmax;
+            res.phi_approx = (uint64_t)phi + 2ull * res.radius;
         }
     }
-    if (tid == 0) {
+    if (br == 0 && tid == 0) {
         out->r = res;
         out->status = status;
     }
-    __syncthreads();
 }
 
+// One job: CLUSTER + quotient + Phi(G_C) of one arena graph by CTA br of nb; CTA 0 stores the result.
+template <class Barrier>
 __device__ void run_job(const Job& job, const ArenaDesc& d, const uint64_t* __restrict__ arena_off,
                         const uint2* __restrict__ arena_adj, const uint32_t* __restrict__ arena_row,
-                        const Workspace& ws, BatchSmem& sm, uint32_t* dyn, JobOut* out) {
-    Counters* ctr = ws.ctr;
-    volatile Counters* vc = ctr;
+                        const Workspace& ws, BatchSmem& sm, uint32_t* dyn, JobOut* out, uint32_t br, uint32_t nb,
+                        Barrier barrier) {
     const unsigned tid = threadIdx.x;
     const uint32_t n = d.n;
     const uint64_t* off = arena_off + d.off_base;
     const uint2* adj = arena_adj + d.adj_base;
     const uint32_t* row = arena_row + d.adj_base;
-    cldiam_result res;
-    memset(&res, 0, sizeof res);
-    uint32_t status = kJobOk;
-
-    for (uint32_t v = tid; v < n; v += BT) {
+    for (uint32_t v = br * BT + tid; v < n; v += nb * BT) {
         ws.center[v] = kNone;
         ws.D[v] = 0;
         ws.R[v] = 0;
         ws.stamp[v] = 0;
         ws.key[v] = kInfKey;
     }
-    if (tid == 0) memset(ctr, 0, sizeof(Counters));
-    __syncthreads();
-
-    uint64_t U = n, frozen_deg = 0, covered = 0;
-    uint32_t stage = 1, stepid = 0, delta = job.delta0, cur = 0;
-    const bool pull_ok = d.nnz < 0x80000000ull;
-    uint32_t nf = 0, E = 0;
-    for (;;) {
-        uint64_t thr = 0;
-        if (!stage_threshold(U, job.tau, job.L, &thr)) break;
-        if (stage > kMaxStages) {
-            status = kJobDiverged;
-            break;
-        }
-        if (tid == 0) {
-            ctr->selected = 0;
-            ctr->front = 0;
-        }
-        __syncthreads();
-        dev_select(n, ws.center, ws.key, job.seed, stage, thr, ctr, 0, 1);
-        __syncthreads();
-        {
-            const bool pull = pull_ok && (d.nnz - frozen_deg) < frozen_deg;
-            dev_rebuild(n, ws.key, ws.center, job.cumulative ? ws.D : nullptr, off, delta, pull, ws.fbase[cur],
-                        ws.fkey[cur], ws.fpre[cur], nullptr,
-                        ctr, sm.scratch, 0, 1);
-        }
-        __syncthreads();
-        covered = vc->selected;
-        res.centers_drawn += vc->selected;
-        nf = (uint32_t)(vc->front >> 32);
-        E = (uint32_t)vc->front;
-        __syncthreads();
-        for (;;) {
-            uint32_t updated, growth_steps = 0;
-            do {
-                ++growth_steps;
-                ++stepid;
-                updated = 0;
-                if (nf > 0) {
-                    if (tid == 0) {
-                        ctr->newly_covered = 0;
-                        ctr->front = 0;
-                        ctr->nnext = 0;
-                    }
-                    __syncthreads();
-                    dev_relax<kRelaxU>(ws.fbase[cur], ws.fkey[cur], ws.fpre[cur], nf, E, adj, ws.center,
-                                 job.cumulative ? ws.D : nullptr, ws.key,
-                                 delta, ws.stamp, stepid, ws.next, ctr, sm.relax, sm.relax_next, 0, 1);
-                    __syncthreads();
-                    const uint32_t nn = vc->nnext;
-                    dev_snapshot(ws.next, nn, ws.key, off, delta, ws.fbase[cur ^ 1], ws.fkey[cur ^ 1],
-                                 ws.fpre[cur ^ 1], nullptr, ctr, sm.scratch, 0, 1);
-                    __syncthreads();
-                    updated = nn;
-                    covered += vc->newly_covered;
-                    res.edges_scanned += E;
-                    nf = (uint32_t)(vc->front >> 32);
-                    E = (uint32_t)vc->front;
-                    cur ^= 1;
-                    __syncthreads();
-                }
-                res.steps++;
-                res.node_updates += updated;
-            } while (updated != 0 && 2 * covered < U && (job.step_cap == 0 || growth_steps < job.step_cap));
-            if (2 * covered >= U) break;
-            bool growable = false;
-            if (delta < kDeltaMax && d.connected) {
-                growable = covered > 0 || U < n;
-            } else if (delta < kDeltaMax && d.nnz) {
-                if (tid == 0) ctr->growable = 0;
-                __syncthreads();
-                dev_growable(row, adj, d.nnz, ws.key, ctr, 0, 1);
-                __syncthreads();
-                growable = vc->growable != 0;
-                __syncthreads();
-            }
-            if (!growable) {
-                res.guard_exits++;
-                break;
-            }
-            delta = (delta > kDeltaMax / 2) ? kDeltaMax : 2 * delta;
-            res.doublings++;
-            if (tid == 0) ctr->front = 0;
-            __syncthreads();
-            {
-                const bool pull = pull_ok && (d.nnz - frozen_deg) < frozen_deg;
-                dev_rebuild(n, ws.key, ws.center, job.cumulative ? ws.D : nullptr, off, delta, pull, ws.fbase[cur],
-                        ws.fkey[cur], ws.fpre[cur], nullptr,
-                            ctr, sm.scratch, 0, 1);
-            }
-            __syncthreads();
-            nf = (uint32_t)(vc->front >> 32);
-            E = (uint32_t)vc->front;
-            __syncthreads();
-        }
-        if (tid == 0) {
-            ctr->frozen = 0;
-            ctr->frozen_deg = 0;
-        }
-        __syncthreads();
-        dev_finalize_d(n, ws.key, ws.center, job.cumulative ? nullptr : ws.R, ws.D, ctr, 0, 1);
-        __syncthreads();
-        dev_finalize_freeze(n, ws.key, ws.center, ws.R, ws.D, off, ctr, 0, 1);
-        __syncthreads();
-        if (vc->overflow) status = kJobOverflow;
-        U -= vc->frozen;
-        frozen_deg += vc->frozen_deg;
-        res.stages++;
-        ++stage;
-        __syncthreads();
-        if (status != kJobOk) break;
+    if (br == 0 && tid == 0) {
+        memset(ws.ring, 0, 3 * sizeof(Counters));
+        FinishCtl* fin = ws.fin;
+        fin->entries = fin->wsum = 0;
+        fin->wmax = fin->rmax = fin->best = fin->nsrc = fin->err = 0;
     }
-    finish_job(job, d, off, adj, row, ws, sm, dyn, out, res, status, delta);
+    if (tid == 0) {
+        GrowArgs& a = sm.args;
+        a.off = off;
+        a.adj = adj;
+        a.key = ws.key;
+        a.keyS = nullptr;
+        for (int i = 0; i < 2; ++i) {
+            a.fkey[i] = ws.fkey[i];
+            a.fbase[i] = ws.fbase[i];
+            a.fpre[i] = ws.fpre[i];
+            a.cfirst[i] = ws.cfirst[i];
+        }
+        a.center = ws.center;
+        a.D = ws.D;
+        a.R = ws.R;
+        a.stamp = ws.stamp;
+        a.next = ws.next;
+        a.ring = ws.ring;
+        a.out = nullptr;
+        a.row = row;
+        a.tau = job.tau;
+        a.L = job.L;
+        a.seed = job.seed;
+        a.nnz = d.nnz;
+        a.n = n;
+        a.step_cap = job.step_cap;
+        a.max_entries = a.max_epochs = 0xFFFFFFFFu;
+        a.cumulative = job.cumulative != 0;
+        a.pull_ok = d.nnz < 0x80000000ull;
+        a.stages = true;
+        a.connected = d.connected != 0;
+    }
+    GrowState g;
+    memset(&g, 0, sizeof g);
+    g.U = n;
+    g.phase = kPhaseStage;
+    g.stage = 1;
+    g.delta = job.delta0;
+    barrier();
+    grow_run(sm.args, g, *reinterpret_cast<GrowSmem*>(dyn), br, nb, barrier);
+    uint32_t status = kJobOk;
+    if (g.phase != kPhaseDone)
+        status = g.stage > kMaxStages || g.unfrozen != g.U ? kJobDiverged : kJobOverflow;
+    cldiam_result res;
+    memset(&res, 0, sizeof res);
+    res.stages = g.stages;
+    res.steps = g.steps;
+    res.doublings = g.doublings;
+    res.delta_end = g.delta;
+    res.guard_exits = g.guard_exits;
+    res.node_updates = g.node_updates;
+    res.edges_scanned = g.edges_scanned;
+    res.centers_drawn = g.centers_drawn;
+    finish_job(job, d, off, adj, row, ws, sm, dyn, out, res, status, br, nb, barrier);
 }
 
+// The jobs of a queue (largest first), one after another, by one CTA each (GROUP: by a thread-block cluster each).
+template <bool GROUP>
 __global__ void __launch_bounds__(BT, kBatchCtasPerSm)
     k_batch(const ArenaDesc* __restrict__ descs, const Job* __restrict__ jobs, uint32_t count,
             const uint64_t* __restrict__ arena_off, const uint2* __restrict__ arena_adj,
@@ -491,17 +689,34 @@ __global__ void __launch_bounds__(BT, kBatchCtasPerSm)
             JobOut* __restrict__ outs) {
     extern __shared__ __align__(16) uint32_t dyn[];
     __shared__ BatchSmem sm;
-    const Workspace ws = wss[blockIdx.x];
+    uint32_t br = 0, nb = 1;
+    if constexpr (GROUP) {
+        asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(br));
+        asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(nb));
+    }
+    const auto barrier = [] {
+        if constexpr (GROUP) cluster_barrier();
+        else __syncthreads();
+    };
+    const Workspace ws = wss[blockIdx.x / nb];
     for (;;) {
-        if (threadIdx.x == 0) sm.job = atomicAdd(queue, 1u);
-        __syncthreads();
-        const uint32_t j = sm.job;
-        __syncthreads();
+        uint32_t j;
+        if constexpr (GROUP) {
+            if (br == 0 && threadIdx.x == 0) ws.fin->job = atomicAdd(queue, 1u);
+            barrier();
+            j = __ldcg(&ws.fin->job);
+        } else {
+            if (threadIdx.x == 0) sm.word = atomicAdd(queue, 1u);
+            __syncthreads();
+            j = sm.word;
+            __syncthreads();
+        }
         if (j >= count) break;
         const Job job = jobs[j];
         const uint64_t t0 = global_ns();
-        run_job(job, descs[job.graph], arena_off, arena_adj, arena_row, ws, sm, dyn, &outs[job.out]);
-        if (threadIdx.x == 0) {
+        run_job(job, descs[job.graph], arena_off, arena_adj, arena_row, ws, sm, dyn, &outs[job.out], br, nb, barrier);
+        barrier();  // (every CTA is done with the job's workspace)
+        if (br == 0 && threadIdx.x == 0) {
             outs[job.out].t_start = t0;
             outs[job.out].t_end = global_ns();
         }
@@ -560,7 +775,7 @@ __global__ void __launch_bounds__(BT, kBatchCtasPerSm)
                 }
                 __nanosleep(2000);
             }
-            sm.job = claimed;
+            sm.word = claimed;
             if (claimed != kNone) {
                 const volatile Job* vj = ring + claimed;
                 s_job.tau = vj->tau;
@@ -575,11 +790,12 @@ __global__ void __launch_bounds__(BT, kBatchCtasPerSm)
             }
         }
         __syncthreads();
-        const uint32_t slot = sm.job;
+        const uint32_t slot = sm.word;
         if (slot == kNone) break;
         const Job job = s_job;
         __syncthreads();
-        run_job(job, descs[job.graph], arena_off, arena_adj, arena_row, ws, sm, dyn, &outs[job.out]);
+        run_job(job, descs[job.graph], arena_off, arena_adj, arena_row, ws, sm, dyn, &outs[job.out], 0u, 1u,
+                [] { __syncthreads(); });
         if (threadIdx.x == 0) {
             __threadfence_system();
             st_release_sys(&done[job.out], 1u);
@@ -739,14 +955,16 @@ uint64_t arena_entries(const cldiam_arena* a, const uint32_t* ids, uint32_t coun
 }
 uint64_t arena_device_bytes(const cldiam_arena* a) { return arena_bytes(a); }
 
-// Per-CTA workspaces for graphs of up to nmax nodes, carved from one (cached) device buffer.
-static cldiam_status make_workspaces(uint32_t nmax, int ctas, cudaStream_t s, void** buf, size_t* buf_bytes,
-                                     std::vector<Workspace>* out) {
+// Workspaces for graphs of up to nmax nodes and zmax entries, one per CTA (or group of CTAs), carved from one (cached)
+// device buffer.
+static cldiam_status make_workspaces(uint32_t nmax, uint64_t zmax, int ctas, cudaStream_t s, void** buf,
+                                     size_t* buf_bytes, std::vector<Workspace>* out) {
     auto al = [](size_t b) { return (b + 255) & ~(size_t)255; };
     const size_t n8 = al((size_t)nmax * 8), n4 = al((size_t)nmax * 4), f8 = al((size_t)nmax * 16),
                  f4 = al((size_t)nmax * 8), mm = al((size_t)kDenseCap * kDenseCap * 4),
-                 qo = al(((size_t)kDenseCap + 1) * 4), ctrb = al(sizeof(Counters));
-    const size_t slice = n8 + 2 * f8 + 6 * n4 + 4 * f4 + mm + qo + 2 * mm + ctrb;
+                 cf = al((size_t)(2 * zmax / QC + 2) * 4),  // a frontier has at most 2 x nnz entries (push + pull)
+                 qo = al(((size_t)kDenseCap + 1) * 4), ctrb = al(3 * sizeof(Counters)), finb = al(sizeof(FinishCtl));
+    const size_t slice = n8 + 2 * f8 + 5 * n4 + 4 * f4 + 2 * cf + mm + qo + 2 * mm + ctrb + finb;
     const size_t need = slice * ctas;
     if (need > *buf_bytes) {
         dfree(*buf, s);
@@ -767,16 +985,18 @@ static cldiam_status make_workspaces(uint32_t nmax, int ctas, cudaStream_t s, vo
         w.R = reinterpret_cast<uint32_t*>(p); p += n4;
         w.stamp = reinterpret_cast<uint32_t*>(p); p += n4;
         w.next = reinterpret_cast<uint32_t*>(p); p += n4;
-        w.cid = reinterpret_cast<uint32_t*>(p); p += n4;
         w.fbase[0] = reinterpret_cast<uint32_t*>(p); p += f4;
         w.fbase[1] = reinterpret_cast<uint32_t*>(p); p += f4;
         w.fpre[0] = reinterpret_cast<uint32_t*>(p); p += f4;
         w.fpre[1] = reinterpret_cast<uint32_t*>(p); p += f4;
+        w.cfirst[0] = reinterpret_cast<uint32_t*>(p); p += cf;
+        w.cfirst[1] = reinterpret_cast<uint32_t*>(p); p += cf;
         w.M = reinterpret_cast<uint32_t*>(p); p += mm;
         w.qoff = reinterpret_cast<uint32_t*>(p); p += qo;
         w.qcol = reinterpret_cast<uint32_t*>(p); p += mm;
         w.qw = reinterpret_cast<uint32_t*>(p); p += mm;
-        w.ctr = reinterpret_cast<Counters*>(p);
+        w.ring = reinterpret_cast<Counters*>(p); p += ctrb;
+        w.fin = reinterpret_cast<FinishCtl*>(p);
     }
     return CLDIAM_OK;
 }
@@ -792,10 +1012,7 @@ struct CudaEvent {
     }
 };
 
-static size_t batch_dyn_smem() {
-    // shared Floyd-Warshall matrix, or the quotient SSSP's k x 8 distances and two words of change bits per node
-    return std::max<size_t>((size_t)kSmemFwK * kSmemFwK * 4, (size_t)kDenseCap * (8 * 4 + 8));
-}
+static size_t batch_dyn_smem() { return kBatchDyn; }
 
 template <class Kern>
 static cldiam_status set_dyn_smem(Kern k, std::atomic<bool>* done_flags) {
@@ -856,7 +1073,7 @@ cldiam_status batch_run(cldiam_arena* a, const uint32_t* ids, const double* tau,
     });
     static std::atomic<bool> attr[64];
     int cps = 1;
-    CLD_TRY(resident_per_sm(k_batch, attr, &cps));
+    CLD_TRY(resident_per_sm(k_batch<false>, attr, &cps));
     const int nsm = num_sms() * cps;  // CTAs of the launch
     // The launch ends with its largest graph on one CTA, or with the even split of all work over the CTAs,
     // whichever is later.  The k largest graphs can instead run first on the one-graph path, each with the
@@ -921,9 +1138,13 @@ cldiam_status batch_run(cldiam_arena* a, const uint32_t* ids, const double* tau,
     const uint32_t nrest = count - nbig;
     if (nrest > 0) {
         uint32_t nmax_rest = 1;
-        for (uint32_t j = nbig; j < count; ++j) nmax_rest = std::max(nmax_rest, a->graphs[jobs[j].graph].n);
+        uint64_t zmax_rest = 0;
+        for (uint32_t j = nbig; j < count; ++j) {
+            nmax_rest = std::max(nmax_rest, a->graphs[jobs[j].graph].n);
+            zmax_rest = std::max(zmax_rest, a->graphs[jobs[j].graph].nnz);
+        }
         std::vector<Workspace> wsh;
-        CLD_TRY(make_workspaces(nmax_rest, nsm, s, &a->ws, &a->ws_bytes, &wsh));
+        CLD_TRY(make_workspaces(nmax_rest, zmax_rest, nsm, s, &a->ws, &a->ws_bytes, &wsh));
         DBuf<ArenaDesc> ddesc;
         DBuf<Job> djobs;
         DBuf<Workspace> dws;
@@ -940,7 +1161,7 @@ cldiam_status batch_run(cldiam_arena* a, const uint32_t* ids, const double* tau,
         CLD_CUDA(cudaMemcpyAsync(dws.get(), wsh.data(), nsm * sizeof(Workspace), cudaMemcpyHostToDevice, s));
         CLD_CUDA(cudaMemsetAsync(queue.get(), 0, 4, s));
         const size_t dyn = batch_dyn_smem();
-        CLD_K(K_MISC, s, k_batch<<<nsm, BT, dyn, s>>>(ddesc.get(), djobs.get(), nrest, a->off, a->adj, a->row, dws.get(),
+        CLD_K(K_MISC, s, k_batch<false><<<nsm, BT, dyn, s>>>(ddesc.get(), djobs.get(), nrest, a->off, a->adj, a->row, dws.get(),
                                                        queue.get(), douts.get()));
         CLD_LAUNCH_CHECK();
         std::vector<JobOut> hl(count);
@@ -1147,10 +1368,14 @@ cldiam_status server_create(cldiam_arena* a, const cldiam_server_opts* o, cldiam
     if (st != CLDIAM_OK) return cleanup(st);
     // device state: descriptors, head counter, workspaces for the graphs the kernel serves
     uint32_t nmax = 1;
+    uint64_t zmax = 0;
     for (const ArenaDesc& d : a->graphs)
-        if (d.n <= sv->big_nodes) nmax = std::max(nmax, d.n);
+        if (d.n <= sv->big_nodes) {
+            nmax = std::max(nmax, d.n);
+            zmax = std::max(zmax, d.nnz);
+        }
     std::vector<Workspace> wsh;
-    if ((st = make_workspaces(nmax, (int)sv->ctas, sv->kstream, &sv->ws, &sv->ws_bytes, &wsh)) != CLDIAM_OK)
+    if ((st = make_workspaces(nmax, zmax, (int)sv->ctas, sv->kstream, &sv->ws, &sv->ws_bytes, &wsh)) != CLDIAM_OK)
         return cleanup(st);
     if (sv->budget && arena_bytes(a) + sv->ws_bytes > sv->budget)
         return cleanup(fail(CLDIAM_ERR_OOM, "arena plus serving workspace exceed the budget"));

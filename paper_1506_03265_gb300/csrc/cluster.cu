@@ -7,7 +7,7 @@
 #include <vector>
 
 
-#include "cluster_dev.cuh"
+#include "grow.cuh"
 #include "internal.cuh"
 #include "prof.cuh"
 
@@ -92,202 +92,6 @@ __global__ void k_assign_cid(uint32_t n, const uint32_t* __restrict__ center, co
 // atomic minimum when it undercuts the snapshot; the per-step stamp decides
 // "first change" (next list) and "newly covered" as in the pushed form.  No
 // block barrier: warps run independently, so many gathers stay in flight.
-
-// a5, pushed form: the frontier's adjacency lists are one flattened range of E
-// positions; each warp takes QC consecutive positions (4 groups of 32), finds
-// the entries they span from the chunk table (cfirst, written by the frontier
-// producers) and maps positions to entries with the start words.  A pushing
-// entry (start-of-step key of its node) sends (d_u + w, c_u) to each
-// neighbour: a key read (evict-last) filters candidates that cannot win, the
-// rest lower the neighbour's key with a no-return atomic minimum.  A pulling
-// entry (an unfrozen node that reads the candidates of its contracted
-// neighbours, kPullTag | v) reduces its candidates over its lanes first, so
-// it lowers its own key once per group segment.  No block barrier.
-// RESIDENT: the kernel runs many steps (k_grow), so node state is read past L1, whose lines may be older than a
-// stage's reset; a one-step launch reads through L1 (a stale line only lets an extra candidate through).  Its
-// positions and ids come from lists that other CTAs wrote earlier in the same launch, so they are checked against the
-// graph's sizes (n, nnz) before use; one outside them would set ctr->bad.
-template <int WARPS>
-struct PushSmem {
-    unsigned long long skey[WARPS][QC + 2];
-    uint32_t spre[WARPS][QC + 1];  // first positions of the entries after the chunk's first
-    uint32_t sbase[WARPS][QC + 2];
-    uint32_t sbuf[WARPS][PNB];
-};
-
-template <bool RESIDENT, int WARPS>
-__device__ __forceinline__ void dev_push(const uint32_t* __restrict__ fbase, const unsigned long long* __restrict__ fkey,
-                                         const uint32_t* __restrict__ fpre, const uint32_t* __restrict__ cfirst,
-                                         uint32_t nf, uint32_t E, const uint2* __restrict__ adj,
-                                         const uint32_t* __restrict__ center, const uint32_t* __restrict__ Dcum,
-                                         unsigned long long* __restrict__ key, uint32_t delta,
-                                         uint32_t* __restrict__ stamp, uint32_t stepid,
-                                         uint32_t* __restrict__ next, Counters* ctr, PushSmem<WARPS>& smp, uint32_t br,
-                                         uint32_t nb, uint32_t n = 0, uint32_t nnz = 0) {
-    auto& spre = smp.spre;
-    auto& sbase = smp.sbase;
-    auto& skey = smp.skey;
-    auto& sbuf = smp.sbuf;
-    const uint32_t lane = lane_id(), warp = threadIdx.x >> 5;
-    const uint64_t pol_stream = l2_evict_first_policy(), pol_keep = l2_evict_last_policy();
-    const unsigned le_mask = 0xffffffffu >> (31u - lane);
-    WarpNext wn{sbuf[warp], 0};
-    unsigned long long newly = 0;
-    bool bad = false;
-    const uint32_t nq = (uint32_t)(((uint64_t)E + QC - 1) / QC);
-    const uint32_t nwarps = nb * WARPS;
-    for (uint32_t q = br * WARPS + warp; q < nq; q += nwarps) {
-        const uint32_t p0 = q * QC, e1 = min(E, p0 + QC);
-        // entry i0 holds p0; entries i0 + 1 .. il start inside (p0, p0 + QC] (at most QC of them)
-        const uint32_t i0 = __ldcg(&cfirst[q]);
-        const uint32_t il = q + 1 < nq ? __ldcg(&cfirst[q + 1]) : nf - 1;
-        if (RESIDENT && (i0 > il || il >= nf)) {
-            bad = true;
-            continue;
-        }
-        const uint32_t ne = min(il - i0 + 1, (uint32_t)QC + 1);
-        if (RESIDENT) __syncwarp();  // the previous chunk's entries have been read
-        for (uint32_t j = lane; j < ne; j += 32) {
-            if (j) spre[warp][j - 1] = __ldcg(&fpre[i0 + j]);
-            sbase[warp][j] = __ldcg(&fbase[i0 + j]);
-            skey[warp][j] = __ldcg(&fkey[i0 + j]);
-        }
-        __syncwarp();
-        uint32_t word[4], own[4];
-        {
-            uint32_t B = 0;
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                word[u] = group_starts(spre[warp] + B, ne - 1 - B, p0 + 32u * u, B, lane, le_mask, &own[u]);
-                B += (uint32_t)__popc(word[u]);
-            }
-        }
-        uint2 ed[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const uint32_t p = p0 + 32u * u + lane;
-            bool in = p < e1;
-            if (RESIDENT && in && (own[u] >= ne || sbase[warp][own[u]] + p >= nnz)) {
-                bad = true;
-                in = false;
-            }
-            ed[u] = in ? ld_stream_u2(adj + (sbase[warp][own[u]] + p), pol_stream) : make_uint2(0u, 0xFFFFFFFFu);
-        }
-        // RESIDENT: the groups' loads and exchanges are issued level by level for all four groups, since few warps
-        // share the latency (one group after another, a push took 14,000 cycles, so 8,200)
-        uint32_t pcu[4], pdu[4], tgt[4];
-        unsigned long long cnk[4];
-        if constexpr (RESIDENT) {
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                pcu[u] = kNone;
-                pdu[u] = 0;
-                if ((skey[warp][own[u]] & kPullTag) == kPullTag && ed[u].y <= delta) {
-                    pcu[u] = __ldcg(&center[ed[u].x]);
-                    if (Dcum) pdu[u] = __ldcg(&Dcum[ed[u].x]);
-                }
-            }
-        }
-        unsigned long long carry = kInfKey;  // pull entry still open at the previous group's end
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const unsigned long long ku = skey[warp][own[u]];
-            const bool is_pull = (ku & kPullTag) == kPullTag;
-            const bool live = p0 + 32u * u + lane < e1;
-            unsigned long long nk = kInfKey;
-            uint32_t target = 0;
-            if (live && !is_pull) {
-                const uint64_t cand = (ku >> 32) + ed[u].y;
-                if (cand <= delta) {
-                    target = ed[u].x;
-                    nk = (cand << 32) | (ku & 0xFFFFFFFFull);
-                }
-            } else if (live && ed[u].y <= delta) {  // pull: candidate of a contracted neighbour
-                uint32_t cu, du = 0;
-                if constexpr (RESIDENT) {
-                    cu = pcu[u];
-                    du = pdu[u];
-                } else {
-                    cu = __ldg(&center[ed[u].x]);
-                    if (cu != kNone && Dcum) du = __ldg(&Dcum[ed[u].x]);
-                }
-                const uint64_t cand = (uint64_t)du + ed[u].y;
-                if (cu != kNone && cand <= delta) nk = (cand << 32) | cu;
-            }
-            // pulling entries: one candidate per segment (all lanes of an entry share its kind)
-            if (__any_sync(0xffffffffu, is_pull)) {
-                unsigned long long pv = is_pull ? nk : kInfKey;
-                if (lane == 0 && !(word[u] & 1u)) pv = carry < pv ? carry : pv;
-                pv = segment_min(pv, word[u], lane);
-                const uint32_t last_head = word[u] ? 31u - (uint32_t)__clz(word[u]) : 0u;
-                const bool cont = u < 3 && !(word[(u + 1) & 3] & 1u);
-                carry = __shfl_sync(0xffffffffu, pv, last_head);
-                const unsigned le = word[u] & le_mask;
-                const uint32_t head = le ? 31u - (uint32_t)__clz(le) : 0u;
-                if (is_pull) {
-                    const bool flush = lane == head && !(cont && head == last_head);
-                    nk = flush ? pv : kInfKey;
-                    target = (uint32_t)ku;
-                }
-            } else {
-                carry = kInfKey;
-            }
-            if constexpr (RESIDENT) {
-                if (nk != kInfKey && target >= n) {
-                    bad = true;
-                    nk = kInfKey;
-                }
-                cnk[u] = nk;
-                tgt[u] = target;
-            } else {
-                bool first = false;
-                if (nk != kInfKey) {
-                    // the target's key and stamp in one round trip, through L1 (a stale line only lets an
-                    // extra candidate through: keys only fall within a launch, and the atomics decide); most
-                    // candidates lose to the current key
-                    const unsigned long long cur = ld_keep_u64(&key[target], pol_keep);
-                    const uint32_t stp = ld_keep_u32(&stamp[target], pol_keep);
-                    if (nk < cur) {
-                        red_min_keep_u64(&key[target], nk, pol_keep);
-                        if (stp != stepid) {  // hubs see many lowerings: only the first ones exchange
-                            const uint32_t old = atomicExch(&stamp[target], stepid);
-                            first = old != stepid;
-                            newly += old == 0u ? 1 : 0;
-                        }
-                    }
-                }
-                wn.put(first, target, lane);
-            }
-        }
-        if constexpr (RESIDENT) {
-            unsigned long long cur[4];
-            uint32_t stp[4], old[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const bool has = cnk[u] != kInfKey;
-                cur[u] = has ? ld_cg_keep_u64(&key[tgt[u]], pol_keep) : 0ull;
-                stp[u] = has ? ld_cg_keep_u32(&stamp[tgt[u]], pol_keep) : stepid;
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                old[u] = stepid;
-                if (cnk[u] < cur[u]) {
-                    red_min_keep_u64(&key[tgt[u]], cnk[u], pol_keep);
-                    if (stp[u] != stepid) old[u] = atomicExch(&stamp[tgt[u]], stepid);
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                newly += old[u] == 0u ? 1 : 0;
-                wn.put(old[u] != stepid, tgt[u], lane);
-            }
-        }
-        if (wn.cnt >= (uint32_t)PW) wn.flush(next, &ctr->nnext, lane);
-    }
-    if (wn.cnt) wn.flush(next, &ctr->nnext, lane);
-    warp_add_u64(&ctr->newly_covered, newly);
-    if (RESIDENT && __any_sync(0xffffffffu, bad) && lane == 0) atomicExch(&ctr->bad, 1u);
-}
 
 __global__ void __launch_bounds__(PT, 6) k_push(const uint32_t* __restrict__ fbase,
                                                 const unsigned long long* __restrict__ fkey,
@@ -427,180 +231,11 @@ __global__ void __launch_bounds__(PT, 6) k_pull(uint32_t n, uint32_t nnz, uint32
                     blockIdx.x, gridDim.x);
 }
 
-// ---------------------------------------------------------------- resident growth
-// Small steps are latency: as separate launches a step is a push, a snapshot, a counter reset and a counter read
-// that the host waits for, 37 us on a 1,001 x 1,001 mesh for frontiers of a few thousand entries.  k_grow runs them
-// in one launch: one thread-block cluster (its CTAs are resident together, and its barrier orders their memory)
-// takes growing steps back to back, every CTA deciding from the same counters, until a step is too large for it or
-// the growth ends; on small graphs it runs whole stages (draw, listing, doubling, contraction) too.
-// Bound by dependent L2 round trips (chunk table, entries, adjacency, keys, stamps, append; then the snapshot's): 16,000
-// cycles a step up to 65,000 entries, 33,000 at 100,000, of which a cluster barrier is 1,050.  Clustering alone, host
-// loop / resident: 64^2 mesh (44 steps) 1,602 / 504 us, 300^2 mesh (101) 3,101 / 1,326 us, 1,001^2 mesh (206) 7,405 /
-// 4,779 us, road mesh 4,096^2 (134) 12,520 / 11,555 us.  Above 2^18 entries a step of the whole device (push and
-// snapshot 13 to 40 us and 22 us between them) is the faster one; a whole-node pass over more than 2^17 nodes by 16
-// SMs likewise.
-constexpr int GT = 1024;                     // threads per CTA
-constexpr int GCTAS = 16;                    // CTAs of the cluster
-constexpr uint32_t kGrowEntries = 1u << 18;  // largest step: 16 passes of a warp's 128 positions over the cluster's warps
-constexpr uint32_t kGrowNodes = 1u << 17;    // whole stages up to this many nodes: 8 rounds of a node per thread
-constexpr uint32_t kGrowEpochs = 1u << 20;   // phases per launch, after which the host launches it again
-
-enum GrowPhase : uint32_t { kPhaseStage = 0, kPhaseStep = 1, kPhaseGrown = 2, kPhaseDone = 3, kPhaseFailed = 4 };
-
-// The control state of CLUSTER between phases, kept by the host and by every thread of k_grow alike.
-struct GrowState {
-    uint64_t U;           // unfrozen nodes at the stage's start
-    uint64_t covered;     // of them, nodes holding a key
-    uint64_t frozen_deg;  // adjacency entries of frozen nodes
-    uint64_t node_updates, edges_scanned, centers_drawn;
-    uint64_t unfrozen;    // what the last draw saw
-    uint32_t phase, stage, stepid, delta;
-    uint32_t nf, E, cur;  // the frontier and which pair of buffers holds it
-    uint32_t growth_steps;
-    uint32_t steps, stages, doublings, guard_exits;
-};
-
-struct GrowArgs {
-    const uint64_t* off;
-    const uint2* adj;
-    unsigned long long* key;
-    unsigned long long* keyS;
-    unsigned long long* fkey[2];
-    uint32_t *center, *D, *R, *stamp, *next;
-    uint32_t *fbase[2], *fpre[2], *cfirst[2];
-    Counters* ring;  // three counter blocks, zeroed
-    GrowState* out;
-    double tau, L;
-    uint64_t seed, nnz;
-    uint32_t n, step_cap, max_entries;
-    bool cumulative, pull_ok, stages;
-};
-
-struct GrowSmem {
-    PushSmem<GT / 32> push;
-    unsigned long long scratch[33];
-    Counters seen;
-};
-
-__device__ __forceinline__ void grow_barrier() {
-    __syncwarp();
-    asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
-}
-
+// resident growth (grow.cuh) by one thread-block cluster
 __global__ void __launch_bounds__(GT, 1) k_grow(const GrowArgs a, GrowState g) {
     extern __shared__ __align__(16) unsigned char grow_smem[];
-    GrowSmem& sm = *reinterpret_cast<GrowSmem*>(grow_smem);
-    const uint32_t br = blockIdx.x, nb = gridDim.x;  // one cluster: the CTA's rank and the cluster's size
-    uint32_t epoch = 0;
-    // Counter block of the current epoch (between two closing barriers).  An epoch clears the next one's block, last
-    // read two epochs ago: every CTA has passed the barrier that closed the epoch in between.
-    const auto ctr = [&]() { return a.ring + epoch % 3; };
-    const auto close_epoch = [&]() {  // every thread gets the epoch's counters
-        if (br == 0 && threadIdx.x < sizeof(Counters) / 8)
-            reinterpret_cast<unsigned long long*>(a.ring + (epoch + 1) % 3)[threadIdx.x] = 0ull;
-        grow_barrier();
-        if (threadIdx.x < sizeof(Counters) / 8)
-            reinterpret_cast<unsigned long long*>(&sm.seen)[threadIdx.x] =
-                __ldcg(reinterpret_cast<const unsigned long long*>(ctr()) + threadIdx.x);
-        __syncthreads();
-        ++epoch;
-    };
-    const auto rebuild = [&]() {
-        const bool pull = a.pull_ok && (a.nnz - g.frozen_deg) < g.frozen_deg;
-        dev_rebuild(a.n, a.key, a.center, a.cumulative ? a.D : nullptr, a.off, g.delta, pull, a.fbase[g.cur],
-                    a.fkey[g.cur], a.fpre[g.cur], a.cfirst[g.cur], ctr(), sm.scratch, br, nb);
-        close_epoch();
-        g.nf = (uint32_t)(sm.seen.front >> 32);
-        g.E = (uint32_t)sm.seen.front;
-    };
-    while (epoch < kGrowEpochs) {
-        if (g.phase == kPhaseStep) {
-            if (g.E > a.max_entries) break;
-            uint32_t updated = 0;
-            ++g.growth_steps;
-            ++g.stepid;
-            if (g.nf > 0) {
-                dev_push<true>(a.fbase[g.cur], a.fkey[g.cur], a.fpre[g.cur], a.cfirst[g.cur], g.nf, g.E, a.adj, a.center,
-                               a.cumulative ? a.D : nullptr, a.key, g.delta, a.stamp, g.stepid, a.next, ctr(), sm.push,
-                               br, nb, a.n, (uint32_t)a.nnz);
-                grow_barrier();
-                const uint32_t nn = min(__ldcg(&ctr()->nnext), a.n), o = g.cur ^ 1;
-                dev_snapshot(a.next, nn, a.key, a.off, g.delta, a.fbase[o], a.fkey[o], a.fpre[o], a.cfirst[o], ctr(),
-                             sm.scratch, br, nb, a.keyS, a.n);
-                close_epoch();
-                if (sm.seen.bad) {
-                    g.phase = kPhaseFailed;
-                    g.unfrozen = ~g.U;
-                    break;
-                }
-                updated = sm.seen.nnext;
-                g.covered += sm.seen.newly_covered;
-                g.edges_scanned += g.E;
-                g.nf = (uint32_t)(sm.seen.front >> 32);
-                g.E = (uint32_t)sm.seen.front;
-                g.cur = o;
-            }
-            g.steps++;
-            g.node_updates += updated;
-            if (!(updated != 0 && 2 * g.covered < g.U && (a.step_cap == 0 || g.growth_steps < a.step_cap)))
-                g.phase = kPhaseGrown;
-        } else if (!a.stages) {
-            break;
-        } else if (g.phase == kPhaseStage) {
-            uint64_t thr = 0;
-            if (!stage_threshold(g.U, a.tau, a.L, &thr)) {
-                g.phase = kPhaseDone;
-                break;
-            }
-            if (g.stage > kMaxStages) {
-                g.phase = kPhaseFailed;
-                break;
-            }
-            dev_select(a.n, a.center, a.key, a.seed, g.stage, thr, ctr(), br, nb, a.keyS);
-            close_epoch();
-            g.covered = sm.seen.selected;
-            g.centers_drawn += sm.seen.selected;
-            g.unfrozen = sm.seen.unfrozen;
-            if (g.unfrozen != g.U) {
-                g.phase = kPhaseFailed;
-                break;
-            }
-            rebuild();
-            g.growth_steps = 0;
-            g.phase = kPhaseStep;
-        } else if (g.phase == kPhaseGrown) {
-            if (2 * g.covered < g.U) {
-                // (connected graph: some covered or frozen node touches an uncovered one iff any exists)
-                if (g.delta < kDeltaMax && (g.covered > 0 || g.U < a.n)) {
-                    g.delta = (g.delta > kDeltaMax / 2) ? kDeltaMax : 2 * g.delta;
-                    g.doublings++;
-                    rebuild();
-                    g.growth_steps = 0;
-                    g.phase = kPhaseStep;
-                    continue;
-                }
-                g.guard_exits++;
-            }
-            dev_finalize_d(a.n, a.key, a.center, a.cumulative ? nullptr : a.R, a.D, ctr(), br, nb);
-            grow_barrier();
-            dev_finalize_freeze(a.n, a.key, a.center, a.R, a.D, a.off, ctr(), br, nb, a.keyS, a.cumulative);
-            close_epoch();
-            const bool overflow = sm.seen.overflow != 0;
-            g.U -= sm.seen.frozen;
-            g.frozen_deg += sm.seen.frozen_deg;
-            if (overflow) {
-                g.phase = kPhaseFailed;
-                g.unfrozen = g.U = 0;
-                break;
-            }
-            g.stages++;
-            ++g.stage;
-            g.phase = kPhaseStage;
-        } else {
-            break;
-        }
-    }
-    if (br == 0 && threadIdx.x == 0) *a.out = g;
+    grow_run(a, g, *reinterpret_cast<GrowSmem*>(grow_smem), blockIdx.x, gridDim.x, [] { cluster_barrier(); });
+    if (blockIdx.x == 0 && threadIdx.x == 0) *a.out = g;
 }
 
 // CTAs of k_grow's cluster on this device: 16 where such a cluster can be resident, else the portable 8, else 0 (not
@@ -847,6 +482,8 @@ cldiam_status cluster(cldiam_graph* g, double tau, uint64_t seed, const cldiam_o
         a.n = n;
         a.step_cap = step_cap;
         a.max_entries = grow_entries;
+        a.max_epochs = kGrowEpochs;
+        a.connected = true;
         a.cumulative = cumulative;
         a.pull_ok = pull_ok;
         a.stages = grow_stages;

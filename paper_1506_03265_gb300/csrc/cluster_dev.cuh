@@ -54,7 +54,6 @@ struct Counters {
 static_assert(offsetof(Counters, bad) + 4 - offsetof(Counters, newly_covered) == 24,
               "the per-step counters form one block");
 
-constexpr int RC = 1024;  // adjacency entries per relax chunk of one CTA (the many-graph form)
 constexpr int QC = 128;   // frontier positions per chunk-table slot (one warp chunk of the one-graph form)
 // In shared memory a pull entry's key is kPullTag | v: a pushed key has
 // d < Delta <= 2^31, so its high word is never all ones.
@@ -302,225 +301,6 @@ __device__ __forceinline__ void dev_rebuild(uint32_t n, const unsigned long long
             }
         }
     }
-}
-
-// Shared memory of the relax chunks: the frontier entries a chunk spans,
-// double-buffered so that one block barrier per chunk separates staging from
-// use (a buffer is restaged only after every thread has passed the barrier
-// that follows its last use).
-struct RelaxSmem {
-    uint32_t pre[2][RC + 1];              // entry's first position in the flattened list
-    uint32_t base[2][RC + 1];             // off[v] - pre (mod 2^32): adjacency index = base + position
-    unsigned long long key[2][RC + 1];    // start-of-step key, or kPullTag | v for a pull entry
-};
-// Changed nodes waiting to be appended to the next list: 2 x U x 32 words per
-// warp, flushed once half full.
-template <int U>
-constexpr int relax_nbuf_words(int warps) { return warps * 2 * U * 32; }
-
-// largest i < n with a[i] <= x, for nondecreasing a with a[lo] <= x: a
-// blockDim-ary search, one probe per thread and one barrier per round.
-__device__ __forceinline__ uint32_t block_last_le(const uint32_t* __restrict__ a, uint32_t lo, uint32_t n, uint32_t x) {
-    uint32_t len = n - lo;
-    while (len > 1) {
-        const uint32_t step = (len + blockDim.x - 1) / blockDim.x;
-        const uint64_t idx = (uint64_t)lo + (uint64_t)threadIdx.x * step;
-        const bool pred = threadIdx.x > 0 && idx < (uint64_t)lo + len && __ldcg(&a[idx]) <= x;
-        const uint32_t c = (uint32_t)__syncthreads_count(pred);  // probes 1..c hold, the rest do not
-        const uint32_t nlo = lo + c * step;
-        len = min(step, lo + len - nlo);
-        lo = nlo;
-    }
-    return lo;
-}
-
-__device__ __forceinline__ void cp_async_4(void* smem, const void* gmem) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"((unsigned)__cvta_generic_to_shared(smem)),
-                 "l"(gmem)
-                 : "memory");
-}
-__device__ __forceinline__ void cp_async_8(void* smem, const void* gmem) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"((unsigned)__cvta_generic_to_shared(smem)),
-                 "l"(gmem)
-                 : "memory");
-}
-__device__ __forceinline__ void cp_async_commit_wait_all() {
-    asm volatile("cp.async.commit_group;\n" ::: "memory");
-    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
-}
-
-// a5: one synchronous Delta-growing step over the frontier, edge-balanced:
-// the frontier's adjacency lists are viewed as one flattened range of E
-// entries cut into chunks of U x blockDim.x; each CTA takes chunks, each warp
-// U x 32 consecutive positions of it, and maps every position to its
-// frontier entry from the entries the chunk spans, held in shared memory, so
-// hubs spread over many CTAs.  A block-wide search finds a chunk's entries.  The entries of the
-// next chunk are copied into the other shared buffer (cp.async) while the
-// current one is processed, so one barrier per chunk remains.  Every thread
-// handles U positions per chunk with their loads issued together; a key is
-// lowered with a plain atomicMin whose result is not needed, and the
-// per-step stamp decides both "first change this step" (the node joins the
-// next list) and "newly covered" (a node that was never lowered before had
-// no key: centers and frozen nodes cannot be lowered).  Changed nodes gather
-// in a per-warp shared buffer that is appended to the next list with one
-// atomic per U x 32 or more nodes.  L2STAGE: the frontier entries are staged
-// with L2 loads instead of cp.async through L1 (several CTAs of one job write
-// the frontier, and none of them ends its kernel between steps).
-template <int U, bool L2STAGE = false>
-__device__ __forceinline__ void dev_relax(const uint32_t* __restrict__ fbase, const unsigned long long* __restrict__ fkey,
-                                          const uint32_t* __restrict__ fpre,
-                                          uint32_t nf, uint32_t E, const uint2* __restrict__ adj,
-                                          const uint32_t* __restrict__ center, const uint32_t* __restrict__ Dcum,
-                                          unsigned long long* __restrict__ key, uint32_t delta,
-                                          uint32_t* __restrict__ stamp, uint32_t stepid,
-                                          uint32_t* __restrict__ next, Counters* ctr, RelaxSmem& sm,
-                                          uint32_t* nbuf, uint32_t br, uint32_t nb) {
-    constexpr uint32_t kNB = 2 * U * 32;  // a chunk adds at most U x 32 nodes per warp
-    const uint32_t tid = threadIdx.x, nt = blockDim.x, CL = U * nt;  // CL <= RC
-    const uint64_t pol_stream = l2_evict_first_policy(), pol_keep = l2_evict_last_policy();
-    unsigned long long newly = 0;
-    uint32_t* wbuf = nbuf + (tid >> 5) * kNB;
-    uint32_t wcnt = 0;  // entries in this warp's buffer (warp-uniform)
-    const auto flush = [&]() {  // one atomic per kNB / 2 or more changed nodes
-        uint32_t wb = 0;
-        if (lane_id() == 0) wb = atomicAdd(&ctr->nnext, wcnt);
-        wb = __shfl_sync(0xffffffffu, wb, 0);
-        for (uint32_t j = lane_id(); j < wcnt; j += 32) next[wb + j] = wbuf[j];
-        wcnt = 0;
-        __syncwarp();
-    };
-    // entries [i0, i0 + cnt) that chunk c spans (cnt <= CL + 1: every entry has >= 1 adjacency entry)
-    const auto range_of = [&](uint32_t c, uint32_t& i0, uint32_t& cnt) {
-        const uint32_t e0 = c * CL;
-        const uint32_t e1 = (uint32_t)min((uint64_t)E, (uint64_t)e0 + CL);
-        i0 = block_last_le(fpre, 0, nf, e0);
-        const uint32_t il = block_last_le(fpre, i0, nf, e1 - 1);
-        cnt = il - i0 + 1;
-    };
-    const auto stage = [&](uint32_t b, uint32_t i0, uint32_t cnt) {
-        for (uint32_t j = tid; j < cnt; j += nt) {
-            if constexpr (L2STAGE) {
-                sm.pre[b][j] = __ldcg(&fpre[i0 + j]);
-                sm.base[b][j] = __ldcg(&fbase[i0 + j]);
-                sm.key[b][j] = __ldcg(&fkey[i0 + j]);
-            } else {
-                cp_async_4(&sm.pre[b][j], &fpre[i0 + j]);
-                cp_async_4(&sm.base[b][j], &fbase[i0 + j]);
-                cp_async_8(&sm.key[b][j], &fkey[i0 + j]);
-            }
-        }
-    };
-    uint32_t chunk = br;  // chunks br, br + nb, ...
-    if ((uint64_t)chunk * CL >= E) return;
-    uint32_t i0, cnt;
-    range_of(chunk, i0, cnt);
-    stage(0, i0, cnt);
-    cp_async_commit_wait_all();
-    __syncthreads();
-    for (uint32_t b = 0;; b ^= 1) {
-        const uint32_t e0 = chunk * CL;
-        const uint32_t e1 = (uint32_t)min((uint64_t)E, (uint64_t)e0 + CL);
-        const uint32_t nchunk = chunk + nb;
-        const bool has_next = (uint64_t)nchunk * CL < E;
-        uint32_t ni0 = 0, ncnt = 0;
-        if (has_next) {
-            range_of(nchunk, ni0, ncnt);
-            stage(b ^ 1, ni0, ncnt);  // buffer b ^ 1 was last read before the previous barrier
-        }
-        // owners of this warp's U x 32 consecutive positions: one binary search for the first, then
-        // per group of 32 the entries starting inside it are found with one OR-reduction (at most 32
-        // entries start in 32 positions, and they follow the previous group's last owner)
-        uint32_t pos[U], own[U];
-        {
-            const uint32_t lane = lane_id();
-            const uint32_t wp0 = e0 + (tid >> 5) * 32u * U;
-            uint32_t B = 0;
-            if (wp0 < e1) {
-                // entry j >= 1 starts at or after e0 + j, so the owner of position r is <= r
-                uint32_t lo = 0, hi = min(cnt - 1, wp0 - e0);
-                while (lo < hi) {
-                    const uint32_t mid = (lo + hi + 1) >> 1;
-                    if (sm.pre[b][mid] <= wp0) lo = mid; else hi = mid - 1;
-                }
-                B = lo;
-            }
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const uint32_t p0 = wp0 + 32u * u;
-                pos[u] = p0 + lane;
-                const uint32_t jj = B + 1 + lane;
-                const uint32_t pj = jj < cnt ? sm.pre[b][jj] : 0xFFFFFFFFu;
-                const uint32_t d = pj - p0;  // entries after B start at or after p0
-                const unsigned word = __reduce_or_sync(0xffffffffu, d < 32u ? 1u << d : 0u);
-                own[u] = B + (uint32_t)__popc(word & (0xffffffffu >> (31u - lane)));
-                B += (uint32_t)__popc(word);
-            }
-        }
-        uint2 ed[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-            ed[u] = pos[u] < e1 ? ld_stream_u2(adj + (sm.base[b][own[u]] + pos[u]), pol_stream)
-                                : make_uint2(0u, 0xFFFFFFFFu);
-        uint32_t target[U];
-        unsigned long long nk[U], cur[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const unsigned long long ku = sm.key[b][own[u]];
-            nk[u] = kInfKey;
-            target[u] = 0;
-            if (pos[u] < e1) {
-                if ((ku & kPullTag) != kPullTag) {
-                    const uint64_t cand = (ku >> 32) + ed[u].y;
-                    if (cand <= delta) {
-                        target[u] = ed[u].x;
-                        nk[u] = (cand << 32) | (ku & 0xFFFFFFFFull);
-                    }
-                } else if (ed[u].y <= delta) {
-                    const uint32_t cu = __ldcg(&center[ed[u].x]);
-                    if (cu != kNone) {
-                        const uint64_t cand = (uint64_t)(Dcum ? __ldcg(&Dcum[ed[u].x]) : 0u) + ed[u].y;
-                        if (cand <= delta) {
-                            target[u] = (uint32_t)ku;
-                            nk[u] = (cand << 32) | cu;
-                        }
-                    }
-                }
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) cur[u] = nk[u] != kInfKey ? ld_cg_keep_u64(&key[target[u]], pol_keep) : 0ull;
-        bool first[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            first[u] = false;
-            if (nk[u] < cur[u]) {
-                // the key is below its start-of-step value after this, whoever wins the minimum
-                red_min_keep_u64(&key[target[u]], nk[u], pol_keep);
-                // only the first changers of a node this step need the exchange (hubs see many)
-                if (__ldcg(&stamp[target[u]]) != stepid) {
-                    const uint32_t old = atomicExch(&stamp[target[u]], stepid);
-                    first[u] = old != stepid;
-                    newly += old == 0u ? 1 : 0;
-                }
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const unsigned m = __ballot_sync(0xffffffffu, first[u]);
-            if (first[u]) wbuf[wcnt + (uint32_t)__popc(m & lanemask_lt())] = target[u];
-            wcnt += (uint32_t)__popc(m);
-        }
-        __syncwarp();
-        if (wcnt >= kNB / 2) flush();
-        cp_async_commit_wait_all();
-        __syncthreads();
-        if (!has_next) break;
-        chunk = nchunk;
-        i0 = ni0;
-        cnt = ncnt;
-    }
-    if (wcnt) flush();
-    warp_add_u64(&ctr->newly_covered, newly);
 }
 
 // the changed nodes become the next frontier, with their end-of-step keys
