@@ -292,9 +292,10 @@ cldiam_status cldiam_run(const uint32_t* src, const uint32_t* dst, const uint32_
  * cluster): graphs are packed into one device-resident CSR arena and a batch
  * of (graph, tau, seed) jobs runs the whole method -- CLUSTER (Algorithm 1),
  * the weighted quotient graph and Phi_approx (Section 4) -- in one persistent
- * launch, one graph per CTA at a time, largest graphs first.  The launch
- * ends with its largest graph on one CTA or with the even split of all work,
- * whichever is later; the largest graphs may therefore run first on the
+ * launch, one graph per CTA at a time, longest jobs first.  The launch
+ * ends with its longest job on one CTA or with the even split of all work,
+ * whichever is later; the largest graphs may therefore run on groups of CTAs
+ * beside the others, or, larger still, first on the
  * one-graph path with the whole device (cldiam_tuning.batch_split).  Every result is
  * identical to cldiam_cluster + cldiam_quotient_build + cldiam_estimate on the
  * same graph, tau and seed with the same options.
@@ -380,11 +381,11 @@ typedef struct {
                                       Floyd-Warshall in shared memory; 0 = 200                     */
     float sssp_delta_scale;        /* Delta-stepping with delta = 0: Delta = this x the average
                                       weight (>= 1); 0 = 1                                          */
-    uint32_t batch_split;          /* many-graph form: 2 = the k largest graphs (each with at least
-                                      2^16 entries) run first on the one-graph path with the whole
-                                      device, k chosen by a makespan model (one CTA's rate in the
-                                      launch against a fixed cost per graph on the one-graph path);
-                                      1 = every graph in the persistent launch; 0 = 2              */
+    uint32_t batch_split;          /* many-graph form: 2 = the largest graphs (each with at least 2^16
+                                      entries) run on groups of CTAs, or first on the one-graph path
+                                      with the whole device, how many by a time model (one CTA's rate,
+                                      a group's, a fixed cost per graph on the one-graph path);
+                                      1 = every graph on one CTA; 0 = 2                             */
     uint32_t reserved[8];          /* must be 0                                                     */
 } cldiam_tuning;
 

@@ -1,11 +1,12 @@
 // Many-graph form: graphs packed into one device CSR arena and processed by
 // one persistent launch.  Each CTA (1024 threads, one per SM) takes whole
-// graphs from a work queue (largest first) and runs CLUSTER(tau) (the phase
-// bodies of cluster_dev.cuh, rank 0 of 1, block barriers between phases),
-// the weighted quotient graph (Section 4) and the exact Phi(G_C) for it.
-// Results are identical to the one-graph-per-launch path: the same phase
-// bodies run in the same order on the same data, and the stage control uses
-// the same host-computed log2 n.
+// graphs from a work queue (longest first) and runs CLUSTER(tau) (the growth
+// loop of grow.cuh), the weighted quotient graph (Section 4) and the exact
+// Phi(G_C) for it; large graphs are shared by a group of CTAs (a thread-block
+// cluster) that run the same code, every phase split over them.  Results are
+// identical to the one-graph-per-launch path: the same phase bodies run in
+// the same order on the same data, and the stage control uses the same
+// host-computed log2 n.
 //
 // The quotient is deduplicated in a dense k x k matrix (atomicMin per
 // inter-cluster edge) instead of a sort; its row order equals the sorted
@@ -41,12 +42,16 @@ constexpr int BW = BT / 32;
 constexpr int kJobCtas = 8;  // CTAs that share a large job: the portable cluster size
 constexpr uint32_t kDenseCap = 1024;  // largest quotient deduplicated in the dense matrix
 constexpr uint64_t kSplitMinEntries = 1u << 16;  // graphs below this many entries always stay in the launch
-// makespan model of the many-graph split (GB300): seconds per unit of work (entry or node) on one 1,024-thread
-// CTA of the launch, and a graph's cost on the one-graph path (a fixed part for its launches and counter
-// reads, and a per-unit part with the whole device)
-constexpr double kCtaSecPerUnit = kBatchCtasPerSm == 1 ? 37e-9 : 63e-9;
-constexpr double kPlainSecPerGraph = 1.5e-3;
-constexpr double kPlainSecPerUnit = 0.05e-9;
+// Time model of the many-graph split (GB300; unit = entry or node): a job on one CTA, on a group of kJobCtas CTAs, and
+// on the one-graph path (launches and counter reads, then the whole device).  Graphs of fewer than 8 entries per node
+// (meshes, roads) take many small steps, others few large ones.  Measured on one CTA: meshes 15 ns a unit from 10^5 to
+// 10^6 units, R-MAT 4 to 5; on a group meshes of 4.6 / 6.2 / 10.7 x 10^5 units 2.4 / 3.0 / 3.6 ms, R-MAT 0.8 to 1.1 ns.
+// A batch of 200 graphs (10^3 to 10^6 units): every job on one CTA 15.8 ms, with groups 5.9 ms.
+inline double job_cta_s(double units, bool sparse) { return units * (sparse ? 15e-9 : 4.5e-9); }
+inline double job_group_s(double units, bool sparse) {
+    return sparse ? 1.6e-3 * std::min(1.0, units / 4e5) + units * 1.9e-9 : units * 1.0e-9;
+}
+inline double job_plain_s(double units, bool sparse) { return (sparse ? 3.0e-3 : 1.0e-3) + units * 0.1e-9; }
 // quotients up to this size are closed by Floyd-Warshall in shared memory (the k x k matrix, next to the
 // static shared memory, must fit kBatchCtasPerSm times per SM)
 constexpr uint32_t kSmemFwK = kBatchCtasPerSm == 1 ? 200 : 128;
@@ -143,8 +148,11 @@ __device__ __forceinline__ T block_all_reduce(T v, Op op, T ident, T* red) {
     return r;
 }
 
-struct BatchSmem {
+struct BatchSmem {  // (a CTA's copies of what every thread would otherwise hold in registers)
     GrowArgs args;
+    GrowState grown;  // CLUSTER's control state at its end
+    Workspace ws;
+    Job job;
     uint32_t red32[33];
     uint32_t woff[33];
     uint32_t word;
@@ -280,45 +288,49 @@ struct QuotientView {
     const uint32_t* gw;
 };
 
-// Exact SSSP from `source` by one warp: dist[k] and one bit per node to be relaxed again, both its own; a lane relaxes
-// one node's entries, improved nodes get their bit back, until no bit is left.  No path sum can reach 2^32 - 1.  Returns
-// the largest distance at every lane; *err when the sweeps exceed their limit.
-__device__ uint32_t warp_sssp(uint32_t k, const QuotientView& q, uint32_t source, uint32_t* dist, uint32_t* bits,
-                              uint32_t* err) {
+// Exact SSSP from `source` by one warp, in its own memory: dist[k], one bit per node to be relaxed again and the list of
+// a round's nodes.  A round lists the nodes of the set bits and clears them, then a lane relaxes one node's entries and
+// gives improved nodes their bit back; the last round sets none.  (A lane per node of a 32-node word, without the list,
+// left most lanes idle: 90 of 480 nodes are improved in a round of a mesh's quotient.)  No path sum can reach 2^32 - 1.
+// Returns the largest distance at every lane; *err when the rounds exceed their limit.
+__device__ __forceinline__ uint32_t warp_sssp(uint32_t k, const QuotientView& q, uint32_t source, uint32_t* dist,
+                                              uint32_t* bits, uint16_t* list, uint32_t* err) {
     const uint32_t l = lane_id(), words = (k + 31) / 32;
     for (uint32_t v = l; v < k; v += 32) dist[v] = v == source ? 0u : kNone;
     for (uint32_t i = l; i < words; i += 32) bits[i] = i == source / 32 ? 1u << (source % 32) : 0u;
     __syncwarp();
-    for (uint32_t sweep = 0;; ++sweep) {
-        bool any = false;
-        for (uint32_t i = 0; i < words; ++i) {
-            const uint32_t b = *(volatile uint32_t*)&bits[i];
-            if (!b) continue;
-            any = true;
-            __syncwarp();
-            if (l == 0) bits[i] = 0;
-            __syncwarp();
-            if ((b >> l) & 1u) {
-                const uint32_t v = 32 * i + l, d = *(volatile uint32_t*)&dist[v];
-                for (uint32_t j = q.off[v]; j < q.off[v + 1]; ++j) {
-                    const uint32_t u = q.scol ? q.scol[j] : __ldcg(&q.gcol[j]);
-                    const uint32_t nd = d + (q.scol ? q.sw[j] : __ldcg(&q.gw[j]));
-                    if (nd < *(volatile uint32_t*)&dist[u] && nd < atomicMin(&dist[u], nd))
-                        atomicOr(&bits[u / 32], 1u << (u % 32));
-                }
-            }
-            __syncwarp();
+    for (uint32_t round = 0;; ++round) {
+        uint32_t m = 0;  // listed nodes; words <= 32: one word per lane
+        {
+            const uint32_t b = l < words ? bits[l] : 0u;
+            const uint32_t c = (uint32_t)__popc(b), incl = warp_incl_scan(c);
+            m = __shfl_sync(0xffffffffu, incl, 31);
+            if (m == 0) break;
+            uint32_t at = incl - c;
+            for (uint32_t x = b; x; x &= x - 1) list[at++] = (uint16_t)(32 * l + (uint32_t)__ffs(x) - 1);
+            if (l < words) bits[l] = 0;
         }
-        if (!any) break;
-        if (sweep > 4 * k + 64) {  // far above any real count: a guard, reported as an error
+        __syncwarp();
+        if (round > 4 * k + 64) {  // far above any real count: a guard, reported as an error
             if (l == 0) atomicExch(err, 1u);
             break;
         }
+        for (uint32_t g = l; g < m; g += 32) {
+            const uint32_t v = list[g], d = *(volatile uint32_t*)&dist[v];
+            for (uint32_t j = q.off[v]; j < q.off[v + 1]; ++j) {
+                const uint32_t u = q.scol ? q.scol[j] : __ldcg(&q.gcol[j]);
+                const uint32_t nd = d + (q.scol ? q.sw[j] : __ldcg(&q.gw[j]));
+                if (nd < *(volatile uint32_t*)&dist[u] && nd < atomicMin(&dist[u], nd))
+                    atomicOr(&bits[u / 32], 1u << (u % 32));
+            }
+        }
+        __syncwarp();
     }
     uint32_t ecc = 0;
     for (uint32_t v = l; v < k; v += 32) ecc = dist[v] != kNone ? max(ecc, dist[v]) : ecc;
     return __reduce_max_sync(0xffffffffu, ecc);
 }
+static_assert(kDenseCap <= 1024, "one word of a round's bits per lane");
 
 constexpr size_t kBatchDyn = 208 * 1024;  // dynamic shared memory of a CTA
 static_assert(kBatchDyn >= sizeof(GrowSmem) && kBatchDyn >= (size_t)kSmemFwK * kSmemFwK * 4 &&
@@ -331,8 +343,8 @@ template <class Barrier>
 __device__ void group_bound_diameter(uint32_t k, uint32_t entries, const Workspace& ws, uint32_t* ub, uint32_t* lb,
                                      uint32_t* src, uint32_t* soff, BatchSmem& sm, uint32_t br, uint32_t nb,
                                      Barrier barrier) {
-    // shared memory behind the offsets: the CSR if it leaves room for 16 warps, then dist and bits per warp
-    const uint32_t words = (k + 31) / 32, per = k + words;  // words of one warp's SSSP
+    // shared memory behind the offsets: the CSR if it leaves room for 16 warps, then dist, bits and list per warp
+    const uint32_t words = (k + 31) / 32, per = k + words + (k + 1) / 2;  // words of one warp's SSSP
     uint32_t* mem = soff + k + 1;
     const size_t room = kBatchDyn / 4 - (k + 1);
     const size_t csr = entries + (entries + 1) / 2;
@@ -359,7 +371,8 @@ __device__ void group_bound_diameter(uint32_t k, uint32_t entries, const Workspa
         if (w < warps && i < ns) {
             uint32_t* dist = mem + (size_t)w * per;
             const uint32_t source = first ? (uint32_t)((uint64_t)i * k / ns) : __ldcg(&src[i]);
-            const uint32_t ecc = warp_sssp(k, q, source, dist, dist + k, &ws.fin->err);
+            const uint32_t ecc = warp_sssp(k, q, source, dist, dist + k,
+                                           reinterpret_cast<uint16_t*>(dist + k + words), &ws.fin->err);
             if (l == 0) atomicMax(&ws.fin->best, ecc);
             for (uint32_t v = l; v < k; v += 32) {
                 const uint32_t d = dist[v];
@@ -387,26 +400,27 @@ __device__ void group_bound_diameter(uint32_t k, uint32_t entries, const Workspa
     }
 }
 
-// The end of a job: singletons, relabel, the dense quotient and Phi(G_C); CTA 0 stores the result.  `res` holds the
-// CLUSTER counters so far.  Every phase is split over the job's CTAs (br of nb), a barrier between phases.
+// The end of a job: singletons, relabel, the dense quotient and Phi(G_C); CTA 0 stores the result, with the counters of
+// sm.grown.  Every phase is split over the job's CTAs (br of nb), a barrier between phases.
 template <class Barrier>
 __device__ void finish_job(const Job& job, const ArenaDesc& d, const uint64_t* __restrict__ off,
                            const uint2* __restrict__ adj, const uint32_t* __restrict__ row, const Workspace& ws,
-                           BatchSmem& sm, uint32_t* dyn, JobOut* out, cldiam_result res, uint32_t status,
-                           uint32_t br, uint32_t nb, Barrier barrier) {
+                           BatchSmem& sm, uint32_t* dyn, JobOut* out, uint32_t status, uint32_t br, uint32_t nb,
+                           Barrier barrier) {
     const unsigned tid = threadIdx.x, w = tid >> 5, l = lane_id();
     const uint32_t n = d.n, gt = br * BT + tid, gw = br * BW + w;  // thread and warp among the job's
     const uint32_t nt = nb * BT, nw = nb * BW;
     FinishCtl* fin = ws.fin;
     uint2* cd = reinterpret_cast<uint2*>(ws.fkey[0]);  // (cluster id, D) of every node
     const auto pack = [](uint2 x) { return (unsigned long long)x.y << 32 | x.x; };
+    uint32_t k = 0, qe = 0;
     if (status == kJobOk) {
         dev_singletons(n, ws.center, ws.D, br, nb);
         barrier();
         // cluster id = rank of the center among the centers: counts of the CTAs' shares, then ranks
         const uint32_t share = (uint32_t)(((uint64_t)n + (uint64_t)nb * 4096 - 1) / ((uint64_t)nb * 4096) * 4096);
         const uint32_t lo = min(n, br * share), hi = (uint32_t)min((uint64_t)n, (uint64_t)lo + share);
-        uint32_t first = 0, k = 0;
+        uint32_t first = 0;
         if (nb > 1) {
             const uint32_t c = block_centers(lo, hi, ws.center, nullptr, 0, sm);
             if (tid == 0) fin->part[br] = c;
@@ -419,7 +433,6 @@ __device__ void finish_job(const Job& job, const ArenaDesc& d, const uint64_t* _
         }
         const uint32_t mine = block_centers(lo, hi, ws.center, ws.stamp, first, sm);  // stamp reused as rank
         if (nb == 1) k = mine;
-        res.k = k;
         barrier();
         uint32_t* ub = ws.R;
         uint32_t* lb = ws.next;
@@ -526,8 +539,7 @@ __device__ void finish_job(const Job& job, const ArenaDesc& d, const uint64_t* _
                 atomicMax(&fin->wmax, wmax);
             }
             barrier();
-            const uint32_t qe = (uint32_t)__ldcg(&fin->entries);
-            res.quotient_edges = qe;
+            qe = (uint32_t)__ldcg(&fin->entries);
             bool ovf2 = false;
             // No path sum of an SSSP can reach 2^32 - 1 when the sum of the rows' heaviest entries and one more entry do
             // not; Floyd-Warshall also adds two paths.  Up to fw_k nodes it takes dense quotients, and those whose two
@@ -587,14 +599,26 @@ __device__ void finish_job(const Job& job, const ArenaDesc& d, const uint64_t* _
             }
             if (__any_sync(0xffffffffu, ovf2) && l == 0) atomicExch(&fin->err, 2u);
             barrier();
-            const uint32_t err = __ldcg(&fin->err), phi = __ldcg(&fin->best);
-            if (err) status = err == 1u ? kJobDiverged : kJobOverflow;
-            res.radius = __ldcg(&fin->rmax);
-            res.phi_gc = phi;
-            res.phi_approx = (uint64_t)phi + 2ull * res.radius;
+            if (const uint32_t err = __ldcg(&fin->err)) status = err == 1u ? kJobDiverged : kJobOverflow;
         }
     }
     if (br == 0 && tid == 0) {
+        const GrowState& g = sm.grown;
+        cldiam_result res;
+        memset(&res, 0, sizeof res);
+        res.stages = g.stages;
+        res.steps = g.steps;
+        res.doublings = g.doublings;
+        res.delta_end = g.delta;
+        res.guard_exits = g.guard_exits;
+        res.node_updates = g.node_updates;
+        res.edges_scanned = g.edges_scanned;
+        res.centers_drawn = g.centers_drawn;
+        res.k = k;
+        res.quotient_edges = qe;
+        res.radius = __ldcg(&fin->rmax);
+        res.phi_gc = __ldcg(&fin->best);
+        res.phi_approx = res.phi_gc + 2ull * res.radius;
         out->r = res;
         out->status = status;
     }
@@ -656,28 +680,23 @@ __device__ void run_job(const Job& job, const ArenaDesc& d, const uint64_t* __re
         a.stages = true;
         a.connected = d.connected != 0;
     }
-    GrowState g;
-    memset(&g, 0, sizeof g);
-    g.U = n;
-    g.phase = kPhaseStage;
-    g.stage = 1;
-    g.delta = job.delta0;
+    GrowSmem& gsm = *reinterpret_cast<GrowSmem*>(dyn);
+    GrowState& g = gsm.g;
+    if (tid == 0) {
+        memset(&g, 0, sizeof g);
+        g.U = n;
+        g.phase = kPhaseStage;
+        g.stage = 1;
+        g.delta = job.delta0;
+    }
     barrier();
-    grow_run(sm.args, g, *reinterpret_cast<GrowSmem*>(dyn), br, nb, barrier);
+    grow_run(sm.args, gsm, br, nb, barrier);
     uint32_t status = kJobOk;
     if (g.phase != kPhaseDone)
         status = g.stage > kMaxStages || g.unfrozen != g.U ? kJobDiverged : kJobOverflow;
-    cldiam_result res;
-    memset(&res, 0, sizeof res);
-    res.stages = g.stages;
-    res.steps = g.steps;
-    res.doublings = g.doublings;
-    res.delta_end = g.delta;
-    res.guard_exits = g.guard_exits;
-    res.node_updates = g.node_updates;
-    res.edges_scanned = g.edges_scanned;
-    res.centers_drawn = g.centers_drawn;
-    finish_job(job, d, off, adj, row, ws, sm, dyn, out, res, status, br, nb, barrier);
+    if (tid == 0) sm.grown = g;
+    __syncthreads();  // the state has been read: the end of the job uses its shared memory
+    finish_job(job, d, off, adj, row, ws, sm, dyn, out, status, br, nb, barrier);
 }
 
 // The jobs of a queue (largest first), one after another, by one CTA each (GROUP: by a thread-block cluster each).
@@ -698,13 +717,14 @@ __global__ void __launch_bounds__(BT, kBatchCtasPerSm)
         if constexpr (GROUP) cluster_barrier();
         else __syncthreads();
     };
-    const Workspace ws = wss[blockIdx.x / nb];
+    if (threadIdx.x == 0) sm.ws = wss[blockIdx.x / nb];
+    __syncthreads();
     for (;;) {
         uint32_t j;
         if constexpr (GROUP) {
-            if (br == 0 && threadIdx.x == 0) ws.fin->job = atomicAdd(queue, 1u);
+            if (br == 0 && threadIdx.x == 0) sm.ws.fin->job = atomicAdd(queue, 1u);
             barrier();
-            j = __ldcg(&ws.fin->job);
+            j = __ldcg(&sm.ws.fin->job);
         } else {
             if (threadIdx.x == 0) sm.word = atomicAdd(queue, 1u);
             __syncthreads();
@@ -712,13 +732,15 @@ __global__ void __launch_bounds__(BT, kBatchCtasPerSm)
             __syncthreads();
         }
         if (j >= count) break;
-        const Job job = jobs[j];
+        if (threadIdx.x == 0) sm.job = jobs[j];
+        __syncthreads();
         const uint64_t t0 = global_ns();
-        run_job(job, descs[job.graph], arena_off, arena_adj, arena_row, ws, sm, dyn, &outs[job.out], br, nb, barrier);
-        barrier();  // (every CTA is done with the job's workspace)
+        run_job(sm.job, descs[sm.job.graph], arena_off, arena_adj, arena_row, sm.ws, sm, dyn, &outs[sm.job.out], br, nb,
+                barrier);
+        barrier();  // (every CTA is done with the job and its workspace)
         if (br == 0 && threadIdx.x == 0) {
-            outs[job.out].t_start = t0;
-            outs[job.out].t_end = global_ns();
+            outs[sm.job.out].t_start = t0;
+            outs[sm.job.out].t_end = global_ns();
         }
     }
 }
@@ -752,8 +774,7 @@ __global__ void __launch_bounds__(BT, kBatchCtasPerSm)
             uint32_t* done, long long idle_cycles) {
     extern __shared__ __align__(16) uint32_t dyn[];
     __shared__ BatchSmem sm;
-    __shared__ Job s_job;
-    const Workspace ws = wss[blockIdx.x];
+    if (threadIdx.x == 0) sm.ws = wss[blockIdx.x];
     for (;;) {
         if (threadIdx.x == 0) {
             uint32_t claimed = kNone;
@@ -778,27 +799,26 @@ __global__ void __launch_bounds__(BT, kBatchCtasPerSm)
             sm.word = claimed;
             if (claimed != kNone) {
                 const volatile Job* vj = ring + claimed;
-                s_job.tau = vj->tau;
-                s_job.L = vj->L;
-                s_job.seed = vj->seed;
-                s_job.graph = vj->graph;
-                s_job.delta0 = vj->delta0;
-                s_job.out = vj->out;
-                s_job.step_cap = vj->step_cap;
-                s_job.cumulative = vj->cumulative;
-                s_job.fw_k = vj->fw_k;
+                sm.job.tau = vj->tau;
+                sm.job.L = vj->L;
+                sm.job.seed = vj->seed;
+                sm.job.graph = vj->graph;
+                sm.job.delta0 = vj->delta0;
+                sm.job.out = vj->out;
+                sm.job.step_cap = vj->step_cap;
+                sm.job.cumulative = vj->cumulative;
+                sm.job.fw_k = vj->fw_k;
             }
         }
         __syncthreads();
         const uint32_t slot = sm.word;
         if (slot == kNone) break;
-        const Job job = s_job;
         __syncthreads();
-        run_job(job, descs[job.graph], arena_off, arena_adj, arena_row, ws, sm, dyn, &outs[job.out], 0u, 1u,
+        run_job(sm.job, descs[sm.job.graph], arena_off, arena_adj, arena_row, sm.ws, sm, dyn, &outs[sm.job.out], 0u, 1u,
                 [] { __syncthreads(); });
         if (threadIdx.x == 0) {
             __threadfence_system();
-            st_release_sys(&done[job.out], 1u);
+            st_release_sys(&done[sm.job.out], 1u);
         }
         __syncthreads();
     }
@@ -822,12 +842,15 @@ struct cldiam_arena {
     uint64_t off_cap = 0, adj_cap = 0, off_used = 0, adj_used = 0;
     void* ws = nullptr;  // cached per-CTA workspaces
     size_t ws_bytes = 0;
+    void* gws = nullptr;  // cached workspaces of the groups that share large jobs
+    size_t gws_bytes = 0;
+    cudaStream_t aux = nullptr;  // the one-CTA jobs run here beside the groups' on `stream`
     std::vector<double> last_start, last_end;  // per-job device times of the last batch (seconds)
 };
 
 namespace cld {
 
-static uint64_t arena_bytes(const cldiam_arena* a) { return a->off_cap * 8 + a->adj_cap * 12 + a->ws_bytes; }
+static uint64_t arena_bytes(const cldiam_arena* a) { return a->off_cap * 8 + a->adj_cap * 12 + a->ws_bytes + a->gws_bytes; }
 
 // grow a device array to hold `need` elements (doubling), keeping the first `used`
 template <class T>
@@ -859,7 +882,9 @@ void arena_free(cldiam_arena* a) {
     dfree(a->adj, a->stream);
     dfree(a->row, a->stream);
     dfree(a->ws, a->stream);
+    dfree(a->gws, a->stream);
     cudaStreamSynchronize(a->stream);
+    if (a->aux) cudaStreamDestroy(a->aux);
     delete a;
 }
 
@@ -1038,6 +1063,38 @@ static cldiam_status resident_per_sm(Kern k, std::atomic<bool>* done_flags, int*
     return CLDIAM_OK;
 }
 
+// launch configuration of `groups` job groups, one CTA per SM each of kJobCtas in a thread-block cluster
+static void job_group_config(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* at, int groups) {
+    at->id = cudaLaunchAttributeClusterDimension;
+    at->val.clusterDim.x = kJobCtas;
+    at->val.clusterDim.y = at->val.clusterDim.z = 1;
+    cfg->gridDim = dim3((unsigned)groups * kJobCtas);
+    cfg->blockDim = dim3(BT);
+    cfg->dynamicSmemBytes = batch_dyn_smem();
+    cfg->attrs = at;
+    cfg->numAttrs = 1;
+}
+// job groups that this device holds at once (0: none); asked once per device, concurrent first calls store the same
+static cldiam_status max_job_groups(int dev, int* out) {
+    static std::atomic<int> cached[64];  // 0 = not asked yet, else number + 1
+    *out = 0;
+    if (dev < 0 || dev >= 64) return CLDIAM_OK;
+    if (cached[dev].load() == 0) {
+        CLD_CUDA(cudaFuncSetAttribute(k_batch<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)batch_dyn_smem()));
+        cudaLaunchConfig_t cfg{};
+        cudaLaunchAttribute at{};
+        job_group_config(&cfg, &at, 1);
+        int m = 0;
+        if (cudaOccupancyMaxActiveClusters(&m, k_batch<true>, &cfg) != cudaSuccess) {
+            cudaGetLastError();
+            m = 0;
+        }
+        cached[dev].store(m + 1);
+    }
+    *out = cached[dev].load() - 1;
+    return CLDIAM_OK;
+}
+
 cldiam_status batch_run(cldiam_arena* a, const uint32_t* ids, const double* tau, const uint64_t* seed, uint32_t count,
                         const cldiam_opts* o, cldiam_result* out, cldiam_status* status) {
     if (!a || (count && (!ids || !tau || !seed || !out))) return fail(CLDIAM_ERR_INVALID_ARG, "NULL argument");
@@ -1067,39 +1124,58 @@ cldiam_status batch_run(cldiam_arena* a, const uint32_t* ids, const double* tau,
         jobs[i].cumulative = opts.contract_mode == CLDIAM_CONTRACT_CUMULATIVE ? 1u : 0u;
         jobs[i].fw_k = fw_k;
     }
-    // largest graphs first: the work queue then balances the tail
+    // longest jobs first: the work queue then balances the tail
+    const auto units = [&](const Job& j) { return (double)(a->graphs[j.graph].nnz + a->graphs[j.graph].n); };
+    const auto sparse = [&](const Job& j) { return a->graphs[j.graph].nnz < 8ull * a->graphs[j.graph].n; };
     std::stable_sort(jobs.begin(), jobs.end(), [&](const Job& x, const Job& y) {
-        return a->graphs[x.graph].nnz + a->graphs[x.graph].n > a->graphs[y.graph].nnz + a->graphs[y.graph].n;
+        return job_cta_s(units(x), sparse(x)) > job_cta_s(units(y), sparse(y));
     });
     static std::atomic<bool> attr[64];
     int cps = 1;
     CLD_TRY(resident_per_sm(k_batch<false>, attr, &cps));
     const int nsm = num_sms() * cps;  // CTAs of the launch
-    // The launch ends with its largest graph on one CTA, or with the even split of all work over the CTAs,
-    // whichever is later.  The k largest graphs can instead run first on the one-graph path, each with the
-    // whole device at a fixed cost per graph; k is chosen to minimise the estimated makespan
-    // (batch_split = 2; 1 keeps every graph in the launch).  Work = adjacency entries + nodes.
+    // The launch ends with its largest graph on one CTA, or with the even split of all work over the CTAs, whichever is
+    // later.  So the largest graphs may run elsewhere (batch_split = 2; 1 keeps every graph on one CTA): on groups of
+    // kJobCtas CTAs beside the others, or, larger still, first on the one-graph path, each with the whole device at a
+    // fixed cost per graph.  Both are prefixes of the jobs, chosen to minimise the estimated end.  Work = adjacency
+    // entries + nodes.
     const uint32_t split = tuning_for_batch(arena_entries(a, ids, count)).batch_split;
-    std::vector<double> cost(count);
-    double rest = 0.0;
-    for (uint32_t j = 0; j < count; ++j) {
-        cost[j] = (double)(a->graphs[jobs[j].graph].nnz + a->graphs[jobs[j].graph].n);
-        rest += cost[j];
+    int dev = 0;
+    CLD_CUDA(cudaGetDevice(&dev));
+    int max_groups = 0;
+    if (split == 2 && !serving_kernel_alive(dev)) CLD_TRY(max_job_groups(dev, &max_groups));
+    std::vector<double> one(count + 1, 0.0), grp(count + 1, 0.0);          // seconds of job j on one CTA, on a group
+    std::vector<double> one_from(count + 1, 0.0), grp_from(count + 1, 0.0);  // their sums over jobs[j ..)
+    for (uint32_t j = count; j-- > 0;) {
+        one[j] = job_cta_s(units(jobs[j]), sparse(jobs[j]));
+        grp[j] = job_group_s(units(jobs[j]), sparse(jobs[j]));
+        one_from[j] = one_from[j + 1] + one[j];
+        grp_from[j] = grp_from[j + 1] + grp[j];
     }
-    uint32_t nbig = 0;  // jobs[0 .. nbig) take the one-graph path (largest first, so a prefix)
+    uint32_t nbig = 0, ngrp = 0;  // jobs[0 .. nbig): one-graph path; jobs[nbig .. nbig + ngrp): groups
     if (split == 2) {
-        const auto launch_s = [&](uint32_t k, double rest_work) {
-            return k < count ? std::max(cost[k] * kCtaSecPerUnit, rest_work * kCtaSecPerUnit / nsm) : 0.0;
+        const auto big = [&](uint32_t j) { return a->graphs[jobs[j].graph].nnz >= kSplitMinEntries; };
+        // end of the launch when jobs[k .. k + g) run on groups and jobs[k + g ..) on one CTA each
+        const auto launch_s = [&](uint32_t k, uint32_t g) {
+            const double group_s = grp_from[k] - grp_from[k + g];
+            const double even = (group_s * kJobCtas + one_from[k + g]) / nsm;
+            const double groups = g ? std::max(grp[k], group_s / max_groups) : 0.0;
+            return std::max(std::max(even, groups), one[k + g]);
         };
-        double plain_s = 0.0, best = launch_s(0, rest);
-        for (uint32_t k = 1; k <= count && a->graphs[jobs[k - 1].graph].nnz >= kSplitMinEntries; ++k) {
-            plain_s += kPlainSecPerGraph + cost[k - 1] * kPlainSecPerUnit;
-            rest -= cost[k - 1];
-            const double t = plain_s + launch_s(k, rest);
-            if (t < best) {
-                best = t;
-                nbig = k;
+        double plain_s = 0.0, best = -1.0;
+        for (uint32_t k = 0; k <= count; ++k) {
+            if (k > 0) plain_s += job_plain_s(units(jobs[k - 1]), sparse(jobs[k - 1]));
+            if (best >= 0.0 && plain_s >= best) break;
+            for (uint32_t g = 0; k + g <= count; ++g) {
+                if (g > 0 && (max_groups == 0 || !big(k + g - 1))) break;
+                const double t = plain_s + launch_s(k, g);
+                if (best < 0.0 || t < best) {
+                    best = t;
+                    nbig = k;
+                    ngrp = g;
+                }
             }
+            if (k < count && !big(k)) break;
         }
     }
     a->last_start.assign(count, 0.0);
@@ -1137,14 +1213,23 @@ cldiam_status batch_run(cldiam_arena* a, const uint32_t* ids, const double* tau,
     }
     const uint32_t nrest = count - nbig;
     if (nrest > 0) {
-        uint32_t nmax_rest = 1;
-        uint64_t zmax_rest = 0;
-        for (uint32_t j = nbig; j < count; ++j) {
-            nmax_rest = std::max(nmax_rest, a->graphs[jobs[j].graph].n);
-            zmax_rest = std::max(zmax_rest, a->graphs[jobs[j].graph].nnz);
-        }
-        std::vector<Workspace> wsh;
-        CLD_TRY(make_workspaces(nmax_rest, zmax_rest, nsm, s, &a->ws, &a->ws_bytes, &wsh));
+        const auto workspaces = [&](uint32_t j0, uint32_t j1, int slices, void** buf, size_t* bytes,
+                                    std::vector<Workspace>* out) {
+            uint32_t nmax = 1;
+            uint64_t zmax = 0;
+            for (uint32_t j = j0; j < j1; ++j) {
+                nmax = std::max(nmax, a->graphs[jobs[j].graph].n);
+                zmax = std::max(zmax, a->graphs[jobs[j].graph].nnz);
+            }
+            return make_workspaces(nmax, zmax, slices, s, buf, bytes, out);
+        };
+        std::vector<Workspace> wsh, gwsh;
+        const int groups = std::min<int>((int)ngrp, max_groups);
+        if (ngrp > 0 && workspaces(nbig, nbig + ngrp, groups, &a->gws, &a->gws_bytes, &gwsh) != CLDIAM_OK)
+            ngrp = 0;  // no memory for the groups' workspaces: every job on one CTA
+        const uint32_t nones = nrest - ngrp;  // jobs on one CTA each
+        CLD_TRY(workspaces(nbig + ngrp, count, nsm, &a->ws, &a->ws_bytes, &wsh));
+        if (ngrp > 0) wsh.insert(wsh.end(), gwsh.begin(), gwsh.end());
         DBuf<ArenaDesc> ddesc;
         DBuf<Job> djobs;
         DBuf<Workspace> dws;
@@ -1152,18 +1237,50 @@ cldiam_status batch_run(cldiam_arena* a, const uint32_t* ids, const double* tau,
         DBuf<JobOut> douts;
         CLD_TRY(ddesc.alloc(a->graphs.size(), s));
         CLD_TRY(djobs.alloc(nrest, s));
-        CLD_TRY(dws.alloc(nsm, s));
-        CLD_TRY(queue.alloc(1, s));
+        CLD_TRY(dws.alloc(wsh.size(), s));
+        CLD_TRY(queue.alloc(2, s));
         CLD_TRY(douts.alloc(count, s));
         CLD_CUDA(cudaMemcpyAsync(ddesc.get(), a->graphs.data(), a->graphs.size() * sizeof(ArenaDesc),
                                  cudaMemcpyHostToDevice, s));
         CLD_CUDA(cudaMemcpyAsync(djobs.get(), jobs.data() + nbig, nrest * sizeof(Job), cudaMemcpyHostToDevice, s));
-        CLD_CUDA(cudaMemcpyAsync(dws.get(), wsh.data(), nsm * sizeof(Workspace), cudaMemcpyHostToDevice, s));
-        CLD_CUDA(cudaMemsetAsync(queue.get(), 0, 4, s));
+        CLD_CUDA(cudaMemcpyAsync(dws.get(), wsh.data(), wsh.size() * sizeof(Workspace), cudaMemcpyHostToDevice, s));
+        CLD_CUDA(cudaMemsetAsync(queue.get(), 0, 8, s));
         const size_t dyn = batch_dyn_smem();
-        CLD_K(K_MISC, s, k_batch<false><<<nsm, BT, dyn, s>>>(ddesc.get(), djobs.get(), nrest, a->off, a->adj, a->row, dws.get(),
-                                                       queue.get(), douts.get()));
-        CLD_LAUNCH_CHECK();
+        cudaStream_t ones = s;
+        CudaEvent fork, join;
+        if (ngrp > 0) {
+            // the groups first, on s; the one-CTA jobs beside them on the arena's second stream, on the SMs left and
+            // those that the groups leave.  Everything they use was allocated and filled on s before the fork, and s
+            // waits for them before anything is read or released.
+            if (nones > 0 && !a->aux) CLD_CUDA(cudaStreamCreateWithFlags(&a->aux, cudaStreamNonBlocking));
+            if (nones > 0) {
+                ones = a->aux;
+                CLD_TRY(fork.create());
+                CLD_TRY(join.create());
+                CLD_CUDA(cudaEventRecord(fork.e, s));
+                CLD_CUDA(cudaStreamWaitEvent(ones, fork.e, 0));
+            }
+            cudaLaunchConfig_t cfg{};
+            cudaLaunchAttribute at{};
+            job_group_config(&cfg, &at, groups);
+            cfg.stream = s;
+            const uint64_t* off = a->off;
+            const uint2* adj = a->adj;
+            const uint32_t* row = a->row;
+            CLD_K(K_MISC, s, CLD_CUDA(cudaLaunchKernelEx(&cfg, k_batch<true>, (const ArenaDesc*)ddesc.get(),
+                                                         (const Job*)djobs.get(), ngrp, off, adj, row, dws.get() + nsm,
+                                                         queue.get() + 1, douts.get())));
+        }
+        if (nones > 0) {
+            CLD_K(K_MISC, ones, k_batch<false><<<std::min<uint32_t>(nsm, nones), BT, dyn, ones>>>(
+                                    ddesc.get(), djobs.get() + ngrp, nones, a->off, a->adj, a->row, dws.get(), queue.get(),
+                                    douts.get()));
+            CLD_LAUNCH_CHECK();
+            if (ones != s) {
+                CLD_CUDA(cudaEventRecord(join.e, ones));
+                CLD_CUDA(cudaStreamWaitEvent(s, join.e, 0));
+            }
+        }
         std::vector<JobOut> hl(count);
         CLD_CUDA(cudaMemcpyAsync(hl.data(), douts.get(), count * sizeof(JobOut), cudaMemcpyDeviceToHost, s));
         CLD_CUDA(cudaStreamSynchronize(s));

@@ -232,10 +232,12 @@ __global__ void __launch_bounds__(PT, 6) k_pull(uint32_t n, uint32_t nnz, uint32
 }
 
 // resident growth (grow.cuh) by one thread-block cluster
-__global__ void __launch_bounds__(GT, 1) k_grow(const GrowArgs a, GrowState g) {
+__global__ void __launch_bounds__(GT, 1) k_grow(const GrowArgs a, const GrowState g) {
     extern __shared__ __align__(16) unsigned char grow_smem[];
-    grow_run(a, g, *reinterpret_cast<GrowSmem*>(grow_smem), blockIdx.x, gridDim.x, [] { cluster_barrier(); });
-    if (blockIdx.x == 0 && threadIdx.x == 0) *a.out = g;
+    GrowSmem& sm = *reinterpret_cast<GrowSmem*>(grow_smem);
+    if (threadIdx.x == 0) sm.g = g;
+    grow_run(a, sm, blockIdx.x, gridDim.x, [] { cluster_barrier(); });
+    if (blockIdx.x == 0 && threadIdx.x == 0) *a.out = sm.g;
 }
 
 // CTAs of k_grow's cluster on this device: 16 where such a cluster can be resident, else the portable 8, else 0 (not

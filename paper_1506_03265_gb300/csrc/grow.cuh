@@ -223,7 +223,7 @@ constexpr uint32_t kGrowEpochs = 1u << 20;   // phases per launch of k_grow, aft
 
 enum GrowPhase : uint32_t { kPhaseStage = 0, kPhaseStep = 1, kPhaseGrown = 2, kPhaseDone = 3, kPhaseFailed = 4 };
 
-// The control state of CLUSTER between phases, kept by the host and by every thread of k_grow alike.
+// The control state of CLUSTER between phases, kept by the host and by every CTA alike.
 struct GrowState {
     uint64_t U;           // unfrozen nodes at the stage's start
     uint64_t covered;     // of them, nodes holding a key
@@ -253,10 +253,15 @@ struct GrowArgs {
     bool cumulative, pull_ok, stages, connected;
 };
 
+// what a CTA does next, decided by its thread 0
+enum GrowWork : uint32_t { kWorkPush, kWorkDraw, kWorkList, kWorkGuard, kWorkFinal, kWorkLeave };
+
 struct GrowSmem {
     PushSmem<GT / 32> push;
     unsigned long long scratch[33];
-    Counters seen;
+    GrowState g;
+    uint64_t thr;  // draw threshold of the stage
+    uint32_t work;
 };
 
 // barrier of a thread-block cluster: all its threads, and their memory in order
@@ -264,126 +269,145 @@ __device__ __forceinline__ void cluster_barrier() {
     __syncwarp();
     asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
 }
-// The loop: phases until one that this launch may not take (a step of more than max_entries entries, a whole-node phase
-// when `stages` is off), the end, or a failure.  CTA br of nb that share the graph; `barrier` synchronises all their
-// threads and orders their memory.
-template <class Barrier>
-__device__ __forceinline__ void grow_run(const GrowArgs& a, GrowState& g, GrowSmem& sm, uint32_t br, uint32_t nb,
-                                         Barrier barrier) {
-    uint32_t epoch = 0;
-    // Counter block of the current epoch (between two closing barriers).  An epoch clears the next one's block, last
-    // read two epochs ago: every CTA has passed the barrier that closed the epoch in between.
-    const auto ctr = [&]() { return a.ring + epoch % 3; };
-    const auto close_epoch = [&]() {  // every thread gets the epoch's counters
-        if (br == 0 && threadIdx.x < sizeof(Counters) / 8)
-            reinterpret_cast<unsigned long long*>(a.ring + (epoch + 1) % 3)[threadIdx.x] = 0ull;
-        barrier();
-        if (threadIdx.x < sizeof(Counters) / 8)
-            reinterpret_cast<unsigned long long*>(&sm.seen)[threadIdx.x] =
-                __ldcg(reinterpret_cast<const unsigned long long*>(ctr()) + threadIdx.x);
-        __syncthreads();
-        ++epoch;
-    };
-    const auto rebuild = [&]() {
-        const bool pull = a.pull_ok && (a.nnz - g.frozen_deg) < g.frozen_deg;
-        dev_rebuild(a.n, a.key, a.center, a.cumulative ? a.D : nullptr, a.off, g.delta, pull, a.fbase[g.cur],
-                    a.fkey[g.cur], a.fpre[g.cur], a.cfirst[g.cur], ctr(), sm.scratch, br, nb);
-        close_epoch();
-        g.nf = (uint32_t)(sm.seen.front >> 32);
-        g.E = (uint32_t)sm.seen.front;
-    };
-    while (epoch < a.max_epochs) {
+// Control decisions up to the next work (thread 0 of every CTA, from the same values).
+__device__ __forceinline__ uint32_t grow_decide(const GrowArgs& a, GrowState& g, uint64_t* thr) {
+    for (;;) {
         if (g.phase == kPhaseStep) {
-            if (g.E > a.max_entries) break;
-            uint32_t updated = 0;
+            if (g.E > a.max_entries) return kWorkLeave;
             ++g.growth_steps;
             ++g.stepid;
-            if (g.nf > 0) {
-                dev_push<true>(a.fbase[g.cur], a.fkey[g.cur], a.fpre[g.cur], a.cfirst[g.cur], g.nf, g.E, a.adj, a.center,
-                               a.cumulative ? a.D : nullptr, a.key, g.delta, a.stamp, g.stepid, a.next, ctr(), sm.push,
-                               br, nb, a.n, (uint32_t)a.nnz);
-                barrier();
-                const uint32_t nn = min(__ldcg(&ctr()->nnext), a.n), o = g.cur ^ 1;
-                dev_snapshot(a.next, nn, a.key, a.off, g.delta, a.fbase[o], a.fkey[o], a.fpre[o], a.cfirst[o], ctr(),
-                             sm.scratch, br, nb, a.keyS, a.n);
-                close_epoch();
-                if (sm.seen.bad) {
-                    g.phase = kPhaseFailed;
-                    g.unfrozen = ~g.U;
-                    break;
-                }
-                updated = sm.seen.nnext;
-                g.covered += sm.seen.newly_covered;
-                g.edges_scanned += g.E;
-                g.nf = (uint32_t)(sm.seen.front >> 32);
-                g.E = (uint32_t)sm.seen.front;
-                g.cur = o;
-            }
+            if (g.nf > 0) return kWorkPush;
             g.steps++;
-            g.node_updates += updated;
-            if (!(updated != 0 && 2 * g.covered < g.U && (a.step_cap == 0 || g.growth_steps < a.step_cap)))
-                g.phase = kPhaseGrown;
+            g.phase = kPhaseGrown;
         } else if (!a.stages) {
-            break;
+            return kWorkLeave;
         } else if (g.phase == kPhaseStage) {
-            uint64_t thr = 0;
-            if (!stage_threshold(g.U, a.tau, a.L, &thr)) {
+            if (!stage_threshold(g.U, a.tau, a.L, thr)) {
                 g.phase = kPhaseDone;
-                break;
+                return kWorkLeave;
             }
             if (g.stage > kMaxStages) {
                 g.phase = kPhaseFailed;
-                break;
+                return kWorkLeave;
             }
-            dev_select(a.n, a.center, a.key, a.seed, g.stage, thr, ctr(), br, nb, a.keyS);
-            close_epoch();
-            g.covered = sm.seen.selected;
-            g.centers_drawn += sm.seen.selected;
-            g.unfrozen = sm.seen.unfrozen;
-            if (g.unfrozen != g.U) {
-                g.phase = kPhaseFailed;
-                break;
-            }
-            rebuild();
-            g.growth_steps = 0;
-            g.phase = kPhaseStep;
+            return kWorkDraw;
         } else if (g.phase == kPhaseGrown) {
-            if (2 * g.covered < g.U) {
-                // (connected graph: some covered or frozen node touches an uncovered one iff any exists)
-                bool growable = g.delta < kDeltaMax && (g.covered > 0 || g.U < a.n);
-                if (growable && !a.connected) {
-                    dev_growable(a.row, a.adj, a.nnz, a.key, ctr(), br, nb);
-                    close_epoch();
-                    growable = sm.seen.growable != 0;
-                }
-                if (growable) {
-                    g.delta = (g.delta > kDeltaMax / 2) ? kDeltaMax : 2 * g.delta;
-                    g.doublings++;
-                    rebuild();
-                    g.growth_steps = 0;
-                    g.phase = kPhaseStep;
-                    continue;
-                }
-                g.guard_exits++;
+            if (2 * g.covered >= g.U) return kWorkFinal;
+            // (connected graph: some covered or frozen node touches an uncovered one iff any exists)
+            if (g.delta < kDeltaMax && (g.covered > 0 || g.U < a.n)) {
+                if (!a.connected) return kWorkGuard;
+                g.delta = (g.delta > kDeltaMax / 2) ? kDeltaMax : 2 * g.delta;
+                g.doublings++;
+                return kWorkList;
             }
-            dev_finalize_d(a.n, a.key, a.center, a.cumulative ? nullptr : a.R, a.D, ctr(), br, nb);
-            barrier();
-            dev_finalize_freeze(a.n, a.key, a.center, a.R, a.D, a.off, ctr(), br, nb, a.keyS, a.cumulative);
-            close_epoch();
-            const bool overflow = sm.seen.overflow != 0;
-            g.U -= sm.seen.frozen;
-            g.frozen_deg += sm.seen.frozen_deg;
-            if (overflow) {
-                g.phase = kPhaseFailed;
-                g.unfrozen = g.U = 0;
-                break;
-            }
-            g.stages++;
-            ++g.stage;
-            g.phase = kPhaseStage;
+            g.guard_exits++;
+            return kWorkFinal;
         } else {
-            break;
+            return kWorkLeave;
         }
+    }
+}
+
+// What a finished work changes, from the epoch's counters; returns the next work.
+__device__ __forceinline__ uint32_t grow_apply(const GrowArgs& a, GrowState& g, uint32_t work, const Counters* c,
+                                               uint64_t* thr) {
+    if (work == kWorkPush) {
+        const uint32_t updated = __ldcg(&c->nnext);
+        const unsigned long long front = __ldcg(&c->front);
+        if (__ldcg(&c->bad)) {
+            g.phase = kPhaseFailed;
+            g.unfrozen = ~g.U;
+            return kWorkLeave;
+        }
+        g.covered += __ldcg(&c->newly_covered);
+        g.edges_scanned += g.E;
+        g.nf = (uint32_t)(front >> 32);
+        g.E = (uint32_t)front;
+        g.cur ^= 1;
+        g.steps++;
+        g.node_updates += updated;
+        if (!(updated != 0 && 2 * g.covered < g.U && (a.step_cap == 0 || g.growth_steps < a.step_cap)))
+            g.phase = kPhaseGrown;
+    } else if (work == kWorkDraw) {
+        g.covered = __ldcg(&c->selected);
+        g.centers_drawn += g.covered;
+        g.unfrozen = __ldcg(&c->unfrozen);
+        if (g.unfrozen != g.U) {
+            g.phase = kPhaseFailed;
+            return kWorkLeave;
+        }
+        return kWorkList;
+    } else if (work == kWorkList) {
+        const unsigned long long front = __ldcg(&c->front);
+        g.nf = (uint32_t)(front >> 32);
+        g.E = (uint32_t)front;
+        g.growth_steps = 0;
+        g.phase = kPhaseStep;
+    } else if (work == kWorkGuard) {
+        if (!__ldcg(&c->growable)) {
+            g.guard_exits++;
+            return kWorkFinal;
+        }
+        g.delta = (g.delta > kDeltaMax / 2) ? kDeltaMax : 2 * g.delta;
+        g.doublings++;
+        return kWorkList;
+    } else {
+        if (__ldcg(&c->overflow)) {
+            g.phase = kPhaseFailed;
+            g.unfrozen = g.U = 0;
+            return kWorkLeave;
+        }
+        g.U -= __ldcg(&c->frozen);
+        g.frozen_deg += __ldcg(&c->frozen_deg);
+        g.stages++;
+        ++g.stage;
+        g.phase = kPhaseStage;
+    }
+    return grow_decide(a, g, thr);
+}
+
+// The loop: works until one that this launch may not take (a step of more than max_entries entries, a whole-node phase
+// when `stages` is off), the end, or a failure; sm.g holds the control state before and after.  CTA br of nb that share
+// the graph; `barrier` synchronises all their threads and orders their memory.  The state stays in shared memory and
+// thread 0 decides (kept in every thread's registers it spilled the pushes' at 64 of them).
+template <class Barrier>
+__device__ __forceinline__ void grow_run(const GrowArgs& a, GrowSmem& sm, uint32_t br, uint32_t nb, Barrier barrier) {
+    GrowState& g = sm.g;
+    __syncthreads();  // the state is set
+    if (threadIdx.x == 0) sm.work = grow_decide(a, g, &sm.thr);
+    __syncthreads();
+    // Counter block of the current epoch (one work, up to its closing barrier).  An epoch clears the next one's block,
+    // last read two epochs ago: every CTA has passed the barrier that closed the epoch in between.
+    for (uint32_t epoch = 0; sm.work != kWorkLeave && epoch < a.max_epochs; ++epoch) {
+        const uint32_t work = sm.work;
+        Counters* ctr = a.ring + epoch % 3;
+        if (work == kWorkPush) {
+            const uint32_t c = g.cur, o = c ^ 1;
+            dev_push<true>(a.fbase[c], a.fkey[c], a.fpre[c], a.cfirst[c], g.nf, g.E, a.adj, a.center,
+                           a.cumulative ? a.D : nullptr, a.key, g.delta, a.stamp, g.stepid, a.next, ctr, sm.push, br, nb,
+                           a.n, (uint32_t)a.nnz);
+            barrier();
+            const uint32_t nn = min(__ldcg(&ctr->nnext), a.n);
+            dev_snapshot(a.next, nn, a.key, a.off, g.delta, a.fbase[o], a.fkey[o], a.fpre[o], a.cfirst[o], ctr,
+                         sm.scratch, br, nb, a.keyS, a.n);
+        } else if (work == kWorkDraw) {
+            dev_select(a.n, a.center, a.key, a.seed, g.stage, sm.thr, ctr, br, nb, a.keyS);
+        } else if (work == kWorkList) {
+            const bool pull = a.pull_ok && (a.nnz - g.frozen_deg) < g.frozen_deg;
+            dev_rebuild(a.n, a.key, a.center, a.cumulative ? a.D : nullptr, a.off, g.delta, pull, a.fbase[g.cur],
+                        a.fkey[g.cur], a.fpre[g.cur], a.cfirst[g.cur], ctr, sm.scratch, br, nb);
+        } else if (work == kWorkGuard) {
+            dev_growable(a.row, a.adj, a.nnz, a.key, ctr, br, nb);
+        } else {
+            dev_finalize_d(a.n, a.key, a.center, a.cumulative ? nullptr : a.R, a.D, ctr, br, nb);
+            barrier();
+            dev_finalize_freeze(a.n, a.key, a.center, a.R, a.D, a.off, ctr, br, nb, a.keyS, a.cumulative);
+        }
+        if (br == 0 && threadIdx.x < sizeof(Counters) / 8)
+            reinterpret_cast<unsigned long long*>(a.ring + (epoch + 1) % 3)[threadIdx.x] = 0ull;
+        barrier();
+        if (threadIdx.x == 0) sm.work = grow_apply(a, g, work, ctr, &sm.thr);
+        __syncthreads();
     }
 }
 

@@ -69,3 +69,36 @@ def test_mixture_equals_one_graph_path():
         for i in range(40):
             c = cd.cluster(a.graph(i), 0.4, i, contract_mode=mode)
             assert res[i] == cd.estimate(cd.quotient_build(c)), i
+
+
+@pytest.mark.parametrize("mode,cap", [(0, 0), (1, 2)])
+def test_groups_beside_small_jobs(mode, cap):
+    """Few large jobs among many small ones: the large ones run on groups of CTAs."""
+    import paper_1506_03265_gb300 as cd
+    a, taus = cd.arena_create(), []
+    big = [(inputs.grid(140, 1000, 1), True, 0.5), (inputs.grid(333, 1000, 2), True, 0.7),
+           (inputs.rmat(15, 8, 1000, 3), False, 0.5), (inputs.road_mesh(400, 1000, 4), False, 0.8),
+           (inputs.rmat(16, 8, 1000, 5), True, 30.0),  # k above the dense capacity: finished on the one-graph path
+           (inputs.grid(250, 1 << 24, 6), True, 0.6)]  # path sums that may overflow
+    for e, lcc, tau in big:
+        a.add(e.src, e.dst, e.w, e.n, lcc=lcc)
+        taus.append(tau)
+    for i in range(30):
+        e = inputs.grid(8 + i, 100, i)
+        a.add(e.src, e.dst, e.w, e.n)
+        taus.append(0.1)
+    ids = np.arange(len(taus))
+    res, sts = a.run(ids, taus, ids, raise_on_error=False, contract_mode=mode, step_cap=cap)
+    start, end = a.job_times(len(ids))
+    assert np.all(end >= start)
+    for i in ids:
+        try:
+            c = cd.cluster(a.graph(int(i)), taus[i], int(i), contract_mode=mode, step_cap=cap)
+            want, st = cd.estimate(cd.quotient_build(c)), 0
+        except cd.CldiamError as e:
+            want, st = None, e.status
+        assert sts[i] == st, i
+        if st == 0:
+            assert res[i] == want, i
+    again, _ = a.run(ids, taus, ids, raise_on_error=False, contract_mode=mode, step_cap=cap)
+    assert [r for r, s in zip(again, sts) if s == 0] == [r for r, s in zip(res, sts) if s == 0]
