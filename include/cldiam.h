@@ -268,13 +268,13 @@ cldiam_status cldiam_apsp_max_noalloc(uint32_t k, const uint64_t* off, const uin
 cldiam_status cldiam_sssp_source(const cldiam_graph* g, uint64_t seed, uint32_t* source);
 /*
  * Delta-stepping SSSP (Meyer and Sanders) from `source` with bucket width
- * `delta` (>= 1; 0 = average edge weight times cldiam_tuning.sssp_delta_scale):
+ * `delta` (>= 1; 0 = average edge weight times a factor, cldiam_tuning.sssp_delta_scale):
  * exact distances, so any delta gives the same result.  dist[n] (may be NULL;
  * 0xFFFFFFFF = unreachable) and *ecc = largest finite distance (host pointer);
  * 2 * ecc is the SSSP 2-approximation of Section 5.  *rounds (may be NULL) =
- * light/heavy phases run; *edges_scanned (may be NULL) = adjacency entries the
- * phases read (0 on graphs with 2^32 or more entries, which are not counted).
- * Errors: INVALID_ARG, OVERFLOW, OOM, CUDA.
+ * relaxation phases run; *edges_scanned (may be NULL) = adjacency entries the
+ * phases read.
+ * Errors: INVALID_ARG, OVERFLOW, DIVERGED (an internal list was inconsistent), OOM, CUDA.
  */
 cldiam_status cldiam_sssp_delta(cldiam_graph* g, uint32_t source, uint32_t delta, uint32_t* dist,
                                 uint64_t* ecc, uint64_t* rounds, uint64_t* edges_scanned);
@@ -380,7 +380,7 @@ typedef struct {
     uint32_t batch_fw_k;           /* many-graph form: quotients up to this k (<= 200) are closed by
                                       Floyd-Warshall in shared memory; 0 = 200                     */
     float sssp_delta_scale;        /* Delta-stepping with delta = 0: Delta = this x the average
-                                      weight (>= 1); 0 = 1                                          */
+                                      weight (> 1); 0 or 1 = by the graph's size and degree        */
     uint32_t batch_split;          /* many-graph form: 2 = the largest graphs (each with at least 2^16
                                       entries) run on groups of CTAs, or first on the one-graph path
                                       with the whole device, how many by a time model (one CTA's rate,

@@ -240,34 +240,11 @@ __global__ void __launch_bounds__(GT, 1) k_grow(const GrowArgs a, const GrowStat
     if (blockIdx.x == 0 && threadIdx.x == 0) *a.out = sm.g;
 }
 
-// CTAs of k_grow's cluster on this device: 16 where such a cluster can be resident, else the portable 8, else 0 (not
-// used).  Decided once per device; concurrent first calls store the same value.
+// CTAs of k_grow's cluster on this device; asked once per device, concurrent first calls store the same value
 int grow_cluster_size(int dev) {
     static std::atomic<int> cached[64];  // 0 = not asked yet, else size + 1
     if (dev < 0 || dev >= 64) return 0;
-    if (cached[dev].load() == 0) {
-        int size = 0;
-        if (cudaFuncSetAttribute(k_grow, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(GrowSmem)) ==
-                cudaSuccess &&
-            cudaFuncSetAttribute(k_grow, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
-            for (int c = GCTAS; c >= 8 && size == 0; c /= 2) {
-                cudaLaunchConfig_t cfg{};
-                cudaLaunchAttribute at{};
-                at.id = cudaLaunchAttributeClusterDimension;
-                at.val.clusterDim.x = (unsigned)c;
-                at.val.clusterDim.y = at.val.clusterDim.z = 1;
-                cfg.gridDim = dim3((unsigned)c);
-                cfg.blockDim = dim3(GT);
-                cfg.dynamicSmemBytes = sizeof(GrowSmem);
-                cfg.attrs = &at;
-                cfg.numAttrs = 1;
-                int m = 0;
-                if (cudaOccupancyMaxActiveClusters(&m, k_grow, &cfg) == cudaSuccess && m > 0) size = c;
-            }
-        }
-        cudaGetLastError();
-        cached[dev].store(size + 1);
-    }
+    if (cached[dev].load() == 0) cached[dev].store(1 + resident_cluster_size(k_grow, sizeof(GrowSmem)));
     return cached[dev].load() - 1;
 }
 
@@ -492,15 +469,7 @@ cldiam_status cluster(cldiam_graph* g, double tau, uint64_t seed, const cldiam_o
         CLD_CUDA(cudaMemsetAsync(ring.get(), 0, 3 * sizeof(Counters), s));
         cudaLaunchConfig_t cfg{};
         cudaLaunchAttribute at{};
-        at.id = cudaLaunchAttributeClusterDimension;
-        at.val.clusterDim.x = (unsigned)grow_ctas;
-        at.val.clusterDim.y = at.val.clusterDim.z = 1;
-        cfg.gridDim = dim3((unsigned)grow_ctas);
-        cfg.blockDim = dim3(GT);
-        cfg.dynamicSmemBytes = sizeof(GrowSmem);
-        cfg.stream = s;
-        cfg.attrs = &at;
-        cfg.numAttrs = 1;
+        resident_config(&cfg, &at, grow_ctas, sizeof(GrowSmem), s);
         const uint64_t scanned0 = gs.edges_scanned, updates0 = gs.node_updates;
         CLD_K(K_RELAX, s, CLD_CUDA(cudaLaunchKernelEx(&cfg, k_grow, a, gs)));
         GrowState* hg = static_cast<GrowState*>(g->host.h);

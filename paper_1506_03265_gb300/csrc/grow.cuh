@@ -411,4 +411,36 @@ __device__ __forceinline__ void grow_run(const GrowArgs& a, GrowSmem& sm, uint32
     }
 }
 
+// ---------------------------------------------------------------- launching a resident kernel
+// Launch configuration of one cluster of `ctas` CTAs of GT threads.
+inline void resident_config(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* at, int ctas, size_t smem, cudaStream_t s) {
+    at->id = cudaLaunchAttributeClusterDimension;
+    at->val.clusterDim.x = (unsigned)ctas;
+    at->val.clusterDim.y = at->val.clusterDim.z = 1;
+    cfg->gridDim = dim3((unsigned)ctas);
+    cfg->blockDim = dim3(GT);
+    cfg->dynamicSmemBytes = smem;
+    cfg->stream = s;
+    cfg->attrs = at;
+    cfg->numAttrs = 1;
+}
+// CTAs of a resident kernel's cluster on the current device: 16 where such a cluster can be resident, else the portable
+// 8, else 0 (not used).
+template <class Kern>
+int resident_cluster_size(Kern kern, size_t smem) {
+    int size = 0;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess &&
+        cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
+        for (int c = GCTAS; c >= 8 && size == 0; c /= 2) {
+            cudaLaunchConfig_t cfg{};
+            cudaLaunchAttribute at{};
+            resident_config(&cfg, &at, c, smem, nullptr);
+            int m = 0;
+            if (cudaOccupancyMaxActiveClusters(&m, kern, &cfg) == cudaSuccess && m > 0) size = c;
+        }
+    }
+    cudaGetLastError();
+    return size;
+}
+
 }  // namespace cld

@@ -1,26 +1,33 @@
 // Delta-stepping SSSP (Meyer and Sanders, J. Algorithms 2003), the parallel
 // SSSP the paper compares against (Sections 1 and 5): bucket i holds the
 // nodes with tentative distance in [i Delta, (i+1) Delta).  The current
-// bucket is settled by repeated rounds over its light edges (w <= Delta);
-// then the heavy edges (w > Delta) of every node settled in it are relaxed
-// once; the next non-empty bucket is then taken from the far pile.  Twice
-// the source's eccentricity is the SSSP 2-approximation of the diameter.
+// bucket is settled by repeated rounds; the next non-empty bucket is then
+// taken from the far pile.  Twice the source's eccentricity is the SSSP
+// 2-approximation of the diameter.
 //
-// Dedup: a node enters a light round's frontier at most once per round
-// (round stamp), the bucket's settled list once per bucket and the far pile
-// once per bucket epoch (epoch stamps); stale far entries are dropped when
-// the next bucket is chosen.
+// A round relaxes every edge of its nodes, light and heavy alike: with rows
+// sorted by column a light round reads the heavy edges too, so settling the
+// light ones first only adds a pass over the bucket's adjacency and its
+// rounds (R-MAT 24 read 2.2G entries in 34 rounds that way; DSCOUNT).
+//
+// Dedup: a node enters a round's frontier at most once per round (round
+// stamp) and the far pile once per bucket epoch (epoch stamp); stale far
+// entries are dropped when the next bucket is taken.
 //
 // Work distribution: each round's node list becomes a frontier with the
 // first position of every node's adjacency in one flattened range (one packed
-// atomic per CTA hands out slots and positions) and a chunk table; the relax
-// kernel gives each warp PW consecutive positions, so a hub's adjacency is
-// spread over many warps instead of one (edge-balanced, as the growing step of
-// CLUSTER).  Graphs with 2^32 or more adjacency entries keep one warp per node.
+// atomic per CTA hands out slots and positions) and a chunk table; each warp
+// takes PW consecutive positions, so a hub's adjacency is spread over many
+// warps instead of one (edge-balanced, as the growing step of CLUSTER).
+//
+// Small rounds run back to back in one launch by one thread-block cluster
+// (k_ds_resident), as CLUSTER's growing steps do (grow.cuh): a round as
+// separate launches costs 30 us however small it is, and a mesh takes a
+// thousand.
 #include <algorithm>
 #include <atomic>
 
-#include "cluster_dev.cuh"
+#include "grow.cuh"
 #include "internal.cuh"
 #include "prof.cuh"
 
@@ -28,87 +35,136 @@ namespace cld {
 
 namespace {
 
-struct SCounters {
-    uint32_t nnext;      // next light-round frontier
-    uint32_t nsettled;   // nodes settled in the current bucket
-    uint32_t nfar;       // far pile entries appended
-    uint32_t nfar2;      // far pile after compaction
-    uint32_t overflow;
-    uint32_t minbucket;  // smallest bucket index in the far pile
+// A count that either form of append can raise: 32-bit additions to `count`, or front_append_n's 64-bit ones, whose low
+// words are 0 here.
+struct DsCount {
+    uint32_t zero;
+    uint32_t count;
+    __device__ unsigned long long* packed() { return reinterpret_cast<unsigned long long*>(this); }
+};
+// Far pile of one bucket epoch: two take turns (what a new bucket leaves is rewritten into the other).
+struct __align__(8) DsPile {
+    DsCount n;
+    uint32_t min;  // smallest distance at which a node was put on it
+    uint32_t pad;
+};
+// counters of one round or split
+struct __align__(8) DsRound {
     unsigned long long front;  // listed frontier: (entries << 32) | adjacency positions
+    DsCount next;              // nodes of the next round
+    uint32_t bad;              // a list held an id out of range
+    uint32_t pad;
+};
+struct DsCounters {
+    DsRound r;  // reset before every round
+    DsPile pile[2];
+    uint32_t overflow;  // some candidate reached 2^32 - 1
+    uint32_t pad;
 };
 
-// A round's node list as a frontier: slot, first position and adjacency base of every node with
-// entries, its distance when listed, and the chunk table; light rounds also record the bucket's
-// settled nodes (once per bucket epoch).
-__global__ void k_ds_list(const uint32_t* __restrict__ list, uint32_t nl, const uint32_t* __restrict__ dist,
-                          const uint64_t* __restrict__ off, bool settle, uint32_t* __restrict__ sstamp, uint32_t epoch,
-                          uint32_t* __restrict__ settled, uint32_t* __restrict__ fbase, uint32_t* __restrict__ fdist,
-                          uint32_t* __restrict__ fpre, uint32_t* __restrict__ cfirst, SCounters* ctr) {
-    __shared__ unsigned long long scratch[33];
-    for (uint32_t base = blockIdx.x * blockDim.x; base < nl; base += gridDim.x * blockDim.x) {
-        const uint32_t i = base + threadIdx.x;
-        bool take = false, settle_now = false;
-        uint32_t u = 0, deg = 0, b0 = 0, du = 0;
-        if (i < nl) {
-            u = list[i];
-            du = __ldcg(&dist[u]);
-            const uint64_t o = off[u];
-            b0 = (uint32_t)o;
-            deg = (uint32_t)(off[u + 1] - o);
-            take = deg > 0;
-            settle_now = settle && atomicExch(&sstamp[u], epoch) != epoch;
+// The control state between rounds, kept by the host and by every CTA of k_ds_resident alike.
+struct DsState {
+    uint64_t hi;       // end of the current bucket
+    uint64_t scanned;  // adjacency entries read
+    uint32_t ncur;     // nodes of the next round, in list[cur]
+    uint32_t cur;
+    uint32_t pile;     // the far pile in use
+    uint32_t nfar, min;  // its entries and smallest distance
+    uint32_t round_id, epoch, rounds;
+    uint32_t done, bad;
+};
+
+struct DsArgs {
+    const uint64_t* off;
+    const uint2* adj;
+    uint32_t *dist, *rstamp, *fstamp;
+    uint32_t *list[2], *far[2];
+    uint32_t *fbase, *fdist, *fpre, *cfirst;
+    DsCounters* ctr;        // host-driven rounds and the kept counters
+    DsRound* ring;          // resident rounds: three blocks, zeroed
+    DsState* out;
+    uint64_t nnz;
+    uint32_t n, delta;
+    uint32_t max_list, max_far, max_epochs;  // resident rounds: largest list and pile, phases per launch
+};
+
+// A round's node list as a frontier: slot, first position and adjacency base of every node with entries, its distance
+// when listed, and the chunk table.
+__device__ __forceinline__ void ds_list(const DsArgs& a, const uint32_t* list, uint32_t nl, unsigned long long* front,
+                                        unsigned long long* scratch, uint32_t br, uint32_t nb, uint32_t* bad) {
+    const uint32_t per = nodes_per_thread(nl, nb);
+    const uint64_t stride = (uint64_t)nb * blockDim.x * per;
+    for (uint64_t base = (uint64_t)br * blockDim.x * per; base < nl; base += stride) {
+        uint32_t v[NU], deg[NU], b0[NU], d[NU], slot[NU], pre[NU], kinds = 0;
+#pragma unroll
+        for (uint32_t u = 0; u < NU; ++u) {
+            const uint64_t i = base + u * blockDim.x + threadIdx.x;
+            v[u] = u < per && i < nl ? __ldcg(&list[i]) : kNone;
+            if (u < per && i < nl && v[u] >= a.n) atomicExch(bad, 1u);
         }
-        const uint32_t s1 = warp_append(&ctr->nsettled, settle_now);
-        if (settle_now) settled[s1] = u;
-        uint32_t slot = 0, pre = 0;
-        front_append(&ctr->front, take, deg, slot, pre, scratch);
-        if (take) {
-            fbase[slot] = b0 - pre;
-            fdist[slot] = du;
-            fpre[slot] = pre;
-            chunk_table_put(cfirst, slot, pre, deg);
+#pragma unroll
+        for (uint32_t u = 0; u < NU; ++u) {
+            deg[u] = b0[u] = d[u] = 0;
+            if (v[u] < a.n) {
+                d[u] = __ldcg(&a.dist[v[u]]);
+                const uint64_t o = a.off[v[u]];
+                b0[u] = (uint32_t)o;
+                deg[u] = (uint32_t)(a.off[v[u] + 1] - o);
+            }
+            kinds |= (deg[u] ? 1u : 0u) << u;
+        }
+        front_append_n<NU>(front, kinds, deg, slot, pre, scratch);
+#pragma unroll
+        for (uint32_t u = 0; u < NU; ++u) {
+            if (!deg[u]) continue;
+            a.fbase[slot[u]] = b0[u] - pre[u];
+            a.fdist[slot[u]] = d[u];
+            a.fpre[slot[u]] = pre[u];
+            chunk_table_put(a.cfirst, slot[u], pre[u], deg[u]);
         }
     }
 }
 
-// One light round (heavy = false) or the heavy phase over a listed frontier: each warp takes PW
-// consecutive positions of the flattened adjacency; a candidate that undercuts the target's distance
-// lowers it with an atomic minimum, and an improved target goes to the next round (below hi) or to
-// the far pile, each deduplicated by its stamp.
-__global__ void __launch_bounds__(PT, 6) k_ds_push(const uint32_t* __restrict__ fbase,
-                                                   const uint32_t* __restrict__ fdist,
-                                                   const uint32_t* __restrict__ fpre,
-                                                   const uint32_t* __restrict__ cfirst,
-                                                   const uint2* __restrict__ adj, bool heavy,
-                                                   uint32_t* __restrict__ dist, uint32_t delta, uint64_t hi,
-                                                   uint32_t* __restrict__ rstamp, uint32_t round_id,
-                                                   uint32_t* __restrict__ fstamp, uint32_t epoch,
-                                                   uint32_t* __restrict__ next, uint32_t* __restrict__ far,
-                                                   SCounters* ctr) {
-    __shared__ uint32_t spre[PT / 32][PW + 1];
-    __shared__ uint32_t sbase[PT / 32][PW + 2];
-    __shared__ uint32_t sdist[PT / 32][PW + 2];
-    __shared__ uint32_t snext[PT / 32][PNB];
-    __shared__ uint32_t sfar[PT / 32][PNB];
+template <int WARPS>
+struct DsPushSmem {
+    uint32_t spre[WARPS][PW + 1];
+    uint32_t sbase[WARPS][PW + 2];
+    uint32_t sdist[WARPS][PW + 2];
+    uint32_t snext[WARPS][PNB];
+    uint32_t sfar[WARPS][PNB];
+};
+
+// One round over a listed frontier: each warp takes PW consecutive positions of the flattened adjacency; a candidate
+// that undercuts the target's distance lowers it with an atomic minimum, and an improved target goes to the next round
+// (below hi) or to the far pile, each deduplicated by its stamp.  RESIDENT: distances are read past L1 and positions
+// and ids checked, as in dev_push.
+template <bool RESIDENT, int WARPS>
+__device__ __forceinline__ void ds_push(const DsArgs& a, uint32_t nf, uint32_t E, uint64_t hi, uint32_t round_id,
+                                        uint32_t epoch, uint32_t* next, uint32_t* nnext, uint32_t* far, DsPile* pile,
+                                        DsPushSmem<WARPS>& sm, uint32_t br, uint32_t nb, uint32_t* overflow,
+                                        uint32_t* badp) {
     const uint32_t lane = lane_id(), warp = threadIdx.x >> 5;
     const uint64_t pol_stream = l2_evict_first_policy(), pol_keep = l2_evict_last_policy();
     const unsigned le_mask = 0xffffffffu >> (31u - lane);
-    const unsigned long long fr = __ldcg(&ctr->front);
-    const uint32_t nf = (uint32_t)(fr >> 32), E = (uint32_t)fr;
-    WarpNext wn{snext[warp], 0}, wf{sfar[warp], 0};
-    bool ovf = false;
+    WarpNext wn{sm.snext[warp], 0}, wf{sm.sfar[warp], 0};
+    bool ovf = false, bad = false;
+    uint32_t fmin = kNone;
     const uint32_t nq = (uint32_t)(((uint64_t)E + PW - 1) / PW);
-    const uint32_t nwarps = gridDim.x * (PT / 32);
-    for (uint32_t q = blockIdx.x * (PT / 32) + warp; q < nq; q += nwarps) {
+    const uint32_t nwarps = nb * WARPS;
+    for (uint32_t q = br * WARPS + warp; q < nq; q += nwarps) {
         const uint32_t p0 = q * PW, e1 = min(E, p0 + PW);
-        const uint32_t i0 = __ldcg(&cfirst[q]);
-        const uint32_t il = q + 1 < nq ? __ldcg(&cfirst[q + 1]) : nf - 1;
+        const uint32_t i0 = __ldcg(&a.cfirst[q]);
+        const uint32_t il = q + 1 < nq ? __ldcg(&a.cfirst[q + 1]) : nf - 1;
+        if (RESIDENT && (i0 > il || il >= nf)) {
+            bad = true;
+            continue;
+        }
         const uint32_t ne = min(il - i0 + 1, (uint32_t)PW + 1);
+        __syncwarp();  // the previous chunk's entries have been read
         for (uint32_t j = lane; j < ne; j += 32) {
-            if (j) spre[warp][j - 1] = __ldcg(&fpre[i0 + j]);
-            sbase[warp][j] = __ldcg(&fbase[i0 + j]);
-            sdist[warp][j] = __ldcg(&fdist[i0 + j]);
+            if (j) sm.spre[warp][j - 1] = __ldcg(&a.fpre[i0 + j]);
+            sm.sbase[warp][j] = __ldcg(&a.fbase[i0 + j]);
+            sm.sdist[warp][j] = __ldcg(&a.fdist[i0 + j]);
         }
         __syncwarp();
         uint32_t own[PWG];
@@ -116,134 +172,244 @@ __global__ void __launch_bounds__(PT, 6) k_ds_push(const uint32_t* __restrict__ 
             uint32_t B = 0;
 #pragma unroll
             for (int u = 0; u < PWG; ++u) {
-                const uint32_t word = group_starts(spre[warp] + B, ne - 1 - B, p0 + 32u * u, B, lane, le_mask, &own[u]);
+                const uint32_t word =
+                    group_starts(sm.spre[warp] + B, ne - 1 - B, p0 + 32u * u, B, lane, le_mask, &own[u]);
                 B += (uint32_t)__popc(word);
             }
         }
         uint2 ed[PWG];
+        uint32_t live = 0;
 #pragma unroll
         for (int u = 0; u < PWG; ++u) {
             const uint32_t p = p0 + 32u * u + lane;
-            ed[u] = p < e1 ? ld_stream_u2(adj + (sbase[warp][own[u]] + p), pol_stream) : make_uint2(0u, 0u);
+            bool in = p < e1;
+            if (RESIDENT && in && (own[u] >= ne || sm.sbase[warp][own[u]] + p >= (uint32_t)a.nnz)) {
+                bad = true;
+                in = false;
+            }
+            live |= (in ? 1u : 0u) << u;
+            ed[u] = in ? ld_stream_u2(a.adj + (sm.sbase[warp][own[u]] + p), pol_stream) : make_uint2(0u, 0u);
         }
         uint64_t nd[PWG];
         uint32_t cur[PWG];
 #pragma unroll
         for (int u = 0; u < PWG; ++u) {
-            const bool live = p0 + 32u * u + lane < e1 && ((ed[u].y <= delta) != heavy);
-            nd[u] = live ? (uint64_t)sdist[warp][own[u]] + ed[u].y : ~0ull;
-            cur[u] = nd[u] != ~0ull ? ld_keep_u32(&dist[ed[u].x], pol_keep) : 0u;  // filter through L1
+            nd[u] = (live >> u) & 1u ? (uint64_t)sm.sdist[warp][own[u]] + ed[u].y : ~0ull;
+            cur[u] = 0;
+            if ((live >> u) & 1u) {  // (a one-round launch filters through L1)
+                if constexpr (RESIDENT) cur[u] = ld_cg_keep_u32(&a.dist[ed[u].x], pol_keep);
+                else cur[u] = ld_keep_u32(&a.dist[ed[u].x], pol_keep);
+            }
+        }
+        uint32_t old[PWG];
+#pragma unroll
+        for (int u = 0; u < PWG; ++u) {
+            old[u] = 0;
+            if (nd[u] >= 0xFFFFFFFFull) {
+                ovf |= nd[u] != ~0ull;
+                nd[u] = ~0ull;
+            } else if (nd[u] < cur[u]) {
+                old[u] = atomicMin(&a.dist[ed[u].x], (uint32_t)nd[u]);
+            }
+        }
+        uint32_t st[PWG];
+#pragma unroll
+        for (int u = 0; u < PWG; ++u) {
+            // an improved target: was it listed (next round or far pile) before?
+            const bool better = nd[u] < old[u];
+            const bool near = nd[u] < hi;
+            st[u] = 0;
+            if (better) st[u] = near ? atomicExch(&a.rstamp[ed[u].x], round_id) != round_id
+                                     : atomicExch(&a.fstamp[ed[u].x], epoch) != epoch;
+            if (better && !near) fmin = min(fmin, (uint32_t)nd[u]);
         }
 #pragma unroll
         for (int u = 0; u < PWG; ++u) {
-            bool to_next = false, to_far = false;
-            if (nd[u] != ~0ull && nd[u] >= 0xFFFFFFFFull) {
-                ovf = true;
-            } else if (nd[u] < cur[u]) {
-                const uint32_t v = ed[u].x;
-                if ((uint32_t)nd[u] < atomicMin(&dist[v], (uint32_t)nd[u])) {
-                    if (nd[u] < hi) to_next = atomicExch(&rstamp[v], round_id) != round_id;
-                    else to_far = atomicExch(&fstamp[v], epoch) != epoch;
-                }
-            }
-            wn.put(to_next, ed[u].x, lane);
-            wf.put(to_far, ed[u].x, lane);
+            wn.put(st[u] && nd[u] < hi, ed[u].x, lane);
+            wf.put(st[u] && nd[u] >= hi, ed[u].x, lane);
         }
-        if (wn.cnt >= (uint32_t)PW) wn.flush(next, &ctr->nnext, lane);
-        if (wf.cnt >= (uint32_t)PW) wf.flush(far, &ctr->nfar, lane);
+        if (wn.cnt >= (uint32_t)PW) wn.flush(next, nnext, lane);
+        if (wf.cnt >= (uint32_t)PW) wf.flush(far, &pile->n.count, lane);
     }
-    if (wn.cnt) wn.flush(next, &ctr->nnext, lane);
-    if (wf.cnt) wf.flush(far, &ctr->nfar, lane);
-    if (__any_sync(0xffffffffu, ovf) && lane == 0) atomicExch(&ctr->overflow, 1u);
+    if (wn.cnt) wn.flush(next, nnext, lane);
+    if (wf.cnt) wf.flush(far, &pile->n.count, lane);
+    fmin = __reduce_min_sync(0xffffffffu, fmin);
+    if (lane == 0 && fmin != kNone) atomicMin(&pile->min, fmin);
+    if (__any_sync(0xffffffffu, ovf) && lane == 0) atomicExch(overflow, 1u);
+    if (RESIDENT && __any_sync(0xffffffffu, bad) && lane == 0) atomicExch(badp, 1u);
 }
 
-// one light round (heavy = false) over `list`, or the heavy phase (heavy = true); one warp per node
-__global__ void __launch_bounds__(256) k_ds_relax(const uint32_t* __restrict__ list, uint32_t nl, bool heavy,
-                                                  const uint64_t* __restrict__ off, const uint2* __restrict__ adj,
-                                                  uint32_t* __restrict__ dist, uint32_t delta, uint64_t hi,
-                                                  uint32_t* __restrict__ rstamp, uint32_t round_id,
-                                                  uint32_t* __restrict__ sstamp, uint32_t* __restrict__ fstamp,
-                                                  uint32_t epoch, uint32_t* __restrict__ next,
-                                                  uint32_t* __restrict__ settled, uint32_t* __restrict__ far,
-                                                  SCounters* ctr) {
+// Split the far pile (nfar entries): those below hi become the next round's list, later ones move to the other pile
+// (re-stamped); entries that were improved below lo meanwhile are dropped.  *taken and pile2->count are counters of
+// front_append_n: the number of entries in their high words.
+__device__ __forceinline__ void ds_split(const DsArgs& a, const uint32_t* far, uint32_t nfar, uint64_t lo, uint64_t hi,
+                                         uint32_t epoch, uint32_t* next, unsigned long long* taken, uint32_t* far2,
+                                         DsPile* pile2, unsigned long long* scratch, uint32_t br, uint32_t nb,
+                                         uint32_t* bad) {
+    unsigned long long* kept = pile2->n.packed();
+    const uint32_t per = nodes_per_thread(nfar, nb);
+    const uint64_t stride = (uint64_t)nb * blockDim.x * per;
+    uint32_t kmin = kNone;
+    for (uint64_t base = (uint64_t)br * blockDim.x * per; base < nfar; base += stride) {
+        uint32_t v[NU], d[NU];
+#pragma unroll
+        for (uint32_t u = 0; u < NU; ++u) {
+            const uint64_t i = base + u * blockDim.x + threadIdx.x;
+            v[u] = u < per && i < nfar ? __ldcg(&far[i]) : kNone;
+            if (u < per && i < nfar && v[u] >= a.n) atomicExch(bad, 1u);
+        }
+#pragma unroll
+        for (uint32_t u = 0; u < NU; ++u) d[u] = v[u] < a.n ? __ldcg(&a.dist[v[u]]) : 0u;
+        uint32_t takes = 0, keeps = 0, slot[NU], one[NU], pre[NU];
+#pragma unroll
+        for (uint32_t u = 0; u < NU; ++u) {
+            one[u] = 0;
+            if (v[u] >= a.n) continue;
+            if ((uint64_t)d[u] >= hi) {
+                keeps |= (atomicExch(&a.fstamp[v[u]], epoch) != epoch ? 1u : 0u) << u;
+                kmin = min(kmin, d[u]);
+            } else {
+                takes |= ((uint64_t)d[u] >= lo ? 1u : 0u) << u;
+            }
+        }
+        // one append per block and list (with one per warp the 6.5M entries of R-MAT 24's first split queued at the two
+        // counters for 636 us; 68 us so)
+        front_append_n<NU>(taken, takes, one, slot, pre, scratch);
+#pragma unroll
+        for (uint32_t u = 0; u < NU; ++u)
+            if ((takes >> u) & 1u) next[slot[u]] = v[u];
+        front_append_n<NU>(kept, keeps, one, slot, pre, scratch);
+#pragma unroll
+        for (uint32_t u = 0; u < NU; ++u)
+            if ((keeps >> u) & 1u) far2[slot[u]] = v[u];
+    }
+    kmin = __reduce_min_sync(0xffffffffu, kmin);
+    if (lane_id() == 0 && kmin != kNone) atomicMin(&pile2->min, kmin);
+}
+
+__global__ void __launch_bounds__(256) k_ds_list(const DsArgs a, uint32_t cur, uint32_t nl) {
+    __shared__ unsigned long long scratch[33];
+    ds_list(a, a.list[cur], nl, &a.ctr->r.front, scratch, blockIdx.x, gridDim.x, &a.ctr->r.bad);
+}
+__global__ void __launch_bounds__(PT, 6) k_ds_push(const DsArgs a, uint32_t cur, uint32_t pile, uint64_t hi,
+                                                   uint32_t round_id, uint32_t epoch) {
+    __shared__ DsPushSmem<PT / 32> sm;
+    const unsigned long long fr = __ldcg(&a.ctr->r.front);
+    ds_push<false>(a, (uint32_t)(fr >> 32), (uint32_t)fr, hi, round_id, epoch, a.list[cur ^ 1], &a.ctr->r.next.count,
+                   a.far[pile], &a.ctr->pile[pile], sm, blockIdx.x, gridDim.x, &a.ctr->overflow, &a.ctr->r.bad);
+}
+__global__ void __launch_bounds__(256) k_ds_split(const DsArgs a, uint32_t cur, uint32_t pile, uint32_t nfar, uint64_t lo,
+                                                  uint64_t hi, uint32_t epoch) {
+    __shared__ unsigned long long scratch[33];
+    if (blockIdx.x == 0 && threadIdx.x == 0) a.ctr->pile[pile] = DsPile{{0u, 0u}, kNone, 0u};  // (its values are known)
+    ds_split(a, a.far[pile], nfar, lo, hi, epoch, a.list[cur], a.ctr->r.next.packed(), a.far[pile ^ 1],
+             &a.ctr->pile[pile ^ 1], scratch, blockIdx.x, gridDim.x, &a.ctr->r.bad);
+}
+
+// What follows a finished round or split (host, or thread 0 of every CTA): false when the SSSP is done.
+__host__ __device__ inline bool ds_next_bucket(DsState& g, uint32_t delta, uint64_t* lo) {
+    if (g.nfar == 0) {
+        g.done = 1;
+        return false;
+    }
+    *lo = (uint64_t)g.min / delta * delta;
+    if (*lo < g.hi) *lo = g.hi;  // (the pile's minimum may be a node that has moved below since)
+    g.hi = (uint64_t)g.min / delta * delta + delta;
+    if (g.hi <= *lo) g.hi = *lo + delta;
+    ++g.epoch;
+    return true;
+}
+
+struct DsSmem {
+    DsPushSmem<GT / 32> push;
+    unsigned long long scratch[33];
+    DsState g;
+    uint64_t lo;
+    uint32_t work;
+};
+enum DsWork : uint32_t { kDsRound, kDsSplit, kDsLeave };
+
+__device__ __forceinline__ uint32_t ds_decide(const DsArgs& a, DsState& g, uint64_t* lo) {
+    if (g.ncur > 0) {
+        if (g.ncur > a.max_list) return kDsLeave;
+        ++g.round_id;
+        return kDsRound;
+    }
+    if (g.nfar > a.max_far) return kDsLeave;
+    return ds_next_bucket(g, a.delta, lo) ? kDsSplit : kDsLeave;
+}
+
+// Rounds and splits back to back by one thread-block cluster, until one that is too large for it, or the end.
+__global__ void __launch_bounds__(GT, 1) k_ds_resident(const DsArgs a, const DsState start) {
+    extern __shared__ __align__(16) unsigned char ds_smem[];
+    DsSmem& sm = *reinterpret_cast<DsSmem*>(ds_smem);
+    DsState& g = sm.g;
+    const uint32_t br = blockIdx.x, nb = gridDim.x;
+    if (threadIdx.x == 0) {
+        g = start;
+        sm.work = ds_decide(a, g, &sm.lo);
+    }
+    __syncthreads();
+    // Counters of the epoch; an epoch clears the next one's, last read two epochs ago.
+    for (uint32_t epoch = 0; sm.work != kDsLeave && epoch < a.max_epochs; ++epoch) {
+        DsRound* r = a.ring + epoch % 3;
+        const uint32_t work = sm.work, p = g.pile;
+        unsigned long long fr = 0;
+        if (work == kDsRound) {
+            ds_list(a, a.list[g.cur], g.ncur, &r->front, sm.scratch, br, nb, &r->bad);
+            cluster_barrier();
+            fr = __ldcg(&r->front);
+            ds_push<true>(a, (uint32_t)(fr >> 32), (uint32_t)fr, g.hi, g.round_id, g.epoch, a.list[g.cur ^ 1],
+                          &r->next.count, a.far[p], &a.ctr->pile[p], sm.push, br, nb, &a.ctr->overflow, &r->bad);
+        } else {
+            cluster_barrier();  // every CTA has read the old pile's counters
+            if (br == 0 && threadIdx.x == 0) a.ctr->pile[p] = DsPile{{0u, 0u}, kNone, 0u};
+            ds_split(a, a.far[p], g.nfar, sm.lo, g.hi, g.epoch, a.list[g.cur], r->next.packed(), a.far[p ^ 1],
+                     &a.ctr->pile[p ^ 1], sm.scratch, br, nb, &r->bad);
+        }
+        if (br == 0 && threadIdx.x < sizeof(DsRound) / 8)
+            reinterpret_cast<unsigned long long*>(a.ring + (epoch + 1) % 3)[threadIdx.x] = 0ull;
+        cluster_barrier();
+        if (threadIdx.x == 0) {
+            if (work == kDsRound) {
+                g.cur ^= 1;
+                ++g.rounds;
+                g.scanned += (uint32_t)fr;
+            } else {
+                g.pile ^= 1;
+            }
+            g.ncur = __ldcg(&r->next.count);
+            g.bad = __ldcg(&r->bad);
+            // (while a round follows, other CTAs may already be adding to the pile: its counters decide only when none
+            // does, and then nobody writes them before the next barrier)
+            g.nfar = __ldcg(&a.ctr->pile[g.pile].n.count);
+            g.min = __ldcg(&a.ctr->pile[g.pile].min);
+            sm.work = g.bad ? (uint32_t)kDsLeave : ds_decide(a, g, &sm.lo);
+        }
+        __syncthreads();
+    }
+    if (br == 0 && threadIdx.x == 0) *a.out = g;
+}
+
+// some edge (u, v) of a reached node has dist[u] + w >= 2^32 - 1: a distance does not fit
+__global__ void k_ds_overflow(const uint64_t* __restrict__ off, const uint2* __restrict__ adj, uint32_t n,
+                              const uint32_t* __restrict__ dist, uint32_t* __restrict__ overflow) {
     const uint32_t warps = (gridDim.x * blockDim.x) >> 5;
-    const uint32_t lane = lane_id();
-    for (uint32_t i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < nl; i += warps) {
-        const uint32_t u = list[i];
-        if (!heavy && lane == 0 && atomicExch(&sstamp[u], epoch) != epoch) settled[atomicAdd(&ctr->nsettled, 1u)] = u;
-        const uint64_t du = dist[u];
-        const uint64_t beg = off[u], end = off[u + 1];
-        for (uint64_t b = beg; b < end; b += 32) {
-            const uint64_t j = b + lane;
-            bool to_next = false, to_far = false;
-            uint32_t v = 0;
-            if (j < end) {
-                const uint2 e = adj[j];
-                v = e.x;
-                const bool light = e.y <= delta;
-                if (light != heavy) {
-                    const uint64_t nd = du + e.y;
-                    if (nd >= 0xFFFFFFFFull) {
-                        atomicExch(&ctr->overflow, 1u);
-                    } else if ((uint32_t)nd < dist[v]) {
-                        const uint32_t old = atomicMin(&dist[v], (uint32_t)nd);
-                        if ((uint32_t)nd < old) {
-                            if (nd < hi) to_next = atomicExch(&rstamp[v], round_id) != round_id;
-                            else to_far = atomicExch(&fstamp[v], epoch) != epoch;
-                        }
-                    }
-                }
-            }
-            uint32_t s1 = warp_append(&ctr->nnext, to_next);
-            if (to_next) next[s1] = v;
-            uint32_t s2 = warp_append(&ctr->nfar, to_far);
-            if (to_far) far[s2] = v;
-        }
+    bool ovf = false;
+    for (uint32_t v = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; v < n; v += warps) {
+        const uint32_t d = dist[v];
+        if (d == kNone) continue;
+        for (uint64_t j = off[v] + lane_id(); j < off[v + 1]; j += 32) ovf |= (uint64_t)d + adj[j].y >= 0xFFFFFFFFull;
     }
+    if (ovf) atomicExch(overflow, 2u);
 }
 
-// smallest bucket among far entries still beyond the settled range
-__global__ void k_ds_minbucket(const uint32_t* __restrict__ far, uint32_t nfar, const uint32_t* __restrict__ dist,
-                               uint64_t hi, uint32_t delta, SCounters* ctr) {
-    uint32_t m = 0xFFFFFFFFu;
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < nfar; i += gridDim.x * blockDim.x) {
-        uint32_t d = dist[far[i]];
-        if ((uint64_t)d >= hi) m = min(m, d / delta);
-    }
-    m = block_reduce(m, [](uint32_t a, uint32_t b) { return a < b ? a : b; }, 0xFFFFFFFFu);
-    if (threadIdx.x == 0) atomicMin(&ctr->minbucket, m);
-}
-
-// split the far pile: entries of the new bucket become the frontier, later ones stay (re-stamped)
-__global__ void k_ds_split(const uint32_t* __restrict__ far, uint32_t nfar, const uint32_t* __restrict__ dist,
-                           uint64_t old_hi, uint64_t new_hi, uint32_t* __restrict__ fstamp, uint32_t new_epoch,
-                           uint32_t* __restrict__ cur, uint32_t* __restrict__ far2, SCounters* ctr) {
-    for (uint32_t base = blockIdx.x * blockDim.x; base < nfar; base += gridDim.x * blockDim.x) {
-        uint32_t i = base + threadIdx.x;
-        bool to_cur = false, keep = false;
-        uint32_t v = 0;
-        if (i < nfar) {
-            v = far[i];
-            uint64_t d = dist[v];
-            if (d >= old_hi) {
-                if (d < new_hi) to_cur = true;
-                else keep = atomicExch(&fstamp[v], new_epoch) != new_epoch;
-            }
-        }
-        uint32_t s1 = warp_append(&ctr->nnext, to_cur);
-        if (to_cur) cur[s1] = v;
-        uint32_t s2 = warp_append(&ctr->nfar2, keep);
-        if (keep) far2[s2] = v;
-    }
-}
-
-__global__ void k_ds_init(uint32_t* __restrict__ dist, uint32_t* __restrict__ a, uint32_t* __restrict__ b,
-                          uint32_t* __restrict__ c, uint32_t n, uint32_t source) {
+__global__ void k_ds_init(uint32_t* __restrict__ dist, uint32_t* __restrict__ a, uint32_t* __restrict__ b, uint32_t n,
+                          uint32_t source) {
     for (uint32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
         dist[v] = v == source ? 0u : 0xFFFFFFFFu;
         a[v] = 0;
         b[v] = 0;
-        c[v] = 0;
     }
 }
 
@@ -255,156 +421,174 @@ __global__ void k_ds_ecc(const uint32_t* __restrict__ dist, uint32_t n, uint32_t
     if (threadIdx.x == 0) atomicMax(out, m);
 }
 
+// CTAs of the resident form's cluster: 16, else 8, else 0 (not used); asked once per device, concurrent first calls
+// store the same value
+int ds_cluster_size(int dev) {
+    static std::atomic<int> cached[64];  // 0 = not asked yet, else size + 1
+    if (dev < 0 || dev >= 64) return 0;
+    if (cached[dev].load() == 0) cached[dev].store(1 + resident_cluster_size(k_ds_resident, sizeof(DsSmem)));
+    return cached[dev].load() - 1;
+}
+
 }  // namespace
 
 cldiam_status sssp_delta(cldiam_graph* g, uint32_t source, uint32_t delta, uint32_t* dist_out, uint64_t* ecc,
                          uint64_t* rounds_out, uint64_t* scanned_out) {
     if (!g || !ecc) return fail(CLDIAM_ERR_INVALID_ARG, "NULL graph or ecc");
     if (source >= g->n) return fail(CLDIAM_ERR_INVALID_ARG, "source >= n");
+    if (g->nnz >= 0xFFFFFFFFull) return fail(CLDIAM_ERR_UNSUPPORTED, "2^32 - 1 or more adjacency entries");
     const uint32_t n = g->n;
     const cudaStream_t s = g->stream;
     if (delta == 0) {
         uint32_t d0 = 1;
         CLD_TRY(cld::delta0(g, CLDIAM_DELTA0_AVG, 0, &d0));
-        const double scaled = (double)d0 * (double)tuning_for(g->nnz).sssp_delta_scale;
+        // Width of a bucket.  A round costs 10 to 30 us, an adjacency entry read 8 ps with the whole device: sparse graphs
+        // (rounds by the hundred) and small ones want wide buckets, large dense ones few repeated reads.  ms at 16 / 8 /
+        // 1 / 0.35 times the average weight: 400^2 mesh 9.0 / 9.7 / 18.1 / 30.4; road mesh 2,000^2 4.4 / 4.7 / 8.8 / 14.2;
+        // R-MAT of 31M entries 1.29 / 1.30 / 1.46 / 1.63, of 128M 6.11 / 6.13 / 6.19 / 7.06, of 166M 4.61 / 4.61 / 4.10 /
+        // 4.18 (0.25: 4.03), of 521M 14.1 / 14.1 / 14.8 / 10.1 (0.25: 10.8).
+        double scale = (double)tuning_for(g->nnz).sssp_delta_scale;
+        if (scale == 1.0) scale = g->nnz < 8ull * n ? 16.0 : g->nnz < (1ull << 27) ? 8.0 : 0.3;
+        const double scaled = (double)d0 * scale;
         delta = (uint32_t)std::min(std::max(scaled, 1.0), 2147483648.0);
     }
-    // edge-balanced rounds index positions with 32 bits
-    const bool chunked = g->nnz < 0xFFFFFFFFull;
-    DBuf<uint32_t> dist, rstamp, sstamp, fstamp, cur, next, settled, far, far2, ecc_d;
-    DBuf<uint32_t> fbase, fdist, fpre, cfirst;
-    DBuf<SCounters> ctr;
+    DBuf<uint32_t> dist, rstamp, fstamp, listA, listB, farA, farB, ecc_d, fbase, fdist, fpre, cfirst;
+    DBuf<DsCounters> ctr;
+    DBuf<DsRound> ring;
+    DBuf<DsState> gdev;
     CLD_TRY(dist.alloc(n, s));
     CLD_TRY(rstamp.alloc(n, s));
-    CLD_TRY(sstamp.alloc(n, s));
     CLD_TRY(fstamp.alloc(n, s));
-    CLD_TRY(cur.alloc(n, s));
-    CLD_TRY(next.alloc(n, s));
-    CLD_TRY(settled.alloc(n, s));
-    CLD_TRY(far.alloc(n, s));
-    CLD_TRY(far2.alloc(n, s));
+    CLD_TRY(listA.alloc(n, s));
+    CLD_TRY(listB.alloc(n, s));
+    CLD_TRY(farA.alloc(n, s));
+    CLD_TRY(farB.alloc(n, s));
     CLD_TRY(ecc_d.alloc(1, s));
     CLD_TRY(ctr.alloc(1, s));
-    if (chunked) {
-        CLD_TRY(fbase.alloc(n, s));
-        CLD_TRY(fdist.alloc(n, s));
-        CLD_TRY(fpre.alloc(n, s));
-        CLD_TRY(cfirst.alloc(g->nnz / PW + 2, s));
-    }
-    SCounters* hc = reinterpret_cast<SCounters*>(static_cast<char*>(g->host.h) + 192);
-    static_assert(sizeof(SCounters) <= 64, "counter block must fit the pinned area");
+    CLD_TRY(fbase.alloc(n, s));
+    CLD_TRY(fdist.alloc(n, s));
+    CLD_TRY(fpre.alloc(n, s));
+    CLD_TRY(cfirst.alloc(g->nnz / PW + 2, s));
+    CLD_TRY(ring.alloc(3, s));
+    CLD_TRY(gdev.alloc(1, s));
+    DsCounters* hc = reinterpret_cast<DsCounters*>(static_cast<char*>(g->host.h) + 96);
+    DsState* hg = reinterpret_cast<DsState*>(static_cast<char*>(g->host.h) + 176);
+    uint32_t* he = reinterpret_cast<uint32_t*>(static_cast<char*>(g->host.h) + 240);
+    static_assert(sizeof(DsCounters) <= 80 && sizeof(DsState) <= 64, "read-back blocks must fit the pinned area");
+    DsArgs a{};
+    a.off = g->off;
+    a.adj = g->adj;
+    a.dist = dist.get();
+    a.rstamp = rstamp.get();
+    a.fstamp = fstamp.get();
+    a.list[0] = listA.get();
+    a.list[1] = listB.get();
+    a.far[0] = farA.get();
+    a.far[1] = farB.get();
+    a.fbase = fbase.get();
+    a.fdist = fdist.get();
+    a.fpre = fpre.get();
+    a.cfirst = cfirst.get();
+    a.ctr = ctr.get();
+    a.ring = ring.get();
+    a.out = gdev.get();
+    a.nnz = g->nnz;
+    a.n = n;
+    a.delta = delta;
+    // resident rounds: lists of about 2^18 adjacency entries, piles of 2^18 nodes (as CLUSTER's resident steps)
+    a.max_list = (uint32_t)std::max<uint64_t>(1, (uint64_t)kGrowEntries / (g->nnz / n + 1));
+    a.max_far = kGrowEntries;
+    a.max_epochs = kGrowEpochs;
     const unsigned gb = grid_for(n, 256);
-    CLD_K(K_SSSP, s, k_ds_init<<<gb, 256, 0, s>>>(dist.get(), rstamp.get(), sstamp.get(), fstamp.get(), n, source));
+    CLD_K(K_SSSP, s, k_ds_init<<<gb, 256, 0, s>>>(dist.get(), rstamp.get(), fstamp.get(), n, source));
     CLD_LAUNCH_CHECK();
-    CLD_CUDA(cudaMemcpyAsync(cur.get(), &source, 4, cudaMemcpyHostToDevice, s));
-    CLD_CUDA(cudaMemsetAsync(ctr.get(), 0, sizeof(SCounters), s));
+    hc[0] = DsCounters{};
+    hc->pile[0].min = hc->pile[1].min = kNone;
+    CLD_CUDA(cudaMemcpyAsync(ctr.get(), hc, sizeof(DsCounters), cudaMemcpyHostToDevice, s));
+    he[0] = source;
+    CLD_CUDA(cudaMemcpyAsync(listA.get(), he, 4, cudaMemcpyHostToDevice, s));
 
-    auto sync = [&]() -> cldiam_status {
-        CLD_CUDA(cudaMemcpyAsync(hc, ctr.get(), sizeof(SCounters), cudaMemcpyDeviceToHost, s));
+    DsState st{};
+    st.hi = delta;
+    st.ncur = 1;
+    st.min = kNone;
+    st.epoch = 1;
+    const auto bad_list = [] { return fail(CLDIAM_ERR_DIVERGED, "inconsistent list in a shortest-path round"); };
+    const auto read = [&]() -> cldiam_status {
+        CLD_CUDA(cudaMemcpyAsync(hc, ctr.get(), sizeof(DsCounters), cudaMemcpyDeviceToHost, s));
         CLD_CUDA(cudaStreamSynchronize(s));
-        if (hc->overflow) return fail(CLDIAM_ERR_OVERFLOW, "a distance reached 2^32 - 1");
+        if (hc->r.bad) return bad_list();
+        st.ncur = hc->r.next.count;
+        st.nfar = hc->pile[st.pile].n.count;
+        st.min = hc->pile[st.pile].min;
         return CLDIAM_OK;
     };
     static std::atomic<int> push_per_sm[64];  // concurrent first calls store the same value
     int dev = 0;
     CLD_CUDA(cudaGetDevice(&dev));
     const int di = (dev >= 0 && dev < 64) ? dev : 0;
-    if (chunked && push_per_sm[di].load() == 0) {
-        int a = 0;
-        CLD_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_ds_push, PT, 0));
-        push_per_sm[di] = std::max(1, a);
+    if (push_per_sm[di].load() == 0) {
+        int b = 0;
+        CLD_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_ds_push, PT, 0));
+        push_per_sm[di] = std::max(1, b);
     }
     const unsigned push_grid = (unsigned)num_sms() * (unsigned)std::max(1, push_per_sm[di].load());
-    const unsigned relax_grid = (unsigned)num_sms() * 8;
-    uint32_t ncur = 1, round_id = 0, epoch = 1, nfar = 0;
-    uint64_t lo = 0, hi = delta, rounds = 0, scanned = 0;
-    uint32_t* pcur = cur.get();
-    uint32_t* pnext = next.get();
-    uint32_t* pfar = far.get();
-    uint32_t* pfar2 = far2.get();
-    // one light round or the heavy phase over `list`
-    auto relax = [&](const uint32_t* list, uint32_t nl, bool heavy) -> cldiam_status {
-        if (chunked) {
-            CLD_CUDA(cudaMemsetAsync(&ctr.get()->front, 0, 8, s));
-            CLD_K(K_SSSP, s, k_ds_list<<<grid_for(nl, 256), 256, 0, s>>>(list, nl, dist.get(), g->off, !heavy,
-                                                                         sstamp.get(), epoch, settled.get(),
-                                                                         fbase.get(), fdist.get(), fpre.get(),
-                                                                         cfirst.get(), ctr.get()));
+    const int ctas = ds_cluster_size(dev);
+    while (!st.done && (st.ncur > 0 || st.nfar > 0)) {
+        const bool small = st.ncur > 0 ? st.ncur <= a.max_list : st.nfar <= a.max_far;
+        if (small && ctas && !serving_kernel_alive(dev)) {
+            CLD_CUDA(cudaMemsetAsync(ring.get(), 0, 3 * sizeof(DsRound), s));
+            cudaLaunchConfig_t cfg{};
+            cudaLaunchAttribute at{};
+            resident_config(&cfg, &at, ctas, sizeof(DsSmem), s);
+            const uint64_t scanned0 = st.scanned;
+            CLD_K(K_SSSP, s, CLD_CUDA(cudaLaunchKernelEx(&cfg, k_ds_resident, a, st)));
+            CLD_CUDA(cudaMemcpyAsync(hg, gdev.get(), sizeof(DsState), cudaMemcpyDeviceToHost, s));
+            CLD_TRY(read());
+            st = *hg;
+            if (st.bad) return bad_list();
+            prof_add_bytes(K_SSSP, 18.0 * (double)(st.scanned - scanned0));
+        } else if (st.ncur > 0) {
+            ++st.round_id;
+            CLD_CUDA(cudaMemsetAsync(ctr.get(), 0, sizeof(DsRound), s));
+            CLD_K(K_SSSP, s, k_ds_list<<<grid_for(((size_t)st.ncur + NU - 1) / NU, 256), 256, 0, s>>>(a, st.cur, st.ncur));
+            CLD_K(K_SSSP, s, k_ds_push<<<push_grid, PT, 0, s>>>(a, st.cur, st.pile, st.hi, st.round_id, st.epoch));
             CLD_LAUNCH_CHECK();
-            CLD_K(K_SSSP, s, k_ds_push<<<push_grid, PT, 0, s>>>(fbase.get(), fdist.get(), fpre.get(), cfirst.get(),
-                                                                g->adj, heavy, dist.get(), delta, hi, rstamp.get(),
-                                                                round_id, fstamp.get(), epoch, pnext, pfar,
-                                                                ctr.get()));
-        } else {
-            const unsigned rg = (unsigned)std::min<uint64_t>((nl + 7) / 8, relax_grid);
-            CLD_K(K_SSSP, s, k_ds_relax<<<rg, 256, 0, s>>>(list, nl, heavy, g->off, g->adj, dist.get(), delta, hi,
-                                                           rstamp.get(), round_id, sstamp.get(), fstamp.get(), epoch,
-                                                           pnext, settled.get(), pfar, ctr.get()));
-        }
-        CLD_LAUNCH_CHECK();
-        return CLDIAM_OK;
-    };
-    for (;;) {
-        // light rounds of the current bucket
-        CLD_CUDA(cudaMemsetAsync(&ctr.get()->nsettled, 0, 4, s));
-        while (ncur > 0) {
-            ++round_id;
-            CLD_CUDA(cudaMemsetAsync(&ctr.get()->nnext, 0, 4, s));
-            CLD_CUDA(cudaMemcpyAsync(&ctr.get()->nfar, &nfar, 4, cudaMemcpyHostToDevice, s));
-            CLD_TRY(relax(pcur, ncur, false));
-            CLD_TRY(sync());
-            ++rounds;
-            ncur = hc->nnext;
-            nfar = hc->nfar;
-            scanned += (uint32_t)hc->front;
+            CLD_TRY(read());
+            st.cur ^= 1;
+            ++st.rounds;
+            st.scanned += (uint32_t)hc->r.front;
             // list: 16 B per node (+ its chunk-table share); relax: 8 B (col, w) + 4 B target distance per
             // position (+ 8 B per improved target: distance, stamp, list slot)
-            prof_add_bytes(K_SSSP, 24.0 * (double)(uint32_t)(hc->front >> 32) + 12.0 * (double)(uint32_t)hc->front +
-                                       8.0 * ncur);
-            std::swap(pcur, pnext);
+            prof_add_bytes(K_SSSP, 24.0 * (double)(uint32_t)(hc->r.front >> 32) + 12.0 * (double)(uint32_t)hc->r.front +
+                                       8.0 * st.ncur);
+        } else {
+            uint64_t lo = 0;
+            if (!ds_next_bucket(st, delta, &lo)) break;
+            CLD_CUDA(cudaMemsetAsync(ctr.get(), 0, sizeof(DsRound), s));
+            CLD_K(K_SSSP, s, k_ds_split<<<grid_for(((size_t)st.nfar + NU - 1) / NU, 256), 256, 0, s>>>(
+                                 a, st.cur, st.pile, st.nfar, lo, st.hi, st.epoch));
+            CLD_LAUNCH_CHECK();
+            st.pile ^= 1;
+            CLD_TRY(read());
         }
-        // heavy phase of the bucket
-        uint32_t ns = hc->nsettled;
-        if (ns > 0) {
-            CLD_CUDA(cudaMemcpyAsync(&ctr.get()->nfar, &nfar, 4, cudaMemcpyHostToDevice, s));
-            CLD_TRY(relax(settled.get(), ns, true));
-            CLD_TRY(sync());
-            ++rounds;
-            nfar = hc->nfar;
-            scanned += (uint32_t)hc->front;
-            prof_add_bytes(K_SSSP, 24.0 * (double)(uint32_t)(hc->front >> 32) + 12.0 * (double)(uint32_t)hc->front);
-        }
-        if (nfar == 0) break;
-        // next bucket
-        CLD_CUDA(cudaMemsetAsync(&ctr.get()->minbucket, 0xFF, 4, s));
-        CLD_K(K_SSSP, s, k_ds_minbucket<<<grid_for(nfar, 256), 256, 0, s>>>(pfar, nfar, dist.get(), hi, delta, ctr.get()));
-        CLD_LAUNCH_CHECK();
-        CLD_TRY(sync());
-        if (hc->minbucket == 0xFFFFFFFFu) break;
-        const uint64_t old_hi = hi;
-        lo = (uint64_t)hc->minbucket * delta;
-        hi = lo + delta;
-        ++epoch;
-        CLD_CUDA(cudaMemsetAsync(&ctr.get()->nnext, 0, 4, s));
-        CLD_CUDA(cudaMemsetAsync(&ctr.get()->nfar2, 0, 4, s));
-        CLD_K(K_SSSP, s, k_ds_split<<<grid_for(nfar, 256), 256, 0, s>>>(pfar, nfar, dist.get(), old_hi, hi, fstamp.get(), epoch, pcur,
-                                                      pfar2, ctr.get()));
-        CLD_LAUNCH_CHECK();
-        CLD_TRY(sync());
-        ncur = hc->nnext;
-        nfar = hc->nfar2;
-        std::swap(pfar, pfar2);
     }
     CLD_CUDA(cudaMemsetAsync(ecc_d.get(), 0, 4, s));
     CLD_K(K_SSSP, s, k_ds_ecc<<<gb, 256, 0, s>>>(dist.get(), n, ecc_d.get()));
     CLD_LAUNCH_CHECK();
-    uint32_t* he = reinterpret_cast<uint32_t*>(static_cast<char*>(g->host.h) + 240);
+    if (hc->overflow) {
+        // a candidate did not fit: an error if one from a final distance does not (an unsettled one may be larger)
+        CLD_K(K_SSSP, s, k_ds_overflow<<<gb, 256, 0, s>>>(g->off, g->adj, n, dist.get(), &ctr.get()->overflow));
+        CLD_LAUNCH_CHECK();
+        CLD_TRY(read());
+        if (hc->overflow == 2u) return fail(CLDIAM_ERR_OVERFLOW, "a distance reached 2^32 - 1");
+    }
     CLD_CUDA(cudaMemcpyAsync(he, ecc_d.get(), 4, cudaMemcpyDeviceToHost, s));
     if (dist_out) CLD_CUDA(cudaMemcpyAsync(dist_out, dist.get(), (size_t)n * 4, cudaMemcpyDefault, s));
     CLD_CUDA(cudaStreamSynchronize(s));
     *ecc = *he;
-    if (rounds_out) *rounds_out = rounds;
-    if (scanned_out) *scanned_out = scanned;
+    if (rounds_out) *rounds_out = st.rounds;
+    if (scanned_out) *scanned_out = st.scanned;
     return CLDIAM_OK;
 }
 
