@@ -225,9 +225,19 @@ struct ListAdj {
 // first passes: link every node with its r-th neighbour (ids >= n, which a consistent graph never holds,
 // are skipped rather than followed).  One launch per r with pointer jumping in between: linking several
 // neighbours in one pass builds long parent chains on meshes, which every later link then walks.
+// The pass that joins the first pass's trees is bound by exactly those walks on a large graph: every node
+// of a tree links at once, against roots that are being hooked.  So a sixteenth of the warps links first
+// (part 1), a jump follows, and the rest (part 2) finds nearly all of its pairs joined already, two reads
+// a node.  Second pass with its jumps, us, in one part -> in two: road grids of 16.8M nodes 2126 -> 367,
+// 9M 911 -> 253, 4.2M 284 -> 107; R-MAT 2^24 607 -> 291, 2^22 100 -> 88; an unblocked 4M mesh 36 -> 51.
+// Below kSplitNodes the two more launches are what shows (R-MAT 2^20 23 -> 34, road 1M 50 -> 48).
+constexpr uint32_t kSplitNodes = 1u << 22;
+constexpr uint32_t kSplitMask = 15;
 template <class A>
-__global__ void k_cc_link_nth(A g, uint32_t n, uint32_t r, uint32_t* __restrict__ parent) {
+__global__ void k_cc_link_nth(A g, uint32_t n, uint32_t r, uint32_t part, uint32_t* __restrict__ parent) {
     for (uint32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
+        // (hashed, so that no period of the node order picks one side of a grid)
+        if (part != 0 && (((((v >> 5) * 2654435761u) >> 16) & kSplitMask) == 0) != (part == 1)) continue;
         if (r >= g.deg(v)) continue;
         const uint32_t c = g.nbr(v, r);
         if (c < n) cc_link(v, c, parent);
@@ -736,10 +746,14 @@ cldiam_status build_csr(const uint32_t* src, const uint32_t* dst, const uint32_t
         // Afforest-style: link two neighbours per node, find the dominant tree by sampling,
         // then link the remaining edges of the nodes outside it (all no-ops on a graph without edges)
         constexpr uint32_t kNeighbourRounds = 2;
+        const bool split = n >= kSplitNodes;
         for (uint32_t r = 0; r < kNeighbourRounds; ++r) {
-            if (packed) CLD_K(K_CC, s, k_cc_link_nth<<<grid_for(n, 256), 256, 0, s>>>(la, n, r, parent.get()));
-            else CLD_K(K_CC, s, k_cc_link_nth<<<grid_for(n, 256), 256, 0, s>>>(ca, n, r, parent.get()));
-            CLD_K(K_CC, s, k_cc_compress<<<grid_for(n, 256), 256, 0, s>>>(parent.get(), n));
+            const uint32_t first = split && r > 0 ? 1 : 0, last = split && r > 0 ? 2 : 0;
+            for (uint32_t part = first; part <= last; ++part) {
+                if (packed) CLD_K(K_CC, s, k_cc_link_nth<<<grid_for(n, 256), 256, 0, s>>>(la, n, r, part, parent.get()));
+                else CLD_K(K_CC, s, k_cc_link_nth<<<grid_for(n, 256), 256, 0, s>>>(ca, n, r, part, parent.get()));
+                CLD_K(K_CC, s, k_cc_compress<<<grid_for(n, 256), 256, 0, s>>>(parent.get(), n));
+            }
         }
         CLD_LAUNCH_CHECK();
         constexpr uint32_t kSamples = 1024;
