@@ -272,16 +272,25 @@ cldiam_status reduce_sum_u32_to_u64(const uint32_t* in, size_t n, uint64_t* out,
 // look-back over a per-(tile, digit) status word, so no per-pass histogram
 // read or separate scan is needed.  Items are staged in shared memory in
 // digit order and written out as contiguous runs.
-constexpr int OS_THREADS = 256;
-constexpr int OS_WARPS = OS_THREADS / 32;
-template <class K, bool KV>
-struct OsCfg {  // items per thread: fewer for 64-bit (key, value) pairs to keep registers (and occupancy) in check
-    static constexpr int ITEMS = (sizeof(K) == 8 && KV) ? 8 : 12;
-    static constexpr int TILE = OS_THREADS * ITEMS;
+// Two tile sizes.  A pass is bound by instructions (the ALU pipe is the busiest unit), and per item they are
+// the ranking's ballots plus a share of the tile's fixed work: clearing and summing the warps' counts, the scan
+// over the digits, the look-back.  The large tile (512 threads, as many items as fit 64 registers, two CTAs an
+// SM) halves that share, the status words and the length of the look-back.  Against 256 threads of 12 (8 for
+// 64-bit pairs) items with a look-back that branched on every tile, a pass, us: 268M keys 1587 -> 1277,
+// 16.8M 105 -> 89, 1M 11.9 -> 9.6; 67M 64-bit pairs 1166 -> 831.  (14 keys rather than 12: 1277 for 1323;
+// 16 spill; 1024 threads of 12: 1550; 11 pairs rather than 8: 831 for 933.)
+// Below OS_BIG_MIN items the chip has room for every tile at once and one tile's latency is what shows:
+// 256 threads of 4.  A pass there, us, 12 items -> 4 -> the large tile: 8K keys 5.0 -> 3.4 -> 6.8, 65K 5.9 ->
+// 4.5 -> 7.5, 262K 7.1 -> 6.1 -> 8.4, 523K 8.8 -> 9.5 -> 8.9.
+constexpr size_t OS_BIG_MIN = 3u << 17;  // items from which the large tile is used
+template <class K, bool KV, bool BIG>
+struct OsCfg {
+    static constexpr int THREADS = BIG ? 512 : 256;
+    static constexpr int ITEMS = BIG ? ((sizeof(K) == 8 && KV) ? 11 : 14) : 4;
+    static constexpr int TILE = THREADS * ITEMS;
 };
+constexpr int OS_HIST_WARPS = 8;
 constexpr int OS_RADIX = 256;
-constexpr unsigned long long OS_AGG = 1ull << 32;   // status: tile's own count
-constexpr unsigned long long OS_PRE = 2ull << 32;   // status: inclusive prefix over tiles 0..t
 constexpr long long OS_WAIT_CYCLES = 4000000000ll;  // ~2 s at 2 GHz: a look-back that waits longer gives up
 
 // Digit histograms of every pass from one read of the keys: one private histogram per warp and pass
@@ -291,7 +300,7 @@ __global__ void __launch_bounds__(256) k_os_hist(const K* __restrict__ keys, siz
                                                  uint32_t* __restrict__ hist) {
     extern __shared__ uint32_t hs[];
     const unsigned w = threadIdx.x >> 5;
-    for (int i = threadIdx.x; i < OS_WARPS * npass * OS_RADIX; i += blockDim.x) hs[i] = 0;
+    for (int i = threadIdx.x; i < OS_HIST_WARPS * npass * OS_RADIX; i += blockDim.x) hs[i] = 0;
     __syncthreads();
     uint32_t* h = hs + (size_t)w * npass * OS_RADIX;
     constexpr int U = 8;  // keys loaded per thread before counting, to keep loads in flight
@@ -317,14 +326,14 @@ __global__ void __launch_bounds__(256) k_os_hist(const K* __restrict__ keys, siz
     __syncthreads();
     for (int i = threadIdx.x; i < npass * OS_RADIX; i += blockDim.x) {
         uint32_t c = 0;
-        for (int ww = 0; ww < OS_WARPS; ++ww) c += hs[(size_t)ww * npass * OS_RADIX + i];
+        for (int ww = 0; ww < OS_HIST_WARPS; ++ww) c += hs[(size_t)ww * npass * OS_RADIX + i];
         if (c) atomicAdd(&hist[i], c);
     }
 }
 
 // exclusive scan of each pass's 256 digit counts (one block, 256 threads)
 __global__ void k_os_hist_scan(uint32_t* __restrict__ hist, int npass) {
-    __shared__ uint32_t wsum[OS_WARPS];
+    __shared__ uint32_t wsum[OS_HIST_WARPS];
     const unsigned d = threadIdx.x, w = d >> 5, l = lane_id();
     for (int p = 0; p < npass; ++p) {
         uint32_t c = hist[p * OS_RADIX + d];
@@ -412,11 +421,17 @@ __device__ __forceinline__ void os_load_rank(const K* __restrict__ kt, const uin
 }
 
 // KV: items carry a 32-bit value (vin/vout); otherwise keys only.  sh = shift mod 32 (HI: shift >= 32).
-template <class K, bool KV, bool HI, int OS_ITEMS = OsCfg<K, KV>::ITEMS, int OS_TILE = OsCfg<K, KV>::TILE>
-__global__ void __launch_bounds__(OS_THREADS, 4)
+// A status word holds a count and, in its upper half, fl (the tile's own count) or fl + 1 (the inclusive
+// prefix over tiles 0..t); fl differs from pass to pass, so the words are cleared once a sort, not once a pass.
+template <class K, bool KV, bool HI, bool BIG>
+__global__ void __launch_bounds__(OsCfg<K, KV, BIG>::THREADS, 1024 / OsCfg<K, KV, BIG>::THREADS)
     k_os_pass(const K* __restrict__ kin, const uint32_t* __restrict__ vin, K* __restrict__ kout,
               uint32_t* __restrict__ vout, size_t n, uint32_t sh, uint32_t dm, const uint32_t* __restrict__ goff,
-              unsigned long long* __restrict__ status, uint32_t* __restrict__ tile_ctr, uint32_t* __restrict__ err) {
+              unsigned long long* __restrict__ status, uint32_t fl, uint32_t* __restrict__ tile_ctr,
+              uint32_t* __restrict__ err) {
+    constexpr int OS_THREADS = OsCfg<K, KV, BIG>::THREADS, OS_WARPS = OS_THREADS / 32;
+    constexpr int OS_ITEMS = OsCfg<K, KV, BIG>::ITEMS, OS_TILE = OsCfg<K, KV, BIG>::TILE;
+    const unsigned long long own = (unsigned long long)fl << 32, prefix = (unsigned long long)(fl + 1) << 32;
     extern __shared__ __align__(16) unsigned char os_smem[];
     K* s_key = reinterpret_cast<K*>(os_smem);
     uint32_t* s_val = reinterpret_cast<uint32_t*>(os_smem + sizeof(K) * OS_TILE);
@@ -450,13 +465,15 @@ __global__ void __launch_bounds__(OS_THREADS, 4)
 
     // per digit (thread d): tile count, publication, tile-local scan, look-back
     const unsigned d = tid;
-    const uint32_t g0 = goff[d];
+    const bool dig = OS_THREADS == OS_RADIX || d < OS_RADIX;
+    const uint32_t g0 = dig ? goff[d] : 0;
     uint32_t cnt = 0;
-#pragma unroll
-    for (int ww = 0; ww < OS_WARPS; ++ww) cnt += whist[ww][d];
     volatile unsigned long long* vst = status;
-    if (tile == 0) vst[d] = OS_PRE | cnt;
-    else vst[(size_t)tile * OS_RADIX + d] = OS_AGG | cnt;
+    if (dig) {
+#pragma unroll
+        for (int ww = 0; ww < OS_WARPS; ++ww) cnt += whist[ww][d];
+        vst[(size_t)tile * OS_RADIX + d] = (tile == 0 ? prefix : own) | cnt;
+    }
     uint32_t tst;
     {
         const uint32_t incl = warp_incl_scan(cnt);
@@ -466,7 +483,7 @@ __global__ void __launch_bounds__(OS_THREADS, 4)
         for (unsigned ww = 0; ww < w; ++ww) off += wsum[ww];
         tst = off + incl - cnt;
     }
-    {
+    if (dig) {
         uint32_t run = tst;  // only thread d touches column d of whist here
 #pragma unroll
         for (int ww = 0; ww < OS_WARPS; ++ww) {
@@ -489,38 +506,44 @@ __global__ void __launch_bounds__(OS_THREADS, 4)
         }
     }
     uint32_t excl = 0;
-    if (tile > 0) {
-        // windowed look-back: read the statuses of LB earlier tiles at once, add their counts
-        // back to the first inclusive prefix; wait (bounded) only on a tile not yet published
+    if (dig && tile > 0) {
+        // windowed look-back: read the statuses of LB earlier tiles at once, add their counts back to the
+        // first inclusive prefix (selects, no branch per tile); a window with a tile that has not published
+        // before that prefix is read again (bounded)
         constexpr int LB = 8;
         const long long t0 = clock64();
         long long t = (long long)tile - 1;
-        bool done = false, timed_out = false;
-        while (!done && !timed_out) {
+        bool done = false;
+        while (!done) {
             unsigned long long sw[LB];
 #pragma unroll
             for (int j = 0; j < LB; ++j)
-                sw[j] = (t - j >= 0) ? (unsigned long long)vst[(size_t)(t - j) * OS_RADIX + d] : (unsigned long long)OS_PRE;
+                sw[j] = (t - j >= 0) ? (unsigned long long)vst[(size_t)(t - j) * OS_RADIX + d] : prefix;
+            // entries up to the first prefix count; one of them not yet published: this window again
+            bool open = true, miss = false;
+            uint32_t sum = 0;
 #pragma unroll
             for (int j = 0; j < LB; ++j) {
-                if (done || timed_out) break;
-                while ((sw[j] & ~0xFFFFFFFFull) == 0) {
-                    if (clock64() - t0 > OS_WAIT_CYCLES) {
-                        atomicExch(err, 1u);
-                        timed_out = true;
-                        break;
-                    }
-                    __nanosleep(32);
-                    sw[j] = vst[(size_t)(t - j) * OS_RADIX + d];
-                }
-                excl += (uint32_t)sw[j];
-                if ((sw[j] & ~0xFFFFFFFFull) == OS_PRE) done = true;
+                const uint32_t f = (uint32_t)(sw[j] >> 32);
+                sum += open ? (uint32_t)sw[j] : 0u;
+                miss |= open && f - fl > 1u;
+                open = open && f != fl + 1u;
             }
+            if (miss) {
+                if (clock64() - t0 > OS_WAIT_CYCLES) {
+                    atomicExch(err, 1u);
+                    break;
+                }
+                __nanosleep(32);
+                continue;
+            }
+            excl += sum;
+            done = !open;
             t -= LB;
         }
-        vst[(size_t)tile * OS_RADIX + d] = OS_PRE | (excl + cnt);
+        vst[(size_t)tile * OS_RADIX + d] = prefix | (excl + cnt);
     }
-    gdiff[d] = g0 + excl - tst;  // modulo 2^32; positions are < 2^32
+    if (dig) gdiff[d] = g0 + excl - tst;  // modulo 2^32; positions are < 2^32
     __syncthreads();
     // write out: consecutive threads take consecutive staged items, i.e. runs of equal digits
     if (rem == (uint32_t)OS_TILE) {
@@ -555,23 +578,27 @@ static cldiam_status radix_sort_impl(K* keys, uint32_t* vals, K* keys_alt, uint3
     if (n > 0xFFFFFFFFull) return fail(CLDIAM_ERR_UNSUPPORTED, "radix sort limited to 2^32 - 1 items");
     const bool kv = vals != nullptr;
     const int npass = (bits + 7) / 8;
-    const int tile = kv ? OsCfg<K, true>::TILE : OsCfg<K, false>::TILE;
+    const bool big = n >= OS_BIG_MIN;
+    const int tile = big ? (kv ? OsCfg<K, true, true>::TILE : OsCfg<K, false, true>::TILE)
+                         : (kv ? OsCfg<K, true, false>::TILE : OsCfg<K, false, false>::TILE);
+    const int threads = big ? OsCfg<K, true, true>::THREADS : OsCfg<K, true, false>::THREADS;
     const uint32_t ntiles = (uint32_t)((n + tile - 1) / tile);
     const size_t smem = (sizeof(K) + (kv ? sizeof(uint32_t) : 0)) * tile;
-    static std::atomic<bool> attr_set[2][64];  // first call per device sets the attributes (idempotent)
+    static std::atomic<bool> attr_set[4][64];  // first call per device sets the attributes (idempotent)
     static std::atomic<bool> hist_attr_set[64];
+    const auto pick = [&](bool hi) {
+        if (kv) return big ? (hi ? k_os_pass<K, true, true, true> : k_os_pass<K, true, false, true>)
+                           : (hi ? k_os_pass<K, true, true, false> : k_os_pass<K, true, false, false>);
+        return big ? (hi ? k_os_pass<K, false, true, true> : k_os_pass<K, false, false, true>)
+                   : (hi ? k_os_pass<K, false, true, false> : k_os_pass<K, false, false, false>);
+    };
     int dev = 0;
     CLD_CUDA(cudaGetDevice(&dev));
-    if (dev < 0 || dev >= 64 || !attr_set[kv][dev]) {
-        const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
-        if (kv) {
-            CLD_CUDA(cudaFuncSetAttribute(k_os_pass<K, true, false>, a, (int)smem));
-            CLD_CUDA(cudaFuncSetAttribute(k_os_pass<K, true, true>, a, (int)smem));
-        } else {
-            CLD_CUDA(cudaFuncSetAttribute(k_os_pass<K, false, false>, a, (int)smem));
-            CLD_CUDA(cudaFuncSetAttribute(k_os_pass<K, false, true>, a, (int)smem));
-        }
-        if (dev >= 0 && dev < 64) attr_set[kv][dev] = true;
+    const int form = (kv ? 2 : 0) + (big ? 1 : 0);
+    if (dev < 0 || dev >= 64 || !attr_set[form][dev]) {
+        for (int hi = 0; hi < 2; ++hi)
+            CLD_CUDA(cudaFuncSetAttribute(pick(hi), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        if (dev >= 0 && dev < 64) attr_set[form][dev] = true;
     }
     DBuf<uint32_t> hist_own, ctl;
     DBuf<unsigned long long> status;
@@ -583,10 +610,10 @@ static cldiam_status radix_sort_impl(K* keys, uint32_t* vals, K* keys_alt, uint3
         CLD_TRY(hist_own.alloc((size_t)npass * OS_RADIX, s));
         hist = hist_own.get();
         CLD_CUDA(cudaMemsetAsync(hist, 0, (size_t)npass * OS_RADIX * 4, s));
-        const size_t hsm = (size_t)OS_WARPS * npass * OS_RADIX * 4;  // <= 64 KB (at most 8 passes)
+        const size_t hsm = (size_t)OS_HIST_WARPS * npass * OS_RADIX * 4;  // <= 64 KB (at most 8 passes)
         if (dev < 0 || dev >= 64 || !hist_attr_set[dev]) {
             CLD_CUDA(cudaFuncSetAttribute(k_os_hist<K>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          8 * OS_WARPS * OS_RADIX * 4));
+                                          8 * OS_HIST_WARPS * OS_RADIX * 4));
             if (dev >= 0 && dev < 64) hist_attr_set[dev] = true;
         }
         CLD_K(K_RADIX_HIST, s, k_os_hist<K><<<grid_for(n, 256, 4), 256, hsm, s>>>(first_in ? first_in : keys, n, npass,
@@ -601,8 +628,8 @@ static cldiam_status radix_sort_impl(K* keys, uint32_t* vals, K* keys_alt, uint3
     K* ko = keys_alt;
     uint32_t* vo = vals_alt;
     bool alt = false;
+    CLD_CUDA(cudaMemsetAsync(status.get(), 0, (size_t)ntiles * OS_RADIX * 8, s));
     for (int p = 0; p < npass; ++p) {
-        CLD_CUDA(cudaMemsetAsync(status.get(), 0, (size_t)ntiles * OS_RADIX * 8, s));
         const int shift = shift0 + 8 * p;
         const bool hi = sizeof(K) == 8 && shift >= 32;
         const uint32_t sh = (uint32_t)shift & 31u;
@@ -610,19 +637,8 @@ static cldiam_status radix_sort_impl(K* keys, uint32_t* vals, K* keys_alt, uint3
         const uint32_t* go = hist + p * OS_RADIX;
         uint32_t* tc = ctl.get() + p;
         uint32_t* er = err_dev ? err_dev : ctl.get() + 2 * npass;
-        if (kv && hi) {
-            CLD_K(K_RADIX_SCATTER, s, k_os_pass<K, true, true><<<ntiles, OS_THREADS, smem, s>>>(ki, vi, ko, vo, n, sh, dm, go,
-                                                                                              status.get(), tc, er));
-        } else if (kv) {
-            CLD_K(K_RADIX_SCATTER, s, k_os_pass<K, true, false><<<ntiles, OS_THREADS, smem, s>>>(ki, vi, ko, vo, n, sh, dm, go,
-                                                                                               status.get(), tc, er));
-        } else if (hi) {
-            CLD_K(K_RADIX_SCATTER, s, k_os_pass<K, false, true><<<ntiles, OS_THREADS, smem, s>>>(ki, nullptr, ko, nullptr, n,
-                                                                                               sh, dm, go, status.get(), tc, er));
-        } else {
-            CLD_K(K_RADIX_SCATTER, s, k_os_pass<K, false, false><<<ntiles, OS_THREADS, smem, s>>>(ki, nullptr, ko, nullptr, n,
-                                                                                                sh, dm, go, status.get(), tc, er));
-        }
+        CLD_K(K_RADIX_SCATTER, s, pick(hi)<<<ntiles, threads, smem, s>>>(ki, vi, ko, vo, n, sh, dm, go, status.get(),
+                                                                         2u * p + 1u, tc, er));
         CLD_LAUNCH_CHECK();
         // algorithmic bytes: every item (key and value) read once and written once
         prof_add_bytes(K_RADIX_SCATTER, 2.0 * (double)n * (sizeof(K) + (kv ? sizeof(uint32_t) : 0)));
@@ -1076,8 +1092,10 @@ cldiam_status radix_sort_pairs_u32(uint32_t* keys, uint32_t* vals, uint32_t* key
 cldiam_status load_prims_kernels() {
     return load_kernels(k_tile_reduce<uint32_t>, k_tile_scan<uint32_t>, k_tile_reduce<uint64_t>, k_tile_scan<uint64_t>,
                         k_offsets_from_rows, k_reduce_max_u32, k_reduce_min_u32, k_reduce_sum_u32, k_os_hist<uint32_t>,
-                        k_os_hist<uint64_t>, k_os_hist_scan, k_os_pass<uint32_t, true, false>,
-                        k_os_pass<uint64_t, true, false>, k_os_pass<uint64_t, true, true>, k_unique_count<uint32_t>,
+                        k_os_hist<uint64_t>, k_os_hist_scan, k_os_pass<uint32_t, true, false, false>,
+                        k_os_pass<uint64_t, true, false, false>, k_os_pass<uint64_t, true, true, false>,
+                        k_os_pass<uint32_t, true, false, true>, k_os_pass<uint64_t, true, false, true>,
+                        k_os_pass<uint64_t, true, true, true>, k_unique_count<uint32_t>,
                         k_unique_count<uint64_t>, k_unique_write<uint32_t>, k_unique_write<uint64_t>);
 }
 
