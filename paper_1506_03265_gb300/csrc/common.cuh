@@ -360,7 +360,9 @@ cldiam_status reduce_min_u32(const uint32_t* in, size_t n, uint32_t* out, cudaSt
 // key.  Buffers *_alt are scratch of the same size; on return *result_in_alt
 // tells which pair of buffers holds the sorted sequence.
 cldiam_status radix_sort_pairs_u64(uint64_t* keys, uint32_t* vals, uint64_t* keys_alt, uint32_t* vals_alt,
-                                   size_t n, int bits, bool* result_in_alt, cudaStream_t s);
+                                   size_t n, int bits, bool* result_in_alt, cudaStream_t s,
+                                   uint32_t* err_dev = nullptr, const uint64_t* first_in = nullptr,
+                                   const uint32_t* first_vin = nullptr, uint32_t* hist_in = nullptr);
 cldiam_status radix_sort_pairs_u32(uint32_t* keys, uint32_t* vals, uint32_t* keys_alt, uint32_t* vals_alt,
                                    size_t n, int bits, bool* result_in_alt, cudaStream_t s);
 // Stable LSD radix sort of 64-bit keys alone on key bits [shift0, shift0 + bits).  With err_dev the
@@ -369,29 +371,30 @@ cldiam_status radix_sort_pairs_u32(uint32_t* keys, uint32_t* vals, uint32_t* key
 // read from there (never written) and keys / keys_alt serve only as the ping-pong buffers.  With hist_in
 // the digit counts of every pass (ceil(bits / 8) x 256 words, in pass order, digits as the sort takes
 // them) were accumulated by the producer of the keys: the sort scans them in place instead of reading
-// the keys once more to count.
+// the keys once more to count.  (All of this holds for the 64-bit pairs too, first_vin beside first_in.)
 cldiam_status radix_sort_keys_u64(uint64_t* keys, uint64_t* keys_alt, size_t n, int shift0, int bits,
                                   bool* result_in_alt, cudaStream_t s, uint32_t* err_dev = nullptr,
                                   const uint64_t* first_in = nullptr, uint32_t* hist_in = nullptr);
 
 // Unique keys of a sorted sequence with the minimum value of each run:
-// row_out[r] = key / div (row_out may be null), col_out[r*cs] = key % div,
-// w_out[r*cs] = run minimum (w_out must hold 0xFFFFFFFF beforehand);
-// keys >= sentinel are skipped; *total_dev = number of unique keys.  With
-// off_out (may be null), off_out[0..nrows] = CSR offsets of the rows.
+// col_out[r] = key % div, w_out[r] = run minimum (w_out must hold 0xFFFFFFFF
+// beforehand), off_out[0..nrows] = CSR offsets of the rows key / div;
+// keys >= sentinel are skipped; *total_dev = number of unique keys.
 cldiam_status unique_min_sorted_u64(const uint64_t* keys, const uint32_t* vals, size_t cnt, uint64_t sentinel,
-                                    uint64_t div, uint32_t* row_out, uint32_t* col_out, uint32_t* w_out, int cs,
-                                    uint64_t* off_out, uint32_t nrows, uint32_t* total_dev, cudaStream_t s);
+                                    uint64_t div, uint32_t* col_out, uint32_t* w_out, uint64_t* off_out,
+                                    uint32_t nrows, uint32_t* total_dev, cudaStream_t s);
 cldiam_status unique_min_sorted_u32(const uint32_t* keys, const uint32_t* vals, size_t cnt, uint32_t sentinel,
-                                    uint64_t div, uint32_t* row_out, uint32_t* col_out, uint32_t* w_out, int cs,
-                                    uint64_t* off_out, uint32_t nrows, uint32_t* total_dev, cudaStream_t s);
-// De-duplication of packed edge items (a << vb | b) << (64 - 2 vb) | w sorted on their (a, b) bits (~0 marks
-// a dropped item): out[r] = the r-th distinct (a, b) item with its smallest weight; *total_dev = their
-// number.  With hist2 (ceil(vb / 8) x 256 words, zeroed) the counting pass also adds up the 8-bit digits
-// of every distinct item's b (bits [wb, wb + vb)), pass by pass: the histograms of a following sort on b.
-cldiam_status unique_items_u64(const uint64_t* items, size_t cnt, int vb, uint64_t* out, uint32_t* total_dev,
-                               cudaStream_t s, uint32_t* hist2 = nullptr, uint32_t* ustart = nullptr,
-                               uint32_t* uend = nullptr);
+                                    uint64_t div, uint32_t* col_out, uint32_t* w_out, uint64_t* off_out,
+                                    uint32_t nrows, uint32_t* total_dev, cudaStream_t s);
+// De-duplication of edge items sorted on their (a, b) bits: packed words (a << vb | b) << (64 - 2 vb) | w when
+// vals is null, else keys a << vb | b with the weight beside them in vals; ~0 marks a dropped item.  out[r] = the
+// r-th distinct (a, b) item with its smallest weight (w_out[r] with vals: cnt words); *total_dev = their number.
+// The counting pass also adds up the 8-bit digits of every distinct item's b, pass by pass, into hist2
+// (ceil(vb / 8) x 256 words, zeroed): the histograms of a following sort on b.  ustart / uend (zeroed): the run
+// bounds of every row a.
+cldiam_status unique_items_u64(const uint64_t* items, const uint32_t* vals, size_t cnt, int vb, uint64_t* out,
+                               uint32_t* w_out, uint32_t* total_dev, cudaStream_t s, uint32_t* hist2, uint32_t* ustart,
+                               uint32_t* uend);
 
 // CSR offsets off[0..n] of entries whose (sorted) row ids are row[0..nnz):
 // off[u] = index of the first entry with row >= u.  No atomics, no scan.

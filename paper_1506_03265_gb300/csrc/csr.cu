@@ -8,8 +8,11 @@
 // parallel edge.  The distinct edges sorted again on max alone (stable, so
 // by (max, min)) give each row's entries below the diagonal; row x of the
 // CSR is those, then its entries above the diagonal from the first order.
-// Otherwise every edge becomes two directed (row * n + col, weight) pairs,
-// sorted and de-duplicated the same way.  Components come from min-label
+// With wider weights the words hold the ids alone and the weights travel
+// beside them through the same steps (before, every edge became two directed
+// (row * n + col, weight) pairs, 12 sorted items an edge to 9 here: R-MAT 2^20
+// x 16 with 31-bit weights 2.66 -> 1.92 ms, R-MAT of 10.4M nodes x 8 with
+// 20-bit weights, whole estimate, 18.2 -> 14.1).  Components come from min-label
 // hooking with pointer jumping: every tree points to a smaller id of its
 // component, so roots are component minima and the labelling is
 // deterministic.
@@ -24,42 +27,29 @@ namespace cld {
 
 namespace {
 
-__global__ void k_emit_directed(const uint32_t* __restrict__ src, const uint32_t* __restrict__ dst,
-                                const uint32_t* __restrict__ w, uint64_t m, uint32_t n, uint64_t sentinel,
-                                uint64_t* __restrict__ keys, uint32_t* __restrict__ vals, uint32_t* __restrict__ bad) {
-    for (uint64_t e = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m; e += (uint64_t)gridDim.x * blockDim.x) {
-        uint32_t u = src[e], v = dst[e], ww = w[e];
-        bool ok = u < n && v < n && ww != 0;
-        if (!ok) atomicExch(bad, 1u);
-        uint64_t k0 = sentinel, k1 = sentinel;
-        if (ok && u != v) {
-            k0 = (uint64_t)u * n + v;
-            k1 = (uint64_t)v * n + u;
-        }
-        keys[2 * e] = k0;
-        keys[2 * e + 1] = k1;
-        vals[2 * e] = ww;
-        vals[2 * e + 1] = ww;
-    }
-}
-
 // one item per edge, (min(u,v) << vb | max(u,v)) << wb | w, a self-loop as ~0 (dropped, sorts last); also
 // the input check (ids < n, weights >= 1 -> *bad) and whether a weight needs more than wb bits (*wide: the
-// caller falls back to (key, weight) pairs)
+// caller emits again as PAIRS: wb = 0, the weights in vals).  The first wide weight ends its CTA's part and by
+// the flag the others': what has to be done again costs little (R-MAT 2^20 x 16 with 31-bit weights 93 -> 43 us;
+// a flag that every thread stored to, 303).
 // The same pass counts the digits of every pass of the sort that follows (8-bit digits of the item's
 // 2 vb (a, b) bits, the last one masked to the bits left) into per-warp shared histograms
 // (warps x npass x 256 words of dynamic shared memory), flushed into hist (npass x 256) at the end: the
 // sort then needs no read of its own to count them.
+template <bool PAIRS>
 __global__ void k_emit_canon(const uint32_t* __restrict__ src, const uint32_t* __restrict__ dst,
                              const uint32_t* __restrict__ w, uint64_t m, uint32_t n, int vb, int wb,
-                             uint64_t* __restrict__ items, uint32_t* __restrict__ bad, uint32_t* __restrict__ wide,
-                             uint32_t* __restrict__ hist) {
+                             uint64_t* __restrict__ items, uint32_t* __restrict__ vals, uint32_t* __restrict__ bad,
+                             uint32_t* __restrict__ wide, uint32_t* __restrict__ hist) {
     extern __shared__ uint32_t eh[];
+    __shared__ uint32_t s_wide;
+    volatile uint32_t* const wide_here = &s_wide;
+    if (!PAIRS && threadIdx.x == 0) s_wide = 0;
     const int npass = (2 * vb + 7) / 8;
     for (int i = threadIdx.x; i < (int)(blockDim.x >> 5) * npass * 256; i += blockDim.x) eh[i] = 0;
     __syncthreads();
     uint32_t* h = eh + (threadIdx.x >> 5) * npass * 256;
-    bool b = false, wd = false;
+    bool b = false;
     const uint64_t wlim = wb >= 32 ? ~0ull : (1ull << wb);
     // EU edges per thread and iteration, their loads issued before the counting (which would otherwise
     // hold back the next loads: fewer CTAs fit per SM with the histograms)
@@ -67,6 +57,7 @@ __global__ void k_emit_canon(const uint32_t* __restrict__ src, const uint32_t* _
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     for (uint64_t base = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; base < m; base += stride * EU) {
         uint32_t su[EU], sv[EU], sw[EU];
+        const uint32_t stop = PAIRS ? 0u : *static_cast<volatile uint32_t*>(wide) | *wide_here;
 #pragma unroll
         for (int k = 0; k < EU; ++k) {
             const uint64_t e = base + k * stride;
@@ -74,16 +65,18 @@ __global__ void k_emit_canon(const uint32_t* __restrict__ src, const uint32_t* _
             sv[k] = e < m ? dst[e] : 0u;
             sw[k] = e < m ? w[e] : 1u;
         }
+        if (stop) break;
 #pragma unroll
         for (int k = 0; k < EU; ++k) {
             const uint64_t e = base + k * stride;
             if (e >= m) break;
             const uint64_t u = su[k], v = sv[k], ww = sw[k];
             b |= u >= n || v >= n || ww == 0;
-            wd |= ww >= wlim;
+            if (!PAIRS && ww >= wlim) *wide_here = 1u;
             const uint64_t lo = u < v ? u : v, hi = u < v ? v : u;
-            const uint64_t it = u != v ? (((lo << vb) | hi) << wb) | ww : ~0ull;
+            const uint64_t it = u != v ? (((lo << vb) | hi) << wb) | (PAIRS ? 0ull : ww) : ~0ull;
             items[e] = it;
+            if (PAIRS) vals[e] = (uint32_t)ww;
             for (int p = 0; p < npass; ++p) {
                 const int left = 2 * vb - 8 * p;
                 const uint32_t dm = left >= 8 ? 0xFFu : ((1u << left) - 1u);
@@ -92,8 +85,8 @@ __global__ void k_emit_canon(const uint32_t* __restrict__ src, const uint32_t* _
         }
     }
     if (__any_sync(0xffffffffu, b) && lane_id() == 0) atomicExch(bad, 1u);
-    if (__any_sync(0xffffffffu, wd) && lane_id() == 0) atomicExch(wide, 1u);
     __syncthreads();
+    if (!PAIRS && threadIdx.x == 0 && s_wide) *static_cast<volatile uint32_t*>(wide) = 1u;
     for (int i = threadIdx.x; i < npass * 256; i += blockDim.x) {
         uint32_t c = 0;
         for (int ww = 0; ww < (int)(blockDim.x >> 5); ++ww) c += eh[ww * npass * 256 + i];
@@ -150,35 +143,6 @@ __global__ void k_canon_deg(uint32_t n, const uint32_t* __restrict__ ustart, con
         deg[x] = (uint64_t)(uend[x] - ustart[x]) + (tend[x] - tstart[x]);
 }
 
-// (a position outside its row's part means inconsistent runs: recorded in *err, the write skipped)
-__global__ void k_canon_scatter(const uint64_t* __restrict__ U, const uint64_t* __restrict__ T, uint32_t mu, int vb,
-                                int wb, const uint32_t* __restrict__ ustart, const uint32_t* __restrict__ tstart,
-                                const uint32_t* __restrict__ tend, const uint64_t* __restrict__ off,
-                                uint32_t* __restrict__ row, uint2* __restrict__ adj, uint32_t* __restrict__ err) {
-    const int ash = 64 - vb;
-    const uint32_t cmask = vb >= 32 ? 0xFFFFFFFFu : ((1u << vb) - 1u);
-    const uint32_t wmask = wb >= 32 ? 0xFFFFFFFFu : ((1u << wb) - 1u);
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < mu; i += gridDim.x * blockDim.x) {
-        const uint64_t u = U[i], t = T[i];
-        const uint32_t a = (uint32_t)(u >> ash), b = (uint32_t)(u >> wb) & cmask;
-        const uint64_t pu = off[a] + (tend[a] - tstart[a]) + (i - ustart[a]);  // after row a's lower entries
-        if (i >= ustart[a] && pu < off[a + 1]) {
-            adj[pu] = make_uint2(b, (uint32_t)u & wmask);
-            row[pu] = a;
-        } else {
-            atomicExch(err, 1u);
-        }
-        const uint32_t ta = (uint32_t)(t >> ash), tb = (uint32_t)(t >> wb) & cmask;
-        const uint64_t pt = off[tb] + (i - tstart[tb]);
-        if (i >= tstart[tb] && i < tend[tb]) {
-            adj[pt] = make_uint2(ta, (uint32_t)t & wmask);
-            row[pt] = tb;
-        } else {
-            atomicExch(err, 1u);
-        }
-    }
-}
-
 __global__ void k_iota(uint32_t* __restrict__ a, uint32_t n) {
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) a[i] = i;
 }
@@ -199,18 +163,13 @@ __device__ __forceinline__ void cc_link(uint32_t u, uint32_t v, uint32_t* parent
     }
 }
 
-// A node's neighbours in CSR order, from the CSR ...
-struct CsrAdj {
-    const uint64_t* off;
-    const uint2* adj;
-    __device__ uint32_t deg(uint32_t v) const { return (uint32_t)(off[v + 1] - off[v]); }
-    __device__ uint32_t nbr(uint32_t v, uint32_t r) const { return adj[off[v] + r].x; }
-};
-// ... or from the two orders of the distinct edges (a, b), a < b: first the lower neighbours (the a of
-// v's run in T, sorted by (b, a)), then the upper ones (the b of v's run in U, sorted by (a, b))
+// A node's neighbours in CSR order, from the two orders of the distinct edges (a, b), a < b: first the lower
+// neighbours (the a of v's run in T, sorted by (b, a)), then the upper ones (the b of v's run in U, sorted by
+// (a, b)).  The weights are in the words' low wb bits, or (wb = 0) beside them in UW and TW.
 struct ListAdj {
     const uint64_t* U;
     const uint64_t* T;
+    const uint32_t *UW, *TW;
     const uint32_t *ustart, *uend, *tstart, *tend;
     int ash, wb;
     uint32_t cmask;
@@ -221,6 +180,32 @@ struct ListAdj {
         return r < l ? (uint32_t)(T[tstart[v] + r] >> ash) : (uint32_t)(U[ustart[v] + (r - l)] >> wb) & cmask;
     }
 };
+
+// (a position outside its row's part means inconsistent runs: recorded in *err, the write skipped)
+__global__ void k_canon_scatter(ListAdj g, uint32_t mu, const uint64_t* __restrict__ off, uint32_t* __restrict__ row,
+                                uint2* __restrict__ adj, uint32_t* __restrict__ err) {
+    const uint32_t wmask = g.wb >= 32 ? 0xFFFFFFFFu : ((1u << g.wb) - 1u);
+    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < mu; i += gridDim.x * blockDim.x) {
+        const uint64_t u = g.U[i], t = g.T[i];
+        const uint32_t uw = g.UW ? g.UW[i] : (uint32_t)u & wmask, tw = g.TW ? g.TW[i] : (uint32_t)t & wmask;
+        const uint32_t a = (uint32_t)(u >> g.ash), b = (uint32_t)(u >> g.wb) & g.cmask;
+        const uint64_t pu = off[a] + g.lo(a) + (i - g.ustart[a]);  // after row a's lower entries
+        if (i >= g.ustart[a] && pu < off[a + 1]) {
+            adj[pu] = make_uint2(b, uw);
+            row[pu] = a;
+        } else {
+            atomicExch(err, 1u);
+        }
+        const uint32_t ta = (uint32_t)(t >> g.ash), tb = (uint32_t)(t >> g.wb) & g.cmask;
+        const uint64_t pt = off[tb] + (i - g.tstart[tb]);
+        if (i >= g.tstart[tb] && i < g.tend[tb]) {
+            adj[pt] = make_uint2(ta, tw);
+            row[pt] = tb;
+        } else {
+            atomicExch(err, 1u);
+        }
+    }
+}
 
 // first passes: link every node with its r-th neighbour (ids >= n, which a consistent graph never holds,
 // are skipped rather than followed).  One launch per r with pointer jumping in between: linking several
@@ -233,8 +218,7 @@ struct ListAdj {
 // Below kSplitNodes the two more launches are what shows (R-MAT 2^20 23 -> 34, road 1M 50 -> 48).
 constexpr uint32_t kSplitNodes = 1u << 22;
 constexpr uint32_t kSplitMask = 15;
-template <class A>
-__global__ void k_cc_link_nth(A g, uint32_t n, uint32_t r, uint32_t part, uint32_t* __restrict__ parent) {
+__global__ void k_cc_link_nth(ListAdj g, uint32_t n, uint32_t r, uint32_t part, uint32_t* __restrict__ parent) {
     for (uint32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
         // (hashed, so that no period of the node order picks one side of a grid)
         if (part != 0 && (((((v >> 5) * 2654435761u) >> 16) & kSplitMask) == 0) != (part == 1)) continue;
@@ -247,8 +231,7 @@ __global__ void k_cc_link_nth(A g, uint32_t n, uint32_t r, uint32_t part, uint32
 // final pass: nodes outside the dominant tree link all their remaining
 // neighbours (an edge with both ends in the dominant tree adds nothing; an
 // edge with one end outside is linked from that end)
-template <class A>
-__global__ void k_cc_link_rest(A g, uint32_t n, uint32_t skip, uint32_t giant, uint32_t* __restrict__ parent) {
+__global__ void k_cc_link_rest(ListAdj g, uint32_t n, uint32_t skip, uint32_t giant, uint32_t* __restrict__ parent) {
     for (uint32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
         uint32_t r = parent[v];
         while (parent[r] != r) r = parent[r];
@@ -333,74 +316,13 @@ __global__ void k_cc_keep(const uint32_t* __restrict__ parent, uint32_t n, const
         keep[v] = parent[v] == root ? 1u : 0u;
 }
 
-template <class A>
-__global__ void k_lcc_degrees(const uint32_t* __restrict__ keep, const uint32_t* __restrict__ newid, A g, uint32_t n,
+__global__ void k_lcc_degrees(const uint32_t* __restrict__ keep, const uint32_t* __restrict__ newid, ListAdj g, uint32_t n,
                               uint32_t* __restrict__ ndeg, uint32_t* __restrict__ orig) {
     for (uint32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x)
         if (keep[v]) {
             ndeg[newid[v]] = g.deg(v);
             orig[newid[v]] = v;
         }
-}
-
-// new offsets (widened from the 32-bit scan of the kept degrees) and, for each kept node orig[i], its
-// new id and the shift from its old adjacency positions to its new ones (positions are < 2^32, so
-// the shift is taken modulo 2^32); map of a dropped node keeps its 0xFFFFFFFF pre-fill
-__global__ void k_lcc_offsets(const uint32_t* __restrict__ excl, uint32_t n, const uint32_t* __restrict__ n_out_dev,
-                              const uint32_t* __restrict__ total_dev, const uint32_t* __restrict__ orig,
-                              const uint64_t* __restrict__ off, uint64_t* __restrict__ noff, uint2* __restrict__ map) {
-    const uint32_t n_out = *n_out_dev, total = *total_dev;  // n_out <= n
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i <= n_out; i += gridDim.x * blockDim.x) {
-        noff[i] = (i == n_out) ? (uint64_t)total : (uint64_t)excl[i];
-        if (map && i < n_out) {
-            const uint32_t u = orig[i];
-            map[u] = make_uint2(i, excl[i] - (uint32_t)off[u]);
-        }
-    }
-}
-
-// copy of the kept rows with new ids (monotone, so rows stay sorted), and the
-// weight statistics of the copy: sum over u < v and minimum.  Each thread
-// handles LU entries a grid stride apart with all their loads issued first.
-__global__ void __launch_bounds__(256) k_lcc_copy(const uint2* __restrict__ map, const uint32_t* __restrict__ newid,
-                                                  const uint32_t* __restrict__ row, const uint2* __restrict__ adj,
-                                                  uint64_t nnz, uint32_t* __restrict__ nrow, uint2* __restrict__ nadj,
-                                                  unsigned long long* __restrict__ wsum, uint32_t* __restrict__ wmin) {
-    constexpr int LU = 4;
-    unsigned long long sum = 0;
-    uint32_t mn = 0xFFFFFFFFu;
-    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    for (uint64_t b = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; b < nnz; b += stride * LU) {
-        uint32_t u[LU];
-        uint2 e[LU], mp[LU];
-        uint32_t nv[LU];
-#pragma unroll
-        for (int k = 0; k < LU; ++k) {
-            const uint64_t i = b + (uint64_t)k * stride;
-            u[k] = i < nnz ? row[i] : 0u;
-            e[k] = i < nnz ? adj[i] : make_uint2(0u, 0u);
-        }
-#pragma unroll
-        for (int k = 0; k < LU; ++k) {
-            const uint64_t i = b + (uint64_t)k * stride;
-            mp[k] = i < nnz ? map[u[k]] : make_uint2(0xFFFFFFFFu, 0u);
-            nv[k] = i < nnz ? newid[e[k].x] : 0u;
-        }
-#pragma unroll
-        for (int k = 0; k < LU; ++k) {
-            if (mp[k].x == 0xFFFFFFFFu) continue;  // dropped row, or past the end
-            const uint64_t i = b + (uint64_t)k * stride;
-            const uint32_t pos = (uint32_t)i + mp[k].y;
-            nadj[pos] = make_uint2(nv[k], e[k].y);
-            nrow[pos] = mp[k].x;
-            if (u[k] < e[k].x) sum += e[k].y;
-            mn = e[k].y < mn ? e[k].y : mn;
-        }
-    }
-    sum = block_reduce(sum, [](unsigned long long a, unsigned long long b) { return a + b; }, 0ull);
-    if (threadIdx.x == 0 && sum) atomicAdd(wsum, sum);
-    mn = block_reduce(mn, [](uint32_t a, uint32_t b) { return a < b ? a : b; }, 0xFFFFFFFFu);
-    if (threadIdx.x == 0 && mn != 0xFFFFFFFFu) atomicMin(wmin, mn);
 }
 
 // New offsets of the LCC from the scan of its degrees, and per kept node u = orig[i] one word of four:
@@ -426,6 +348,7 @@ __global__ void k_lcc_offsets_lists(const uint32_t* __restrict__ excl, const uin
 // A position past the output (inconsistent input) is recorded in *err and the write skipped.  The row's
 // own record (info, 16 B) is read in runs (U is sorted on a, T on b); the far end's new id comes from
 // the 4-byte newid array (evict-last: it stays in L2 while the two edge lists stream through, evict-first).
+template <bool PAIRS>
 __global__ void __launch_bounds__(256, 4) k_lcc_assemble(ListAdj g, uint32_t mu, const uint4* __restrict__ info,
                                                          const uint32_t* __restrict__ newid, uint64_t cap,
                                                          uint2* __restrict__ nadj, unsigned long long* __restrict__ wsum,
@@ -441,11 +364,16 @@ __global__ void __launch_bounds__(256, 4) k_lcc_assemble(ListAdj g, uint32_t mu,
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     for (uint64_t base = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; base < mu; base += stride * AU) {
         uint64_t u[AU], t[AU];
+        uint32_t uw[PAIRS ? AU : 1], tw[PAIRS ? AU : 1];
 #pragma unroll
         for (int k = 0; k < AU; ++k) {
             const uint64_t i = base + k * stride;
             u[k] = i < mu ? ld_stream_u64(g.U + i, pol_stream) : 0ull;
             t[k] = i < mu ? ld_stream_u64(g.T + i, pol_stream) : 0ull;
+            if constexpr (PAIRS) {
+                uw[k] = i < mu ? g.UW[i] : 0u;
+                tw[k] = i < mu ? g.TW[i] : 0u;
+            }
         }
         // position shifts of the kept rows' entries, and which rows are kept (bit k: the edge's row in U,
         // bit AU + k: its row in T)
@@ -472,7 +400,8 @@ __global__ void __launch_bounds__(256, 4) k_lcc_assemble(ListAdj g, uint32_t mu,
         for (int k = 0; k < AU; ++k) {
             const uint32_t i = (uint32_t)(base + k * stride);  // < mu when the row is kept
             if ((kept >> k) & 1u) {  // kept (then b is kept too)
-                const uint32_t w = (uint32_t)u[k] & wmask;
+                uint32_t w = (uint32_t)u[k] & wmask;
+                if constexpr (PAIRS) w = uw[k];
                 const uint32_t pos = iy[k] + i;
                 if (pos < cap) {
                     nadj[pos] = make_uint2(nb[k], w);
@@ -483,9 +412,11 @@ __global__ void __launch_bounds__(256, 4) k_lcc_assemble(ListAdj g, uint32_t mu,
                 mn = w < mn ? w : mn;
             }
             if ((kept >> (AU + k)) & 1u) {
+                uint32_t w = (uint32_t)t[k] & wmask;
+                if constexpr (PAIRS) w = tw[k];
                 const uint32_t pos = jz[k] + i;
                 if (pos < cap) {
-                    nadj[pos] = make_uint2(na[k], (uint32_t)t[k] & wmask);
+                    nadj[pos] = make_uint2(na[k], w);
                 } else {
                     atomicExch(err, 1u);
                 }
@@ -596,36 +527,29 @@ cldiam_status build_csr(const uint32_t* src, const uint32_t* dst, const uint32_t
     CLD_TRY(scal.alloc(9, s));
     CLD_CUDA(cudaMemsetAsync(scal.get(), 0, 9 * sizeof(uint32_t), s));
     const int vb = std::max(1, bits_for((uint64_t)n - 1));
-    const int wb = 64 - 2 * vb;  // weight bits of a packed item
+    const int wfit = 64 - 2 * vb;  // weight bits of a packed item
 
     DBuf<uint32_t> row, deg, degx;
     DBuf<uint64_t> off;
     DBuf<uint2> adj;
-    // the whole graph's row / adj arrays are allocated only where they are built (the packed path with the
-    // LCC goes from the edge lists straight to the LCC's CSR)
-    const auto alloc_full = [&]() -> cldiam_status {
-        CLD_TRY(row.alloc(cnt ? cnt : 1, s));
-        CLD_TRY(adj.alloc(cnt ? cnt : 1, s));
-        return CLDIAM_OK;
-    };
-    CLD_TRY(deg.alloc((size_t)n + 1, s));
-    CLD_TRY(degx.alloc((size_t)n + 1, s));
-    CLD_TRY(off.alloc((size_t)n + 1, s));
     const bool lcc = (flags & CLDIAM_CSR_LCC) != 0;
-    bool packed = wb >= 1;
-    // packed path: the distinct edges in two orders and their run bounds (the adjacency in list form)
+    // the distinct edges in two orders (with their weights beside them when these do not fit the words) and
+    // their run bounds: the adjacency in list form
+    bool pairs = wfit < 1;
     DBuf<uint64_t> items, items2, uniq;
+    DBuf<uint32_t> vals, vals2, uniqw;
     DBuf<uint32_t> hist1;  // digit counts of the first sort, accumulated by the emission
     DBuf<uint32_t> hist2;  // digit counts of the second sort, accumulated by the de-duplication
     DBuf<uint32_t> runs;
     ListAdj la{};
     uint32_t mu = 0;
-    if (packed) {
-        // one item per edge, sorted on (a, b) and de-duplicated (U); the same distinct edges sorted on b alone
-        // (stable, so by (b, a): T) give every row's entries below the diagonal
-        CLD_TRY(items.alloc(m ? m : 1, s));
-        const int npass1 = (2 * vb + 7) / 8;
-        CLD_TRY(hist1.alloc((size_t)npass1 * 256, s));
+    // one item per edge, sorted on (a, b) and de-duplicated (U); the same distinct edges sorted on b alone
+    // (stable, so by (b, a): T) give every row's entries below the diagonal
+    CLD_TRY(items.alloc(m ? m : 1, s));
+    const int npass1 = (2 * vb + 7) / 8;
+    CLD_TRY(hist1.alloc((size_t)npass1 * 256, s));
+    for (;;) {
+        if (pairs) CLD_TRY(vals.alloc(m ? m : 1, s));
         CLD_CUDA(cudaMemsetAsync(hist1.get(), 0, (size_t)npass1 * 256 * 4, s));
         if (m > 0) {
             const size_t esm = (size_t)8 * npass1 * 256 * 4;  // 8 warps; <= 64 KB
@@ -633,98 +557,87 @@ cldiam_status build_csr(const uint32_t* src, const uint32_t* dst, const uint32_t
             int dev = 0;
             CLD_CUDA(cudaGetDevice(&dev));
             if (dev < 0 || dev >= 64 || !emit_attr[dev]) {
-                CLD_CUDA(cudaFuncSetAttribute(k_emit_canon, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024));
+                const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
+                CLD_CUDA(cudaFuncSetAttribute(k_emit_canon<false>, a, 64 * 1024));
+                CLD_CUDA(cudaFuncSetAttribute(k_emit_canon<true>, a, 64 * 1024));
                 if (dev >= 0 && dev < 64) emit_attr[dev] = true;
             }
-            CLD_K(K_CSR, s, k_emit_canon<<<grid_for(m, 256, 4), 256, esm, s>>>(
-                                (const uint32_t*)dsrc, (const uint32_t*)ddst, (const uint32_t*)dw, m, n, vb, wb, items.get(),
-                                scal.get(), scal.get() + 2, hist1.get()));
+            const auto emit = pairs ? k_emit_canon<true> : k_emit_canon<false>;
+            CLD_K(K_CSR, s, emit<<<grid_for(m, 256, 4), 256, esm, s>>>(
+                                (const uint32_t*)dsrc, (const uint32_t*)ddst, (const uint32_t*)dw, m, n, vb,
+                                pairs ? 0 : wfit, items.get(), vals.get(), scal.get(), scal.get() + 2, hist1.get()));
             CLD_LAUNCH_CHECK();
         }
         CLD_CUDA(cudaMemcpyAsync(hbad, scal.get(), 3 * sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
         CLD_CUDA(cudaStreamSynchronize(s));
         if (hbad[0]) return fail(CLDIAM_ERR_INVALID_ARG, "edge with node id >= n or weight 0");
-        packed = hbad[2] == 0;
-        if (packed) {
-            CLD_TRY(items2.alloc(m ? m : 1, s));
-            CLD_TRY(uniq.alloc(m ? m : 1, s));
-            bool alt = false;
-            CLD_TRY(radix_sort_keys_u64(items.get(), items2.get(), m, wb, 2 * vb, &alt, s, scal.get() + 8, nullptr,
-                                        hist1.get()));
-            const int npass2 = (vb + 7) / 8;
-            CLD_TRY(hist2.alloc((size_t)npass2 * 256, s));
-            CLD_CUDA(cudaMemsetAsync(hist2.get(), 0, (size_t)npass2 * 256 * 4, s));
-            // every row's run bounds in both orders; the de-duplication writes the first order's
-            CLD_TRY(runs.alloc(4 * (size_t)n, s));
-            CLD_CUDA(cudaMemsetAsync(runs.get(), 0, 4 * (size_t)n * 4, s));
-            CLD_TRY(unique_items_u64(alt ? items2.get() : items.get(), m, vb, uniq.get(), scal.get() + 1, s, hist2.get(),
-                                     runs.get(), runs.get() + n));
-            CLD_CUDA(cudaMemcpyAsync(hbad + 1, scal.get() + 1, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
-            CLD_CUDA(cudaStreamSynchronize(s));
-            mu = hbad[1];  // distinct undirected edges
-            bool alt2 = false;
-            CLD_TRY(radix_sort_keys_u64(items.get(), items2.get(), mu, wb, vb, &alt2, s, scal.get() + 8, uniq.get(),
-                                        hist2.get()));
-            la.U = uniq.get();
-            la.T = alt2 ? items2.get() : items.get();
-            la.ustart = runs.get();
-            la.uend = runs.get() + n;
-            la.tstart = runs.get() + 2 * (size_t)n;
-            la.tend = runs.get() + 3 * (size_t)n;
-            la.ash = 64 - vb;
-            la.wb = wb;
-            la.cmask = vb >= 32 ? 0xFFFFFFFFu : ((1u << vb) - 1u);
-            uint32_t* r0 = runs.get();
-            if (mu > 0) {
-                CLD_K(K_CSR, s, k_canon_runs<<<grid_for(mu, 256), 256, 0, s>>>(la.T, mu, vb, wb, r0 + 2 * (size_t)n,
-                                                                              r0 + 3 * (size_t)n, scal.get() + 1));
-                CLD_LAUNCH_CHECK();
-            }
-            if (!lcc) {
-                // the whole graph's CSR: row x = its lower entries, then its upper entries
-                CLD_TRY(alloc_full());
-                DBuf<uint64_t> degs;
-                CLD_TRY(degs.alloc(n, s));
-                CLD_K(K_CSR, s, k_canon_deg<<<grid_for(n, 256), 256, 0, s>>>(n, la.ustart, la.uend, la.tstart, la.tend,
-                                                                            degs.get()));
-                CLD_LAUNCH_CHECK();
-                CLD_TRY(scan_exclusive_u64(degs.get(), off.get(), n, off.get() + n, s));
-                if (mu > 0) {
-                    CLD_K(K_CSR, s, k_canon_scatter<<<grid_for(mu, 256), 256, 0, s>>>(la.U, la.T, mu, vb, wb, la.ustart,
-                                                                                     la.tstart, la.tend, off.get(),
-                                                                                     row.get(), adj.get(),
-                                                                                     scal.get() + 8));
-                    CLD_LAUNCH_CHECK();
-                }
-            }
-        }
+        if (pairs || hbad[2] == 0) break;
+        pairs = true;
     }
-    if (!packed) {
-        // keys u*n + v (u != v) are at most n^2 - 2; n^2 - 1 marks a dropped self-loop
-        CLD_TRY(alloc_full());
-        CLD_CUDA(cudaMemsetAsync(adj.get(), 0xFF, (size_t)(cnt ? cnt : 1) * 8, s));  // run minima fold in
-        const uint64_t sentinel = (uint64_t)n * (uint64_t)n - 1;
-        DBuf<uint64_t> keys, keys2;
-        DBuf<uint32_t> vals, vals2;
-        CLD_TRY(keys.alloc(cnt ? cnt : 1, s));
-        CLD_TRY(keys2.alloc(cnt ? cnt : 1, s));
-        CLD_TRY(vals.alloc(cnt ? cnt : 1, s));
-        CLD_TRY(vals2.alloc(cnt ? cnt : 1, s));
-        if (m > 0) {
-            CLD_K(K_CSR, s, k_emit_directed<<<grid_for(m, 256), 256, 0, s>>>((const uint32_t*)dsrc,
-                                                                            (const uint32_t*)ddst, (const uint32_t*)dw,
-                                                                            m, n, sentinel, keys.get(), vals.get(),
-                                                                            scal.get()));
+    const int wb = pairs ? 0 : wfit;
+    CLD_TRY(items2.alloc(m ? m : 1, s));
+    CLD_TRY(uniq.alloc(m ? m : 1, s));
+    bool alt = false;
+    if (pairs) {
+        CLD_TRY(vals2.alloc(m ? m : 1, s));
+        CLD_TRY(uniqw.alloc(m ? m : 1, s));
+        CLD_TRY(radix_sort_pairs_u64(items.get(), vals.get(), items2.get(), vals2.get(), m, 2 * vb, &alt, s,
+                                     scal.get() + 8, nullptr, nullptr, hist1.get()));
+    } else {
+        CLD_TRY(radix_sort_keys_u64(items.get(), items2.get(), m, wb, 2 * vb, &alt, s, scal.get() + 8, nullptr,
+                                    hist1.get()));
+    }
+    const int npass2 = (vb + 7) / 8;
+    CLD_TRY(hist2.alloc((size_t)npass2 * 256, s));
+    CLD_CUDA(cudaMemsetAsync(hist2.get(), 0, (size_t)npass2 * 256 * 4, s));
+    // every row's run bounds in both orders; the de-duplication writes the first order's
+    CLD_TRY(runs.alloc(4 * (size_t)n, s));
+    CLD_CUDA(cudaMemsetAsync(runs.get(), 0, 4 * (size_t)n * 4, s));
+    CLD_TRY(unique_items_u64(alt ? items2.get() : items.get(), pairs ? (alt ? vals2.get() : vals.get()) : nullptr, m, vb,
+                             uniq.get(), uniqw.get(), scal.get() + 1, s, hist2.get(), runs.get(), runs.get() + n));
+    CLD_CUDA(cudaMemcpyAsync(hbad + 1, scal.get() + 1, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+    CLD_CUDA(cudaStreamSynchronize(s));
+    mu = hbad[1];  // distinct undirected edges
+    bool alt2 = false;
+    if (pairs)
+        CLD_TRY(radix_sort_pairs_u64(items.get(), vals.get(), items2.get(), vals2.get(), mu, vb, &alt2, s,
+                                     scal.get() + 8, uniq.get(), uniqw.get(), hist2.get()));
+    else
+        CLD_TRY(radix_sort_keys_u64(items.get(), items2.get(), mu, wb, vb, &alt2, s, scal.get() + 8, uniq.get(),
+                                    hist2.get()));
+    la.U = uniq.get();
+    la.T = alt2 ? items2.get() : items.get();
+    la.UW = pairs ? uniqw.get() : nullptr;
+    la.TW = pairs ? (alt2 ? vals2.get() : vals.get()) : nullptr;
+    la.ustart = runs.get();
+    la.uend = runs.get() + n;
+    la.tstart = runs.get() + 2 * (size_t)n;
+    la.tend = runs.get() + 3 * (size_t)n;
+    la.ash = vb + wb;
+    la.wb = wb;
+    la.cmask = vb >= 32 ? 0xFFFFFFFFu : ((1u << vb) - 1u);
+    if (mu > 0) {
+        uint32_t* r0 = runs.get();
+        CLD_K(K_CSR, s, k_canon_runs<<<grid_for(mu, 256), 256, 0, s>>>(la.T, mu, vb, wb, r0 + 2 * (size_t)n,
+                                                                      r0 + 3 * (size_t)n, scal.get() + 1));
+        CLD_LAUNCH_CHECK();
+    }
+    if (!lcc) {
+        // the whole graph's CSR: row x = its lower entries, then its upper entries
+        CLD_TRY(row.alloc(cnt ? cnt : 1, s));
+        CLD_TRY(adj.alloc(cnt ? cnt : 1, s));
+        CLD_TRY(off.alloc((size_t)n + 1, s));
+        DBuf<uint64_t> degs;
+        CLD_TRY(degs.alloc(n, s));
+        CLD_K(K_CSR, s, k_canon_deg<<<grid_for(n, 256), 256, 0, s>>>(n, la.ustart, la.uend, la.tstart, la.tend,
+                                                                    degs.get()));
+        CLD_LAUNCH_CHECK();
+        CLD_TRY(scan_exclusive_u64(degs.get(), off.get(), n, off.get() + n, s));
+        if (mu > 0) {
+            CLD_K(K_CSR, s, k_canon_scatter<<<grid_for(mu, 256), 256, 0, s>>>(la, mu, off.get(), row.get(), adj.get(),
+                                                                             scal.get() + 8));
             CLD_LAUNCH_CHECK();
         }
-        CLD_CUDA(cudaMemcpyAsync(hbad, scal.get(), sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
-        CLD_CUDA(cudaStreamSynchronize(s));
-        if (hbad[0]) return fail(CLDIAM_ERR_INVALID_ARG, "edge with node id >= n or weight 0");
-        bool alt = false;
-        CLD_TRY(radix_sort_pairs_u64(keys.get(), vals.get(), keys2.get(), vals2.get(), cnt, bits_for(sentinel), &alt,
-                                     s));
-        CLD_TRY(unique_min_sorted_u64(alt ? keys2.get() : keys.get(), alt ? vals2.get() : vals.get(), cnt, sentinel, n,
-                                      row.get(), &adj.get()->x, &adj.get()->y, 2, off.get(), n, scal.get() + 1, s));
     }
     // (the entry count stays on the device until the host needs it, read together with the next result)
     uint32_t nnz = 0;
@@ -742,7 +655,6 @@ cldiam_status build_csr(const uint32_t* src, const uint32_t* dst, const uint32_t
         CLD_TRY(best.alloc(1, s));
         CLD_K(K_MISC, s, k_iota<<<grid_for(n, 256), 256, 0, s>>>(parent.get(), n));
         CLD_LAUNCH_CHECK();
-        const CsrAdj ca{off.get(), adj.get()};
         // Afforest-style: link two neighbours per node, find the dominant tree by sampling,
         // then link the remaining edges of the nodes outside it (all no-ops on a graph without edges)
         constexpr uint32_t kNeighbourRounds = 2;
@@ -750,8 +662,7 @@ cldiam_status build_csr(const uint32_t* src, const uint32_t* dst, const uint32_t
         for (uint32_t r = 0; r < kNeighbourRounds; ++r) {
             const uint32_t first = split && r > 0 ? 1 : 0, last = split && r > 0 ? 2 : 0;
             for (uint32_t part = first; part <= last; ++part) {
-                if (packed) CLD_K(K_CC, s, k_cc_link_nth<<<grid_for(n, 256), 256, 0, s>>>(la, n, r, part, parent.get()));
-                else CLD_K(K_CC, s, k_cc_link_nth<<<grid_for(n, 256), 256, 0, s>>>(ca, n, r, part, parent.get()));
+                CLD_K(K_CC, s, k_cc_link_nth<<<grid_for(n, 256), 256, 0, s>>>(la, n, r, part, parent.get()));
                 CLD_K(K_CC, s, k_cc_compress<<<grid_for(n, 256), 256, 0, s>>>(parent.get(), n));
             }
         }
@@ -778,12 +689,8 @@ cldiam_status build_csr(const uint32_t* src, const uint32_t* dst, const uint32_t
                 if (j - i > best_run) { best_run = (uint32_t)(j - i); giant = hs[i]; }
                 i = j;
             }
-            if (packed)
-                CLD_K(K_CC, s, k_cc_link_rest<<<grid_for(n, 256), 256, 0, s>>>(la, n, kNeighbourRounds, giant,
-                                                                                parent.get()));
-            else
-                CLD_K(K_CC, s, k_cc_link_rest<<<grid_for(n, 256), 256, 0, s>>>(ca, n, kNeighbourRounds, giant,
-                                                                                parent.get()));
+            CLD_K(K_CC, s, k_cc_link_rest<<<grid_for(n, 256), 256, 0, s>>>(la, n, kNeighbourRounds, giant,
+                                                                            parent.get()));
             CLD_K(K_CC, s, k_cc_compress<<<grid_for(n, 256), 256, 0, s>>>(parent.get(), n));
             CLD_LAUNCH_CHECK();
             CLD_CUDA(cudaMemsetAsync(scal.get() + 3, 0, 4, s));
@@ -805,60 +712,42 @@ cldiam_status build_csr(const uint32_t* src, const uint32_t* dst, const uint32_t
         CLD_TRY(newid.alloc(n, s));
         CLD_K(K_CC, s, k_cc_keep<<<grid_for(n, 256), 256, 0, s>>>(parent.get(), n, best.get(), keep.get()));
         CLD_LAUNCH_CHECK();
+        parent.release();
+        size.release();
         CLD_TRY(scan_exclusive_u32(keep.get(), newid.get(), n, scal.get() + 4, s));
         // the LCC's node and entry counts stay on the device: its arrays are sized by the bounds n and
         // nnz, and the kernels read the counts from scal[4] / scal[5]
         CLD_TRY(orig.alloc(n, s));
+        CLD_TRY(deg.alloc((size_t)n + 1, s));
+        CLD_TRY(degx.alloc((size_t)n + 1, s));
         CLD_CUDA(cudaMemsetAsync(deg.get(), 0, ((size_t)n + 1) * 4, s));
-        if (packed)
-            CLD_K(K_CSR, s, k_lcc_degrees<<<grid_for(n, 256), 256, 0, s>>>(keep.get(), newid.get(), la, n, deg.get(),
-                                                                          orig.get()));
-        else
-            CLD_K(K_CSR, s, k_lcc_degrees<<<grid_for(n, 256), 256, 0, s>>>(keep.get(), newid.get(), ca, n, deg.get(),
-                                                                          orig.get()));
+        CLD_K(K_CSR, s, k_lcc_degrees<<<grid_for(n, 256), 256, 0, s>>>(keep.get(), newid.get(), la, n, deg.get(),
+                                                                      orig.get()));
         CLD_LAUNCH_CHECK();
+        keep.release();
         CLD_TRY(scan_exclusive_u32(deg.get(), degx.get(), n, scal.get() + 5, s));  // zeros past the kept nodes
+        deg.release();  // (the largest node counts fit beside the records below: 52 bytes a node at most)
         DBuf<uint64_t> noff;
         DBuf<uint2> nadj;
-        DBuf<uint32_t> nrow;
         CLD_TRY(noff.alloc((size_t)n + 1, s));
         CLD_TRY(nadj.alloc(nnz ? nnz : 1, s));
-        // the row of every entry (COO form) is written only by the (key, weight) copy; a CSR assembled from the
-        // lists leaves it out (its users build it from the offsets when they need it: fill_rows)
-        if (!packed) CLD_TRY(nrow.alloc(nnz ? nnz : 1, s));
-        if (packed) {
-            // the LCC's CSR straight from the lists: the whole graph's CSR is never built
-            DBuf<uint4> info;
-            CLD_TRY(info.alloc(n, s));
-            CLD_CUDA(cudaMemsetAsync(info.get(), 0xFF, (size_t)n * 16, s));
-            CLD_K(K_CSR, s, k_lcc_offsets_lists<<<grid_for((size_t)n + 1, 256), 256, 0, s>>>(
-                                degx.get(), scal.get() + 4, scal.get() + 5, orig.get(), la, noff.get(), info.get()));
+        // the LCC's CSR straight from the lists: the whole graph's CSR is never built, and the row of every entry
+        // (COO form) is left out (its users build it from the offsets when they need it: fill_rows)
+        DBuf<uint4> info;
+        CLD_TRY(info.alloc(n, s));
+        CLD_CUDA(cudaMemsetAsync(info.get(), 0xFF, (size_t)n * 16, s));
+        CLD_K(K_CSR, s, k_lcc_offsets_lists<<<grid_for((size_t)n + 1, 256), 256, 0, s>>>(
+                            degx.get(), scal.get() + 4, scal.get() + 5, orig.get(), la, noff.get(), info.get()));
+        CLD_LAUNCH_CHECK();
+        if (mu > 0) {
+            const auto assemble = pairs ? k_lcc_assemble<true> : k_lcc_assemble<false>;
+            CLD_K(K_CSR, s, assemble<<<grid_for(mu, 256, 4), 256, 0, s>>>(la, mu, info.get(), newid.get(), nnz ? nnz : 1,
+                                                                         nadj.get(), wsum.get(), scal.get() + 6,
+                                                                         scal.get() + 8));
             CLD_LAUNCH_CHECK();
-            if (mu > 0) {
-                CLD_K(K_CSR, s, k_lcc_assemble<<<grid_for(mu, 256, 4), 256, 0, s>>>(la, mu, info.get(), newid.get(),
-                                                                                nnz ? nnz : 1, nadj.get(),
-                                                                                wsum.get(), scal.get() + 6,
-                                                                                scal.get() + 8));
-                CLD_LAUNCH_CHECK();
-            }
-        } else {
-            DBuf<uint2> map;
-            CLD_TRY(map.alloc(n, s));
-            CLD_CUDA(cudaMemsetAsync(map.get(), 0xFF, (size_t)n * 8, s));
-            CLD_K(K_CSR, s, k_lcc_offsets<<<grid_for((size_t)n + 1, 256), 256, 0, s>>>(degx.get(), n, scal.get() + 4,
-                                                                                    scal.get() + 5, orig.get(),
-                                                                                    off.get(), noff.get(), map.get()));
-            CLD_LAUNCH_CHECK();
-            if (nnz) {
-                CLD_K(K_CSR, s, k_lcc_copy<<<grid_for(nnz, 256), 256, 0, s>>>(map.get(), newid.get(), row.get(),
-                                                                             adj.get(), nnz, nrow.get(), nadj.get(),
-                                                                             wsum.get(), scal.get() + 6));
-                CLD_LAUNCH_CHECK();
-            }
         }
         g->off = noff.detach();
         g->adj = nadj.detach();
-        g->row = nrow.detach();
         CLD_K(K_CSR, s, k_degree_max<<<grid_for(n, 256), 256, 0, s>>>(g->off, n, scal.get() + 4, scal.get() + 7));
         CLD_LAUNCH_CHECK();
     } else {

@@ -569,10 +569,12 @@ __global__ void __launch_bounds__(OsCfg<K, KV, BIG>::THREADS, 1024 / OsCfg<K, KV
 template <class K>
 static cldiam_status radix_sort_impl(K* keys, uint32_t* vals, K* keys_alt, uint32_t* vals_alt, size_t n, int shift0,
                                      int bits, bool* in_alt, cudaStream_t s, uint32_t* err_dev = nullptr,
-                                     const K* first_in = nullptr, uint32_t* hist_in = nullptr) {
+                                     const K* first_in = nullptr, uint32_t* hist_in = nullptr,
+                                     const uint32_t* first_vin = nullptr) {
     *in_alt = false;
     if (n <= 1 || bits <= 0) {
         if (first_in && n) CLD_CUDA(cudaMemcpyAsync(keys, first_in, n * sizeof(K), cudaMemcpyDeviceToDevice, s));
+        if (first_vin && n) CLD_CUDA(cudaMemcpyAsync(vals, first_vin, n * 4, cudaMemcpyDeviceToDevice, s));
         return CLDIAM_OK;
     }
     if (n > 0xFFFFFFFFull) return fail(CLDIAM_ERR_UNSUPPORTED, "radix sort limited to 2^32 - 1 items");
@@ -622,9 +624,9 @@ static cldiam_status radix_sort_impl(K* keys, uint32_t* vals, K* keys_alt, uint3
     }
     CLD_K(K_RADIX_HIST, s, k_os_hist_scan<<<1, OS_RADIX, 0, s>>>(hist, npass));
     CLD_LAUNCH_CHECK();
-    // first_in (keys only): the first pass reads it and writes keys_alt, so first_in is never written
+    // first_in / first_vin: the first pass reads them and writes keys_alt / vals_alt, so they are never written
     const K* ki = first_in ? first_in : keys;
-    uint32_t* vi = vals;
+    const uint32_t* vi = first_vin ? first_vin : vals;
     K* ko = keys_alt;
     uint32_t* vo = vals_alt;
     bool alt = false;
@@ -642,10 +644,10 @@ static cldiam_status radix_sort_impl(K* keys, uint32_t* vals, K* keys_alt, uint3
         CLD_LAUNCH_CHECK();
         // algorithmic bytes: every item (key and value) read once and written once
         prof_add_bytes(K_RADIX_SCATTER, 2.0 * (double)n * (sizeof(K) + (kv ? sizeof(uint32_t) : 0)));
-        const K* done_in = ki;
         ki = ko;
-        ko = (first_in && p == 0) ? keys : const_cast<K*>(done_in);  // first_in is never written
-        uint32_t* tv = vi; vi = vo; vo = tv;
+        ko = alt ? keys_alt : keys;
+        vi = vo;
+        vo = alt ? vals_alt : vals;
         alt = !alt;
     }
     *in_alt = alt;
@@ -666,10 +668,9 @@ static cldiam_status radix_sort_impl(K* keys, uint32_t* vals, K* keys_alt, uint3
 // (With one atomicMin per item, runs of millions of equal keys -- the cluster
 // pairs of a power-law graph's quotient -- queue at one address: the 521M items
 // of R-MAT 24 took 202 ms; the whole quotient by sort went from 225 to 20-24 ms.)
-// Output per unique key: row_out[r] = key / div (if row_out), col_out[r*cs] =
-// key % div, w_out[r*cs] = min value (w_out pre-filled with 0xFFFFFFFF).
-// Keys >= sentinel are ignored (they sort last).
-// With off_out, the run heads also write the CSR offsets of rows
+// Output per unique key: col_out[r] = key % div, w_out[r] = min value (w_out
+// pre-filled with 0xFFFFFFFF).  Keys >= sentinel are ignored (they sort last).
+// The run heads also write the CSR offsets of rows
 // 0..nrows: off_out[q] = index of the first unique key with row >= q (a head
 // fills the rows after its predecessor's row up to its own; the last run
 // fills the rows after it with the total).
@@ -707,13 +708,15 @@ __global__ void __launch_bounds__(UQ_THREADS) k_unique_count(const K* __restrict
     }
 }
 
-// second pass: tile t's heads get indices from first[t] on
-template <class K>
+// second pass: tile t's heads get indices from first[t] on.  LIST: the keys are edges row << vb | col of a list
+// that stays one (key_out), with the run bounds ustart / uend of its rows; otherwise they are row * div + col and
+// become a CSR (col_out, off_out).
+template <class K, bool LIST>
 __global__ void __launch_bounds__(UQ_THREADS, 4)
     k_unique_write(const K* __restrict__ keys, const uint32_t* __restrict__ vals, size_t cnt, K sentinel,
-                   uint64_t div, uint32_t* __restrict__ row_out, uint32_t* __restrict__ col_out,
-                   uint32_t* __restrict__ w_out, int cs, uint64_t* __restrict__ off_out, uint32_t nrows,
-                   const uint32_t* __restrict__ first) {
+                   uint64_t div, uint32_t* __restrict__ col_out, uint32_t* __restrict__ w_out,
+                   uint64_t* __restrict__ off_out, uint32_t nrows, const uint32_t* __restrict__ first, int vb,
+                   K* __restrict__ key_out, uint32_t* __restrict__ ustart, uint32_t* __restrict__ uend) {
     __shared__ uint32_t s_woff[UQ_THREADS / 32], s_prefix;
     const unsigned tid = threadIdx.x, w = tid >> 5, l = lane_id();
     const uint32_t tile = blockIdx.x;
@@ -758,7 +761,7 @@ __global__ void __launch_bounds__(UQ_THREADS, 4)
     // carried from one group of 32 to the next) before anything is written: a run that begins and ends in
     // the warp is one plain store, a run shared with other warps one atomicMin per warp (w_out holds
     // 0xFFFFFFFF beforehand).
-    const auto row_of = [&](K kk) -> uint64_t { return (uint64_t)kk / div; };
+    const auto row_of = [&](K kk) -> uint64_t { return LIST ? (uint64_t)kk >> vb : (uint64_t)kk / div; };
     const K wnext = base + UQ_ITEMS * 32 < cnt ? keys[base + UQ_ITEMS * 32] : sentinel;  // item after the warp's
     const K wlast = __shfl_sync(0xffffffffu, key[UQ_ITEMS - 1], 31);
     const bool goes_on = wnext < sentinel && wnext == wlast;  // the warp's last run continues in the next warp
@@ -797,35 +800,44 @@ __global__ void __launch_bounds__(UQ_THREADS, 4)
         if (start && !(i + 1 < UQ_ITEMS && cont && l == last)) {
             const uint32_t r = tbase + ex[i] + (f ? 0u : 0xFFFFFFFFu);  // a piece without its head: the run before
             const bool whole = (f || carry_head) && !(i + 1 == UQ_ITEMS && cont && l == last);
-            if (whole) w_out[(size_t)r * cs] = v;
-            else atomicMin(&w_out[(size_t)r * cs], v);
+            if (whole) w_out[r] = v;
+            else atomicMin(&w_out[r], v);
         }
         carry_head = cont && (word != 0 || carry_head);
         carry = cont ? vlast : 0xFFFFFFFFu;
+        if constexpr (LIST) {
+            if (valid && f) {
+                const uint32_t r = tbase + ex[i];
+                key_out[r] = key[i];
+                // an edge whose row differs from the previous one's starts its row's run and ends the previous
+                // row's (the last row's end is set after the pass)
+                if (idx == 0 || row_of(before) != row_of(key[i])) {
+                    ustart[row_of(key[i])] = r;
+                    if (r > 0) uend[row_of(before)] = r;
+                }
+            }
+            continue;
+        }
         if (valid && f) {
             const uint32_t r = tbase + ex[i];
             const uint64_t q = row_of(key[i]);
-            if (row_out) row_out[r] = (uint32_t)q;
-            col_out[(size_t)r * cs] = (uint32_t)((uint64_t)key[i] - q * div);
-            if (off_out) {
-                const uint64_t q0 = idx == 0 ? 0ull : row_of(before) + 1ull;  // rows after the previous run's row
-                for (uint64_t qq = q0; qq <= q && qq <= nrows; ++qq) off_out[qq] = r;
-            }
+            col_out[r] = (uint32_t)((uint64_t)key[i] - q * div);
+            const uint64_t q0 = idx == 0 ? 0ull : row_of(before) + 1ull;  // rows after the previous run's row
+            for (uint64_t qq = q0; qq <= q && qq <= nrows; ++qq) off_out[qq] = r;
         }
         // the last run: the remaining rows end at the total
-        if (off_out && valid && !(after < sentinel))
+        if (valid && !(after < sentinel))
             for (uint64_t qq = row_of(key[i]) + 1; qq <= nrows; ++qq) off_out[qq] = (uint64_t)(tbase + ex[i] + (f ? 1u : 0u));
     }
 }
 
 template <class K>
 static cldiam_status unique_min_sorted(const K* keys, const uint32_t* vals, size_t cnt, K sentinel,
-                                       uint64_t div, uint32_t* row_out, uint32_t* col_out,
-                                       uint32_t* w_out, int cs, uint64_t* off_out, uint32_t nrows,
-                                       uint32_t* total_dev, cudaStream_t s) {
+                                       uint64_t div, uint32_t* col_out, uint32_t* w_out, uint64_t* off_out,
+                                       uint32_t nrows, uint32_t* total_dev, cudaStream_t s) {
     if (cnt == 0) {
         CLD_CUDA(cudaMemsetAsync(total_dev, 0, 4, s));
-        if (off_out) CLD_CUDA(cudaMemsetAsync(off_out, 0, ((size_t)nrows + 1) * 8, s));
+        CLD_CUDA(cudaMemsetAsync(off_out, 0, ((size_t)nrows + 1) * 8, s));
         return CLDIAM_OK;
     }
     if (cnt > 0xFFFFFFFFull) return fail(CLDIAM_ERR_UNSUPPORTED, "more than 2^32 - 1 items");
@@ -836,14 +848,14 @@ static cldiam_status unique_min_sorted(const K* keys, const uint32_t* vals, size
     CLD_K(K_CSR, s, k_unique_count<K><<<ntiles, UQ_THREADS, 0, s>>>(keys, cnt, sentinel, heads.get()));
     CLD_LAUNCH_CHECK();
     CLD_TRY(scan_exclusive_u32(heads.get(), first.get(), ntiles, total_dev, s));
-    CLD_K(K_CSR, s, k_unique_write<K><<<ntiles, UQ_THREADS, 0, s>>>(keys, vals, cnt, sentinel, div,
-                                                                     row_out, col_out, w_out, cs, off_out, nrows,
-                                                                     first.get()));
+    CLD_K(K_CSR, s, k_unique_write<K, false><<<ntiles, UQ_THREADS, 0, s>>>(keys, vals, cnt, sentinel, div, col_out,
+                                                                           w_out, off_out, nrows, first.get(), 0,
+                                                                           nullptr, nullptr, nullptr));
     CLD_LAUNCH_CHECK();
     uint32_t total = 0;
     CLD_CUDA(cudaMemcpyAsync(&total, total_dev, 4, cudaMemcpyDeviceToHost, s));
     CLD_CUDA(cudaStreamSynchronize(s));
-    if (off_out && total == 0) CLD_CUDA(cudaMemsetAsync(off_out, 0, ((size_t)nrows + 1) * 8, s));  // no valid key
+    if (total == 0) CLD_CUDA(cudaMemsetAsync(off_out, 0, ((size_t)nrows + 1) * 8, s));  // no valid key
     return CLDIAM_OK;
 }
 
@@ -867,12 +879,12 @@ __device__ __forceinline__ bool up_head(uint64_t prev, uint64_t x, uint64_t same
 // b digits are counted too, into per-warp shared histograms (dynamic, warps x npass x 256 words)
 // flushed once per CTA.
 __global__ void __launch_bounds__(UP_THREADS) k_unique_packed_count(const uint64_t* __restrict__ items, uint32_t cnt,
-                                                                    int vb, uint32_t ntiles, uint32_t* __restrict__ heads,
+                                                                    int vb, int wb, uint32_t ntiles,
+                                                                    uint32_t* __restrict__ heads,
                                                                     uint32_t* __restrict__ hist2) {
     extern __shared__ uint32_t uh[];
     __shared__ uint32_t s_w[UP_WARPS];
     const unsigned tid = threadIdx.x, w = tid >> 5, l = lane_id();
-    const int wb = 64 - 2 * vb;
     const int npass = (vb + 7) / 8;
     if (hist2) {
         for (int i = tid; i < UP_WARPS * npass * 256; i += UP_THREADS) uh[i] = 0;
@@ -1037,47 +1049,56 @@ __global__ void k_last_uend(const uint64_t* __restrict__ out, const uint32_t* __
     if (t > 0) uend[(uint32_t)(out[t - 1] >> shift)] = t;
 }
 
-cldiam_status unique_items_u64(const uint64_t* items, size_t cnt, int vb, uint64_t* out, uint32_t* total_dev,
-                               cudaStream_t s, uint32_t* hist2, uint32_t* ustart, uint32_t* uend) {
+cldiam_status unique_items_u64(const uint64_t* items, const uint32_t* vals, size_t cnt, int vb, uint64_t* out,
+                               uint32_t* w_out, uint32_t* total_dev, cudaStream_t s, uint32_t* hist2, uint32_t* ustart,
+                               uint32_t* uend) {
     if (cnt == 0) {
         CLD_CUDA(cudaMemsetAsync(total_dev, 0, 4, s));
         return CLDIAM_OK;
     }
     if (cnt > 0xFFFFFFFFull - UP_TILE) return fail(CLDIAM_ERR_UNSUPPORTED, "too many items");
     if (vb < 1 || vb > 32) return fail(CLDIAM_ERR_INVALID_ARG, "packed items need 1..32 id bits");
+    static_assert(UP_TILE == UQ_TILE, "one tile for both forms");
+    const int wb = vals ? 0 : 64 - 2 * vb;
     const uint32_t ntiles = (uint32_t)((cnt + UP_TILE - 1) / UP_TILE);
     DBuf<uint32_t> heads, first;
     CLD_TRY(heads.alloc(ntiles, s));
     CLD_TRY(first.alloc(ntiles, s));
-    const size_t usm = hist2 ? (size_t)UP_WARPS * ((vb + 7) / 8) * 256 * 4 : 0;  // <= 32 KB
+    const size_t usm = (size_t)UP_WARPS * ((vb + 7) / 8) * 256 * 4;  // <= 32 KB
     CLD_K(K_CSR, s, k_unique_packed_count<<<grid_for((size_t)ntiles * UP_THREADS, UP_THREADS, 4), UP_THREADS, usm, s>>>(
-                        items, (uint32_t)cnt, vb, ntiles, heads.get(), hist2));
+                        items, (uint32_t)cnt, vb, wb, ntiles, heads.get(), hist2));
     CLD_LAUNCH_CHECK();
-    CLD_TRY(scan_exclusive_u32(heads.get(), first.get(), ntiles, nullptr, s));
-    CLD_K(K_CSR, s, k_unique_items<<<ntiles, UP_THREADS, 0, s>>>(items, (uint32_t)cnt, vb,
-                                                                 reinterpret_cast<unsigned long long*>(out), total_dev,
-                                                                 first.get(), ustart, uend));
-    if (ustart) CLD_K(K_CSR, s, k_last_uend<<<1, 1, 0, s>>>(out, total_dev, 64 - vb, uend));
+    CLD_TRY(scan_exclusive_u32(heads.get(), first.get(), ntiles, vals ? total_dev : nullptr, s));
+    if (vals) {
+        CLD_CUDA(cudaMemsetAsync(w_out, 0xFF, cnt * 4, s));
+        CLD_K(K_CSR, s, k_unique_write<uint64_t, true><<<ntiles, UQ_THREADS, 0, s>>>(
+                            items, vals, cnt, ~0ull, 0, nullptr, w_out, nullptr, 0, first.get(), vb, out, ustart, uend));
+    } else {
+        CLD_K(K_CSR, s, k_unique_items<<<ntiles, UP_THREADS, 0, s>>>(items, (uint32_t)cnt, vb,
+                                                                     reinterpret_cast<unsigned long long*>(out),
+                                                                     total_dev, first.get(), ustart, uend));
+    }
+    CLD_K(K_CSR, s, k_last_uend<<<1, 1, 0, s>>>(out, total_dev, vb + wb, uend));
     CLD_LAUNCH_CHECK();
     return CLDIAM_OK;
 }
 
 cldiam_status unique_min_sorted_u64(const uint64_t* keys, const uint32_t* vals, size_t cnt, uint64_t sentinel,
-                                    uint64_t div, uint32_t* row_out, uint32_t* col_out, uint32_t* w_out, int cs,
-                                    uint64_t* off_out, uint32_t nrows, uint32_t* total_dev, cudaStream_t s) {
-    return unique_min_sorted<uint64_t>(keys, vals, cnt, sentinel, div, row_out, col_out, w_out, cs, off_out,
-                                       nrows, total_dev, s);
+                                    uint64_t div, uint32_t* col_out, uint32_t* w_out, uint64_t* off_out,
+                                    uint32_t nrows, uint32_t* total_dev, cudaStream_t s) {
+    return unique_min_sorted<uint64_t>(keys, vals, cnt, sentinel, div, col_out, w_out, off_out, nrows, total_dev, s);
 }
 cldiam_status unique_min_sorted_u32(const uint32_t* keys, const uint32_t* vals, size_t cnt, uint32_t sentinel,
-                                    uint64_t div, uint32_t* row_out, uint32_t* col_out, uint32_t* w_out, int cs,
-                                    uint64_t* off_out, uint32_t nrows, uint32_t* total_dev, cudaStream_t s) {
-    return unique_min_sorted<uint32_t>(keys, vals, cnt, sentinel, div, row_out, col_out, w_out, cs, off_out,
-                                       nrows, total_dev, s);
+                                    uint64_t div, uint32_t* col_out, uint32_t* w_out, uint64_t* off_out,
+                                    uint32_t nrows, uint32_t* total_dev, cudaStream_t s) {
+    return unique_min_sorted<uint32_t>(keys, vals, cnt, sentinel, div, col_out, w_out, off_out, nrows, total_dev, s);
 }
 
 cldiam_status radix_sort_pairs_u64(uint64_t* keys, uint32_t* vals, uint64_t* keys_alt, uint32_t* vals_alt,
-                                   size_t n, int bits, bool* in_alt, cudaStream_t s) {
-    return radix_sort_impl<uint64_t>(keys, vals, keys_alt, vals_alt, n, 0, bits, in_alt, s);
+                                   size_t n, int bits, bool* in_alt, cudaStream_t s, uint32_t* err_dev,
+                                   const uint64_t* first_in, const uint32_t* first_vin, uint32_t* hist_in) {
+    return radix_sort_impl<uint64_t>(keys, vals, keys_alt, vals_alt, n, 0, bits, in_alt, s, err_dev, first_in, hist_in,
+                                     first_vin);
 }
 cldiam_status radix_sort_keys_u64(uint64_t* keys, uint64_t* keys_alt, size_t n, int shift0, int bits, bool* in_alt,
                                   cudaStream_t s, uint32_t* err_dev, const uint64_t* first_in, uint32_t* hist_in) {
@@ -1096,7 +1117,7 @@ cldiam_status load_prims_kernels() {
                         k_os_pass<uint64_t, true, false, false>, k_os_pass<uint64_t, true, true, false>,
                         k_os_pass<uint32_t, true, false, true>, k_os_pass<uint64_t, true, false, true>,
                         k_os_pass<uint64_t, true, true, true>, k_unique_count<uint32_t>,
-                        k_unique_count<uint64_t>, k_unique_write<uint32_t>, k_unique_write<uint64_t>);
+                        k_unique_count<uint64_t>, k_unique_write<uint32_t, false>, k_unique_write<uint64_t, false>);
 }
 
 }  // namespace cld

@@ -350,10 +350,10 @@ cldiam_status build_quotient(const cldiam_clustering* c, cldiam_quotient* q) {
     CLD_TRY(off.alloc((size_t)k + 1, s));
     CLD_CUDA(cudaMemsetAsync(w.get(), 0xFF, (size_t)(cnt ? cnt : 1) * 4, s));
     if (sizeof(K) == 8)
-        CLD_TRY(unique_min_sorted_u64((const uint64_t*)sk, sv, cnt, ~0ull, k, nullptr, col.get(), w.get(), 1,
+        CLD_TRY(unique_min_sorted_u64((const uint64_t*)sk, sv, cnt, ~0ull, k, col.get(), w.get(),
                                       off.get(), k, scal.get() + 2, s));
     else
-        CLD_TRY(unique_min_sorted_u32((const uint32_t*)sk, sv, cnt, 0xFFFFFFFFu, k, nullptr, col.get(), w.get(), 1,
+        CLD_TRY(unique_min_sorted_u32((const uint32_t*)sk, sv, cnt, 0xFFFFFFFFu, k, col.get(), w.get(),
                                       off.get(), k, scal.get() + 2, s));
     CLD_CUDA(cudaMemcpyAsync(hh + 2, scal.get() + 2, 4, cudaMemcpyDeviceToHost, s));
     CLD_CUDA(cudaStreamSynchronize(s));
