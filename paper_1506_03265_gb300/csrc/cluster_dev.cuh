@@ -50,6 +50,8 @@ struct Counters {
     uint32_t growable;                 // some covered/frozen node touches an uncovered one
     uint32_t overflow;                 // a D_v reached 2^32 - 1
     unsigned long long unfrozen;       // unfrozen nodes the stage's draw saw (checks the tracked |U|)
+    uint32_t heavy;                    // a warp that was to hold its part of the next frontier got too much of it
+    uint32_t pad;
 };
 static_assert(offsetof(Counters, bad) + 4 - offsetof(Counters, newly_covered) == 24,
               "the per-step counters form one block");

@@ -29,6 +29,12 @@ struct PushSmem {
     uint32_t sbuf[WARPS][PNB];
 };
 
+// A frontier that the warps hold in PushSmem instead of the lists: this warp's entries and their positions.
+struct Held {
+    uint32_t ne = 0, total = 0;
+    bool on = false;
+};
+
 template <bool RESIDENT, int WARPS>
 __device__ __forceinline__ void dev_push(const uint32_t* __restrict__ fbase, const unsigned long long* __restrict__ fkey,
                                          const uint32_t* __restrict__ fpre, const uint32_t* __restrict__ cfirst,
@@ -37,7 +43,8 @@ __device__ __forceinline__ void dev_push(const uint32_t* __restrict__ fbase, con
                                          unsigned long long* __restrict__ key, uint32_t delta,
                                          uint32_t* __restrict__ stamp, uint32_t stepid,
                                          uint32_t* __restrict__ next, Counters* ctr, PushSmem<WARPS>& smp, uint32_t br,
-                                         uint32_t nb, uint32_t n = 0, uint32_t nnz = 0) {
+                                         uint32_t nb, uint32_t n = 0, uint32_t nnz = 0,
+                                         const Held held = Held{}) {
     auto& spre = smp.spre;
     auto& sbase = smp.sbase;
     auto& skey = smp.skey;
@@ -50,26 +57,32 @@ __device__ __forceinline__ void dev_push(const uint32_t* __restrict__ fbase, con
     bool bad = false;
     const uint32_t nq = (uint32_t)(((uint64_t)E + QC - 1) / QC);
     const uint32_t nwarps = nb * WARPS;
-    for (uint32_t q = br * WARPS + warp; q < nq; q += nwarps) {
-        const uint32_t p0 = q * QC, e1 = min(E, p0 + QC);
-        // entry i0 holds p0; entries i0 + 1 .. il start inside (p0, p0 + QC] (at most QC of them)
-        const uint32_t i0 = __ldcg(&cfirst[q]);
-        const uint32_t il = q + 1 < nq ? __ldcg(&cfirst[q + 1]) : nf - 1;
-        if (RESIDENT && (i0 > il || il >= nf)) {
-            bad = true;
-            continue;
+    const bool mine = RESIDENT && held.on;  // the warp's own entries, else chunks of the lists
+    const uint32_t qend = mine ? (held.total + QC - 1) / QC : nq, qstep = mine ? 1u : nwarps;
+    uint32_t B = 0;
+    for (uint32_t q = mine ? 0u : br * WARPS + warp; q < qend; q += qstep) {
+        const uint32_t p0 = q * QC, e1 = min(mine ? held.total : E, p0 + QC);
+        uint32_t ne = held.ne;
+        if (!mine) {
+            // entry i0 holds p0; entries i0 + 1 .. il start inside (p0, p0 + QC] (at most QC of them)
+            const uint32_t i0 = __ldcg(&cfirst[q]);
+            const uint32_t il = q + 1 < nq ? __ldcg(&cfirst[q + 1]) : nf - 1;
+            if (RESIDENT && (i0 > il || il >= nf)) {
+                bad = true;
+                continue;
+            }
+            ne = min(il - i0 + 1, (uint32_t)QC + 1);
+            if (RESIDENT) __syncwarp();  // the previous chunk's entries have been read
+            for (uint32_t j = lane; j < ne; j += 32) {
+                if (j) spre[warp][j - 1] = __ldcg(&fpre[i0 + j]);
+                sbase[warp][j] = __ldcg(&fbase[i0 + j]);
+                skey[warp][j] = __ldcg(&fkey[i0 + j]);
+            }
+            __syncwarp();
+            B = 0;
         }
-        const uint32_t ne = min(il - i0 + 1, (uint32_t)QC + 1);
-        if (RESIDENT) __syncwarp();  // the previous chunk's entries have been read
-        for (uint32_t j = lane; j < ne; j += 32) {
-            if (j) spre[warp][j - 1] = __ldcg(&fpre[i0 + j]);
-            sbase[warp][j] = __ldcg(&fbase[i0 + j]);
-            skey[warp][j] = __ldcg(&fkey[i0 + j]);
-        }
-        __syncwarp();
         uint32_t word[4], own[4];
         {
-            uint32_t B = 0;
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 word[u] = group_starts(spre[warp] + B, ne - 1 - B, p0 + 32u * u, B, lane, le_mask, &own[u]);
@@ -209,10 +222,13 @@ __device__ __forceinline__ void dev_push(const uint32_t* __restrict__ fbase, con
 // in one launch: one thread-block cluster (its CTAs are resident together, and its barrier orders their memory)
 // takes growing steps back to back, every CTA deciding from the same counters, until a step is too large for it or
 // the growth ends; on small graphs it runs whole stages (draw, listing, doubling, contraction) too.
-// Bound by dependent L2 round trips (chunk table, entries, adjacency, keys, stamps, append; then the snapshot's): 16,000
-// cycles a step up to 65,000 entries, 33,000 at 100,000, of which a cluster barrier is 1,050.  Clustering alone, host
-// loop / resident: 64^2 mesh (44 steps) 1,602 / 504 us, 300^2 mesh (101) 3,101 / 1,326 us, 1,001^2 mesh (206) 7,405 /
-// 4,779 us, road mesh 4,096^2 (134) 12,520 / 11,555 us.  Above 2^18 entries a step of the whole device (push and
+// Bound by dependent L2 round trips.  With the next frontier in the warps' hands (hold_front) a step takes 15,500 cycles
+// up to 3,000 entries, 19,000 at 24,000, 25,000 at 54,000, 35,000 at 99,000: the push (adjacency, keys and stamps,
+// exchange, append) 7,000 to 21,000 of them, two cluster barriers 3,600, hold_front 2,600 to 7,000, the decision the
+// rest.  (Through lists, that is chunk table, entries and two more appends, the steps of the 1,001^2 mesh took 3.09 ms
+// in place of 2.23, those of the 64^2 mesh with its whole-node phases 400 us in place of 353.)  Clustering alone, host
+// loop / resident: 64^2 mesh (44 steps) 1,602 / 457 us, 1,001^2 mesh (206) 7,405 / 4,200 us, road mesh 4,096^2 (134)
+// 12,520 / 11,400 us.  Above 2^18 entries a step of the whole device (push and
 // snapshot 13 to 40 us and 22 us between them) is the faster one; a whole-node pass over more than 2^17 nodes by 16
 // SMs likewise.
 constexpr int GT = 1024;                     // threads per CTA
@@ -254,7 +270,7 @@ struct GrowArgs {
 };
 
 // what a CTA does next, decided by its thread 0
-enum GrowWork : uint32_t { kWorkPush, kWorkDraw, kWorkList, kWorkGuard, kWorkFinal, kWorkLeave };
+enum GrowWork : uint32_t { kWorkPush, kWorkDraw, kWorkList, kWorkGuard, kWorkFinal, kWorkLeave, kWorkSnap };
 
 struct GrowSmem {
     PushSmem<GT / 32> push;
@@ -262,7 +278,73 @@ struct GrowSmem {
     GrowState g;
     uint64_t thr;  // draw threshold of the stage
     uint32_t work;
+    uint32_t nn;       // changed nodes of the last push
+    uint32_t light;    // the warps took them (hold_front) ...
+    uint32_t held;     // ... and push them
+    uint32_t no_hold;  // a warp's share was too much: lists until the launch ends
 };
+
+// The changed nodes become the next frontier in the warps' hands: each takes up to 128 of them, their end-of-step keys and
+// its own prefix over their degrees into the arrays its next push reads, so a step goes without the lists (two appends
+// and three dependent reads less).  Counted as dev_snapshot counts; a warp with more than kHeldMost positions (a hub)
+// sets ctr->heavy, and the lists are written after all.
+constexpr uint32_t kHeldMost = 4 * QC;
+constexpr uint32_t kHeldNodes = QC;  // entries that the warp's arrays hold
+template <int WARPS>
+__device__ __forceinline__ Held hold_front(const uint32_t* __restrict__ next, uint32_t nn,
+                                           const unsigned long long* __restrict__ key, const uint64_t* __restrict__ off,
+                                           uint32_t delta, Counters* ctr, PushSmem<WARPS>& smp, uint32_t br, uint32_t nb,
+                                           unsigned long long* __restrict__ keyS, uint32_t n) {
+    const uint32_t lane = lane_id(), warp = threadIdx.x >> 5, nwarps = nb * WARPS;
+    // fewer warps with more lanes for small steps; at most kHeldNodes a warp
+    const uint32_t per = max((nn + nwarps - 1) / nwarps, 8u), base = (warp * nb + br) * per;
+    constexpr int HU = kHeldNodes / 32;
+    uint32_t v[HU], deg[HU], b0[HU];
+    unsigned long long k[HU];
+    __syncwarp();  // the last push's entries have been read
+#pragma unroll
+    for (int u = 0; u < HU; ++u) {
+        const uint32_t x = u * 32 + lane;
+        v[u] = x < per && base + x < nn ? __ldcg(&next[base + x]) : kNone;
+    }
+#pragma unroll
+    for (int u = 0; u < HU; ++u) {
+        deg[u] = b0[u] = 0;
+        k[u] = kInfKey;
+        if (v[u] < n) {
+            k[u] = __ldcg(&key[v[u]]);
+            const uint64_t o = off[v[u]];
+            b0[u] = (uint32_t)o;
+            deg[u] = (uint32_t)(off[v[u] + 1] - o);
+        } else if (v[u] != kNone) {
+            atomicExch(&ctr->bad, 1u);
+        }
+    }
+    Held h;
+    h.on = true;
+#pragma unroll
+    for (int u = 0; u < HU; ++u) {
+        if (u > 0 && per <= u * 32u) break;
+        if (keyS && v[u] < n) keyS[v[u]] = k[u];  // the next step's start-of-step key
+        const bool take = (uint32_t)(k[u] >> 32) < delta && deg[u] > 0;
+        const unsigned m = __ballot_sync(0xffffffffu, take);
+        const uint32_t d = take ? deg[u] : 0u, incl = warp_incl_scan(d), pre = h.total + incl - d;
+        if (take) {
+            const uint32_t at = h.ne + (uint32_t)__popc(m & lanemask_lt());
+            if (at) smp.spre[warp][at - 1] = pre;
+            smp.sbase[warp][at] = b0[u] - pre;
+            smp.skey[warp][at] = k[u];
+        }
+        h.ne += (uint32_t)__popc(m);
+        h.total += __shfl_sync(0xffffffffu, incl, 31);
+    }
+    if (lane == 0 && h.ne) {
+        atomicAdd(&ctr->front, ((unsigned long long)h.ne << 32) | h.total);
+        if (h.total > kHeldMost) atomicExch(&ctr->heavy, 1u);
+    }
+    __syncwarp();
+    return h;
+}
 
 // barrier of a thread-block cluster: all its threads, and their memory in order
 __device__ __forceinline__ void cluster_barrier() {
@@ -309,25 +391,37 @@ __device__ __forceinline__ uint32_t grow_decide(const GrowArgs& a, GrowState& g,
 }
 
 // What a finished work changes, from the epoch's counters; returns the next work.
-__device__ __forceinline__ uint32_t grow_apply(const GrowArgs& a, GrowState& g, uint32_t work, const Counters* c,
-                                               uint64_t* thr) {
+__device__ __forceinline__ uint32_t grow_apply(const GrowArgs& a, GrowSmem& sm, uint32_t work, const Counters* c) {
+    GrowState& g = sm.g;
+    sm.held = 0;  // (a held frontier is for the next work alone)
     if (work == kWorkPush) {
-        const uint32_t updated = __ldcg(&c->nnext);
-        const unsigned long long front = __ldcg(&c->front);
-        if (__ldcg(&c->bad)) {
+        // (all of the step's counters in one round trip)
+        const uint32_t updated = __ldcg(&c->nnext), bad = __ldcg(&c->bad), heavy = __ldcg(&c->heavy);
+        const unsigned long long front = __ldcg(&c->front), newly = __ldcg(&c->newly_covered);
+        if (bad) {
             g.phase = kPhaseFailed;
             g.unfrozen = ~g.U;
             return kWorkLeave;
         }
-        g.covered += __ldcg(&c->newly_covered);
+        g.covered += newly;
         g.edges_scanned += g.E;
         g.nf = (uint32_t)(front >> 32);
         g.E = (uint32_t)front;
         g.cur ^= 1;
         g.steps++;
         g.node_updates += updated;
-        if (!(updated != 0 && 2 * g.covered < g.U && (a.step_cap == 0 || g.growth_steps < a.step_cap)))
+        if (!(updated != 0 && 2 * g.covered < g.U && (a.step_cap == 0 || g.growth_steps < a.step_cap))) {
             g.phase = kPhaseGrown;
+        } else if (sm.light) {
+            if (heavy) sm.no_hold = 1;
+            sm.held = !sm.no_hold && g.E <= a.max_entries;
+            if (!sm.held) return kWorkSnap;
+        }
+    } else if (work == kWorkSnap) {
+        if (__ldcg(&c->front) != (((unsigned long long)g.nf << 32) | g.E)) {
+            g.phase = kPhaseFailed;
+            return kWorkLeave;
+        }
     } else if (work == kWorkDraw) {
         g.covered = __ldcg(&c->selected);
         g.centers_drawn += g.covered;
@@ -363,7 +457,7 @@ __device__ __forceinline__ uint32_t grow_apply(const GrowArgs& a, GrowState& g, 
         ++g.stage;
         g.phase = kPhaseStage;
     }
-    return grow_decide(a, g, thr);
+    return grow_decide(a, g, &sm.thr);
 }
 
 // The loop: works until one that this launch may not take (a step of more than max_entries entries, a whole-node phase
@@ -374,8 +468,12 @@ template <class Barrier>
 __device__ __forceinline__ void grow_run(const GrowArgs& a, GrowSmem& sm, uint32_t br, uint32_t nb, Barrier barrier) {
     GrowState& g = sm.g;
     __syncthreads();  // the state is set
-    if (threadIdx.x == 0) sm.work = grow_decide(a, g, &sm.thr);
+    if (threadIdx.x == 0) {
+        sm.held = sm.no_hold = sm.light = 0;
+        sm.work = grow_decide(a, g, &sm.thr);
+    }
     __syncthreads();
+    Held held;
     // Counter block of the current epoch (one work, up to its closing barrier).  An epoch clears the next one's block,
     // last read two epochs ago: every CTA has passed the barrier that closed the epoch in between.
     for (uint32_t epoch = 0; sm.work != kWorkLeave && epoch < a.max_epochs; ++epoch) {
@@ -385,10 +483,23 @@ __device__ __forceinline__ void grow_run(const GrowArgs& a, GrowSmem& sm, uint32
             const uint32_t c = g.cur, o = c ^ 1;
             dev_push<true>(a.fbase[c], a.fkey[c], a.fpre[c], a.cfirst[c], g.nf, g.E, a.adj, a.center,
                            a.cumulative ? a.D : nullptr, a.key, g.delta, a.stamp, g.stepid, a.next, ctr, sm.push, br, nb,
-                           a.n, (uint32_t)a.nnz);
+                           a.n, (uint32_t)a.nnz, held);
             barrier();
             const uint32_t nn = min(__ldcg(&ctr->nnext), a.n);
-            dev_snapshot(a.next, nn, a.key, a.off, g.delta, a.fbase[o], a.fkey[o], a.fpre[o], a.cfirst[o], ctr,
+            // (a launch that ends leaves lists, so its last two epochs hold nothing)
+            const bool light = nn <= nb * (GT / 32) * kHeldNodes && !sm.no_hold && epoch + 2 < a.max_epochs;
+            if (light)
+                held = hold_front(a.next, nn, a.key, a.off, g.delta, ctr, sm.push, br, nb, a.keyS, a.n);
+            else
+                dev_snapshot(a.next, nn, a.key, a.off, g.delta, a.fbase[o], a.fkey[o], a.fpre[o], a.cfirst[o], ctr,
+                             sm.scratch, br, nb, a.keyS, a.n);
+            if (threadIdx.x == 0) {
+                sm.nn = nn;
+                sm.light = light;
+            }
+        } else if (work == kWorkSnap) {
+            const uint32_t c = g.cur;
+            dev_snapshot(a.next, sm.nn, a.key, a.off, g.delta, a.fbase[c], a.fkey[c], a.fpre[c], a.cfirst[c], ctr,
                          sm.scratch, br, nb, a.keyS, a.n);
         } else if (work == kWorkDraw) {
             dev_select(a.n, a.center, a.key, a.seed, g.stage, sm.thr, ctr, br, nb, a.keyS);
@@ -406,8 +517,9 @@ __device__ __forceinline__ void grow_run(const GrowArgs& a, GrowSmem& sm, uint32
         if (br == 0 && threadIdx.x < sizeof(Counters) / 8)
             reinterpret_cast<unsigned long long*>(a.ring + (epoch + 1) % 3)[threadIdx.x] = 0ull;
         barrier();
-        if (threadIdx.x == 0) sm.work = grow_apply(a, g, work, ctr, &sm.thr);
+        if (threadIdx.x == 0) sm.work = grow_apply(a, sm, work, ctr);
         __syncthreads();
+        held.on = sm.held;
     }
 }
 
