@@ -1,7 +1,7 @@
 // Device bodies of the CLUSTER(tau) phases (Algorithm 1), shared by the
-// one-graph-per-launch path (each body runs as its own grid kernel, rank =
-// blockIdx.x) and the many-graph persistent kernel (one CTA runs every body
-// for its graph, rank 0 of 1, with block barriers between phases).
+// one-graph path's grid kernels (rank br = blockIdx.x of nb CTAs) and the
+// resident loop of grow.cuh (the CTAs of a thread-block cluster, or one CTA
+// alone, run every body for their graph with a barrier between phases).
 //
 // Node state (Section 3) is one 64-bit word per node, key = d << 32 | c, so
 // the paper's tie-break (smallest distance, then smallest center index) is
@@ -26,8 +26,8 @@
 // position in the frontier's flattened adjacency) and base = off[v] - pre
 // (mod 2^32), so that adjacency index = base + position.
 //
-// Mutable node state is read with L2 loads (__ldcg): inside one persistent
-// CTA there is no kernel boundary to drop stale L1 lines between phases.
+// Mutable node state is read with L2 loads (__ldcg): inside one resident
+// launch there is no kernel boundary to drop stale L1 lines between phases.
 #pragma once
 
 #include <cstddef>

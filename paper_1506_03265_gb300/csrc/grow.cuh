@@ -227,8 +227,8 @@ __device__ __forceinline__ void dev_push(const uint32_t* __restrict__ fbase, con
 // exchange, append) 7,000 to 21,000 of them, two cluster barriers 3,600, hold_front 2,600 to 7,000, the decision the
 // rest.  (Through lists, that is chunk table, entries and two more appends, the steps of the 1,001^2 mesh took 3.09 ms
 // in place of 2.23, those of the 64^2 mesh with its whole-node phases 400 us in place of 353.)  Clustering alone, host
-// loop / resident: 64^2 mesh (44 steps) 1,602 / 457 us, 1,001^2 mesh (206) 7,405 / 4,200 us, road mesh 4,096^2 (134)
-// 12,520 / 11,400 us.  Above 2^18 entries a step of the whole device (push and
+// loop / resident: 64^2 mesh (44 steps) 1,636 / 502 us, 300^2 mesh (101) 3,073 / 1,043 us, 1,001^2 mesh (206) 7,492 /
+// 4,059 us, road mesh 4,096^2 (134) 11,538 / 10,483 us.  Above 2^18 entries a step of the whole device (push and
 // snapshot 13 to 40 us and 22 us between them) is the faster one; a whole-node pass over more than 2^17 nodes by 16
 // SMs likewise.
 constexpr int GT = 1024;                     // threads per CTA

@@ -8,7 +8,7 @@
 // A round relaxes every edge of its nodes, light and heavy alike: with rows
 // sorted by column a light round reads the heavy edges too, so settling the
 // light ones first only adds a pass over the bucket's adjacency and its
-// rounds (R-MAT 24 read 2.2G entries in 34 rounds that way; DSCOUNT).
+// rounds (R-MAT 24 read 2.2G entries in 34 rounds that way).
 //
 // Dedup: a node enters a round's frontier at most once per round (round
 // stamp) and the far pile once per bucket epoch (epoch stamp); stale far
