@@ -143,7 +143,9 @@ __global__ void k_canon_deg(uint32_t n, const uint32_t* __restrict__ ustart, con
         deg[x] = (uint64_t)(uend[x] - ustart[x]) + (tend[x] - tstart[x]);
 }
 
-__global__ void k_iota(uint32_t* __restrict__ a, uint32_t n) {
+// (and *least = all ones, where a minimum starts)
+__global__ void k_iota(uint32_t* __restrict__ a, uint32_t n, uint32_t* __restrict__ least) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) *least = 0xFFFFFFFFu;
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) a[i] = i;
 }
 
@@ -317,18 +319,20 @@ __global__ void k_cc_keep(const uint32_t* __restrict__ parent, uint32_t n, const
 }
 
 __global__ void k_lcc_degrees(const uint32_t* __restrict__ keep, const uint32_t* __restrict__ newid, ListAdj g, uint32_t n,
-                              uint32_t* __restrict__ ndeg, uint32_t* __restrict__ orig) {
+                              uint32_t* __restrict__ ndeg, uint32_t* __restrict__ orig, uint4* __restrict__ info) {
     for (uint32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x)
         if (keep[v]) {
             ndeg[newid[v]] = g.deg(v);
             orig[newid[v]] = v;
+        } else {
+            info[v] = make_uint4(0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu);
         }
 }
 
 // New offsets of the LCC from the scan of its degrees, and per kept node u = orig[i] one word of four:
 // (i, the position shift of u's upper entries from their index in U, the shift of its lower entries from
-// their index in T, 0), positions and shifts taken modulo 2^32 (positions are < 2^32); dropped nodes keep
-// the all-ones pre-fill
+// their index in T, 0), positions and shifts taken modulo 2^32 (positions are < 2^32); dropped nodes hold
+// all ones (k_lcc_degrees)
 __global__ void k_lcc_offsets_lists(const uint32_t* __restrict__ excl, const uint32_t* __restrict__ n_out_dev,
                                     const uint32_t* __restrict__ total_dev, const uint32_t* __restrict__ orig, ListAdj g,
                                     uint64_t* __restrict__ noff, uint4* __restrict__ info) {
@@ -523,11 +527,21 @@ cldiam_status build_csr(const uint32_t* src, const uint32_t* dst, const uint32_t
     const uint64_t cnt = 2 * m;
     // device words read back by the host: [0] bad input, [1] unique entries, [2] wide weight, [3] sampled
     // giant size, [4] LCC nodes, [5] LCC entries, [6] min weight, [7] max degree, [8] sort look-back error
-    DBuf<uint32_t> scal;
-    CLD_TRY(scal.alloc(9, s));
-    CLD_CUDA(cudaMemsetAsync(scal.get(), 0, 9 * sizeof(uint32_t), s));
     const int vb = std::max(1, bits_for((uint64_t)n - 1));
     const int wfit = 64 - 2 * vb;  // weight bits of a packed item
+    // Everything small that starts at zero is one block with one clear (a clear of its own for each of these was a
+    // device operation of 3 us, of some 300 us of a small build): the words above, the weight sum, the largest
+    // component so far, the digit counts of the two sorts (the first's added up by the emission, the second's by the
+    // de-duplication).  The least weight starts at all ones (k_iota).
+    const int npass1 = (2 * vb + 7) / 8, npass2 = (vb + 7) / 8;
+    DBuf<uint32_t> zero;
+    const size_t zero_words = 32 + (size_t)(npass1 + npass2) * 256;
+    CLD_TRY(zero.alloc(zero_words, s));
+    CLD_CUDA(cudaMemsetAsync(zero.get(), 0, zero_words * 4, s));
+    uint32_t* const scal = zero.get();
+    unsigned long long* const wsum = reinterpret_cast<unsigned long long*>(scal + 16);
+    unsigned long long* const best = wsum + 1;
+    uint32_t *const hist1 = scal + 32, *const hist2 = hist1 + (size_t)npass1 * 256;
 
     DBuf<uint32_t> row, deg, degx;
     DBuf<uint64_t> off;
@@ -538,19 +552,14 @@ cldiam_status build_csr(const uint32_t* src, const uint32_t* dst, const uint32_t
     bool pairs = wfit < 1;
     DBuf<uint64_t> items, items2, uniq;
     DBuf<uint32_t> vals, vals2, uniqw;
-    DBuf<uint32_t> hist1;  // digit counts of the first sort, accumulated by the emission
-    DBuf<uint32_t> hist2;  // digit counts of the second sort, accumulated by the de-duplication
     DBuf<uint32_t> runs;
     ListAdj la{};
     uint32_t mu = 0;
     // one item per edge, sorted on (a, b) and de-duplicated (U); the same distinct edges sorted on b alone
     // (stable, so by (b, a): T) give every row's entries below the diagonal
     CLD_TRY(items.alloc(m ? m : 1, s));
-    const int npass1 = (2 * vb + 7) / 8;
-    CLD_TRY(hist1.alloc((size_t)npass1 * 256, s));
     for (;;) {
         if (pairs) CLD_TRY(vals.alloc(m ? m : 1, s));
-        CLD_CUDA(cudaMemsetAsync(hist1.get(), 0, (size_t)npass1 * 256 * 4, s));
         if (m > 0) {
             const size_t esm = (size_t)8 * npass1 * 256 * 4;  // 8 warps; <= 64 KB
             static std::atomic<bool> emit_attr[64];
@@ -565,14 +574,15 @@ cldiam_status build_csr(const uint32_t* src, const uint32_t* dst, const uint32_t
             const auto emit = pairs ? k_emit_canon<true> : k_emit_canon<false>;
             CLD_K(K_CSR, s, emit<<<grid_for(m, 256, 4), 256, esm, s>>>(
                                 (const uint32_t*)dsrc, (const uint32_t*)ddst, (const uint32_t*)dw, m, n, vb,
-                                pairs ? 0 : wfit, items.get(), vals.get(), scal.get(), scal.get() + 2, hist1.get()));
+                                pairs ? 0 : wfit, items.get(), vals.get(), scal, scal + 2, hist1));
             CLD_LAUNCH_CHECK();
         }
-        CLD_CUDA(cudaMemcpyAsync(hbad, scal.get(), 3 * sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+        CLD_CUDA(cudaMemcpyAsync(hbad, scal, 3 * sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
         CLD_CUDA(cudaStreamSynchronize(s));
         if (hbad[0]) return fail(CLDIAM_ERR_INVALID_ARG, "edge with node id >= n or weight 0");
         if (pairs || hbad[2] == 0) break;
         pairs = true;
+        CLD_CUDA(cudaMemsetAsync(hist1, 0, (size_t)npass1 * 256 * 4, s));
     }
     const int wb = pairs ? 0 : wfit;
     CLD_TRY(items2.alloc(m ? m : 1, s));
@@ -582,29 +592,26 @@ cldiam_status build_csr(const uint32_t* src, const uint32_t* dst, const uint32_t
         CLD_TRY(vals2.alloc(m ? m : 1, s));
         CLD_TRY(uniqw.alloc(m ? m : 1, s));
         CLD_TRY(radix_sort_pairs_u64(items.get(), vals.get(), items2.get(), vals2.get(), m, 2 * vb, &alt, s,
-                                     scal.get() + 8, nullptr, nullptr, hist1.get()));
+                                     scal + 8, nullptr, nullptr, hist1));
     } else {
-        CLD_TRY(radix_sort_keys_u64(items.get(), items2.get(), m, wb, 2 * vb, &alt, s, scal.get() + 8, nullptr,
-                                    hist1.get()));
+        CLD_TRY(radix_sort_keys_u64(items.get(), items2.get(), m, wb, 2 * vb, &alt, s, scal + 8, nullptr,
+                                    hist1));
     }
-    const int npass2 = (vb + 7) / 8;
-    CLD_TRY(hist2.alloc((size_t)npass2 * 256, s));
-    CLD_CUDA(cudaMemsetAsync(hist2.get(), 0, (size_t)npass2 * 256 * 4, s));
     // every row's run bounds in both orders; the de-duplication writes the first order's
     CLD_TRY(runs.alloc(4 * (size_t)n, s));
     CLD_CUDA(cudaMemsetAsync(runs.get(), 0, 4 * (size_t)n * 4, s));
     CLD_TRY(unique_items_u64(alt ? items2.get() : items.get(), pairs ? (alt ? vals2.get() : vals.get()) : nullptr, m, vb,
-                             uniq.get(), uniqw.get(), scal.get() + 1, s, hist2.get(), runs.get(), runs.get() + n));
-    CLD_CUDA(cudaMemcpyAsync(hbad + 1, scal.get() + 1, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+                             uniq.get(), uniqw.get(), scal + 1, s, hist2, runs.get(), runs.get() + n));
+    CLD_CUDA(cudaMemcpyAsync(hbad + 1, scal + 1, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
     CLD_CUDA(cudaStreamSynchronize(s));
     mu = hbad[1];  // distinct undirected edges
     bool alt2 = false;
     if (pairs)
         CLD_TRY(radix_sort_pairs_u64(items.get(), vals.get(), items2.get(), vals2.get(), mu, vb, &alt2, s,
-                                     scal.get() + 8, uniq.get(), uniqw.get(), hist2.get()));
+                                     scal + 8, uniq.get(), uniqw.get(), hist2));
     else
-        CLD_TRY(radix_sort_keys_u64(items.get(), items2.get(), mu, wb, vb, &alt2, s, scal.get() + 8, uniq.get(),
-                                    hist2.get()));
+        CLD_TRY(radix_sort_keys_u64(items.get(), items2.get(), mu, wb, vb, &alt2, s, scal + 8, uniq.get(),
+                                    hist2));
     la.U = uniq.get();
     la.T = alt2 ? items2.get() : items.get();
     la.UW = pairs ? uniqw.get() : nullptr;
@@ -619,7 +626,7 @@ cldiam_status build_csr(const uint32_t* src, const uint32_t* dst, const uint32_t
     if (mu > 0) {
         uint32_t* r0 = runs.get();
         CLD_K(K_CSR, s, k_canon_runs<<<grid_for(mu, 256), 256, 0, s>>>(la.T, mu, vb, wb, r0 + 2 * (size_t)n,
-                                                                      r0 + 3 * (size_t)n, scal.get() + 1));
+                                                                      r0 + 3 * (size_t)n, scal + 1));
         CLD_LAUNCH_CHECK();
     }
     if (!lcc) {
@@ -635,25 +642,17 @@ cldiam_status build_csr(const uint32_t* src, const uint32_t* dst, const uint32_t
         CLD_TRY(scan_exclusive_u64(degs.get(), off.get(), n, off.get() + n, s));
         if (mu > 0) {
             CLD_K(K_CSR, s, k_canon_scatter<<<grid_for(mu, 256), 256, 0, s>>>(la, mu, off.get(), row.get(), adj.get(),
-                                                                             scal.get() + 8));
+                                                                             scal + 8));
             CLD_LAUNCH_CHECK();
         }
     }
     // (the entry count stays on the device until the host needs it, read together with the next result)
     uint32_t nnz = 0;
     DBuf<uint32_t> orig;
-    // weight statistics for the initial Delta (Algorithm 1 / Section 5): sum over u < v, minimum
-    DBuf<unsigned long long> wsum;
-    CLD_TRY(wsum.alloc(1, s));
-    CLD_CUDA(cudaMemsetAsync(wsum.get(), 0, 8, s));
-    CLD_CUDA(cudaMemsetAsync(scal.get() + 6, 0xFF, 4, s));
-    CLD_CUDA(cudaMemsetAsync(scal.get() + 7, 0, 4, s));
     if (lcc) {
         DBuf<uint32_t> parent, size, keep, newid;
-        DBuf<unsigned long long> best;
         CLD_TRY(parent.alloc(n, s));
-        CLD_TRY(best.alloc(1, s));
-        CLD_K(K_MISC, s, k_iota<<<grid_for(n, 256), 256, 0, s>>>(parent.get(), n));
+        CLD_K(K_MISC, s, k_iota<<<grid_for(n, 256), 256, 0, s>>>(parent.get(), n, scal + 6));
         CLD_LAUNCH_CHECK();
         // Afforest-style: link two neighbours per node, find the dominant tree by sampling,
         // then link the remaining edges of the nodes outside it (all no-ops on a graph without edges)
@@ -674,8 +673,8 @@ cldiam_status build_csr(const uint32_t* src, const uint32_t* dst, const uint32_t
         CLD_LAUNCH_CHECK();
         std::vector<uint32_t> hs(kSamples);
         CLD_CUDA(cudaMemcpyAsync(hs.data(), samp.get(), kSamples * 4, cudaMemcpyDeviceToHost, s));
-        CLD_CUDA(cudaMemcpyAsync(hbad + 1, scal.get() + 1, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
-        CLD_CUDA(cudaMemcpyAsync(hbad + 8, scal.get() + 8, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+        CLD_CUDA(cudaMemcpyAsync(hbad + 1, scal + 1, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+        CLD_CUDA(cudaMemcpyAsync(hbad + 8, scal + 8, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
         CLD_CUDA(cudaStreamSynchronize(s));
         // a failed sort leaves the graph unusable: stop before anything indexes by its entries
         if (hbad[8]) return fail(CLDIAM_ERR_TIMEOUT, "radix sort look-back wait expired or CSR assembly inconsistent");
@@ -693,39 +692,37 @@ cldiam_status build_csr(const uint32_t* src, const uint32_t* dst, const uint32_t
                                                                             parent.get()));
             CLD_K(K_CC, s, k_cc_compress<<<grid_for(n, 256), 256, 0, s>>>(parent.get(), n));
             CLD_LAUNCH_CHECK();
-            CLD_CUDA(cudaMemsetAsync(scal.get() + 3, 0, 4, s));
-            CLD_K(K_CC, s, k_cc_size_of<<<grid_for(n, 256), 256, 0, s>>>(parent.get(), n, giant, scal.get() + 3));
-            CLD_CUDA(cudaMemsetAsync(best.get(), 0, 8, s));
-            CLD_K(K_CC, s, k_cc_giant_best<<<1, 1, 0, s>>>(scal.get() + 3, n, giant, best.get()));
+            CLD_K(K_CC, s, k_cc_size_of<<<grid_for(n, 256), 256, 0, s>>>(parent.get(), n, giant, scal + 3));
+            CLD_K(K_CC, s, k_cc_giant_best<<<1, 1, 0, s>>>(scal + 3, n, giant, best));
             CLD_LAUNCH_CHECK();
-        } else {
-            CLD_CUDA(cudaMemsetAsync(best.get(), 0, 8, s));
         }
         CLD_TRY(size.alloc(n, s));
         CLD_CUDA(cudaMemsetAsync(size.get(), 0, (size_t)n * 4, s));
-        const uint32_t* gcount = nnz > 0 ? scal.get() + 3 : nullptr;
+        const uint32_t* gcount = nnz > 0 ? scal + 3 : nullptr;
         CLD_K(K_CC, s, k_cc_count<<<grid_for(n, 256), 256, 0, s>>>(parent.get(), n, size.get(), gcount));
         CLD_LAUNCH_CHECK();
-        CLD_K(K_CC, s, k_cc_best<<<grid_for(n, 256), 256, 0, s>>>(parent.get(), size.get(), n, best.get(), gcount));
+        CLD_K(K_CC, s, k_cc_best<<<grid_for(n, 256), 256, 0, s>>>(parent.get(), size.get(), n, best, gcount));
         CLD_LAUNCH_CHECK();
         CLD_TRY(keep.alloc(n, s));
         CLD_TRY(newid.alloc(n, s));
-        CLD_K(K_CC, s, k_cc_keep<<<grid_for(n, 256), 256, 0, s>>>(parent.get(), n, best.get(), keep.get()));
+        CLD_K(K_CC, s, k_cc_keep<<<grid_for(n, 256), 256, 0, s>>>(parent.get(), n, best, keep.get()));
         CLD_LAUNCH_CHECK();
         parent.release();
         size.release();
-        CLD_TRY(scan_exclusive_u32(keep.get(), newid.get(), n, scal.get() + 4, s));
+        CLD_TRY(scan_exclusive_u32(keep.get(), newid.get(), n, scal + 4, s));
         // the LCC's node and entry counts stay on the device: its arrays are sized by the bounds n and
         // nnz, and the kernels read the counts from scal[4] / scal[5]
         CLD_TRY(orig.alloc(n, s));
+        DBuf<uint4> info;
+        CLD_TRY(info.alloc(n, s));
         CLD_TRY(deg.alloc((size_t)n + 1, s));
         CLD_TRY(degx.alloc((size_t)n + 1, s));
         CLD_CUDA(cudaMemsetAsync(deg.get(), 0, ((size_t)n + 1) * 4, s));
         CLD_K(K_CSR, s, k_lcc_degrees<<<grid_for(n, 256), 256, 0, s>>>(keep.get(), newid.get(), la, n, deg.get(),
-                                                                      orig.get()));
+                                                                      orig.get(), info.get()));
         CLD_LAUNCH_CHECK();
         keep.release();
-        CLD_TRY(scan_exclusive_u32(deg.get(), degx.get(), n, scal.get() + 5, s));  // zeros past the kept nodes
+        CLD_TRY(scan_exclusive_u32(deg.get(), degx.get(), n, scal + 5, s));  // zeros past the kept nodes
         deg.release();  // (the largest node counts fit beside the records below: 52 bytes a node at most)
         DBuf<uint64_t> noff;
         DBuf<uint2> nadj;
@@ -733,46 +730,43 @@ cldiam_status build_csr(const uint32_t* src, const uint32_t* dst, const uint32_t
         CLD_TRY(nadj.alloc(nnz ? nnz : 1, s));
         // the LCC's CSR straight from the lists: the whole graph's CSR is never built, and the row of every entry
         // (COO form) is left out (its users build it from the offsets when they need it: fill_rows)
-        DBuf<uint4> info;
-        CLD_TRY(info.alloc(n, s));
-        CLD_CUDA(cudaMemsetAsync(info.get(), 0xFF, (size_t)n * 16, s));
         CLD_K(K_CSR, s, k_lcc_offsets_lists<<<grid_for((size_t)n + 1, 256), 256, 0, s>>>(
-                            degx.get(), scal.get() + 4, scal.get() + 5, orig.get(), la, noff.get(), info.get()));
+                            degx.get(), scal + 4, scal + 5, orig.get(), la, noff.get(), info.get()));
         CLD_LAUNCH_CHECK();
         if (mu > 0) {
             const auto assemble = pairs ? k_lcc_assemble<true> : k_lcc_assemble<false>;
             CLD_K(K_CSR, s, assemble<<<grid_for(mu, 256, 4), 256, 0, s>>>(la, mu, info.get(), newid.get(), nnz ? nnz : 1,
-                                                                         nadj.get(), wsum.get(), scal.get() + 6,
-                                                                         scal.get() + 8));
+                                                                         nadj.get(), wsum, scal + 6,
+                                                                         scal + 8));
             CLD_LAUNCH_CHECK();
         }
         g->off = noff.detach();
         g->adj = nadj.detach();
-        CLD_K(K_CSR, s, k_degree_max<<<grid_for(n, 256), 256, 0, s>>>(g->off, n, scal.get() + 4, scal.get() + 7));
+        CLD_K(K_CSR, s, k_degree_max<<<grid_for(n, 256), 256, 0, s>>>(g->off, n, scal + 4, scal + 7));
         CLD_LAUNCH_CHECK();
     } else {
-        CLD_CUDA(cudaMemcpyAsync(hbad + 1, scal.get() + 1, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+        CLD_CUDA(cudaMemcpyAsync(hbad + 1, scal + 1, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
         CLD_CUDA(cudaStreamSynchronize(s));
         nnz = hbad[1];
         CLD_TRY(orig.alloc(n, s));
-        CLD_K(K_MISC, s, k_iota<<<grid_for(n, 256), 256, 0, s>>>(orig.get(), n));
+        CLD_K(K_MISC, s, k_iota<<<grid_for(n, 256), 256, 0, s>>>(orig.get(), n, scal + 6));
         CLD_LAUNCH_CHECK();
         g->off = off.detach();
         g->adj = adj.detach();
         g->row = row.detach();
         if (nnz) {
-            CLD_K(K_CSR, s, k_graph_stats<<<grid_for(nnz, 256), 256, 0, s>>>(g->row, g->adj, nnz, wsum.get(),
-                                                                             scal.get() + 6));
+            CLD_K(K_CSR, s, k_graph_stats<<<grid_for(nnz, 256), 256, 0, s>>>(g->row, g->adj, nnz, wsum,
+                                                                             scal + 6));
             CLD_LAUNCH_CHECK();
         }
-        CLD_K(K_CSR, s, k_degree_max<<<grid_for(n, 256), 256, 0, s>>>(g->off, n, nullptr, scal.get() + 7));
+        CLD_K(K_CSR, s, k_degree_max<<<grid_for(n, 256), 256, 0, s>>>(g->off, n, nullptr, scal + 7));
         CLD_LAUNCH_CHECK();
     }
     g->orig = orig.detach();
     g->connected = lcc;
     uint64_t* hsum = reinterpret_cast<uint64_t*>(static_cast<char*>(g->host.h) + 64);
-    CLD_CUDA(cudaMemcpyAsync(hsum, wsum.get(), 8, cudaMemcpyDeviceToHost, s));
-    CLD_CUDA(cudaMemcpyAsync(hbad + 1, scal.get() + 1, 8 * sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+    CLD_CUDA(cudaMemcpyAsync(hsum, wsum, 8, cudaMemcpyDeviceToHost, s));
+    CLD_CUDA(cudaMemcpyAsync(hbad + 1, scal + 1, 8 * sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
     CLD_CUDA(cudaStreamSynchronize(s));
     if (hbad[8]) return fail(CLDIAM_ERR_TIMEOUT, "radix sort look-back wait expired or CSR assembly inconsistent");
     if (lcc) {

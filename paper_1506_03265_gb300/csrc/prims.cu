@@ -602,16 +602,16 @@ static cldiam_status radix_sort_impl(K* keys, uint32_t* vals, K* keys_alt, uint3
             CLD_CUDA(cudaFuncSetAttribute(pick(hi), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         if (dev >= 0 && dev < 64) attr_set[form][dev] = true;
     }
-    DBuf<uint32_t> hist_own, ctl;
+    // one block, cleared once: the status words, the tile counters and the error word, the digit counts if they are
+    // counted here
+    const size_t sw = (size_t)ntiles * OS_RADIX, hw = hist_in ? 0 : (size_t)npass * OS_RADIX;
     DBuf<unsigned long long> status;
-    CLD_TRY(ctl.alloc(2 * npass + 2, s));
-    CLD_TRY(status.alloc((size_t)ntiles * OS_RADIX, s));
-    CLD_CUDA(cudaMemsetAsync(ctl.get(), 0, (2 * npass + 2) * 4, s));
+    CLD_TRY(status.alloc(sw + npass + 1 + hw / 2, s));
+    CLD_CUDA(cudaMemsetAsync(status.get(), 0, status.n * 8, s));
+    uint32_t* const ctl = reinterpret_cast<uint32_t*>(status.get() + sw);
     uint32_t* hist = hist_in;
     if (!hist) {
-        CLD_TRY(hist_own.alloc((size_t)npass * OS_RADIX, s));
-        hist = hist_own.get();
-        CLD_CUDA(cudaMemsetAsync(hist, 0, (size_t)npass * OS_RADIX * 4, s));
+        hist = ctl + 2 * npass + 2;
         const size_t hsm = (size_t)OS_HIST_WARPS * npass * OS_RADIX * 4;  // <= 64 KB (at most 8 passes)
         if (dev < 0 || dev >= 64 || !hist_attr_set[dev]) {
             CLD_CUDA(cudaFuncSetAttribute(k_os_hist<K>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -630,15 +630,14 @@ static cldiam_status radix_sort_impl(K* keys, uint32_t* vals, K* keys_alt, uint3
     K* ko = keys_alt;
     uint32_t* vo = vals_alt;
     bool alt = false;
-    CLD_CUDA(cudaMemsetAsync(status.get(), 0, (size_t)ntiles * OS_RADIX * 8, s));
     for (int p = 0; p < npass; ++p) {
         const int shift = shift0 + 8 * p;
         const bool hi = sizeof(K) == 8 && shift >= 32;
         const uint32_t sh = (uint32_t)shift & 31u;
         const uint32_t dm = bits - 8 * p >= 8 ? 0xFFu : ((1u << (bits - 8 * p)) - 1u);  // key bits only
         const uint32_t* go = hist + p * OS_RADIX;
-        uint32_t* tc = ctl.get() + p;
-        uint32_t* er = err_dev ? err_dev : ctl.get() + 2 * npass;
+        uint32_t* tc = ctl + p;
+        uint32_t* er = err_dev ? err_dev : ctl + 2 * npass;
         CLD_K(K_RADIX_SCATTER, s, pick(hi)<<<ntiles, threads, smem, s>>>(ki, vi, ko, vo, n, sh, dm, go, status.get(),
                                                                          2u * p + 1u, tc, er));
         CLD_LAUNCH_CHECK();
@@ -653,7 +652,7 @@ static cldiam_status radix_sort_impl(K* keys, uint32_t* vals, K* keys_alt, uint3
     *in_alt = alt;
     if (err_dev) return CLDIAM_OK;  // the caller reads the look-back error word with its next result
     uint32_t herr = 0;
-    CLD_CUDA(cudaMemcpyAsync(&herr, ctl.get() + 2 * npass, 4, cudaMemcpyDeviceToHost, s));
+    CLD_CUDA(cudaMemcpyAsync(&herr, ctl + 2 * npass, 4, cudaMemcpyDeviceToHost, s));
     CLD_CUDA(cudaStreamSynchronize(s));
     if (herr) return fail(CLDIAM_ERR_TIMEOUT, "radix sort look-back wait expired");
     return CLDIAM_OK;
