@@ -285,26 +285,31 @@ __global__ void k_cc_giant_best(const uint32_t* __restrict__ count, uint32_t n, 
     if (giant_is_largest(count, n)) *best = ((unsigned long long)*count << 32) | (unsigned long long)(0xFFFFFFFFu - giant);
 }
 
-__global__ void k_cc_count(const uint32_t* __restrict__ parent, uint32_t n, uint32_t* __restrict__ size,
+// Nodes of every tree but the dominant one (its size is known), roots not counted: most of the rest are nodes without
+// an edge, which then cost no atomic (R-MAT of 8.4M nodes x 8, more than half of them alone: 226 -> 8 us).  One atomic
+// per distinct root per warp: the dominant tree may have been hooked under another root since it was sampled.
+__global__ void k_cc_count(const uint32_t* __restrict__ parent, uint32_t n, uint32_t giant, uint32_t* __restrict__ size,
                            const uint32_t* __restrict__ gcount) {
     if (giant_is_largest(gcount, n)) return;
     for (uint32_t base = blockIdx.x * blockDim.x; base < n; base += gridDim.x * blockDim.x) {
         const uint32_t v = base + threadIdx.x;
-        const uint32_t r = v < n ? parent[v] : 0xFFFFFFFFu;
-        // most nodes share one root: one atomic per distinct root per warp
-        const unsigned peers = __match_any_sync(0xffffffffu, r);
-        if (v < n && lane_id() == (unsigned)(__ffs(peers) - 1)) atomicAdd(&size[r], (uint32_t)__popc(peers));
+        const uint32_t r = v < n ? parent[v] : v;
+        const bool counts = r != v && r != giant;
+        if (!__any_sync(0xffffffffu, counts)) continue;
+        const unsigned peers = __match_any_sync(0xffffffffu, counts ? r : 0xFFFFFFFFu);
+        if (counts && lane_id() == (unsigned)(__ffs(peers) - 1)) atomicAdd(&size[r], (uint32_t)__popc(peers));
     }
 }
 
 // best component: largest size, then smallest root id
 __global__ void k_cc_best(const uint32_t* __restrict__ parent, const uint32_t* __restrict__ size, uint32_t n,
-                          unsigned long long* __restrict__ best, const uint32_t* __restrict__ gcount) {
+                          uint32_t giant, unsigned long long* __restrict__ best, const uint32_t* __restrict__ gcount) {
     if (giant_is_largest(gcount, n)) return;
     unsigned long long b = 0;
     for (uint32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x)
         if (parent[v] == v) {
-            unsigned long long key = ((unsigned long long)size[v] << 32) | (unsigned long long)(0xFFFFFFFFu - v);
+            const uint32_t c = v == giant ? *gcount : size[v] + 1u;
+            const unsigned long long key = ((unsigned long long)c << 32) | (unsigned long long)(0xFFFFFFFFu - v);
             b = key > b ? key : b;
         }
     b = block_reduce(b, [](unsigned long long x, unsigned long long y) { return x > y ? x : y; }, 0ull);
@@ -679,9 +684,11 @@ cldiam_status build_csr(const uint32_t* src, const uint32_t* dst, const uint32_t
         // a failed sort leaves the graph unusable: stop before anything indexes by its entries
         if (hbad[8]) return fail(CLDIAM_ERR_TIMEOUT, "radix sort look-back wait expired or CSR assembly inconsistent");
         nnz = hbad[1];
+        uint32_t giant = 0xFFFFFFFFu;  // none
         if (nnz > 0) {
             std::sort(hs.begin(), hs.end());
-            uint32_t giant = hs[0], best_run = 0;
+            uint32_t best_run = 0;
+            giant = hs[0];
             for (size_t i = 0; i < hs.size();) {
                 size_t j = i;
                 while (j < hs.size() && hs[j] == hs[i]) ++j;
@@ -699,9 +706,9 @@ cldiam_status build_csr(const uint32_t* src, const uint32_t* dst, const uint32_t
         CLD_TRY(size.alloc(n, s));
         CLD_CUDA(cudaMemsetAsync(size.get(), 0, (size_t)n * 4, s));
         const uint32_t* gcount = nnz > 0 ? scal + 3 : nullptr;
-        CLD_K(K_CC, s, k_cc_count<<<grid_for(n, 256), 256, 0, s>>>(parent.get(), n, size.get(), gcount));
+        CLD_K(K_CC, s, k_cc_count<<<grid_for(n, 256), 256, 0, s>>>(parent.get(), n, giant, size.get(), gcount));
         CLD_LAUNCH_CHECK();
-        CLD_K(K_CC, s, k_cc_best<<<grid_for(n, 256), 256, 0, s>>>(parent.get(), size.get(), n, best, gcount));
+        CLD_K(K_CC, s, k_cc_best<<<grid_for(n, 256), 256, 0, s>>>(parent.get(), size.get(), n, giant, best, gcount));
         CLD_LAUNCH_CHECK();
         CLD_TRY(keep.alloc(n, s));
         CLD_TRY(newid.alloc(n, s));
