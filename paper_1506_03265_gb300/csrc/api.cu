@@ -325,6 +325,12 @@ cldiam_status cldiam_sssp_delta(cldiam_graph* g, uint32_t source, uint32_t delta
     return guarded([&] { return sssp_delta(g, source, delta, dist, ecc, rounds, edges_scanned); });
 }
 
+// Not in the header: the tests reach the resident form's phase limit with it.
+cldiam_status cldiam_internal_sssp_phases(cldiam_graph* g, uint32_t source, uint32_t delta, uint32_t max_phases,
+                                          uint32_t* dist, uint64_t* ecc) {
+    return guarded([&] { return sssp_delta(g, source, delta, dist, ecc, nullptr, nullptr, max_phases); });
+}
+
 cldiam_status cldiam_arena_job_times(const cldiam_arena* a, uint32_t count, double* start_s, double* end_s) {
     return guarded([&] { return arena_job_times(a, count, start_s, end_s); });
 }

@@ -107,8 +107,9 @@ uint64_t arena_entries(const cldiam_arena* a, const uint32_t* ids, uint32_t coun
 // row[p] = v for every CSR position p of row v (a graph assembled from the sorted lists keeps no row array)
 cldiam_status fill_rows(const uint64_t* off, uint32_t n, uint32_t* row, cudaStream_t s);
 
+// max_phases: rounds and splits that one resident launch takes before the host launches the next (0 = the default)
 cldiam_status sssp_delta(cldiam_graph* g, uint32_t source, uint32_t delta, uint32_t* dist_out, uint64_t* ecc,
-                         uint64_t* rounds, uint64_t* scanned);
+                         uint64_t* rounds, uint64_t* scanned, uint32_t max_phases = 0);
 
 // tuning knobs in effect (defaults filled in) and their validation (tune.cu): the process-wide
 // settings alone, or for a call on `entries` adjacency entries of one graph (or of one batch), where the

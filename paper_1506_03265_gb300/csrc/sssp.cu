@@ -339,19 +339,20 @@ __device__ __forceinline__ uint32_t ds_decide(const DsArgs& a, DsState& g, uint6
     return ds_next_bucket(g, a.delta, lo) ? kDsSplit : kDsLeave;
 }
 
-// Rounds and splits back to back by one thread-block cluster, until one that is too large for it, or the end.
+// Rounds and splits back to back by one thread-block cluster, until one that is too large for it, the phase limit, or the
+// end.  The next work is decided at the head of an iteration, after the limit has been tested: a decision moves the state
+// (a split's bucket), so one that no work followed would leave its bucket out of the next launch.
 __global__ void __launch_bounds__(GT, 1) k_ds_resident(const DsArgs a, const DsState start) {
     extern __shared__ __align__(16) unsigned char ds_smem[];
     DsSmem& sm = *reinterpret_cast<DsSmem*>(ds_smem);
     DsState& g = sm.g;
     const uint32_t br = blockIdx.x, nb = gridDim.x;
-    if (threadIdx.x == 0) {
-        g = start;
-        sm.work = ds_decide(a, g, &sm.lo);
-    }
-    __syncthreads();
+    if (threadIdx.x == 0) g = start;
     // Counters of the epoch; an epoch clears the next one's, last read two epochs ago.
-    for (uint32_t epoch = 0; sm.work != kDsLeave && epoch < a.max_epochs; ++epoch) {
+    for (uint32_t epoch = 0;; ++epoch) {
+        if (threadIdx.x == 0) sm.work = epoch < a.max_epochs && !g.bad ? ds_decide(a, g, &sm.lo) : (uint32_t)kDsLeave;
+        __syncthreads();
+        if (sm.work == kDsLeave) break;
         DsRound* r = a.ring + epoch % 3;
         const uint32_t work = sm.work, p = g.pile;
         unsigned long long fr = 0;
@@ -384,9 +385,7 @@ __global__ void __launch_bounds__(GT, 1) k_ds_resident(const DsArgs a, const DsS
             // does, and then nobody writes them before the next barrier)
             g.nfar = __ldcg(&a.ctr->pile[g.pile].n.count);
             g.min = __ldcg(&a.ctr->pile[g.pile].min);
-            sm.work = g.bad ? (uint32_t)kDsLeave : ds_decide(a, g, &sm.lo);
         }
-        __syncthreads();
     }
     if (br == 0 && threadIdx.x == 0) *a.out = g;
 }
@@ -433,7 +432,7 @@ int ds_cluster_size(int dev) {
 }  // namespace
 
 cldiam_status sssp_delta(cldiam_graph* g, uint32_t source, uint32_t delta, uint32_t* dist_out, uint64_t* ecc,
-                         uint64_t* rounds_out, uint64_t* scanned_out) {
+                         uint64_t* rounds_out, uint64_t* scanned_out, uint32_t max_phases) {
     if (!g || !ecc) return fail(CLDIAM_ERR_INVALID_ARG, "NULL graph or ecc");
     if (source >= g->n) return fail(CLDIAM_ERR_INVALID_ARG, "source >= n");
     if (g->nnz >= 0xFFFFFFFFull) return fail(CLDIAM_ERR_UNSUPPORTED, "2^32 - 1 or more adjacency entries");
@@ -498,7 +497,7 @@ cldiam_status sssp_delta(cldiam_graph* g, uint32_t source, uint32_t delta, uint3
     // resident rounds: lists of about 2^18 adjacency entries, piles of 2^18 nodes (as CLUSTER's resident steps)
     a.max_list = (uint32_t)std::max<uint64_t>(1, (uint64_t)kGrowEntries / (g->nnz / n + 1));
     a.max_far = kGrowEntries;
-    a.max_epochs = kGrowEpochs;
+    a.max_epochs = max_phases ? max_phases : kGrowEpochs;
     const unsigned gb = grid_for(n, 256);
     CLD_K(K_SSSP, s, k_ds_init<<<gb, 256, 0, s>>>(dist.get(), rstamp.get(), fstamp.get(), n, source));
     CLD_LAUNCH_CHECK();
