@@ -325,7 +325,11 @@ cldiam_status cldiam_sssp_delta(cldiam_graph* g, uint32_t source, uint32_t delta
     return guarded([&] { return sssp_delta(g, source, delta, dist, ecc, rounds, edges_scanned); });
 }
 
-// Not in the header: the tests reach the resident form's phase limit with it.
+// Not in the header: the tests reach the resident forms' phase limits with these two.
+cldiam_status cldiam_internal_cluster_phases(cldiam_graph* g, double tau, uint64_t seed, const cldiam_opts* opts,
+                                             uint32_t max_phases, cldiam_clustering** out) {
+    return guarded([&] { return cluster(g, tau, seed, opts, out, max_phases); });
+}
 cldiam_status cldiam_internal_sssp_phases(cldiam_graph* g, uint32_t source, uint32_t delta, uint32_t max_phases,
                                           uint32_t* dist, uint64_t* ecc) {
     return guarded([&] { return sssp_delta(g, source, delta, dist, ecc, nullptr, nullptr, max_phases); });

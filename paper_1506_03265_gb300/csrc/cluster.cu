@@ -304,7 +304,8 @@ void free_clustering(cldiam_clustering* c) {
     delete c;
 }
 
-cldiam_status cluster(cldiam_graph* g, double tau, uint64_t seed, const cldiam_opts* o, cldiam_clustering** out) {
+cldiam_status cluster(cldiam_graph* g, double tau, uint64_t seed, const cldiam_opts* o, cldiam_clustering** out,
+                      uint32_t max_phases) {
     if (!g || !out) return fail(CLDIAM_ERR_INVALID_ARG, "NULL graph or out");
     *out = nullptr;
     if (!(tau > 0.0) || !std::isfinite(tau)) return fail(CLDIAM_ERR_INVALID_ARG, "tau must be a positive number");
@@ -461,7 +462,7 @@ cldiam_status cluster(cldiam_graph* g, double tau, uint64_t seed, const cldiam_o
         a.n = n;
         a.step_cap = step_cap;
         a.max_entries = grow_entries;
-        a.max_epochs = kGrowEpochs;
+        a.max_epochs = max_phases ? max_phases : kGrowEpochs;
         a.connected = true;
         a.cumulative = cumulative;
         a.pull_ok = pull_ok;

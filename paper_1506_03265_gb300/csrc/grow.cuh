@@ -390,8 +390,11 @@ __device__ __forceinline__ uint32_t grow_decide(const GrowArgs& a, GrowState& g,
     }
 }
 
-// What a finished work changes, from the epoch's counters; returns the next work.
-__device__ __forceinline__ uint32_t grow_apply(const GrowArgs& a, GrowSmem& sm, uint32_t work, const Counters* c) {
+// What a finished work changes, from the epoch's counters; returns the next work.  `last`: the launch is to end here if
+// the state can be resumed from, which it can before a decision (that counts a step or doubles Delta) but not between
+// a draw, a doubling or a step and what they ask for next.
+__device__ __forceinline__ uint32_t grow_apply(const GrowArgs& a, GrowSmem& sm, uint32_t work, const Counters* c,
+                                               bool last) {
     GrowState& g = sm.g;
     sm.held = 0;  // (a held frontier is for the next work alone)
     if (work == kWorkPush) {
@@ -457,13 +460,14 @@ __device__ __forceinline__ uint32_t grow_apply(const GrowArgs& a, GrowSmem& sm, 
         ++g.stage;
         g.phase = kPhaseStage;
     }
-    return grow_decide(a, g, &sm.thr);
+    return last ? (uint32_t)kWorkLeave : grow_decide(a, g, &sm.thr);
 }
 
 // The loop: works until one that this launch may not take (a step of more than max_entries entries, a whole-node phase
-// when `stages` is off), the end, or a failure; sm.g holds the control state before and after.  CTA br of nb that share
-// the graph; `barrier` synchronises all their threads and orders their memory.  The state stays in shared memory and
-// thread 0 decides (kept in every thread's registers it spilled the pushes' at 64 of them).
+// when `stages` is off), the end, a failure, or the first state from max_epochs works on that a launch can start from;
+// sm.g holds the control state before and after.  CTA br of nb that share the graph; `barrier` synchronises all their
+// threads and orders their memory.  The state stays in shared memory and thread 0 decides (kept in every thread's
+// registers it spilled the pushes' at 64 of them).
 template <class Barrier>
 __device__ __forceinline__ void grow_run(const GrowArgs& a, GrowSmem& sm, uint32_t br, uint32_t nb, Barrier barrier) {
     GrowState& g = sm.g;
@@ -476,8 +480,9 @@ __device__ __forceinline__ void grow_run(const GrowArgs& a, GrowSmem& sm, uint32
     Held held;
     // Counter block of the current epoch (one work, up to its closing barrier).  An epoch clears the next one's block,
     // last read two epochs ago: every CTA has passed the barrier that closed the epoch in between.
-    for (uint32_t epoch = 0; sm.work != kWorkLeave && epoch < a.max_epochs; ++epoch) {
+    for (uint32_t epoch = 0; sm.work != kWorkLeave; ++epoch) {
         const uint32_t work = sm.work;
+        const bool last = epoch >= a.max_epochs - 1;
         Counters* ctr = a.ring + epoch % 3;
         if (work == kWorkPush) {
             const uint32_t c = g.cur, o = c ^ 1;
@@ -486,8 +491,8 @@ __device__ __forceinline__ void grow_run(const GrowArgs& a, GrowSmem& sm, uint32
                            a.n, (uint32_t)a.nnz, held);
             barrier();
             const uint32_t nn = min(__ldcg(&ctr->nnext), a.n);
-            // (a launch that ends leaves lists, so its last two epochs hold nothing)
-            const bool light = nn <= nb * (GT / 32) * kHeldNodes && !sm.no_hold && epoch + 2 < a.max_epochs;
+            // (a launch that ends leaves lists)
+            const bool light = nn <= nb * (GT / 32) * kHeldNodes && !sm.no_hold && !last;
             if (light)
                 held = hold_front(a.next, nn, a.key, a.off, g.delta, ctr, sm.push, br, nb, a.keyS, a.n);
             else
@@ -517,7 +522,7 @@ __device__ __forceinline__ void grow_run(const GrowArgs& a, GrowSmem& sm, uint32
         if (br == 0 && threadIdx.x < sizeof(Counters) / 8)
             reinterpret_cast<unsigned long long*>(a.ring + (epoch + 1) % 3)[threadIdx.x] = 0ull;
         barrier();
-        if (threadIdx.x == 0) sm.work = grow_apply(a, sm, work, ctr);
+        if (threadIdx.x == 0) sm.work = grow_apply(a, sm, work, ctr, last);
         __syncthreads();
         held.on = sm.held;
     }

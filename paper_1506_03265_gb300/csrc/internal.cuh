@@ -59,7 +59,9 @@ cldiam_status build_csr(const uint32_t* src, const uint32_t* dst, const uint32_t
 void free_graph(cldiam_graph* g);
 
 cldiam_status delta0(const cldiam_graph* g, int mode, uint32_t explicit_value, uint32_t* out);
-cldiam_status cluster(cldiam_graph* g, double tau, uint64_t seed, const cldiam_opts* o, cldiam_clustering** out);
+// max_phases: phases that one resident launch takes before the host launches the next (0 = the default)
+cldiam_status cluster(cldiam_graph* g, double tau, uint64_t seed, const cldiam_opts* o, cldiam_clustering** out,
+                      uint32_t max_phases = 0);
 cldiam_status cluster2(cldiam_graph* g, double tau, uint64_t seed, const cldiam_opts* o, cldiam_clustering** out);
 // cid[v] = rank of center[v] among the centers; *k = their number (synchronises the graph's stream)
 cldiam_status relabel_clusters(cldiam_graph* g, const uint32_t* center, uint32_t* cid, uint32_t* k);
