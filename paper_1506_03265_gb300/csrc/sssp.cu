@@ -62,6 +62,11 @@ struct DsCounters {
     uint32_t pad;
 };
 
+// Most entries of a resident round's nodes.  The list's node count says little where degrees are skewed: 1,500 hubs of
+// 53,000 entries made a list within its limit, and 16 SMs took 16.2 ms for what the whole device does in 4.9.  (2^18 to
+// 2^21 measured alike; at 2^17 rounds of a ring lattice that the launch does faster leave it, 393 -> 678 ms.)
+constexpr uint32_t kDsEntries = 1u << 19;
+
 // The control state between rounds, kept by the host and by every CTA of k_ds_resident alike.
 struct DsState {
     uint64_t hi;       // end of the current bucket
@@ -72,6 +77,7 @@ struct DsState {
     uint32_t nfar, min;  // its entries and smallest distance
     uint32_t round_id, epoch, rounds;
     uint32_t done, bad;
+    uint32_t wide;     // the next round's nodes hold too many entries for the resident form
 };
 
 struct DsArgs {
@@ -86,6 +92,7 @@ struct DsArgs {
     uint64_t nnz;
     uint32_t n, delta;
     uint32_t max_list, max_far, max_epochs;  // resident rounds: largest list and pile, phases per launch
+    uint32_t max_entries;                    // and the entries of a round's nodes
 };
 
 // A round's node list as a frontier: slot, first position and adjacency base of every node with entries, its distance
@@ -339,9 +346,10 @@ __device__ __forceinline__ uint32_t ds_decide(const DsArgs& a, DsState& g, uint6
     return ds_next_bucket(g, a.delta, lo) ? kDsSplit : kDsLeave;
 }
 
-// Rounds and splits back to back by one thread-block cluster, until one that is too large for it, the phase limit, or the
-// end.  The next work is decided at the head of an iteration, after the limit has been tested: a decision moves the state
-// (a split's bucket), so one that no work followed would leave its bucket out of the next launch.
+// Rounds and splits back to back by one thread-block cluster, until one that is too large for it (by its nodes, or by
+// their entries once they are listed: `wide`, the host then runs that round), the phase limit, or the end.  The next work
+// is decided at the head of an iteration, after the limit has been tested: a decision moves the state (a split's bucket),
+// so one that no work followed would leave its bucket out of the next launch.
 __global__ void __launch_bounds__(GT, 1) k_ds_resident(const DsArgs a, const DsState start) {
     extern __shared__ __align__(16) unsigned char ds_smem[];
     DsSmem& sm = *reinterpret_cast<DsSmem*>(ds_smem);
@@ -360,6 +368,11 @@ __global__ void __launch_bounds__(GT, 1) k_ds_resident(const DsArgs a, const DsS
             ds_list(a, a.list[g.cur], g.ncur, &r->front, sm.scratch, br, nb, &r->bad);
             cluster_barrier();
             fr = __ldcg(&r->front);
+            if ((uint32_t)fr > a.max_entries) {  // (the same at every CTA)
+                if (threadIdx.x == 0) g.wide = 1;
+                __syncthreads();
+                break;
+            }
             ds_push<true>(a, (uint32_t)(fr >> 32), (uint32_t)fr, g.hi, g.round_id, g.epoch, a.list[g.cur ^ 1],
                           &r->next.count, a.far[p], &a.ctr->pile[p], sm.push, br, nb, &a.ctr->overflow, &r->bad);
         } else {
@@ -497,6 +510,7 @@ cldiam_status sssp_delta(cldiam_graph* g, uint32_t source, uint32_t delta, uint3
     // resident rounds: lists of about 2^18 adjacency entries, piles of 2^18 nodes (as CLUSTER's resident steps)
     a.max_list = (uint32_t)std::max<uint64_t>(1, (uint64_t)kGrowEntries / (g->nnz / n + 1));
     a.max_far = kGrowEntries;
+    a.max_entries = kDsEntries;
     a.max_epochs = max_phases ? max_phases : kGrowEpochs;
     const unsigned gb = grid_for(n, 256);
     CLD_K(K_SSSP, s, k_ds_init<<<gb, 256, 0, s>>>(dist.get(), rstamp.get(), fstamp.get(), n, source));
@@ -534,7 +548,7 @@ cldiam_status sssp_delta(cldiam_graph* g, uint32_t source, uint32_t delta, uint3
     const unsigned push_grid = (unsigned)num_sms() * (unsigned)std::max(1, push_per_sm[di].load());
     const int ctas = ds_cluster_size(dev);
     while (!st.done && (st.ncur > 0 || st.nfar > 0)) {
-        const bool small = st.ncur > 0 ? st.ncur <= a.max_list : st.nfar <= a.max_far;
+        const bool small = st.ncur > 0 ? st.ncur <= a.max_list && !st.wide : st.nfar <= a.max_far;
         if (small && ctas && !serving_kernel_alive(dev)) {
             CLD_CUDA(cudaMemsetAsync(ring.get(), 0, 3 * sizeof(DsRound), s));
             cudaLaunchConfig_t cfg{};
@@ -555,6 +569,7 @@ cldiam_status sssp_delta(cldiam_graph* g, uint32_t source, uint32_t delta, uint3
             CLD_LAUNCH_CHECK();
             CLD_TRY(read());
             st.cur ^= 1;
+            st.wide = 0;
             ++st.rounds;
             st.scanned += (uint32_t)hc->r.front;
             // list: 16 B per node (+ its chunk-table share); relax: 8 B (col, w) + 4 B target distance per
