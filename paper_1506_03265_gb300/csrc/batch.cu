@@ -835,7 +835,7 @@ struct cldiam_arena {
     uint64_t budget = 0;
     std::vector<cld::ArenaDesc> graphs;
     std::vector<uint64_t> wsum_upper;
-    std::vector<uint32_t> wmin;
+    std::vector<uint32_t> wmin, max_deg;
     uint64_t* off = nullptr;
     uint2* adj = nullptr;
     uint32_t* row = nullptr;
@@ -928,6 +928,7 @@ cldiam_status arena_add(cldiam_arena* a, const uint32_t* src, const uint32_t* ds
     a->graphs.push_back(dsc);
     a->wsum_upper.push_back(g->wsum_upper);
     a->wmin.push_back(g->wmin);
+    a->max_deg.push_back(g->max_deg);
     a->off_used = need_off;
     a->adj_used = need_adj;
     *id = (uint32_t)(a->graphs.size() - 1);
@@ -948,6 +949,7 @@ static void arena_view(const cldiam_arena* a, uint32_t id, cldiam_graph* g) {
     g->orig = nullptr;
     g->wsum_upper = a->wsum_upper[id];
     g->wmin = a->wmin[id];
+    g->max_deg = a->max_deg[id];
     g->connected = d.connected != 0;
     g->borrowed = true;
 }

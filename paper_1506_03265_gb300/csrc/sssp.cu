@@ -454,13 +454,23 @@ cldiam_status sssp_delta(cldiam_graph* g, uint32_t source, uint32_t delta, uint3
     if (delta == 0) {
         uint32_t d0 = 1;
         CLD_TRY(cld::delta0(g, CLDIAM_DELTA0_AVG, 0, &d0));
-        // Width of a bucket.  A round costs 10 to 30 us, an adjacency entry read 8 ps with the whole device: sparse graphs
-        // (rounds by the hundred) and small ones want wide buckets, large dense ones few repeated reads.  ms at 16 / 8 /
-        // 1 / 0.35 times the average weight: 400^2 mesh 9.0 / 9.7 / 18.1 / 30.4; road mesh 2,000^2 4.4 / 4.7 / 8.8 / 14.2;
-        // R-MAT of 31M entries 1.29 / 1.30 / 1.46 / 1.63, of 128M 6.11 / 6.13 / 6.19 / 7.06, of 166M 4.61 / 4.61 / 4.10 /
-        // 4.18 (0.25: 4.03), of 521M 14.1 / 14.1 / 14.8 / 10.1 (0.25: 10.8).
+        // Width of a bucket, in average weights.  Wide buckets have fewer rounds (10 to 30 us each), narrow ones read fewer
+        // entries twice (8 ps each with the whole device).  Which counts, ms at 0.3 / 1 / 8 / 16:
+        // - sparse graphs take rounds by the hundred: road mesh 3,000^2 21.0 / 11.8 / 6.7 / 6.4, 700^2 mesh 56.9 / 31.5 /
+        //   17.2 / 15.6, a uniform graph of 12.6M entries 2.50 / 1.55 / 1.65 / 1.57;
+        // - denser ones without hubs read everything six times and more at 8: uniform, 12.6M entries 1.20 / 1.08 / 1.52 /
+        //   1.50, 100.7M 2.91 / 3.30 / 7.06 / 7.03; 160^3 grid of 26 neighbours 14.9 / 13.4 / 22.1 / 36.0;
+        // - hubs bring every node within a few hops, at any width about the same reads, so the rounds decide: R-MAT of 1.8M
+        //   entries 0.80 / 0.65 / 0.52 / 0.53, 7.6M 1.45 / 1.15 / 0.96 / 0.96, 31M 2.44 / 2.18 / 2.09 / 2.10, 128M 7.69 /
+        //   7.52 / 7.77 / 7.75;
+        // - above 2^27 entries the reads do: uniform, 201M 4.73 / 6.05 / 14.0 / 14.0; R-MAT, 259M 13.8 / 14.5 / 14.8 / 14.7,
+        //   521M 10.1 / 14.8 / 14.1 / 14.1; 180^3 grid 18.8 / 16.8 / 30.1 / 51.3.
+        // (Hub: eight times the average degree.  Uniform graphs of that degree end at four, R-MAT graphs start at ten.)
         double scale = (double)tuning_for(g->nnz).sssp_delta_scale;
-        if (scale == 1.0) scale = g->nnz < 8ull * n ? 16.0 : g->nnz < (1ull << 27) ? 8.0 : 0.3;
+        if (scale == 1.0) {
+            const bool hub = (uint64_t)g->max_deg * n >= 8ull * g->nnz;
+            scale = g->nnz < 8ull * n ? 16.0 : g->nnz >= (1ull << 27) ? 0.3 : hub && g->nnz < (1ull << 26) ? 8.0 : 1.0;
+        }
         const double scaled = (double)d0 * scale;
         delta = (uint32_t)std::min(std::max(scaled, 1.0), 2147483648.0);
     }
