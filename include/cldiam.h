@@ -379,8 +379,9 @@ typedef struct {
                                       batched SSSP otherwise; 0 = 8                                 */
     uint32_t batch_fw_k;           /* many-graph form: quotients up to this k (<= 200) are closed by
                                       Floyd-Warshall in shared memory; 0 = 200                     */
-    float sssp_delta_scale;        /* Delta-stepping with delta = 0: Delta = this x the average
-                                      weight (> 1); 0 or 1 = by the graph's size and degree        */
+    float sssp_delta_scale;        /* Delta-stepping with delta = 0: Delta = this x the average weight
+                                      (>= 1); 0 = by the graph's size and degrees (0.3 to 16 x), which
+                                      filled-in knobs show as 1                                     */
     uint32_t batch_split;          /* many-graph form: 2 = the largest graphs (each with at least 2^16
                                       entries) run on groups of CTAs, or first on the one-graph path
                                       with the whole device, how many by a time model (one CTA's rate,
@@ -414,7 +415,8 @@ cldiam_status cldiam_tuning_set(const cldiam_tuning* t);
  *  graph: pull_ratio, relax_ctas_per_sm, dense_quotient_k, apsp_sources_per_cta,
  *         apsp_fw_density on cldiam_cluster + cldiam_quotient_build + cldiam_estimate;
  *  batch: batch_split, batch_fw_k on cldiam_batch_run of the listed jobs;
- *  sssp:  sssp_delta_scale on cldiam_sssp_delta(delta = 0) from `source`.
+ *  sssp:  sssp_delta_scale on cldiam_sssp_delta(delta = 0) from `source`; where no candidate beats
+ *         the default rule, the cached field stays 0 (the rule) and *out shows 1.
  */
 cldiam_status cldiam_autotune_graph(cldiam_graph* g, double tau, uint64_t seed, const cldiam_opts* opts,
                                     uint32_t reps, cldiam_tuning* out);

@@ -119,6 +119,9 @@ cldiam_status sssp_delta(cldiam_graph* g, uint32_t source, uint32_t delta, uint3
 cldiam_tuning tuning_current();
 cldiam_tuning tuning_for(uint64_t entries);
 cldiam_tuning tuning_for_batch(uint64_t entries);
+// sssp_delta_scale as set process-wide or cached for such a call, 0 where neither: its default is a rule over the graph,
+// which the filled-in knobs show as 1
+float sssp_delta_scale_set(uint64_t entries);
 uint32_t size_class(uint64_t entries);
 cldiam_tuning tuning_defaults_filled(const cldiam_tuning& t);
 cldiam_status tuning_check(const cldiam_tuning& t);

@@ -466,8 +466,8 @@ cldiam_status sssp_delta(cldiam_graph* g, uint32_t source, uint32_t delta, uint3
         // - above 2^27 entries the reads do: uniform, 201M 4.73 / 6.05 / 14.0 / 14.0; R-MAT, 259M 13.8 / 14.5 / 14.8 / 14.7,
         //   521M 10.1 / 14.8 / 14.1 / 14.1; 180^3 grid 18.8 / 16.8 / 30.1 / 51.3.
         // (Hub: eight times the average degree.  Uniform graphs of that degree end at four, R-MAT graphs start at ten.)
-        double scale = (double)tuning_for(g->nnz).sssp_delta_scale;
-        if (scale == 1.0) {
+        double scale = (double)sssp_delta_scale_set(g->nnz);
+        if (scale == 0.0) {
             const bool hub = (uint64_t)g->max_deg * n >= 8ull * g->nnz;
             scale = g->nnz < 8ull * n ? 16.0 : g->nnz >= (1ull << 27) ? 0.3 : hub && g->nnz < (1ull << 26) ? 8.0 : 1.0;
         }

@@ -141,12 +141,19 @@ uint32_t size_class(uint64_t entries) {
     return c;
 }
 
-cldiam_tuning tuning_effective(int device, uint32_t cls) {
+// the knobs set process-wide or cached, the others 0
+static cldiam_tuning tuning_set_for(int device, uint32_t cls) {
     std::lock_guard<std::mutex> lk(g_tmu);
     cldiam_tuning t = g_tuning;
     const auto it = g_measuring ? g_cache.end() : g_cache.find({device, cls});
     if (it != g_cache.end()) merge_unset(t, it->second);
-    return tuning_defaults_filled(t);
+    return t;
+}
+
+cldiam_tuning tuning_effective(int device, uint32_t cls) { return tuning_defaults_filled(tuning_set_for(device, cls)); }
+
+float sssp_delta_scale_set(uint64_t entries) {
+    return tuning_set_for(current_device(), size_class(entries)).sssp_delta_scale;
 }
 
 cldiam_tuning tuning_for(uint64_t entries) { return tuning_effective(current_device(), size_class(entries)); }
@@ -162,7 +169,8 @@ cldiam_tuning tuning_current() {
 
 namespace {
 
-// Coordinate descent over the knobs in `mask`, from `start` (unset knobs take their defaults).
+// Coordinate descent over the knobs in `mask`, from `start` (unset knobs take their defaults; sssp_delta_scale, whose
+// default is a rule over the graph, stays 0 until a candidate beats the rule).
 cldiam_status search(const cldiam_tuning& start, uint32_t mask, cldiam_tune_measure_fn fn, void* user,
                      cldiam_tuning* best, double* best_seconds) {
     if (!fn || !best) return fail(CLDIAM_ERR_INVALID_ARG, "NULL measure function or best");
@@ -170,6 +178,7 @@ cldiam_status search(const cldiam_tuning& start, uint32_t mask, cldiam_tune_meas
     if (mask == 0 || (mask >> table.size()) != 0) return fail(CLDIAM_ERR_INVALID_ARG, "knob mask out of range");
     CLD_TRY(tuning_check(start));
     cldiam_tuning cur = tuning_defaults_filled(start);
+    cur.sssp_delta_scale = start.sssp_delta_scale;
     double cur_t = 0.0;
     uint64_t ref = 0;
     CLD_TRY(fn(&cur, user, &cur_t, &ref));
@@ -450,7 +459,9 @@ cldiam_status cldiam_autotune_search(const cldiam_tuning* start, uint32_t knob_m
                                      void* user, cldiam_tuning* best, double* best_seconds) {
     cldiam_tuning s0{};
     if (start) s0 = *start;
-    return search(s0, knob_mask, measure, user, best, best_seconds);
+    CLD_TRY(search(s0, knob_mask, measure, user, best, best_seconds));
+    *best = tuning_defaults_filled(*best);
+    return CLDIAM_OK;
 }
 
 cldiam_status cldiam_autotune_graph(cldiam_graph* g, double tau, uint64_t seed, const cldiam_opts* opts,
@@ -460,7 +471,7 @@ cldiam_status cldiam_autotune_graph(cldiam_graph* g, double tau, uint64_t seed, 
     cldiam_tuning best{};
     CLD_TRY(search(start_point(), kGraphKnobs, measure_graph, &w, &best, nullptr));
     cache_put(current_device(), size_class(g->nnz), best, kGraphKnobs);
-    *out = best;
+    *out = tuning_defaults_filled(best);
     return CLDIAM_OK;
 }
 
@@ -478,7 +489,7 @@ cldiam_status cldiam_autotune_batch(cldiam_arena* a, const uint32_t* ids, const 
     cldiam_tuning best{};
     CLD_TRY(search(start_point(), kBatchKnobs, measure_batch, &w, &best, nullptr));
     cache_put(current_device(), 64u + size_class(entries), best, kBatchKnobs);
-    *out = best;
+    *out = tuning_defaults_filled(best);
     return CLDIAM_OK;
 }
 
@@ -489,7 +500,7 @@ cldiam_status cldiam_autotune_sssp(cldiam_graph* g, uint32_t source, uint32_t re
     cldiam_tuning best{};
     CLD_TRY(search(start_point(), kSsspKnobs, measure_sssp, &w, &best, nullptr));
     cache_put(current_device(), size_class(g->nnz), best, kSsspKnobs);
-    *out = best;
+    *out = tuning_defaults_filled(best);
     return CLDIAM_OK;
 }
 
