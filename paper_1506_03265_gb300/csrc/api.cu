@@ -122,6 +122,8 @@ static cldiam_status copy_out_adj(const cldiam_graph* g, uint32_t* col, uint32_t
     return CLDIAM_OK;
 }
 
+cldiam_status load_api_kernels() { return load_kernels(k_split_adj); }
+
 // Run f() and turn a stray C++ exception into a status (none may cross the ABI).
 template <class F>
 static cldiam_status guarded(F&& f) {

@@ -1512,8 +1512,10 @@ cldiam_status server_create(cldiam_arena* a, const cldiam_server_opts* o, cldiam
     sv->big_graph.resize(sv->cap);
     sv->big_tau.resize(sv->cap);
     sv->big_seed.resize(sv->cap);
-    for (auto load : {load_prims_kernels, load_csr_kernels, load_cluster_kernels, load_quotient_kernels, load_apsp_kernels})
+    for (auto load : {load_prims_kernels, load_csr_kernels, load_cluster_kernels, load_cluster2_kernels,
+                      load_quotient_kernels, load_apsp_kernels, load_sssp_kernels, load_api_kernels})
         if ((st = load()) != CLDIAM_OK) return cleanup(st);
+    if ((st = load_kernels(k_batch<false>)) != CLDIAM_OK) return cleanup(st);
     {
         std::lock_guard<std::mutex> lk(sv->mu);
         if (sv->device >= 0 && sv->device < 64) {

@@ -422,9 +422,12 @@ cldiam_status cluster(cldiam_graph* g, double tau, uint64_t seed, const cldiam_o
         (unsigned)std::min<uint64_t>((uint64_t)num_sms() * pull_ctas, (pull_chunks + PT / 32 - 1) / (PT / 32));
     DBuf<uint32_t> rows_built;  // COO rows for the guard's edge scan when the graph keeps none
 
-    // Resident growth (k_grow): on connected graphs, while no server's kernel holds the SMs, unless a tuning knob asks for the grid kernels (a set number of
-    // CTAs) or for the dense form at a share of the adjacency that the step reaches (a share other than the default).
-    const int grow_ctas = g->connected && n >= 2 && g->nnz < 0xFFFFFFFFull && tun.relax_ctas_per_sm == 0 ? grow_cluster_size(dev) : 0;
+    // Resident growth (k_grow): on connected graphs, while no server is alive on the device, unless a tuning knob asks for
+    // the grid kernels (a set number of CTAs) or for the dense form at a share of the adjacency that the step reaches (a
+    // share other than the default).
+    // (its kernel is not touched beside a server, which would load it and wait)
+    const bool resident = g->connected && n >= 2 && g->nnz < 0xFFFFFFFFull && tun.relax_ctas_per_sm == 0;
+    const int grow_ctas = resident && !serving_kernel_alive(dev) ? grow_cluster_size(dev) : 0;
     const bool strict_pull = pull_dense && tun.pull_ratio != tuning_defaults_filled(cldiam_tuning{}).pull_ratio;
     const uint32_t grow_entries =
         strict_pull ? (uint32_t)std::min<double>(kGrowEntries, std::max(0.0, std::ceil((double)tun.pull_ratio * (double)g->nnz) - 1))

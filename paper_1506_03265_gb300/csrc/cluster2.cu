@@ -395,4 +395,8 @@ cldiam_status cluster2(cldiam_graph* g, double tau, uint64_t seed, const cldiam_
     return CLDIAM_OK;
 }
 
+cldiam_status load_cluster2_kernels() {
+    return load_kernels(k_c2_fill, k_c2_select, k_c2_list<false>, k_c2_list<true>, k_c2_push, k_c2_finalize, k_c2_distances);
+}
+
 }  // namespace cld

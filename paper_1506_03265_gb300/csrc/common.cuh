@@ -102,9 +102,9 @@ inline unsigned grid_for(size_t n, int block, int max_blocks_per_sm = 8) {
 }
 
 // ---------------------------------------------------------------- kernel loading
-// The runtime loads a kernel's code at its first use, and that load waits for the kernels already running: beside a
-// server's persistent kernel, for as long as it lives.  A server therefore has every kernel of the one-graph path loaded
-// before its own is launched (asking for a kernel's attributes loads it).
+// The runtime loads a kernel's code at its first use (a launch, or asking for or setting its attributes), and that load
+// waits for the kernels already running: beside a server's persistent kernel, for as long as it lives.  A server
+// therefore has every kernel that a call beside it may launch loaded before its own is launched.
 template <class... K>
 cldiam_status load_kernels(K... k) {
     cudaFuncAttributes a;
@@ -114,10 +114,13 @@ cldiam_status load_kernels(K... k) {
     return CLDIAM_OK;
 }
 cldiam_status load_prims_kernels();     // sorts, scans, reductions
+cldiam_status load_csr_kernels();
 cldiam_status load_cluster_kernels();
+cldiam_status load_cluster2_kernels();
 cldiam_status load_quotient_kernels();
 cldiam_status load_apsp_kernels();
-cldiam_status load_csr_kernels();       // the row array of a graph without one
+cldiam_status load_sssp_kernels();
+cldiam_status load_api_kernels();       // the graph copy
 
 // ---------------------------------------------------------------- Philox4x32-10
 // Salmon, Moraes, Dror, Shaw, "Parallel random numbers: as easy as 1, 2, 3"

@@ -841,7 +841,10 @@ cldiam_status delta0(const cldiam_graph* g, int mode, uint32_t explicit_value, u
 }
 
 cldiam_status load_csr_kernels() {
-    return load_kernels(k_fill_rows);
+    return load_kernels(k_emit_canon<false>, k_emit_canon<true>, k_canon_runs, k_canon_deg, k_iota, k_canon_scatter,
+                        k_cc_link_nth, k_cc_link_rest, k_cc_sample, k_cc_compress, k_cc_size_of, k_cc_giant_best,
+                        k_cc_count, k_cc_best, k_cc_keep, k_lcc_degrees, k_lcc_offsets_lists, k_lcc_assemble<false>,
+                        k_lcc_assemble<true>, k_graph_stats, k_degree_max, k_fill_rows);
 }
 
 }  // namespace cld

@@ -1109,14 +1109,21 @@ cldiam_status radix_sort_pairs_u32(uint32_t* keys, uint32_t* vals, uint32_t* key
     return radix_sort_impl<uint32_t>(keys, vals, keys_alt, vals_alt, n, 0, bits, in_alt, s);
 }
 
+// (a sort sets the attributes of both digit forms, so the 32-bit keys' unused one is loaded too)
+template <class K, bool KV>
+static cldiam_status load_sort_kernels() {
+    return load_kernels(k_os_pass<K, KV, false, false>, k_os_pass<K, KV, true, false>, k_os_pass<K, KV, false, true>,
+                        k_os_pass<K, KV, true, true>);
+}
 cldiam_status load_prims_kernels() {
+    CLD_TRY((load_sort_kernels<uint32_t, true>()));
+    CLD_TRY((load_sort_kernels<uint64_t, true>()));
+    CLD_TRY((load_sort_kernels<uint64_t, false>()));
     return load_kernels(k_tile_reduce<uint32_t>, k_tile_scan<uint32_t>, k_tile_reduce<uint64_t>, k_tile_scan<uint64_t>,
-                        k_offsets_from_rows, k_reduce_max_u32, k_reduce_min_u32, k_reduce_sum_u32, k_os_hist<uint32_t>,
-                        k_os_hist<uint64_t>, k_os_hist_scan, k_os_pass<uint32_t, true, false, false>,
-                        k_os_pass<uint64_t, true, false, false>, k_os_pass<uint64_t, true, true, false>,
-                        k_os_pass<uint32_t, true, false, true>, k_os_pass<uint64_t, true, false, true>,
-                        k_os_pass<uint64_t, true, true, true>, k_unique_count<uint32_t>,
-                        k_unique_count<uint64_t>, k_unique_write<uint32_t, false>, k_unique_write<uint64_t, false>);
+                        k_reduce_max_u32, k_os_hist<uint32_t>, k_os_hist<uint64_t>, k_os_hist_scan,
+                        k_unique_count<uint32_t>, k_unique_count<uint64_t>, k_unique_write<uint32_t, false>,
+                        k_unique_write<uint64_t, false>, k_unique_write<uint64_t, true>, k_unique_packed_count,
+                        k_unique_items, k_last_uend);
 }
 
 }  // namespace cld

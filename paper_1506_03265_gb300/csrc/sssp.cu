@@ -556,7 +556,7 @@ cldiam_status sssp_delta(cldiam_graph* g, uint32_t source, uint32_t delta, uint3
         push_per_sm[di] = std::max(1, b);
     }
     const unsigned push_grid = (unsigned)num_sms() * (unsigned)std::max(1, push_per_sm[di].load());
-    const int ctas = ds_cluster_size(dev);
+    const int ctas = serving_kernel_alive(dev) ? 0 : ds_cluster_size(dev);  // (beside a server the query would load the kernel and wait)
     while (!st.done && (st.ncur > 0 || st.nfar > 0)) {
         const bool small = st.ncur > 0 ? st.ncur <= a.max_list && !st.wide : st.nfar <= a.max_far;
         if (small && ctas && !serving_kernel_alive(dev)) {
@@ -614,6 +614,10 @@ cldiam_status sssp_delta(cldiam_graph* g, uint32_t source, uint32_t delta, uint3
     if (rounds_out) *rounds_out = st.rounds;
     if (scanned_out) *scanned_out = st.scanned;
     return CLDIAM_OK;
+}
+
+cldiam_status load_sssp_kernels() {
+    return load_kernels(k_ds_init, k_ds_list, k_ds_push, k_ds_split, k_ds_overflow, k_ds_ecc);
 }
 
 }  // namespace cld
