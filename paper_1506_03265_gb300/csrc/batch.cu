@@ -850,6 +850,14 @@ struct cldiam_arena {
 
 namespace cld {
 
+// the workspaces are a cache for the next batch: given back where their bytes stand in the way of a budget
+static void release_workspaces(cldiam_arena* a) {
+    dfree(a->ws, a->stream);
+    dfree(a->gws, a->stream);
+    a->ws = a->gws = nullptr;
+    a->ws_bytes = a->gws_bytes = 0;
+}
+
 static uint64_t arena_bytes(const cldiam_arena* a) { return a->off_cap * 8 + a->adj_cap * 12 + a->ws_bytes + a->gws_bytes; }
 
 // grow a device array to hold `need` elements (doubling), keeping the first `used`
@@ -881,8 +889,7 @@ void arena_free(cldiam_arena* a) {
     dfree(a->off, a->stream);
     dfree(a->adj, a->stream);
     dfree(a->row, a->stream);
-    dfree(a->ws, a->stream);
-    dfree(a->gws, a->stream);
+    release_workspaces(a);
     cudaStreamSynchronize(a->stream);
     if (a->aux) cudaStreamDestroy(a->aux);
     delete a;
@@ -900,6 +907,7 @@ cldiam_status arena_add(cldiam_arena* a, const uint32_t* src, const uint32_t* ds
     const uint64_t need_off = a->off_used + g->n + 1, need_adj = a->adj_used + g->nnz;
     const uint64_t extra = (need_off > a->off_cap ? (need_off - a->off_cap) * 8 : 0) +
                            (need_adj > a->adj_cap ? (need_adj - a->adj_cap) * 12 : 0);
+    if (a->budget && arena_bytes(a) + extra > a->budget) release_workspaces(a);
     if (a->budget && arena_bytes(a) + extra > a->budget)
         return fail(CLDIAM_ERR_OOM, "graph does not fit the arena's device memory budget");
     CLD_TRY(grow(&a->off, &a->off_cap, a->off_used, need_off, a->stream));
@@ -1230,7 +1238,8 @@ cldiam_status batch_run(cldiam_arena* a, const uint32_t* ids, const double* tau,
         if (ngrp > 0 && workspaces(nbig, nbig + ngrp, groups, &a->gws, &a->gws_bytes, &gwsh) != CLDIAM_OK)
             ngrp = 0;  // no memory for the groups' workspaces: every job on one CTA
         const uint32_t nones = nrest - ngrp;  // jobs on one CTA each
-        CLD_TRY(workspaces(nbig + ngrp, count, nsm, &a->ws, &a->ws_bytes, &wsh));
+        const uint32_t one_ctas = std::min<uint32_t>(nsm, nones);
+        if (nones > 0) CLD_TRY(workspaces(nbig + ngrp, count, (int)one_ctas, &a->ws, &a->ws_bytes, &wsh));
         if (ngrp > 0) wsh.insert(wsh.end(), gwsh.begin(), gwsh.end());
         DBuf<ArenaDesc> ddesc;
         DBuf<Job> djobs;
@@ -1270,11 +1279,11 @@ cldiam_status batch_run(cldiam_arena* a, const uint32_t* ids, const double* tau,
             const uint2* adj = a->adj;
             const uint32_t* row = a->row;
             CLD_K(K_MISC, s, CLD_CUDA(cudaLaunchKernelEx(&cfg, k_batch<true>, (const ArenaDesc*)ddesc.get(),
-                                                         (const Job*)djobs.get(), ngrp, off, adj, row, dws.get() + nsm,
-                                                         queue.get() + 1, douts.get())));
+                                                         (const Job*)djobs.get(), ngrp, off, adj, row,
+                                                         dws.get() + one_ctas, queue.get() + 1, douts.get())));
         }
         if (nones > 0) {
-            CLD_K(K_MISC, ones, k_batch<false><<<std::min<uint32_t>(nsm, nones), BT, dyn, ones>>>(
+            CLD_K(K_MISC, ones, k_batch<false><<<one_ctas, BT, dyn, ones>>>(
                                     ddesc.get(), djobs.get() + ngrp, nones, a->off, a->adj, a->row, dws.get(), queue.get(),
                                     douts.get()));
             CLD_LAUNCH_CHECK();
@@ -1496,6 +1505,7 @@ cldiam_status server_create(cldiam_arena* a, const cldiam_server_opts* o, cldiam
     std::vector<Workspace> wsh;
     if ((st = make_workspaces(nmax, zmax, (int)sv->ctas, sv->kstream, &sv->ws, &sv->ws_bytes, &wsh)) != CLDIAM_OK)
         return cleanup(st);
+    if (sv->budget) release_workspaces(a);
     if (sv->budget && arena_bytes(a) + sv->ws_bytes > sv->budget)
         return cleanup(fail(CLDIAM_ERR_OOM, "arena plus serving workspace exceed the budget"));
     if ((st = dmalloc((void**)&sv->head, 4, sv->kstream)) != CLDIAM_OK ||
