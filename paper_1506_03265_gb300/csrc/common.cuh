@@ -354,10 +354,8 @@ __device__ __forceinline__ void red_min_keep_u64(unsigned long long* p, unsigned
 // Exclusive prefix sum of n values; *total (device pointer, may be null) gets the sum.
 cldiam_status scan_exclusive_u32(const uint32_t* in, uint32_t* out, size_t n, uint32_t* total, cudaStream_t s);
 cldiam_status scan_exclusive_u64(const uint64_t* in, uint64_t* out, size_t n, uint64_t* total, cudaStream_t s);
-// Max / sum reductions into a device scalar (which the call initialises).
+// Maximum into a device scalar (which the call initialises).
 cldiam_status reduce_max_u32(const uint32_t* in, size_t n, uint32_t* out, cudaStream_t s);
-cldiam_status reduce_sum_u32_to_u64(const uint32_t* in, size_t n, uint64_t* out, cudaStream_t s);
-cldiam_status reduce_min_u32(const uint32_t* in, size_t n, uint32_t* out, cudaStream_t s);
 
 // Stable LSD radix sort of (key, value) pairs on the low `bits` bits of the
 // key.  Buffers *_alt are scratch of the same size; on return *result_in_alt
@@ -398,10 +396,6 @@ cldiam_status unique_min_sorted_u32(const uint32_t* keys, const uint32_t* vals, 
 cldiam_status unique_items_u64(const uint64_t* items, const uint32_t* vals, size_t cnt, int vb, uint64_t* out,
                                uint32_t* w_out, uint32_t* total_dev, cudaStream_t s, uint32_t* hist2, uint32_t* ustart,
                                uint32_t* uend);
-
-// CSR offsets off[0..n] of entries whose (sorted) row ids are row[0..nnz):
-// off[u] = index of the first entry with row >= u.  No atomics, no scan.
-cldiam_status offsets_from_rows(const uint32_t* row, uint64_t nnz, uint32_t n, uint64_t* off, cudaStream_t s);
 
 inline int bits_for(uint64_t max_value) {  // bits needed to represent values <= max_value
     int b = 0;

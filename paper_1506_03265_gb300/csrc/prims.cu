@@ -200,25 +200,6 @@ cldiam_status scan_exclusive_u64(const uint64_t* in, uint64_t* out, size_t n, ui
     return scan_exclusive<uint64_t>(in, out, n, total, s);
 }
 
-// ------------------------------------------------------------------ offsets from sorted rows
-__global__ void k_offsets_from_rows(const uint32_t* __restrict__ row, uint64_t nnz, uint32_t n,
-                                    uint64_t* __restrict__ off) {
-    for (uint64_t r = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; r <= nnz; r += (uint64_t)gridDim.x * blockDim.x) {
-        // entry r opens rows row[r-1]+1 .. row[r] (all rows up to row[0] when r = 0); position nnz
-        // closes rows row[nnz-1]+1 .. n
-        if (r > 0 && r < nnz && row[r] == row[r - 1]) continue;
-        const uint64_t lo = (r == 0) ? 0 : (uint64_t)row[r - 1] + 1;
-        const uint64_t hi = (r == nnz) ? n : (uint64_t)row[r];
-        for (uint64_t x = lo; x <= hi; ++x) off[x] = r;
-    }
-}
-
-cldiam_status offsets_from_rows(const uint32_t* row, uint64_t nnz, uint32_t n, uint64_t* off, cudaStream_t s) {
-    CLD_K(K_CSR, s, k_offsets_from_rows<<<grid_for(nnz + 1, 256), 256, 0, s>>>(row, nnz, n, off));
-    CLD_LAUNCH_CHECK();
-    return CLDIAM_OK;
-}
-
 // ------------------------------------------------------------------ reductions
 __global__ void k_reduce_max_u32(const uint32_t* __restrict__ in, size_t n, uint32_t* out) {
     uint32_t m = 0;
@@ -227,39 +208,11 @@ __global__ void k_reduce_max_u32(const uint32_t* __restrict__ in, size_t n, uint
     m = block_reduce(m, [](uint32_t a, uint32_t b) { return a > b ? a : b; }, 0u);
     if (threadIdx.x == 0) atomicMax(out, m);
 }
-__global__ void k_reduce_min_u32(const uint32_t* __restrict__ in, size_t n, uint32_t* out) {
-    uint32_t m = 0xFFFFFFFFu;
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-        m = min(m, in[i]);
-    m = block_reduce(m, [](uint32_t a, uint32_t b) { return a < b ? a : b; }, 0xFFFFFFFFu);
-    if (threadIdx.x == 0) atomicMin(out, m);
-}
-__global__ void k_reduce_sum_u32(const uint32_t* __restrict__ in, size_t n, unsigned long long* out) {
-    unsigned long long m = 0;
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-        m += in[i];
-    m = block_reduce(m, [](unsigned long long a, unsigned long long b) { return a + b; }, 0ull);
-    if (threadIdx.x == 0) atomicAdd(out, m);
-}
 
 cldiam_status reduce_max_u32(const uint32_t* in, size_t n, uint32_t* out, cudaStream_t s) {
     CLD_CUDA(cudaMemsetAsync(out, 0, sizeof(uint32_t), s));
     if (n == 0) return CLDIAM_OK;
     CLD_K(K_REDUCE, s, k_reduce_max_u32<<<grid_for(n, 256, 4), 256, 0, s>>>(in, n, out));
-    CLD_LAUNCH_CHECK();
-    return CLDIAM_OK;
-}
-cldiam_status reduce_min_u32(const uint32_t* in, size_t n, uint32_t* out, cudaStream_t s) {
-    CLD_CUDA(cudaMemsetAsync(out, 0xFF, sizeof(uint32_t), s));
-    if (n == 0) return CLDIAM_OK;
-    CLD_K(K_REDUCE, s, k_reduce_min_u32<<<grid_for(n, 256, 4), 256, 0, s>>>(in, n, out));
-    CLD_LAUNCH_CHECK();
-    return CLDIAM_OK;
-}
-cldiam_status reduce_sum_u32_to_u64(const uint32_t* in, size_t n, uint64_t* out, cudaStream_t s) {
-    CLD_CUDA(cudaMemsetAsync(out, 0, sizeof(uint64_t), s));
-    if (n == 0) return CLDIAM_OK;
-    CLD_K(K_REDUCE, s, k_reduce_sum_u32<<<grid_for(n, 256, 4), 256, 0, s>>>(in, n, reinterpret_cast<unsigned long long*>(out)));
     CLD_LAUNCH_CHECK();
     return CLDIAM_OK;
 }
