@@ -482,7 +482,6 @@ __device__ __forceinline__ void grow_run(const GrowArgs& a, GrowSmem& sm, uint32
     // last read two epochs ago: every CTA has passed the barrier that closed the epoch in between.
     for (uint32_t epoch = 0; sm.work != kWorkLeave; ++epoch) {
         const uint32_t work = sm.work;
-        const bool last = epoch >= a.max_epochs - 1;
         Counters* ctr = a.ring + epoch % 3;
         if (work == kWorkPush) {
             const uint32_t c = g.cur, o = c ^ 1;
@@ -492,7 +491,7 @@ __device__ __forceinline__ void grow_run(const GrowArgs& a, GrowSmem& sm, uint32
             barrier();
             const uint32_t nn = min(__ldcg(&ctr->nnext), a.n);
             // (a launch that ends leaves lists)
-            const bool light = nn <= nb * (GT / 32) * kHeldNodes && !sm.no_hold && !last;
+            const bool light = nn <= nb * (GT / 32) * kHeldNodes && !sm.no_hold && epoch + 1 < a.max_epochs;
             if (light)
                 held = hold_front(a.next, nn, a.key, a.off, g.delta, ctr, sm.push, br, nb, a.keyS, a.n);
             else
@@ -522,7 +521,7 @@ __device__ __forceinline__ void grow_run(const GrowArgs& a, GrowSmem& sm, uint32
         if (br == 0 && threadIdx.x < sizeof(Counters) / 8)
             reinterpret_cast<unsigned long long*>(a.ring + (epoch + 1) % 3)[threadIdx.x] = 0ull;
         barrier();
-        if (threadIdx.x == 0) sm.work = grow_apply(a, sm, work, ctr, last);
+        if (threadIdx.x == 0) sm.work = grow_apply(a, sm, work, ctr, epoch + 1 >= a.max_epochs);
         __syncthreads();
         held.on = sm.held;
     }
