@@ -273,9 +273,9 @@ def batched_leg(cd, stream, mix, sample_every, reps=3, dist=None, total_count=No
                  "makespan_ms": round(1e3 * float(je.max()), 3),
                  "balanced_ms": round(1e3 * float(jt.sum()) / ctas, 3),
                  "last_job_start_ms": round(1e3 * float(js.max()), 3),
-                 "what": ("device time per job (one CTA each: no graph of this batch outweighs the per-CTA average); "
-                          f"balanced_ms = the sum of job times over the {ctas} CTAs, the makespan a perfect split "
-                          "would give")}
+                 "what": ("device time per job (on one CTA, or on a group of CTAs where it would outlast the others); "
+                          f"balanced_ms = the sum of job times (a group's counted once) over the {ctas} CTAs, about the "
+                          "makespan a perfect split would give")}
     # a small batch (the first 50 jobs) is bound by its largest job: one CTA per job vs CTA groups
     small = {}
     sids, staus, sseeds = ids[:50], taus[:50], seeds[:50]
@@ -297,8 +297,8 @@ def batched_leg(cd, stream, mix, sample_every, reps=3, dist=None, total_count=No
     small_same = small.pop("results")
     small["identical_across_forms"] = bool(small_same[0] == small_same[1])
     small["what"] = ("the mixture's first 50 jobs: batch_split = 1 (every graph in the persistent launch, one CTA "
-                     "each) vs 2, the default (a graph that outweighs the per-CTA average runs first on the "
-                     "one-graph path with the whole device)")
+                     "each) vs 2, the default (graphs that would outlast the others on groups of CTAs beside them, or "
+                     "first on the one-graph path with the whole device)")
     # autotuned: the many-graph knobs picked on these jobs (cached for the batch's size class), then timed
     tuned = arena.autotune(ids, taus, seeds, reps=2)
     torch.cuda.synchronize()

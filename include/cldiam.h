@@ -301,7 +301,8 @@ cldiam_status cldiam_run(const uint32_t* src, const uint32_t* dst, const uint32_
  * same graph, tau and seed with the same options.
  */
 /* Empty arena on `stream`; hbm_budget_bytes (0 = unlimited) caps the device memory it may hold
- * (graphs plus the batch workspace); an add that would exceed it fails with OOM. */
+ * (graphs plus the batch workspace); an add that would exceed it releases the workspace of the
+ * last batch, and fails with OOM if that is not enough. */
 cldiam_status cldiam_arena_create(uint64_t hbm_budget_bytes, void* stream, cldiam_arena** out);
 /* Build one graph's CSR (as cldiam_build_csr with `flags`) and append it; *graph_id is its index. */
 cldiam_status cldiam_arena_add(cldiam_arena* a, const uint32_t* src, const uint32_t* dst, const uint32_t* w,
@@ -369,12 +370,16 @@ typedef struct {
     float pull_ratio;              /* a growing step takes the dense pull form (every node reads its
                                       own adjacency) when its relaxers' adjacency is at least this share
                                       of all adjacency entries; < 0 = never; 0 = 0.3                */
-    uint32_t relax_ctas_per_sm;    /* CTAs per SM of the growing-step kernels; 0 = all that fit     */
+    uint32_t relax_ctas_per_sm;    /* CTAs per SM of the growing-step kernels; 0 = all that fit, and
+                                      small steps back to back in one launch (a set number keeps every
+                                      step on the grid kernels: a mesh grows at half the speed)     */
     uint32_t dense_quotient_k;     /* CLDIAM_QUOTIENT_AUTO: dense k x k de-duplication up to this k
                                       (<= 65535), above it (if >= 4096) while k^2 <= nnz, then by
                                       radix sort; 0 = 4096                                          */
-    uint32_t apsp_sources_per_cta; /* quotient diameter by batched SSSP: sources per CTA, 1, 4 or 8;
-                                      0 = by k (8 below 2,048 nodes, else 4)                       */
+    uint32_t apsp_sources_per_cta; /* quotient diameter by batched SSSP from every node: sources per
+                                      CTA, 1, 4 or 8; 0 = from the few nodes that eccentricity bounds
+                                      leave, and where these do not serve from every node, 8 per CTA
+                                      below 2,048 nodes, else 4                                     */
     uint32_t apsp_fw_density;      /* quotient diameter by Floyd-Warshall when nnz >= k^2 / this,
                                       batched SSSP otherwise; 0 = 8                                 */
     uint32_t batch_fw_k;           /* many-graph form: quotients up to this k (<= 200) are closed by

@@ -1448,6 +1448,8 @@ cldiam_status server_free(cldiam_server* sv);
 
 // Servers alive on each device: a server's persistent kernel holds its SMs until it has been idle for long, and the
 // few SMs it leaves need not include a cluster's worth in one GPC, so thread-block clusters are not launched beside it.
+// A server counts until it is freed, also while its kernel is gone: the next request launches it again, possibly before
+// a cluster that was launched in between is running, which would then wait for the whole idle limit.
 static std::atomic<int> g_live_servers[64];
 bool serving_kernel_alive(int dev) { return dev < 0 || dev >= 64 || g_live_servers[dev].load() > 0; }
 

@@ -353,7 +353,7 @@ __global__ void k_lcc_offsets_lists(const uint32_t* __restrict__ excl, const uin
 
 // The LCC's CSR straight from the two orders of the distinct edges: an edge (a, b) of the kept component
 // goes to row newid[a] after its lower entries (from U) and to row newid[b] (from T); new ids are
-// monotone, so rows stay sorted.  Weight statistics as k_lcc_copy (each undirected edge once: from U).
+// monotone, so rows stay sorted.  Weight statistics count each undirected edge once, from U.
 // A position past the output (inconsistent input) is recorded in *err and the write skipped.  The row's
 // own record (info, 16 B) is read in runs (U is sorted on a, T on b); the far end's new id comes from
 // the 4-byte newid array (evict-last: it stays in L2 while the two edge lists stream through, evict-first).
