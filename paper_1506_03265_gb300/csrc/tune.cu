@@ -333,15 +333,12 @@ cldiam_status measure_sssp(const cldiam_tuning* t, void* user, double* seconds, 
 }
 
 void cache_put(int device, uint32_t cls, const cldiam_tuning& t, uint32_t mask) {
-    // only the searched knobs are cached; the others stay unset (0) so they keep their own source
-    cldiam_tuning c{};
-    for (size_t i = 0; i < knob_table().size(); ++i)
-        if (mask & (1u << i)) knob_set(c, i, knob_get(t, i));
+    // only the searched knobs are cached; the others keep what the entry holds (a searched knob whose best is 0, the
+    // default, takes an earlier choice's place too)
     std::lock_guard<std::mutex> lk(g_tmu);
-    auto& slot = g_cache[{device, cls}];
-    cldiam_tuning merged = c;
-    merge_unset(merged, slot);
-    slot = merged;
+    cldiam_tuning& slot = g_cache[{device, cls}];
+    for (size_t i = 0; i < knob_table().size(); ++i)
+        if (mask & (1u << i)) knob_set(slot, i, knob_get(t, i));
 }
 
 constexpr uint32_t kGraphKnobs = (1u << 0) | (1u << 1) | (1u << 2) | (1u << 3) | (1u << 4);

@@ -53,3 +53,18 @@ def test_widths_in_effect():
     best = cd.autotune_sssp(g, 0, reps=2)
     cached = cd.tuning_cache_get(0, cd.size_class(g.nnz))["sssp_delta_scale"]
     assert best["sssp_delta_scale"] == (cached or 1.0) and cd.sssp_delta(g, 0)[2] == want[int(cached) or 16]
+
+
+@pytest.mark.gpu
+def test_tuning_again_replaces_an_earlier_choice():
+    # a tree of small weights: the rule's wide buckets beat every candidate of up to eight average weights
+    n = 1 << 17
+    v = np.arange(1, n, dtype=np.uint32)
+    g = cd.build_csr((v - 1) // 2, v, np.random.default_rng(2).integers(1, 1 << 20, n - 1).astype(np.uint32), n)
+    cls = cd.size_class(g.nnz)
+    cd.tuning_cache_put(0, cls, sssp_delta_scale=2, apsp_fw_density=16)
+    rounds = cd.sssp_delta(g, 0)[2]
+    assert cd.autotune_sssp(g, 0)["sssp_delta_scale"] == 1.0
+    cached = cd.tuning_cache_get(0, cls)
+    assert cached["sssp_delta_scale"] == 0 and cached["apsp_fw_density"] == 16
+    assert cd.sssp_delta(g, 0)[2] < rounds
